@@ -19,10 +19,10 @@
 namespace dpara {
 
 struct AppendParams {
-  const uint16_t *kv;       // [b * J][2 * Hkv * D] bf16: [keys | values] of every candidate row (n_parts == 0)
+  const uint16_t *kv;       // n_parts == 0: layer g of the launch: [b * J][2 * Hkv * D] bf16, [keys | values] of every candidate row, from kv + g * part_stride
   const float *kv_parts;    // layer g of the launch: [n_parts][b * J][2 * Hkv * D] fp32 partial sums from kv_parts + g * n_parts * part_stride
   int n_parts;
-  size_t part_stride;       // elements between two parts
+  size_t part_stride;       // elements between two parts (two layers' rows)
   // per layer of the launch (blockIdx.y)
   const uint16_t *knorm_w[kGemmMaxGroups];  // [D] or null
   uint16_t *k_cache[kGemmMaxGroups], *v_cache[kGemmMaxGroups];
@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
   pdl_wait();
   pdl_launch_dependents();
   const uint16_t *knorm_w = P.knorm_w[g];
+  const uint16_t *kv = P.kv + (size_t)g * P.part_stride;
   const float *kv_parts = P.kv_parts + (size_t)g * P.n_parts * P.part_stride;
   const int r = P.accept_len[n];
   const long long L = P.ctx_len[n];
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
   const size_t src_off = (size_t)blockIdx.x * 2 * P.Hkv * P.D;
   // element `e` of this candidate row as the bf16 value the projection stores (split K: the rounded sum of the parts)
   auto kv_at = [&](size_t e) -> float {
-    if (P.n_parts == 0) return bf16_bits_to_float(P.kv[src_off + e]);
+    if (P.n_parts == 0) return bf16_bits_to_float(kv[src_off + e]);
     float acc = 0.f;
     for (int s = 0; s < P.n_parts; ++s) acc += __ldg(kv_parts + (size_t)s * P.part_stride + src_off + e);
     return __bfloat162float(__float2bfloat16_rn(acc));
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
   const size_t vs = (size_t)P.Hkv * P.D;
   uint16_t *vd = P.v_cache[g] + row * P.Hkv * P.D;
   if (P.n_parts == 0) {
-    for (int c = tid * 8; c < P.Hkv * P.D; c += 128 * 8) *reinterpret_cast<uint4 *>(vd + c) = *reinterpret_cast<const uint4 *>(P.kv + src_off + vs + c);
+    for (int c = tid * 8; c < P.Hkv * P.D; c += 128 * 8) *reinterpret_cast<uint4 *>(vd + c) = *reinterpret_cast<const uint4 *>(kv + src_off + vs + c);
   } else {
     for (int c = tid * 4; c < P.Hkv * P.D; c += 128 * 4) {
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -130,15 +131,14 @@ __global__ void append_commit_kernel(int64_t *ctx_len, const int64_t *capacity, 
   }
 }
 
-// Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: one product per layer with
-// a bf16 store (at most 128 rows: single CTAs, neither grouped nor split).  The parts are chosen to minimise
+// Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores (at most 128 rows: the
+// kernel for few rows splits K inside its clusters.  8 rows, five layers of 2048 x 4096: 29 us a layer one by one -> ~20 us together).  The parts are chosen to minimise
 // rounds x (K slabs per part + ~8 slabs' worth of fixed cost per work unit) over the CTA pairs.
 static void cache_group_plan(const dpara_cache_io *io, int layers_left, int *group, int *parts) {
   const int M = io->batch * io->n_rows, N = 2 * io->n_kv_heads * io->head_dim;
-  *group = 1;
+  *group = layers_left < kGemmMaxGroups ? layers_left : kGemmMaxGroups;
   *parts = 0;
   if (M <= 128) return;
-  *group = layers_left < kGemmMaxGroups ? layers_left : kGemmMaxGroups;
   const int tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = kNumSM / 2, nkb = io->feat_dim / 64;
   int best = 1;
   long best_cost = -1;
@@ -163,7 +163,7 @@ size_t cache_append_workspace_bytes(const dpara_cache_io *io) {
   const size_t M = (size_t)io->batch * io->n_rows, N = (size_t)2 * io->n_kv_heads * io->head_dim;
   int group, parts;
   cache_group_plan(io, io->n_layers, &group, &parts);
-  if (!parts) return align_up(M * io->feat_dim * 2, 256) + align_up(M * N * 2, 256);
+  if (!parts) return (size_t)cache_norm_slots(io) * align_up(M * io->feat_dim * 2, 256) + align_up((size_t)group * M * N * 2, 256);
   // planes of partial sums: the first launch has the most layers, the last (smaller) one may cut K in more parts --
   // sized for the larger of the two
   size_t planes = (size_t)group * parts;
@@ -181,7 +181,7 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
   const size_t xn_bytes = align_up((size_t)M * F * 2, 256);
   int group0, parts0;
   cache_group_plan(io, io->n_layers, &group0, &parts0);
-  const int slots = parts0 ? cache_norm_slots(io) : 1;
+  const int slots = cache_norm_slots(io);
   uint8_t *ws = static_cast<uint8_t *>(workspace);
   uint16_t *kv = reinterpret_cast<uint16_t *>(ws + (size_t)slots * xn_bytes);
   AppendParams P;
@@ -198,17 +198,17 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
     int group, parts;
     cache_group_plan(io, io->n_layers - l0, &group, &parts);
     GemmArgs g{};
-    g.M = M; g.N = N; g.K = F; g.epi = parts ? 3 : 0; g.split_k = parts ? parts : 1; g.n_groups = group;
+    g.M = M; g.N = N; g.K = F; g.epi = parts ? 3 : 0; g.split_k = parts ? parts : 1; g.n_groups = group; g.w_ready = 1;  // the kernel in front is this call's norm or row-wise kernel
     for (int k = 0; k < group; ++k) {
       const int l = l0 + k;
       const void *gain = io->host_norm_w ? io->host_norm_w[l] : nullptr;
       if (l == 0 || gain != prev_gain) {  // layers that share the input norm share the normalised rows
-        slot = parts ? slot + 1 : 0;
+        ++slot;
         dpara_status s = launch_rmsnorm_bf16(io->features, gain, ws + (size_t)slot * xn_bytes, M, F, io->rms_eps, st);
         if (s != DPARA_OK) return s;
         prev_gain = gain;
       }
-      void *out = parts ? static_cast<void *>(reinterpret_cast<float *>(kv) + (size_t)k * parts * M * N) : static_cast<void *>(kv);
+      void *out = parts ? static_cast<void *>(reinterpret_cast<float *>(kv) + (size_t)k * parts * M * N) : static_cast<void *>(kv + (size_t)k * M * N);
       if (k == 0) { g.a = ws + (size_t)slot * xn_bytes; g.w = io->host_w_kv[l]; g.out = out; }
       g.a_g[k] = ws + (size_t)slot * xn_bytes; g.w_g[k] = io->host_w_kv[l]; g.out_g[k] = out;
       P.knorm_w[k] = static_cast<const uint16_t *>(io->host_knorm_w ? io->host_knorm_w[l] : nullptr);

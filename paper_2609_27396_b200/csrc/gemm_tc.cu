@@ -1,8 +1,9 @@
-// bf16 GEMM  out[M][N] = epilogue( a[M][K] * w[N][K]^T )  on the 5th-generation tensor cores.
+// bf16 GEMM  out[M][N] = epilogue( a[M][K] * w[N][K]^T )  on the 5th-generation tensor cores: more than a few activation rows
+// (fewer: gemm_skinny.cu).
 //
-// One CTA computes a 128 x 256 output tile: a TMA producer warp streams 64-wide K slabs of both
-// operands (128-byte swizzle) through a 4-stage shared-memory ring, one elected thread issues
-// tcgen05.mma (M = 128, N = 256, K = 16, fp32 accumulator in 256 TMEM columns), four warps read the
+// A pair of CTAs computes a 256 x 256 output tile: a TMA producer warp per CTA streams 64-wide K slabs of both
+// operands (128-byte swizzle) through a shared-memory ring, one elected thread of the pair issues
+// tcgen05.mma (M = 256, N = 256, K = 16, fp32 accumulator in 256 TMEM columns of each CTA), four warps per CTA read the
 // accumulator back with tcgen05.ld and apply the epilogue:
 //   0  bf16 store                                   (QKV projection)
 //   1  fp32 out = resid + acc  (+ bf16 copy)        (O and down projections with the residual add)
@@ -12,17 +13,15 @@
 //   3  fp32 store                                   (LM head: base logits)
 // Every mbarrier wait is bounded; on expiry the CTA sets DPARA_STATUS_TIMEOUT and drains.
 #include "gemm.cuh"
+#include "gemm_skinny.cuh"
 #include "sm100_ptx.cuh"
 
 namespace dpara {
 using namespace ptx;
 
 namespace {
-constexpr int kBM = 128, kBN = 256, kBK = 64, kStages = 4;
+constexpr int kBM = 128, kBN = 256, kBK = 64;
 constexpr int kABytes = kBM * kBK * 2;         // 16 KB
-constexpr int kBBytes = kBN * kBK * 2;         // 32 KB (two 128-row boxes)
-constexpr int kStageBytes = kABytes + kBBytes;  // 48 KB
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/ + 4 * 32 * 36 * 4 /*epilogue staging*/;
 constexpr int kThreads = 192;                   // warps 0-3 epilogue, 4 TMA, 5 MMA
 }  // namespace
 
@@ -120,130 +119,8 @@ __device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ GemmKernelParams P) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
-  uint64_t *empty = full + kStages;
-  uint64_t *acc_full = empty + kStages;   // [2]: accumulator buffer ready for the epilogue
-  uint64_t *acc_empty = acc_full + 2;     // [2]: accumulator buffer drained
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
-  volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nkb = P.K / kBK;
-  const int tile_cols = P.epi == 2 ? 128 : kBN;
-  const int m_tiles = (P.M + kBM - 1) / kBM, n_tiles = (P.N + tile_cols - 1) / tile_cols;
-  const int total_tiles = m_tiles * n_tiles;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(full + s, 1);
-      mbar_init(empty + s, 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(acc_full + b, 1);
-      mbar_init(acc_empty + b, 4);
-    }
-    *abort_flag = 0;
-    fence_barrier_init();
-  }
-  if (warp == 5) {
-    tmem_alloc(tmem_slot, 512);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  pdl_wait();  // nothing above touches global memory: the set-up overlaps the tail of the kernel before
-  pdl_launch_dependents();
-
-  // Persistent: CTA c computes tiles c, c + gridDim.x, ...; tile id = n_tile * m_tiles + m_tile, so the CTAs
-  // running together cover all M rows of a few weight tiles (A stays in L2, each weight tile is read once).
-  // Two accumulator buffers in TMEM let the epilogue of one tile overlap the main loop of the next.
-  if (warp == 4) {
-    if (lane == 0) {
-      prefetch_tensormap(&P.map_a[0]);
-      prefetch_tensormap(&P.map_b[0]);
-      int stage = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int m_tile = tile % m_tiles, n_tile = tile / m_tiles;
-        const int brow0 = P.epi == 2 ? n_tile * 128 : n_tile * kBN;
-        const int brow1 = P.epi == 2 ? P.up_row_offset + n_tile * 128 : n_tile * kBN + 128;
-        for (int kb = 0; kb < nkb; ++kb) {
-          ok = mbar_wait(empty + stage, ph ^ 1u, abort_flag);
-          if (!ok) break;
-          uint8_t *sa = smem + stage * kStageBytes;
-          mbar_arrive_expect_tx(full + stage, kStageBytes);
-          tma_load_2d(sa, &P.map_a[0], full + stage, kb * kBK, m_tile * kBM);
-          tma_load_2d(sa + kABytes, &P.map_b[0], full + stage, kb * kBK, brow0);
-          tma_load_2d(sa + kABytes + 128 * kBK * 2, &P.map_b[0], full + stage, kb * kBK, brow1);
-          if (++stage == kStages) { stage = 0; ph ^= 1u; }
-        }
-      }
-    }
-  } else if (warp == 5) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kBM, kBN, false, false);
-      // descriptors are built once; stage and K-step offsets are added in 16-byte units
-      const uint64_t adesc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
-      const uint64_t bdesc0 = smem_desc_sw128(smem_u32(smem) + kABytes, 16, 1024);
-      int stage = 0, k = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++k) {
-        const int buf = k & 1;
-        ok = mbar_wait(acc_empty + buf, ((k >> 1) & 1) ^ 1u, abort_flag);  // epilogue of tile k - 2 has drained this buffer
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t acc = tmem + buf * kBN;
-        for (int kb = 0; kb < nkb; ++kb) {
-          ok = mbar_wait(full + stage, ph, abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          const uint64_t so = (uint64_t)(stage * (kStageBytes >> 4));
-          mma_ss(acc, adesc0 + so, bdesc0 + so, idesc, kb != 0);
-#pragma unroll
-          for (int kk = 1; kk < kBK / 16; ++kk) mma_ss_c<true>(acc, adesc0 + so + 2 * kk, bdesc0 + so + 2 * kk, idesc);
-          mma_commit(empty + stage);
-          if (++stage == kStages) { stage = 0; ph ^= 1u; }
-        }
-        if (ok) mma_commit(acc_full + buf);
-      }
-    }
-  } else {
-   int k = 0;
-   bool live = true;
-   for (int tile = blockIdx.x; tile < total_tiles && live; tile += gridDim.x, ++k) {
-    const int m_tile = tile % m_tiles, n_tile = tile / m_tiles;
-    const int buf = k & 1;
-    // ---------------- epilogue: thread = one accumulator row
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (k >> 1) & 1, abort_flag));  // warp-uniform: tcgen05.ld is warp-wide
-    tc_fence_after();
-    const int row_base = m_tile * kBM + warp * 32;
-    const uint32_t taddr = tmem + buf * kBN + ((uint32_t)(warp * 32) << 16);
-    live = ok;
-    if (ok) {
-      gemm_epilogue(P, taddr, row_base, n_tile, reinterpret_cast<float *>(smem + kStages * kStageBytes + 256) + warp * 32 * kEpiPitch, lane, 0, 0);
-    }
-    // this warp has read its part of the accumulator: hand the buffer back to the MMA issuer
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(acc_empty + buf);
-   }
-  }
-  // ---------------- teardown
-  if (threadIdx.x == 0 && *abort_flag && P.status) atomicOr(reinterpret_cast<unsigned int *>(P.status), DPARA_STATUS_TIMEOUT);
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 5) tmem_dealloc(tmem, 512);
-}
-
 // ------------------------------------------------------------------------------------------------ CTA pairs
-// The same GEMM with a pair of CTAs (a cluster of two, tcgen05 cta_group::2) per 256 x 256 output tile.  Each CTA
+// A pair of CTAs (a cluster of two, tcgen05 cta_group::2) per 256 x 256 output tile.  Each CTA
 // holds 128 rows of the activations, HALF of the weight tile (128 of its 256 rows) and the accumulator of its own
 // 128 output rows; the even CTA's thread issues M = 256 products that read both halves.  Per pair and K slab
 // 64 KB enter shared memory instead of the 96 KB two independent 128 x 256 tiles need: these shapes
@@ -392,6 +269,13 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
   if (g.K % kBK != 0 || g.N % 8 != 0) return DPARA_ERR_UNSUPPORTED;
   if (g.epi < 0 || g.epi > 3 || !g.a || !g.w || !g.out || (g.epi == 1 && !g.resid)) return DPARA_ERR_INVALID_ARG;
   if (!aligned16(g.a) || !aligned16(g.w) || !aligned16(g.out) || !aligned16(g.resid) || !aligned16(g.out_bf16)) return DPARA_ERR_INVALID_ARG;
+  // Few rows: the weights as the rows of the product.  Above 128 activation rows only where all tiles run at once (us, pairs / that:
+  // 200 rows, 4096 x 12288 64.5 / 33.7, 6144 x 4096 25.0 / 22.4; 288 rows, 4096 x 4096 29 / 19; but 192 rows, 151936 x 4096 in several
+  // rounds 271 / 326, one accumulator of 512 columns per CTA and nothing under its epilogue).
+  if (g.M <= 512) {
+    const SkinnyShape sh = skinny_shape(g);
+    if (sh.cost >= 0) return launch_gemm_skinny(g, sh, status, st);
+  }
   GemmKernelParams P;
   const int w_rows = g.epi == 2 ? 2 * g.N : g.N;
   int dev = 0, sms = kNumSM;
@@ -429,20 +313,11 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
     if (g.epi != 3 || g.M <= kBM || g.split_k > g.K / kBK) return DPARA_ERR_UNSUPPORTED;
     P.split_k = g.split_k;
   }
-  if (cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return DPARA_ERR_CUDA;
   const int tile_cols = g.epi == 2 ? 128 : P.bn;
-  const int tiles = ((g.N + tile_cols - 1) / tile_cols) * ((g.M + kBM - 1) / kBM);
-  if (g.M > kBM) {
-    // more than one 128-row tile of activations: CTA pairs (one 256 x 256 tile per pair and round)
-    if (cudaFuncSetAttribute(gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) != cudaSuccess) return DPARA_ERR_CUDA;
-    const int pair_tiles = ((g.N + tile_cols - 1) / tile_cols) * ((g.M + 2 * kBM - 1) / (2 * kBM)) * P.split_k * P.n_groups;
-    const int pairs = pair_tiles < sms / 2 ? pair_tiles : sms / 2;
-    launch_pdl(gemm_tc2_kernel, dim3(2 * pairs), dim3(kThreads), kSmemBytes2, st, P);
-    DPARA_CHECK_LAUNCH();
-    count_launches(1);
-    return DPARA_OK;
-  }
-  launch_pdl(gemm_tc_kernel, dim3(tiles < sms ? tiles : sms), dim3(kThreads), kSmemBytes, st, P);
+  if (cudaFuncSetAttribute(gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) != cudaSuccess) return DPARA_ERR_CUDA;
+  const int pair_tiles = ((g.N + tile_cols - 1) / tile_cols) * ((g.M + 2 * kBM - 1) / (2 * kBM)) * P.split_k * P.n_groups;
+  const int pairs = pair_tiles < sms / 2 ? pair_tiles : sms / 2;
+  launch_pdl(gemm_tc2_kernel, dim3(2 * pairs), dim3(kThreads), kSmemBytes2, st, P);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   return DPARA_OK;

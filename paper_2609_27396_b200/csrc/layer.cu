@@ -243,7 +243,7 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   GemmArgs g{};
-  g.a = xn; g.w = L->w_qkv; g.M = M; g.N = QD + 2 * KD; g.K = H; g.epi = 0; g.out = qkv;
+  g.a = xn; g.w = L->w_qkv; g.M = M; g.N = QD + 2 * KD; g.K = H; g.epi = 0; g.out = qkv; g.w_ready = 1;  // the kernels of this chain write no weights
   dpara_status s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
 
@@ -268,18 +268,18 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   if (s != DPARA_OK) return s;
 
   g = GemmArgs{};
-  g.a = a; g.w = L->w_o; g.M = M; g.N = H; g.K = QD; g.epi = 1; g.resid = L->x; g.resid_bf16 = 1; g.out = h1;
+  g.a = a; g.w = L->w_o; g.M = M; g.N = H; g.K = QD; g.epi = 1; g.resid = L->x; g.resid_bf16 = 1; g.out = h1; g.w_ready = 1;
   s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
   launch_pdl(rmsnorm_kernel<true>, dim3(M), dim3(128), 0, st, static_cast<const void *>(h1), static_cast<const uint16_t *>(L->rms2_w), hn, H, L->rms_eps);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   g = GemmArgs{};
-  g.a = hn; g.w = L->w_gate_up; g.M = M; g.N = I; g.K = H; g.epi = 2; g.out = act;
+  g.a = hn; g.w = L->w_gate_up; g.M = M; g.N = I; g.K = H; g.epi = 2; g.out = act; g.w_ready = 1;
   s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
   g = GemmArgs{};
-  g.a = act; g.w = L->w_down; g.M = M; g.N = H; g.K = I; g.epi = 1; g.resid = h1; g.resid_bf16 = 0; g.out = L->y_f32; g.out_bf16 = L->y_bf16;
+  g.a = act; g.w = L->w_down; g.M = M; g.N = H; g.K = I; g.epi = 1; g.resid = h1; g.resid_bf16 = 0; g.out = L->y_f32; g.out_bf16 = L->y_bf16; g.w_ready = 1;
   return launch_gemm_tc(g, status_word, st);
 }
 
