@@ -144,8 +144,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_tc
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
+  // (through shuffles: the compiler then knows that these are the same in the whole warp)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int nkb = P.K / kBK;
   const int tile_cols = P.epi == 2 ? 128 : P.bn;
@@ -173,68 +174,81 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_tc
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers exist before anything signals across the pair
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   pdl_wait();  // nothing above touches global memory: the set-up overlaps the tail of the kernel before
   pdl_launch_dependents();
 
+  // Warps 4 and 5: the whole warp walks the loop and waits, one lane issues, and the barrier of the next stage is asked before this
+  // stage's instructions go out (a wait inside a one-lane branch costs two to three times as many clocks, and the tensor pipe
+  // takes only one product ahead of the running one: what the loop does between two stages' products is idle time of the pipe).
   if (warp == 4) {
-    if (lane == 0) {
-      for (int gi = 0; gi < P.n_groups; ++gi) {
-        prefetch_tensormap(&P.map_a[gi]);
-        prefetch_tensormap(&P.map_b[gi]);
-      }
-      int stage = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int unit0 = pair; unit0 < total_tiles && ok; unit0 += n_pairs) {
-        const int grp = unit0 / group_units, unit = unit0 - grp * group_units;
-        const int tile = unit / P.split_k, ks = unit - tile * P.split_k;
-        const int m_pair = tile % m_pairs, n_tile = tile / m_pairs;
-        const int kb0 = ks * nkb / P.split_k, kb1 = (ks + 1) * nkb / P.split_k;
-        // this CTA's half of the weight tile: rows [rank * 128, +128) of the tile (SwiGLU: gate rows / up rows)
-        const int half = P.epi == 2 ? 128 : P.bn / 2;   // weight rows each CTA of the pair holds
-        const int brow = P.epi == 2 ? (rank == 0 ? n_tile * 128 : P.up_row_offset + n_tile * 128) : n_tile * P.bn + (int)rank * half;
-        const uint32_t tx = 2u * ((uint32_t)kABytes + (uint32_t)half * kBK * 2u);
-        const int arow = (m_pair * 2 + (int)rank) * kBM;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          ok = mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2);
-          if (!ok) break;
-          uint8_t *sa = smem + stage * kStageBytes2;
-          if (rank == 0) mbar_arrive_expect_tx(full + stage, tx);
-          tma_load_2d_pair(sa, &P.map_a[grp], full + stage, kb * kBK, arow);
-          tma_load_2d_pair(sa + kABytes, &P.map_b[grp], full + stage, kb * kBK, brow);
-          if (++stage == kStages2) { stage = 0; ph ^= 1u; }
+    for (int gi = 0; gi < P.n_groups; ++gi) {
+      prefetch_tensormap(&P.map_a[gi]);
+      prefetch_tensormap(&P.map_b[gi]);
+    }
+    int stage = 0;
+    uint32_t ph = 0;
+    bool ok = true, there = false;
+    const int half = P.epi == 2 ? 128 : P.bn / 2;   // weight rows each CTA of the pair holds
+    const uint32_t tx = 2u * ((uint32_t)kABytes + (uint32_t)half * kBK * 2u);
+    for (int unit0 = pair; unit0 < total_tiles && ok; unit0 += n_pairs) {
+      const int grp = unit0 / group_units, unit = unit0 - grp * group_units;
+      const int tile = unit / P.split_k, ks = unit - tile * P.split_k;
+      const int m_pair = tile % m_pairs, n_tile = tile / m_pairs;
+      const int kb0 = ks * nkb / P.split_k, kb1 = (ks + 1) * nkb / P.split_k;
+      // this CTA's half of the weight tile: rows [rank * half, +half) of the tile (SwiGLU: gate rows / up rows)
+      const int brow = P.epi == 2 ? (rank == 0 ? n_tile * 128 : P.up_row_offset + n_tile * 128) : n_tile * P.bn + (int)rank * half;
+      const int arow = (m_pair * 2 + (int)rank) * kBM;
+      const CUtensorMap *map_a = &P.map_a[grp], *map_b = &P.map_b[grp];
+#pragma unroll 1
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!__all_sync(0xffffffffu, there)) ok = __all_sync(0xffffffffu, mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2));
+        if (!ok) break;
+        const int cur = stage;
+        if (++stage == kStages2) { stage = 0; ph ^= 1u; }
+        there = mbar_test(empty + stage, ph ^ 1u);
+        if (elect_one()) {
+          uint8_t *sa = smem + cur * kStageBytes2;
+          if (rank == 0) mbar_arrive_expect_tx(full + cur, tx);
+          tma_load_2d_pair(sa, map_a, full + cur, kb * kBK, arow);
+          tma_load_2d_pair(sa + kABytes, map_b, full + cur, kb * kBK, brow);
         }
+        __syncwarp();
       }
     }
   } else if (warp == 5) {
-    if (rank == 0 && lane == 0) {
+    if (rank == 0) {
       const uint32_t idesc = idesc_bf16_f32(2 * kBM, P.epi == 2 ? kBN : P.bn, false, false);
-      const uint64_t adesc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
-      const uint64_t bdesc0 = smem_desc_sw128(smem_u32(smem) + kABytes, 16, 1024);
+      const uint64_t desc = smem_desc_sw128(smem_u32(smem), 16, 1024);
+      const uint32_t a_lo = (uint32_t)desc, b_lo = a_lo + (kABytes >> 4), hi = (uint32_t)(desc >> 32);
       int stage = 0, k = 0;
       uint32_t ph = 0;
-      bool ok = true;
+      bool ok = true, there = false;
       for (int unit0 = pair; unit0 < total_tiles && ok; unit0 += n_pairs, ++k) {
         const int ks = (unit0 % group_units) % P.split_k;
         const int kb0 = ks * nkb / P.split_k, kb1 = (ks + 1) * nkb / P.split_k;
         const int buf = k & 1;
-        ok = mbar_wait(acc_empty + buf, ((k >> 1) & 1) ^ 1u, abort_flag, 3);  // both CTAs' epilogues of tile k - 2 are done
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + buf, ((k >> 1) & 1) ^ 1u, abort_flag, 3));  // both CTAs' epilogues of tile k - 2 are done
         if (!ok) break;
-        tc_fence_after();
         const uint32_t acc = tmem + buf * kBN;
+#pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
-          ok = mbar_wait(full + stage, ph, abort_flag, 4);
+          if (!__all_sync(0xffffffffu, there)) ok = __all_sync(0xffffffffu, mbar_wait(full + stage, ph, abort_flag, 4));
           if (!ok) break;
-          tc_fence_after();
-          const uint64_t so = (uint64_t)(stage * (kStageBytes2 >> 4));
-          mma2_ss(acc, adesc0 + so, bdesc0 + so, idesc, kb != kb0);
-#pragma unroll
-          for (int kk = 1; kk < kBK / 16; ++kk) mma2_ss_c<true>(acc, adesc0 + so + 2 * kk, bdesc0 + so + 2 * kk, idesc);
-          mma2_commit_both(empty + stage);
+          const int cur = stage;
           if (++stage == kStages2) { stage = 0; ph ^= 1u; }
+          there = mbar_test(full + stage, ph);
+          tc_fence_after();
+          if (elect_one()) {
+            const uint32_t so = cur * (kStageBytes2 >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kBK / 16; ++kk) mma2_ss_lo(acc, a_lo + so + 2 * kk, b_lo + so + 2 * kk, hi, idesc, kk != 0 || kb != kb0);
+            mma2_commit_both(empty + cur);
+          }
+          __syncwarp();
         }
-        if (ok) mma2_commit_both(acc_full + buf);
+        if (ok && elect_one()) mma2_commit_both(acc_full + buf);
+        __syncwarp();
       }
     }
   } else {

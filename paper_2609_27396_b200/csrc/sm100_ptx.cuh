@@ -302,6 +302,15 @@ __device__ __forceinline__ void mma2_ss_c(uint32_t d_tmem, uint64_t adesc, uint6
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "n"(kAcc ? 1 : 0)
       : "memory");
 }
+// The same with the descriptors' low words only (see mma_ss_lo).
+__device__ __forceinline__ void mma2_ss_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.u32 p, %5, 0;\n\t"
+      "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %4, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)accumulate)
+      : "memory");
+}
 // Arrives on the barrier at this offset in BOTH CTAs of the pair once every tcgen05 operation the thread has
 // issued so far has completed (a tcgen05.commit that signals both CTAs; no data moves).
 __device__ __forceinline__ void mma2_commit_both(uint64_t *bar_local) {
