@@ -132,7 +132,8 @@ __global__ void append_commit_kernel(int64_t *ctx_len, const int64_t *capacity, 
 }
 
 // Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores (at most 128 rows: the
-// kernel for few rows splits K inside its clusters.  8 rows, five layers of 2048 x 4096: 29 us a layer one by one -> ~20 us together).  The parts are chosen to minimise
+// kernel for few rows takes all layers at once, one chain of sums over K each.  8 rows, five layers of 2048 x 4096: 29 us a layer one by one ->
+// ~20 us together).  The parts are chosen to minimise
 // rounds x (K slabs per part + ~8 slabs' worth of fixed cost per work unit) over the CTA pairs.
 static void cache_group_plan(const dpara_cache_io *io, int layers_left, int *group, int *parts) {
   const int M = io->batch * io->n_rows, N = 2 * io->n_kv_heads * io->head_dim;
@@ -198,7 +199,7 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
     int group, parts;
     cache_group_plan(io, io->n_layers - l0, &group, &parts);
     GemmArgs g{};
-    g.M = M; g.N = N; g.K = F; g.epi = parts ? 3 : 0; g.split_k = parts ? parts : 1; g.n_groups = group; g.w_ready = 1;  // the kernel in front is this call's norm or row-wise kernel
+    g.M = M; g.N = N; g.K = F; g.epi = parts ? 3 : 0; g.split_k = parts ? parts : 1; g.n_groups = group; g.one_chain = 1; g.w_ready = 1;  // the kernel in front is this call's norm or row-wise kernel
     for (int k = 0; k < group; ++k) {
       const int l = l0 + k;
       const void *gain = io->host_norm_w ? io->host_norm_w[l] : nullptr;

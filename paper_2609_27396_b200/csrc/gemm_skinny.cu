@@ -381,13 +381,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
       const int grp = unit / P.tiles, tile = unit - grp * P.tiles;
       const int buf = n_buf == 2 ? k & 1 : 0;
       const uint32_t use = n_buf == 2 ? k >> 1 : k;
-      live = __all_sync(0xffffffffu, mbar_wait(acc_full + buf, use & 1, abort_flag, 4));
+      // one warp asks for the accumulator, the others sleep on the named barrier: eight polling warps slow down the two that issue
+      live = epilogue_bar(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, use & 1, abort_flag, 4)));
       tc_fence_after();
       const uint32_t taddr = tmem + buf * buf_cols + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
       for (int c0 = 0; c0 < P.T; c0 += P.chunk, ++chunk_no) {
         // ---- this CTA's part of activation rows [c0, c0 + chunk) into its buffer, once the last one has been read
-        if (S > 1 && !P.one_round) live = live && __all_sync(0xffffffffu, mbar_wait_cluster(freed, (chunk_no & 1) ^ 1u, abort_flag, 5));
+        if (S > 1 && !P.one_round) live = epilogue_bar(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(freed, (chunk_no & 1) ^ 1u, abort_flag, 5))));
         else if (!P.one_round) named_bar_sync(1, kEpiThreads);
         const int n_here = min(P.chunk, P.T - c0);
         int piece = 0;   // 32 columns each, handed out to the two warps of a TMEM quarter in turn
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
         live = epilogue_bar(live);
         if (S > 1) {
           if (threadIdx.x < S) mbar_arrive_rank(ready, threadIdx.x);
-          live = live && __all_sync(0xffffffffu, mbar_wait_cluster(ready, chunk_no & 1, abort_flag, 6));
+          live = epilogue_bar(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(ready, chunk_no & 1, abort_flag, 6))));
         }
         const int rows_here = min(P.M - c0, n_here);
         if (live) {
@@ -514,7 +515,7 @@ SkinnyShape skinny_shape(const GemmArgs &g) {
   for (int halves = g.epi == 2 ? 2 : 1; halves <= 2; ++halves) {
     if (halves * T > 512) continue;
     const int per_tile = g.epi == 2 ? 1 : halves;     // output columns per operand row
-    for (int s = 1; s <= kMaxSplit && s <= nkb; ++s) {
+    for (int s = 1; s <= (g.one_chain ? 1 : kMaxSplit) && s <= nkb; ++s) {
       if (cap[s] <= 0) continue;
       int tried = 0;
       for (long k = 1; tried < 3 && k < 4096; ++k) {

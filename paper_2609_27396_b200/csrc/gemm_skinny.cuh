@@ -7,7 +7,7 @@ namespace dpara {
 constexpr int kManyRows = 128;   // above this many activation rows only launches whose tiles all run at once
 
 struct SkinnyShape {
-  double cost;      // model, ns; < 0: the shape is not taken
+  double cost;      // model, ns beside ~3500 of a launch; < 0: the shape is not taken
   int T, rows, halves, tiles, split, clusters, one_round;
   int chunk, stages, slabs, ring_bytes, bar_offset, smem, tmem_cols;
 };

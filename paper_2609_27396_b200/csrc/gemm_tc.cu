@@ -1,15 +1,20 @@
 // bf16 GEMM  out[M][N] = epilogue( a[M][K] * w[N][K]^T )  on the 5th-generation tensor cores: more than a few activation rows
 // (fewer: gemm_skinny.cu).
 //
-// A pair of CTAs computes a 256 x 256 output tile: a TMA producer warp per CTA streams 64-wide K slabs of both
-// operands (128-byte swizzle) through a shared-memory ring, one elected thread of the pair issues
-// tcgen05.mma (M = 256, N = 256, K = 16, fp32 accumulator in 256 TMEM columns of each CTA), four warps per CTA read the
-// accumulator back with tcgen05.ld and apply the epilogue:
+// A pair of CTAs (a cluster of two, tcgen05 cta_group::2) computes a tile of 256 weight rows x nt activation rows (nt <= 256).  The
+// WEIGHTS are the rows of the product, so that nt can be any multiple of 16: a batch of 1152 rows is five tiles of 240, 288 rows are
+// two of 144 (256-row tiles of activations computed 1280 and 512 rows there).  Per 64-wide slab of K each CTA holds 128 of the weight
+// rows and HALF of the activation rows (128-byte swizzle) and the accumulator of its own 128 weight rows; the even CTA's thread
+// issues M = 256 products that read both halves.  These shapes are bound by the L2 -> shared-memory fill and by power: a pair pulls
+// 64 KB per slab for 256 x 256 outputs.  Each CTA's producer fetches its own halves with ordinary tiled copies and counts the bytes
+// on the LEADER's barrier; stage and accumulator hand-offs from the MMA thread reach both CTAs through one tcgen05.commit; the
+// epilogue warps of both CTAs arrive on the leader's accumulator-empty barrier.
+//
+// Epilogues (accumulator: lane = output column, TMEM column = activation row):
 //   0  bf16 store                                   (QKV projection)
 //   1  fp32 out = resid + acc  (+ bf16 copy)        (O and down projections with the residual add)
-//   2  bf16 out = silu(gate) * up                   (gate/up projection: the tile's 256 accumulator
-//                                                    columns are 128 gate columns and the matching 128
-//                                                    up columns, so the activation never leaves the SM)
+//   2  bf16 out = silu(gate) * up                   (gate/up projection: 64 of a CTA's weight rows are gate rows and 64 the matching
+//                                                    up rows, so the activation never leaves the SM)
 //   3  fp32 store                                   (LM head: base logits)
 // Every mbarrier wait is bounded; on expiry the CTA sets DPARA_STATUS_TIMEOUT and drains.
 #include "gemm.cuh"
@@ -20,148 +25,204 @@ namespace dpara {
 using namespace ptx;
 
 namespace {
-constexpr int kBM = 128, kBN = 256, kBK = 64;
-constexpr int kABytes = kBM * kBK * 2;         // 16 KB
-constexpr int kThreads = 192;                   // warps 0-3 epilogue, 4 TMA, 5 MMA
+constexpr int kBK = 64;
+constexpr int kRows = 128;                      // weight rows per CTA
+constexpr int kWBytes = kRows * kBK * 2;        // 16 KB
+constexpr int kThreads = 320;                   // warps 0-3 and 6-9: epilogue; 4: TMA; 5: MMA
+constexpr int kEpiWarps = 8;
+constexpr int kMaxStages = 8;
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kBarBytes = 512;
+constexpr int kEpiBytes = kEpiWarps * 16 * 32 * 4;   // 16 activation rows of 32 columns per warp (SwiGLU, fp32 stores)
 }  // namespace
 
 struct GemmKernelParams {
-  CUtensorMap map_a[kGemmMaxGroups];   // one entry per product of a grouped launch (a plain launch uses entry 0)
-  CUtensorMap map_b[kGemmMaxGroups];
-  void *out_g[kGemmMaxGroups];         // grouped launch: the products' outputs
+  CUtensorMap map_w[kGemmMaxGroups];   // one entry per product of a grouped launch (a plain launch uses entry 0)
+  CUtensorMap map_a[kGemmMaxGroups];
+  void *out_g[kGemmMaxGroups];
   int n_groups;
   int M, N, K;
   int epi;
   int up_row_offset;
-  void *out;
+  int nt, t_tiles, n_tiles;            // activation rows per tile; tiles of one product
+  int stages;
+  int split_k;                         // > 1 (fp32 store only): the K range in split_k parts, part s writes plane s of [split_k][M][N] partial sums
   const void *resid;
   int resid_bf16;
   void *out_bf16;
   int32_t *status;
   int perm_block, perm_b;
-  int bn;        // output columns per tile of the CTA-pair kernel: 256, or 192 where that fills the rounds better (bf16 / fp32 stores)
-  int split_k;   // > 1 (fp32 store only, CTA pairs): the K range in split_k parts, part s writes plane s of [split_k][M][N] partial sums
 };
 
 __device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
 
-// Epilogue of one accumulator tile.  A thread reads one accumulator ROW from tensor memory (lane = row), 32 columns at
-// a time; stored like that, one warp instruction would touch 32 rows x 16 bytes -- 32 cache lines for 512 bytes.  Each
-// 32 x 32 block therefore goes through a per-warp shared-memory buffer (row pitch 36 floats: conflict-free both ways)
-// and comes back with 8 lanes on one row: an instruction then covers 4 rows x 128 contiguous bytes, for the residual
-// read as well as for the stores.  `row_base` = output row of lane 0, `stage` = this warp's 32 x 36 floats.
-constexpr int kEpiPitch = 36;
+// Barrier among the 256 epilogue threads that also makes `live` the same in all of them.
+__device__ __forceinline__ bool epi_bar(bool live) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+      "barrier.red.and.pred q, 1, 256, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(all) : "r"((uint32_t)live) : "memory");
+  return all != 0;
+}
 
-__device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_t taddr, int row_base, int n_tile, float *stage, int lane, int ks,
-                                              int grp) {
-  // fp32 output of this product; split K (fp32 store only): plane ks of the partial sums
-  float *out_f32 = static_cast<float *>(P.n_groups > 1 ? P.out_g[grp] : P.out) + (size_t)ks * P.M * P.N;
-  const int n_chunks = P.epi == 2 ? 4 : P.bn / 32;
-  const int col0 = n_tile * (P.epi == 2 ? 128 : P.bn);
-  const int sub_row = lane >> 3, piece = lane & 7;
+// A unit of work: a tile of one of the products, or one part of its K range (the parts of a tile are neighbours).
+struct Unit {
+  int grp, tile, ks, kb0, kb1;
+  __device__ __forceinline__ Unit(const GemmKernelParams &P, int unit, int nkb) {
+    const int per_group = P.t_tiles * P.n_tiles * P.split_k;
+    grp = unit / per_group;
+    unit -= grp * per_group;
+    tile = unit / P.split_k;
+    ks = unit - tile * P.split_k;
+    kb0 = ks * nkb / P.split_k;
+    kb1 = (ks + 1) * nkb / P.split_k;
+  }
+};
+
+// Epilogue of one accumulator tile.  A thread has one output column (lane) and takes 32 activation rows at a time: an instruction reads or
+// writes 32 neighbouring columns of one activation row (fp32: one 128-byte line), straight from and to registers.  Shared memory is
+// what these products are short of (per slab the products read 64 bytes and the copies write 64 bytes per clock of the 128 an SM
+// has): a transposing buffer here cost 4 % of the whole product.  The two warps of a TMEM quarter take the blocks in turn, and the
+// residual rows of a block are on their way while the one before is worked on.
+__device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_t taddr, const Unit &w, int rank, float *exchange, int quarter, int turn, int lane) {
+  const int grp = w.grp, tile = w.tile;
+  const int t_tile = tile % P.t_tiles, n_tile = tile / P.t_tiles;
+  const int row0 = t_tile * P.nt, rows_all = min(P.M - row0, P.nt);
+  if (P.epi == 2) {
+    // quarters 0 and 1 have gate columns, 2 and 3 the matching up columns: each warp of such a pair hands 16 of the 32 activation rows to the
+    // other and finishes the other 16
+    const int col = n_tile * 128 + rank * 64 + (quarter & 1) * 32 + lane;
+    const bool up_side = quarter >= 2;
+    const int bar = 2 + (quarter & 1) + 2 * turn;
+    float *mine = exchange + (quarter * 2 + turn) * 512 + lane;
+    const float *theirs = exchange + ((quarter ^ 2) * 2 + turn) * 512 + lane;
+    uint16_t *out = static_cast<uint16_t *>(P.out_g[grp]) + (size_t)row0 * P.N + col;
 #pragma unroll 1
-  for (int c = 0; c < n_chunks; ++c) {
-    uint32_t r[32];
-    tmem_ld32(taddr + c * 32, r);
-    if (P.epi == 2) {
-      uint32_t u[32];
-      tmem_ld32(taddr + 128 + c * 32, u);
+    for (int c0 = turn * 32; c0 < rows_all; c0 += 64) {
+      uint32_t r[32];
+      tmem_ld32(taddr + c0, r);
+      tmem_wait_ld();
+      // (selected, not indexed: r stays in registers)
+#pragma unroll
+      for (int j = 0; j < 16; ++j) mine[j * 32] = __uint_as_float(up_side ? r[j] : r[16 + j]);
+      named_bar_sync(bar, 64);
+      const int j0 = c0 + (up_side ? 16 : 0);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float own = __uint_as_float(up_side ? r[16 + j] : r[j]), other = theirs[j * 32];
+        const float v = silu_f(up_side ? other : own) * (up_side ? own : other);
+        if (j0 + j < rows_all && col < P.N) out[(size_t)(j0 + j) * P.N] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+      }
+      named_bar_sync(bar, 64);
+    }
+    return;
+  }
+  if (P.epi == 3) {
+    // four bytes per output and nothing else: 16 activation rows at a time through the buffer, so that an instruction writes 512 bytes
+    // (a split product of 20 slabs per unit, 42 MB of partial sums: 42 -> 39 us)
+    const int sub = lane >> 3, col = n_tile * 256 + rank * 128 + quarter * 32 + (lane & 7) * 4;
+    float *mine = exchange + (quarter * 2 + turn) * 512;
+    float *out = static_cast<float *>(P.out_g[grp]) + (size_t)w.ks * P.M * P.N + col;
+    const int pb = P.perm_block ? P.perm_block : 1 << 30, pm = P.perm_block ? P.perm_b : 0;   // row n * pb + i goes to i * perm_b + n
+#pragma unroll 1
+    for (int c0 = turn * 32; c0 < rows_all; c0 += 64) {
+      uint32_t r[32];
+      tmem_ld32(taddr + c0, r);
       tmem_wait_ld();
 #pragma unroll
-      for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(silu_f(__uint_as_float(r[e])) * __uint_as_float(u[e]));
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) mine[j * 32 + lane] = __uint_as_float(r[16 * h + j]);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int rl = c0 + 16 * h + i * 4 + sub, row = row0 + rl;
+          const float4 x = *reinterpret_cast<const float4 *>(mine + (i * 4 + sub) * 32 + (lane & 7) * 4);
+          const int orow = P.perm_block ? (row % pb) * pm + row / pb : row;
+          if (rl < rows_all && col < P.N) *reinterpret_cast<float4 *>(out + (size_t)orow * P.N) = x;
+        }
+        __syncwarp();
+      }
+    }
+    return;
+  }
+  const int col = n_tile * 256 + rank * 128 + quarter * 32 + lane;
+  const bool in = col < P.N;
+  float rr[32];
+  auto fetch = [&](int c0) {
+    if (P.epi != 1 || !in) return;
+    // (rows behind the last read row M - 1: an unconditional load the compiler can issue early; the value is not used)
+    if (P.resid_bf16) {
+      const uint16_t *src = static_cast<const uint16_t *>(P.resid) + col;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) rr[j] = bf16_bits_to_float(src[(size_t)min(row0 + c0 + j, P.M - 1) * P.N]);
     } else {
-      tmem_wait_ld();
+      const float *src = static_cast<const float *>(P.resid) + col;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) rr[j] = src[(size_t)min(row0 + c0 + j, P.M - 1) * P.N];
     }
-    float4 *mine = reinterpret_cast<float4 *>(stage + lane * kEpiPitch);
+  };
+  if (turn * 32 < rows_all) fetch(turn * 32);
+#pragma unroll 1
+  for (int c0 = turn * 32; c0 < rows_all; c0 += 64) {
+    uint32_t r[32];
+    tmem_ld32(taddr + c0, r);
+    tmem_wait_ld();
+    float x[32];
 #pragma unroll
-    for (int v = 0; v < 8; ++v)
-      mine[v] = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
-    __syncwarp();
-    const int col = col0 + c * 32 + piece * 4;
-    if (col < P.N) {
-      // the residual rows first, all in flight together
-      float4 rr[8];
-      if (P.epi == 1) {
-        // (rows past M read row M - 1: an unconditional load the compiler can issue early; the value is not used)
-        if (P.resid_bf16) {
-          uint2 q[8];
+    for (int j = 0; j < 32; ++j) x[j] = P.epi == 1 ? __uint_as_float(r[j]) + rr[j] : __uint_as_float(r[j]);
+    if (c0 + 64 < rows_all) fetch(c0 + 64);
+    if (!in) continue;
+    const int rows = rows_all - c0;
+    if (P.epi == 0) {
+      uint16_t *out = static_cast<uint16_t *>(P.out_g[grp]) + (size_t)(row0 + c0) * P.N + col;
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            q[i] = *reinterpret_cast<const uint2 *>(static_cast<const uint16_t *>(P.resid) + (size_t)min(row_base + i * 4 + sub_row, P.M - 1) * P.N + col);
+      for (int j = 0; j < 32; ++j)
+        if (j < rows) out[(size_t)j * P.N] = __bfloat16_as_ushort(__float2bfloat16_rn(x[j]));
+    } else {
+      float *out = static_cast<float *>(P.out_g[grp]) + (size_t)(row0 + c0) * P.N + col;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) rr[i] = make_float4(bf16lo(q[i].x), bf16hi(q[i].x), bf16lo(q[i].y), bf16hi(q[i].y));
-        } else {
+      for (int j = 0; j < 32; ++j)
+        if (j < rows) out[(size_t)j * P.N] = x[j];
+      if (P.out_bf16) {
+        uint16_t *o16 = static_cast<uint16_t *>(P.out_bf16) + (size_t)(row0 + c0) * P.N + col;
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            rr[i] = *reinterpret_cast<const float4 *>(static_cast<const float *>(P.resid) + (size_t)min(row_base + i * 4 + sub_row, P.M - 1) * P.N + col);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int rl = i * 4 + sub_row, row = row_base + rl;
-        const float4 a = *reinterpret_cast<const float4 *>(stage + rl * kEpiPitch + piece * 4);
-        if (row < P.M) {
-          if (P.epi == 0 || P.epi == 2) {
-            uint16_t *o = static_cast<uint16_t *>(P.out) + (size_t)row * P.N + col;
-            *reinterpret_cast<uint2 *>(o) = make_uint2(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w));
-          } else {
-            const int orow = P.perm_block ? (row % P.perm_block) * P.perm_b + row / P.perm_block : row;
-            float4 x = a;
-            if (P.epi == 1) { x.x += rr[i].x; x.y += rr[i].y; x.z += rr[i].z; x.w += rr[i].w; }
-            *reinterpret_cast<float4 *>(out_f32 + (size_t)orow * P.N + col) = x;
-            if (P.out_bf16)
-              *reinterpret_cast<uint2 *>(static_cast<uint16_t *>(P.out_bf16) + (size_t)row * P.N + col) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-          }
-        }
+        for (int j = 0; j < 32; ++j)
+          if (j < rows) o16[(size_t)j * P.N] = __bfloat16_as_ushort(__float2bfloat16_rn(x[j]));
       }
     }
-    __syncwarp();
   }
 }
 
-// ------------------------------------------------------------------------------------------------ CTA pairs
-// A pair of CTAs (a cluster of two, tcgen05 cta_group::2) per 256 x 256 output tile.  Each CTA
-// holds 128 rows of the activations, HALF of the weight tile (128 of its 256 rows) and the accumulator of its own
-// 128 output rows; the even CTA's thread issues M = 256 products that read both halves.  Per pair and K slab
-// 64 KB enter shared memory instead of the 96 KB two independent 128 x 256 tiles need: these shapes
-// (M = 256..1024 rows against large weights) are bound by the L2 -> shared-memory fill rate, not by the tensor
-// pipe.  Each CTA's producer fetches its own halves with ordinary tiled copies and counts the bytes on the LEADER's
-// barrier; stage and accumulator hand-offs from the MMA thread reach both CTAs through one tcgen05.commit;
-// the epilogue warps of both CTAs arrive on the leader's accumulator-empty barrier.
-namespace {
-constexpr int kStages2 = 6;
-constexpr int kStageBytes2 = kABytes + 128 * kBK * 2;  // 32 KB: 128 activation rows + 128 weight rows
-constexpr int kSmemBytes2 = kStages2 * kStageBytes2 + 1024 + 256 + 4 * 32 * 36 * 4;
-}  // namespace
-
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_tc2_kernel(const __grid_constant__ GemmKernelParams P) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pair_kernel(const __grid_constant__ GemmKernelParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages2 * kStageBytes2);   // used in the leader only
-  uint64_t *empty = full + kStages2;                                              // local copy in each CTA
-  uint64_t *acc_full = empty + kStages2;                                          // [2] local copy in each CTA
+  const int stage_bytes = kWBytes + P.nt * 64;   // 128 weight rows, nt / 2 activation rows
+  float *exchange = reinterpret_cast<float *>(smem + P.stages * stage_bytes);
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + P.stages * stage_bytes + kEpiBytes);   // used in the leader only
+  uint64_t *empty = full + kMaxStages;                                            // local copy in each CTA
+  uint64_t *acc_full = empty + kMaxStages;                                        // [2] local copy in each CTA
   uint64_t *acc_empty = acc_full + 2;                                             // [2] used in the leader only
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
   // (through shuffles: the compiler then knows that these are the same in the whole warp)
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int rank = __shfl_sync(0xffffffffu, (int)cluster_ctarank(), 0);
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   const int nkb = P.K / kBK;
-  const int tile_cols = P.epi == 2 ? 128 : P.bn;
-  const int m_pairs = (P.M + 2 * kBM - 1) / (2 * kBM), n_tiles = (P.N + tile_cols - 1) / tile_cols;
-  const int group_units = m_pairs * n_tiles * P.split_k;   // work units of one product: (tile, K part), the parts of a tile adjacent
-  const int total_tiles = group_units * P.n_groups;
+  const int units = P.t_tiles * P.n_tiles * P.split_k * P.n_groups;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages2; ++s) {
+    for (int s = 0; s < P.stages; ++s) {
       mbar_init(full + s, 1);
       mbar_init(empty + s, 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(acc_full + b, 1);
-      mbar_init(acc_empty + b, 8);   // four epilogue warps of each CTA
+      mbar_init(acc_empty + b, 2 * kEpiWarps);   // of both CTAs
     }
     *abort_flag = 0;
     fence_barrier_init();
@@ -183,66 +244,65 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_tc
   // takes only one product ahead of the running one: what the loop does between two stages' products is idle time of the pipe).
   if (warp == 4) {
     for (int gi = 0; gi < P.n_groups; ++gi) {
+      prefetch_tensormap(&P.map_w[gi]);
       prefetch_tensormap(&P.map_a[gi]);
-      prefetch_tensormap(&P.map_b[gi]);
     }
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true, there = false;
-    const int half = P.epi == 2 ? 128 : P.bn / 2;   // weight rows each CTA of the pair holds
-    const uint32_t tx = 2u * ((uint32_t)kABytes + (uint32_t)half * kBK * 2u);
-    for (int unit0 = pair; unit0 < total_tiles && ok; unit0 += n_pairs) {
-      const int grp = unit0 / group_units, unit = unit0 - grp * group_units;
-      const int tile = unit / P.split_k, ks = unit - tile * P.split_k;
-      const int m_pair = tile % m_pairs, n_tile = tile / m_pairs;
-      const int kb0 = ks * nkb / P.split_k, kb1 = (ks + 1) * nkb / P.split_k;
-      // this CTA's half of the weight tile: rows [rank * half, +half) of the tile (SwiGLU: gate rows / up rows)
-      const int brow = P.epi == 2 ? (rank == 0 ? n_tile * 128 : P.up_row_offset + n_tile * 128) : n_tile * P.bn + (int)rank * half;
-      const int arow = (m_pair * 2 + (int)rank) * kBM;
-      const CUtensorMap *map_a = &P.map_a[grp], *map_b = &P.map_b[grp];
+    const uint32_t tx = 2u * (uint32_t)stage_bytes;
+    const int half_t = P.nt / 2;
+    // (tile id = weight tile * t_tiles + activation tile: the pairs running together cover all activation rows of a few weight tiles)
+    for (int unit = pair; unit < units && ok; unit += pairs) {
+      const Unit w(P, unit, nkb);
+      const int grp = w.grp, t_tile = w.tile % P.t_tiles, n_tile = w.tile / P.t_tiles;
+      const int wrow = P.epi == 2 ? n_tile * 128 + rank * 64 : n_tile * 256 + rank * 128;
+      const int arow = t_tile * P.nt + rank * half_t;
+      const CUtensorMap *map_w = &P.map_w[grp], *map_a = &P.map_a[grp];
+      const bool swiglu = P.epi == 2;
 #pragma unroll 1
-      for (int kb = kb0; kb < kb1; ++kb) {
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
         if (!__all_sync(0xffffffffu, there)) ok = __all_sync(0xffffffffu, mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2));
         if (!ok) break;
         const int cur = stage;
-        if (++stage == kStages2) { stage = 0; ph ^= 1u; }
+        if (++stage == P.stages) { stage = 0; ph ^= 1u; }
         there = mbar_test(empty + stage, ph ^ 1u);
         if (elect_one()) {
-          uint8_t *sa = smem + cur * kStageBytes2;
+          uint8_t *sw = smem + cur * stage_bytes;
           if (rank == 0) mbar_arrive_expect_tx(full + cur, tx);
-          tma_load_2d_pair(sa, map_a, full + cur, kb * kBK, arow);
-          tma_load_2d_pair(sa + kABytes, map_b, full + cur, kb * kBK, brow);
+          tma_load_2d_pair(sw, map_w, full + cur, kb * kBK, wrow);
+          if (swiglu) tma_load_2d_pair(sw + kWBytes / 2, map_w, full + cur, kb * kBK, P.up_row_offset + wrow);
+          tma_load_2d_pair(sw + kWBytes, map_a, full + cur, kb * kBK, arow);
         }
         __syncwarp();
       }
     }
   } else if (warp == 5) {
     if (rank == 0) {
-      const uint32_t idesc = idesc_bf16_f32(2 * kBM, P.epi == 2 ? kBN : P.bn, false, false);
+      const uint32_t idesc = idesc_bf16_f32(2 * kRows, P.nt, false, false);
       const uint64_t desc = smem_desc_sw128(smem_u32(smem), 16, 1024);
-      const uint32_t a_lo = (uint32_t)desc, b_lo = a_lo + (kABytes >> 4), hi = (uint32_t)(desc >> 32);
+      const uint32_t w_lo = (uint32_t)desc, a_lo = w_lo + (kWBytes >> 4), hi = (uint32_t)(desc >> 32), stage_units = (uint32_t)stage_bytes >> 4;
       int stage = 0, k = 0;
       uint32_t ph = 0;
       bool ok = true, there = false;
-      for (int unit0 = pair; unit0 < total_tiles && ok; unit0 += n_pairs, ++k) {
-        const int ks = (unit0 % group_units) % P.split_k;
-        const int kb0 = ks * nkb / P.split_k, kb1 = (ks + 1) * nkb / P.split_k;
+      for (int unit = pair; unit < units && ok; unit += pairs, ++k) {
+        const Unit w(P, unit, nkb);
         const int buf = k & 1;
         ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + buf, ((k >> 1) & 1) ^ 1u, abort_flag, 3));  // both CTAs' epilogues of tile k - 2 are done
         if (!ok) break;
-        const uint32_t acc = tmem + buf * kBN;
+        const uint32_t acc = tmem + buf * 256;
 #pragma unroll 1
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
           if (!__all_sync(0xffffffffu, there)) ok = __all_sync(0xffffffffu, mbar_wait(full + stage, ph, abort_flag, 4));
           if (!ok) break;
           const int cur = stage;
-          if (++stage == kStages2) { stage = 0; ph ^= 1u; }
+          if (++stage == P.stages) { stage = 0; ph ^= 1u; }
           there = mbar_test(full + stage, ph);
           tc_fence_after();
           if (elect_one()) {
-            const uint32_t so = cur * (kStageBytes2 >> 4);
+            const uint32_t so = cur * stage_units;
 #pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) mma2_ss_lo(acc, a_lo + so + 2 * kk, b_lo + so + 2 * kk, hi, idesc, kk != 0 || kb != kb0);
+            for (int kk = 0; kk < kBK / 16; ++kk) mma2_ss_lo(acc, w_lo + so + 2 * kk, a_lo + so + 2 * kk, hi, idesc, kk != 0 || kb != w.kb0);
             mma2_commit_both(empty + cur);
           }
           __syncwarp();
@@ -252,25 +312,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_tc
       }
     }
   } else {
+    const int quarter = warp & 3, turn = warp >= 4;   // the TMEM lanes a warp may read; which of the two warps that may
     int k = 0;
     bool live = true;
-    for (int unit0 = pair; unit0 < total_tiles && live; unit0 += n_pairs, ++k) {
-      const int grp = unit0 / group_units, unit = unit0 - grp * group_units;
-      const int tile = unit / P.split_k, ks = unit - tile * P.split_k;
-      const int m_pair = tile % m_pairs, n_tile = tile / m_pairs;
+    for (int unit = pair; unit < units && live; unit += pairs, ++k) {
       const int buf = k & 1;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (k >> 1) & 1, abort_flag, 5));
+      // one warp asks for the accumulator, the others sleep on the named barrier
+      live = epi_bar(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (k >> 1) & 1, abort_flag, 5)));
       tc_fence_after();
-      const int row_base = (m_pair * 2 + (int)rank) * kBM + warp * 32;
-      const uint32_t taddr = tmem + buf * kBN + ((uint32_t)(warp * 32) << 16);
-      live = ok;
-      if (ok) gemm_epilogue(P, taddr, row_base, n_tile, reinterpret_cast<float *>(smem + kStages2 * kStageBytes2 + 256) + warp * 32 * kEpiPitch, lane, ks, grp);
+      const uint32_t taddr = tmem + buf * 256 + ((uint32_t)(quarter * 32) << 16);
+      if (live) gemm_epilogue(P, taddr, Unit(P, unit, nkb), rank, exchange, quarter, turn, lane);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(acc_empty + buf);
     }
   }
   // ---------------- teardown
+  __syncwarp();
   if (threadIdx.x == 0 && *abort_flag && P.status) atomicOr(reinterpret_cast<unsigned int *>(P.status), DPARA_STATUS_TIMEOUT);
   tc_fence_before();
   __syncthreads();
@@ -278,60 +336,85 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_tc
   if (warp == 5) tmem_dealloc_pair(tmem, 512);
 }
 
+// ------------------------------------------------------------------------------------------------ host
+namespace {
+int sm_count() {
+  int dev = 0, sms = kNumSM;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 1 ? sms : kNumSM;
+}
+
+struct PairPlan {
+  int t_tiles, nt;
+  double us;   // model
+};
+
+// Activation tiles for n_all weight tiles on `most` pairs.  A slab of a tile takes 0.12 + 0.21 nt / 256 us (fill and products; 0.33 at 256
+// rows), or what its weights take from HBM where no other pair reads them in the same round (0.385 when all pairs run), and a launch 6 us
+// beside them; narrower tiles are taken where they even out the rounds or use more pairs (200 x 6144 x 4096: 24 tiles of 208 rows 21.9 us,
+// 72 of 80 rows 18.5; 1152 x 5120 x 5120: 100 tiles of 240 rows are two rounds of the 74 pairs, the second a third full, 61 us; 140 of 176 rows two
+// rounds of 0.8 the length, 53 us).  Also tried: the tiles of the last rounds shared out by K, their pieces added through L2 by whoever finished
+// last: never faster than this (1152 x 5120 x 17408 165 us against 163, 256 x 151936 x 5120 360 against 355: what the chip saves in
+// idle time it gives back in clocks and in the pieces' traffic).
+PairPlan pair_plan(int M, int n_all, int nkb, int most) {
+  PairPlan best{};
+  best.us = -1;
+  const int t0 = (M + 255) / 256;
+  for (int t = t0; t < t0 + 4 && (t == t0 || (M + t - 1) / t > 64); ++t) {
+    const int nt = ((M + t - 1) / t + 15) / 16 * 16;
+    const long tiles = (long)n_all * t, rounds = (tiles + most - 1) / most;
+    double slab = 0.12 + 0.21 * nt / 256.0;
+    const double hbm = 0.385 * (tiles < most ? (double)tiles / most : 1.0) / t;
+    if (hbm > slab) slab = hbm;
+    const double us = 6.0 + rounds * nkb * slab;
+    if (best.us < 0 || us < 0.97 * best.us) { best.t_tiles = t; best.nt = nt; best.us = us; }
+  }
+  return best;
+}
+}  // namespace
+
 dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0) return DPARA_ERR_INVALID_ARG;
   if (g.K % kBK != 0 || g.N % 8 != 0) return DPARA_ERR_UNSUPPORTED;
   if (g.epi < 0 || g.epi > 3 || !g.a || !g.w || !g.out || (g.epi == 1 && !g.resid)) return DPARA_ERR_INVALID_ARG;
   if (!aligned16(g.a) || !aligned16(g.w) || !aligned16(g.out) || !aligned16(g.resid) || !aligned16(g.out_bf16)) return DPARA_ERR_INVALID_ARG;
-  // Few rows: the weights as the rows of the product.  Above 128 activation rows only where all tiles run at once (us, pairs / that:
-  // 200 rows, 4096 x 12288 64.5 / 33.7, 6144 x 4096 25.0 / 22.4; 288 rows, 4096 x 4096 29 / 19; but 192 rows, 151936 x 4096 in several
-  // rounds 271 / 326, one accumulator of 512 columns per CTA and nothing under its epilogue).
-  if (g.M <= 512) {
-    const SkinnyShape sh = skinny_shape(g);
-    if (sh.cost >= 0) return launch_gemm_skinny(g, sh, status, st);
-  }
+  if (g.n_groups > kGemmMaxGroups) return DPARA_ERR_UNSUPPORTED;
   GemmKernelParams P;
   const int w_rows = g.epi == 2 ? 2 * g.N : g.N;
-  int dev = 0, sms = kNumSM;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int split = g.split_k > 1 ? g.split_k : 1, groups = g.n_groups > 1 ? g.n_groups : 1;
-  // Tile width of the pair kernel: 192 columns when that evens out the rounds (QKV at 1024 x 6144: 96 tiles of 256 are two
-  // rounds of the 74 pairs, the second a third full; 128 tiles of 192 are two rounds of 0.75 the length).  A 192-wide tile
-  // pulls 28 KB per CTA and K slab for 0.75 of the flops of a 256-wide one: its rounds are weighted 1.14x.
-  P.bn = kBN;
-  if (g.M > kBM && g.epi != 2) {
-    const long m_pairs = (g.M + 2 * kBM - 1) / (2 * kBM), pairs = sms / 2 > 0 ? sms / 2 : 1;
-    const long u256 = m_pairs * ((g.N + 255) / 256) * split * groups, u192 = m_pairs * ((g.N + 191) / 192) * split * groups;
-    const double c256 = (double)((u256 + pairs - 1) / pairs) * 256.0, c192 = (double)((u192 + pairs - 1) / pairs) * 192.0 * 1.14;
-    if (c192 < 0.95 * c256) P.bn = 192;
+  const int cols = g.epi == 2 ? 128 : 256;   // output columns per tile
+  P.n_groups = g.n_groups > 1 ? g.n_groups : 1;
+  P.n_tiles = (g.N + cols - 1) / cols;
+  P.split_k = g.split_k > 1 ? g.split_k : 1;
+  const int nkb = g.K / kBK, n_all = P.n_tiles * P.n_groups * P.split_k;
+  if (P.split_k > 1 && (g.epi != 3 || P.split_k > nkb || g.perm_block)) return DPARA_ERR_UNSUPPORTED;
+  const int most = sm_count() / 2 < kNumSM / 2 ? sm_count() / 2 : kNumSM / 2;
+  const PairPlan plan = pair_plan(g.M, n_all, nkb / P.split_k, most);
+  // Few rows: single CTAs that share a tile's K range inside clusters.  Above 128 activation rows by the two models (us, pairs / that:
+  // 200 rows, 4096 x 12288 44.8 / 30.8, 4096 x 4096 19.8 / 16.1, 6144 x 4096 18.5 / 23.3; 400 rows, 4096 x 4096 21.1 / 22.8).
+  if (g.M <= 512) {
+    const SkinnyShape sh = skinny_shape(g);
+    if (sh.cost >= 0 && (g.M <= kManyRows || 1e-3 * sh.cost + 3.5 < plan.us)) return launch_gemm_skinny(g, sh, status, st);
   }
-  P.n_groups = 1;
-  if (g.n_groups > 1) {
-    // several products of one shape in one launch (fp32 stores, CTA pairs): entry 0 of the lists is (a, w, out)
-    if (g.epi != 3 || g.M <= kBM || g.n_groups > kGemmMaxGroups || g.perm_block) return DPARA_ERR_UNSUPPORTED;
-    P.n_groups = g.n_groups;
-  }
+  P.t_tiles = plan.t_tiles; P.nt = plan.nt;
   for (int gi = 0; gi < P.n_groups; ++gi) {
     const void *a = gi ? g.a_g[gi] : g.a, *w = gi ? g.w_g[gi] : g.w;
     void *o = gi ? g.out_g[gi] : g.out;
     if (!a || !w || !o || !aligned16(a) || !aligned16(w) || !aligned16(o)) return DPARA_ERR_INVALID_ARG;
-    if (!make_tmap_bf16_2d(&P.map_a[gi], a, g.K, g.M, (uint64_t)g.K * 2, kBK, kBM)) return DPARA_ERR_CUDA;
-    if (!make_tmap_bf16_2d(&P.map_b[gi], w, g.K, w_rows, (uint64_t)g.K * 2, kBK, P.bn == kBN ? 128 : P.bn / 2)) return DPARA_ERR_CUDA;
+    if (!make_tmap_bf16_2d(&P.map_w[gi], w, g.K, w_rows, (uint64_t)g.K * 2, kBK, g.epi == 2 ? kRows / 2 : kRows)) return DPARA_ERR_CUDA;
+    if (!make_tmap_bf16_2d(&P.map_a[gi], a, g.K, g.M, (uint64_t)g.K * 2, kBK, P.nt / 2)) return DPARA_ERR_CUDA;
     P.out_g[gi] = o;
   }
   P.M = g.M; P.N = g.N; P.K = g.K; P.epi = g.epi; P.up_row_offset = g.N;
-  P.out = g.out; P.resid = g.resid; P.resid_bf16 = g.resid_bf16; P.out_bf16 = g.out_bf16; P.status = status;
+  P.resid = g.resid; P.resid_bf16 = g.resid_bf16; P.out_bf16 = g.out_bf16; P.status = status;
   P.perm_block = g.epi == 3 ? g.perm_block : 0; P.perm_b = g.perm_b;
-  P.split_k = 1;
-  if (g.split_k > 1) {
-    if (g.epi != 3 || g.M <= kBM || g.split_k > g.K / kBK) return DPARA_ERR_UNSUPPORTED;
-    P.split_k = g.split_k;
-  }
-  const int tile_cols = g.epi == 2 ? 128 : P.bn;
-  if (cudaFuncSetAttribute(gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) != cudaSuccess) return DPARA_ERR_CUDA;
-  const int pair_tiles = ((g.N + tile_cols - 1) / tile_cols) * ((g.M + 2 * kBM - 1) / (2 * kBM)) * P.split_k * P.n_groups;
-  const int pairs = pair_tiles < sms / 2 ? pair_tiles : sms / 2;
-  launch_pdl(gemm_tc2_kernel, dim3(2 * pairs), dim3(kThreads), kSmemBytes2, st, P);
+  const int stage_bytes = kWBytes + P.nt * 64;
+  P.stages = (kSmemMax - 1024 - kBarBytes - kEpiBytes) / stage_bytes;
+  if (P.stages > kMaxStages) P.stages = kMaxStages;
+
+  const long units = (long)P.t_tiles * n_all;
+  const int smem = P.stages * stage_bytes + 1024 + kBarBytes + kEpiBytes;
+  if (cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return DPARA_ERR_CUDA;
+  launch_pdl(gemm_pair_kernel, dim3(2 * (unsigned)(units < most ? units : most)), dim3(kThreads), smem, st, P);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   return DPARA_OK;
