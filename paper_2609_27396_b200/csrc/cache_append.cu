@@ -38,20 +38,16 @@ struct AppendParams {
 __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) {
   extern __shared__ float s_cs[];  // cos[D/2], sin[D/2]
   const int n = blockIdx.x / P.J, i = blockIdx.x % P.J, tid = threadIdx.x, g = blockIdx.y;
-  pdl_wait();
-  pdl_launch_dependents();
+  // Outcome, length and angles before the wait: the kernel in front is the projection, which writes none of them, and it lets this one
+  // go only when everything before it has ended (256 rows, five layers: 57.0 -> 54.5 us).
   const uint16_t *knorm_w = P.knorm_w[g];
   const uint16_t *kv = P.kv + (size_t)g * P.part_stride;
   const float *kv_parts = P.kv_parts + (size_t)g * P.n_parts * P.part_stride;
   const int r = P.accept_len[n];
   const long long L = P.ctx_len[n];
-  if (r < 0 || r >= P.J || L + r + 1 > P.capacity[n]) {  // does not fit (or no valid outcome): the request is left alone
-    if (i == 0 && g == 0 && tid == 0 && P.status_word) atomicOr(reinterpret_cast<unsigned int *>(P.status_word), DPARA_STATUS_CACHE_FULL);
-    return;
-  }
-  if (i > r) return;  // rejected suffix: dropped
+  const bool fits = r >= 0 && r < P.J && L + r + 1 <= P.capacity[n];
   const int half = P.D / 2;
-  if (P.use_rope) {
+  if (P.use_rope && fits && i <= r) {
     const double pos = (double)(L + i);
     for (int d = tid; d < half; d += 128) {
       double sn, cs;
@@ -60,6 +56,13 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
       s_cs[half + d] = (float)sn;
     }
   }
+  pdl_wait();
+  pdl_launch_dependents();
+  if (!fits) {  // does not fit (or no valid outcome): the request is left alone
+    if (i == 0 && g == 0 && tid == 0 && P.status_word) atomicOr(reinterpret_cast<unsigned int *>(P.status_word), DPARA_STATUS_CACHE_FULL);
+    return;
+  }
+  if (i > r) return;  // rejected suffix: dropped
   __syncthreads();
   const int warp = tid >> 5, lane = tid & 31;
   const size_t row = (size_t)(P.row_start[n] + L + i);
