@@ -586,7 +586,7 @@ dpara_status launch_gemm_skinny(const GemmArgs &g, const SkinnyShape &sh, int32_
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = sh.split; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = sh.split > 1 ? 2 : 1;
   if (cudaLaunchKernelEx(&cfg, kernel, P) != cudaSuccess) { cudaGetLastError(); return DPARA_ERR_CUDA; }
   DPARA_CHECK_LAUNCH();
   count_launches(1);

@@ -5,7 +5,7 @@
 // The loop is d dependent steps, each a skinny product: all vocab rows of W (vocab x rank, bf16) against the b
 // embedding rows E(y_{i-1}) -- 0.6 GFLOP and one pass over W (78 MB at vocab 151 936, rank 256, which stays in
 // L2) per step.  ONE persistent cooperative kernel runs all d steps:
-//   warp 8      TMA producer: streams this CTA's 128-row tiles of W through a ring of shared-memory stages (the
+//   warp 8      TMA producer: streams this CTA's tiles of W (at most 128 rows) through a ring of shared-memory stages (the
 //               tiles do not depend on the tokens, so the ring runs ahead across steps), and with each tile the
 //               b x 128 block of base logits it will be added to (plain loads of those from the epilogue queued
 //               behind the deep W stream and cost 1.6 us each; as part of the stage they cost nothing);
@@ -45,7 +45,7 @@ __device__ __forceinline__ uint32_t head_key(float f) {
 
 struct ArParams {
   CUtensorMap map_w;
-  CUtensorMap map_l;          // base logits [block * b][vocab] fp32, box = 128 columns x nb rows
+  CUtensorMap map_l;          // base logits [block * b][vocab] fp32, box = one tile's columns x nb rows
   const float *logits;        // [block][b][vocab]: the rows one step reads are contiguous
   const uint16_t *ar_e;       // [vocab][rank]
   const int32_t *bonus;       // [b]
@@ -54,6 +54,7 @@ struct ArParams {
   unsigned int *barrier;      // zeroed before the launch
   int32_t *status;
   int b, block, vocab, rank, n_tiles, nb, stages;
+  int rows;                   // vocabulary rows per tile (<= 128, a multiple of 4)
   float *z_out;               // sampling: [b][vocab] fp32, the logits z of step `step0`
   int step0;                  // sampling: the one step this launch computes
 };
@@ -62,29 +63,28 @@ struct ArParams {
 // loop -- the same producer / MMA / epilogue pipeline, but the epilogue writes z = l + W E(y_prev) to P.z_out instead of
 // tracking maxima, the previous tokens come from P.next_tokens (written by the draw of the step before), and there is no
 // grid barrier (the draw is a launch of its own).
-template <bool kSample>
+template <bool kSample, int kSlabs>
 __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_constant__ ArParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tile_bytes = 128 * P.rank * 2;
   const int lg_bytes = P.nb * 128 * 4;                   // base logits of one tile: [nb rows][128 vocab entries] fp32
   const int stage_bytes = tile_bytes + lg_bytes;
-  const int slabs = P.rank / 64;
+  constexpr int slabs = kSlabs;                          // rank / 64
   uint8_t *sW = smem;                                    // ring of stages: W tile [slab][128 rows][128 B], then the logits block
   uint8_t *sE = smem + P.stages * stage_bytes;           // Ey: [slab][nb rows][128 B]
   uint64_t *bars = reinterpret_cast<uint64_t *>(sE + slabs * P.nb * 128);
-  uint64_t *full = bars, *empty = bars + 4, *acc_full = bars + 8, *acc_empty = bars + 10, *e_ready = bars + 12, *epi_bar = bars + 13;
+  uint64_t *full = bars, *empty = bars + 4, *acc_full = bars + 8, *acc_empty = bars + 10, *e_ready = bars + 12;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 14);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   int *s_tok = reinterpret_cast<int *>(tmem_slot + 2);   // [kMaxBatch] previous tokens of this step
   unsigned long long *s_red = reinterpret_cast<unsigned long long *>(s_tok + kMaxBatch);  // [4 warps][kMaxBatch]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < 4; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1 + kEpiWarps); }  // released by the MMA commit and the epilogue warps
     for (int a = 0; a < 2; ++a) { mbar_init(acc_full + a, 1); mbar_init(acc_empty + a, kEpiWarps); }
     mbar_init(e_ready, kEpiWarps);
-    mbar_init(epi_bar, kEpiWarps);
     *abort_flag = 0;
     fence_barrier_init();
   }
@@ -92,58 +92,69 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  pdl_wait();  // nothing above touches global memory
-  pdl_launch_dependents();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  // Nothing above touches global memory.  In the sampling loop's later steps the kernel in front is the draw of the step before, let
+  // go only when everything before it had ended: W and the base logits are there, and the producer fills its ring while the draw runs.  (The
+  // warps that read tokens and write z wait; only they let the next kernel go.)
+  if (!kSample || P.step0 == 0 || warp < kEpiWarps) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
   // this CTA's tiles: blockIdx.x, blockIdx.x + gridDim.x, ... (the same in every step)
   const int my_tiles = (P.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   const int step_begin = kSample ? P.step0 : 0, step_end = kSample ? P.step0 + 1 : P.block;
 
   if (warp == kProducerWarp) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0) {
-      prefetch_tensormap(&P.map_w);
-      int stage = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int step = step_begin; step < step_end && ok; ++step) {
-        for (int k = 0; k < my_tiles; ++k) {
-          ok = mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2);
-          if (!ok) break;
-          const int row0 = ((int)blockIdx.x + k * (int)gridDim.x) * 128;
-          mbar_arrive_expect_tx(full + stage, (uint32_t)stage_bytes);
-          for (int sb = 0; sb < slabs; ++sb) tma_load_2d(sW + stage * stage_bytes + sb * 16384, &P.map_w, full + stage, sb * 64, row0);
-          tma_load_2d(sW + stage * stage_bytes + tile_bytes, &P.map_l, full + stage, row0, step * P.b);
-          if (++stage == P.stages) { stage = 0; ph ^= 1u; }
+    // (this warp and the next: the whole warp walks the loop and waits, one lane issues; a wait inside a one-lane branch costs two to
+    // three times as many clocks)
+    prefetch_tensormap(&P.map_w);
+    int stage = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    const uint32_t tx = (uint32_t)(slabs * P.rows * 128 + P.nb * P.rows * 4);
+    for (int step = step_begin; step < step_end && ok; ++step) {
+      for (int k = 0; k < my_tiles; ++k) {
+        ok = __all_sync(0xffffffffu, mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2));
+        if (!ok) break;
+        const int row0 = ((int)blockIdx.x + k * (int)gridDim.x) * P.rows;
+        if (elect_one()) {
+          uint8_t *dst = sW + stage * stage_bytes;
+          mbar_arrive_expect_tx(full + stage, tx);
+#pragma unroll
+          for (int sb = 0; sb < slabs; ++sb) tma_load_2d(dst + sb * 16384, &P.map_w, full + stage, sb * 64, row0);
+          tma_load_2d(dst + tile_bytes, &P.map_l, full + stage, row0, step * P.b);
         }
+        __syncwarp();
+        if (++stage == P.stages) { stage = 0; ph ^= 1u; }
       }
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(128, P.nb, false, false);
-      const uint64_t wdesc0 = smem_desc_sw128(smem_u32(sW), 16, 1024);
-      const uint64_t edesc0 = smem_desc_sw128(smem_u32(sE), 16, 1024);
-      int stage = 0, kt = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int step = step_begin; step < step_end && ok; ++step) {
-        ok = mbar_wait(e_ready, (step - step_begin) & 1, abort_flag, 3);   // Ey of this step is in shared memory
-        for (int k = 0; k < my_tiles && ok; ++k, ++kt) {
-          const int buf = kt & 1;
-          ok = mbar_wait(acc_empty + buf, ((kt >> 1) & 1) ^ 1u, abort_flag, 4) && mbar_wait(full + stage, ph, abort_flag, 5);
-          if (!ok) break;
-          tc_fence_after();
-          const uint64_t wd = wdesc0 + (uint64_t)((stage * stage_bytes) >> 4);
-          for (int kk = 0; kk < P.rank / 16; ++kk) {
-            const uint32_t woff = ((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
-            const uint32_t eoff = ((kk >> 2) * (P.nb * 128) + (kk & 3) * 32) >> 4;
-            mma_ss(tmem + buf * kAccCols, wd + woff, edesc0 + eoff, idesc, kk > 0);
-          }
+    const uint32_t idesc = idesc_bf16_f32(128, P.nb, false, false);
+    const uint64_t desc = smem_desc_sw128(smem_u32(sW), 16, 1024);
+    const uint32_t w_lo0 = (uint32_t)desc, e_lo = w_lo0 + ((uint32_t)(sE - sW) >> 4), hi = (uint32_t)(desc >> 32);
+    const uint32_t e_slab = (uint32_t)(P.nb * 128) >> 4, stage_units = (uint32_t)stage_bytes >> 4;
+    int stage = 0, kt = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int step = step_begin; step < step_end && ok; ++step) {
+      ok = __all_sync(0xffffffffu, mbar_wait(e_ready, (step - step_begin) & 1, abort_flag, 3));   // Ey of this step is in shared memory
+      for (int k = 0; k < my_tiles && ok; ++k, ++kt) {
+        const int buf = kt & 1;
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + buf, ((kt >> 1) & 1) ^ 1u, abort_flag, 4) && mbar_wait(full + stage, ph, abort_flag, 5));
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t w_lo = w_lo0 + stage * stage_units;
+#pragma unroll
+          for (int kk = 0; kk < slabs * 4; ++kk)
+            mma_ss_lo(tmem + buf * kAccCols, w_lo + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4), e_lo + (kk >> 2) * e_slab + (kk & 3) * 2, hi, idesc, kk > 0);
           mma_commit(empty + stage);
           mma_commit(acc_full + buf);
-          if (++stage == P.stages) { stage = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == P.stages) { stage = 0; ph ^= 1u; }
       }
     }
   } else {
@@ -152,14 +163,16 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
     int kt = 0, stage = 0;
     bool ok = true;
-    uint32_t ph_epi = 0, ph_full = 0;
-    // barrier of the epilogue warps (bounded like every other wait; orders their shared-memory writes)
-    auto epi_sync = [&]() {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(epi_bar);
-      const bool r = __all_sync(0xffffffffu, mbar_wait(epi_bar, ph_epi, abort_flag, 8));
-      ph_epi ^= 1u;
-      return r;
+    uint32_t ph_full = 0;
+    // barrier of the epilogue warps (orders their shared-memory writes); all of them pass it with the same answer, so that they leave together
+    auto epi_sync = [&](bool good) {
+      uint32_t all;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+          "barrier.red.and.pred q, 1, 256, p;\n\t"
+          "selp.u32 %0, 1, 0, q;\n\t}"
+          : "=r"(all) : "r"((uint32_t)good) : "memory");
+      return all != 0;
     };
     for (int step = step_begin; step < step_end && ok; ++step) {
       // previous tokens: the bonus for the first step, else the winners of the previous step
@@ -184,8 +197,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         }
         s_tok[threadIdx.x] = tok;
       }
-      ok = epi_sync();
-      if (!ok) break;
+      epi_sync(true);
       // Ey[n][k] = E[tok_n][k] in the K-major 128-byte-swizzle layout the MMA reads: slab = k / 64, row n at
       // 128 B pitch, 16-byte chunk c of the row stored at chunk position c ^ (n & 7); rows n >= b are zero
       const int chunks_per_row = P.rank / 8;
@@ -215,18 +227,18 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty + buf);
-        const int v = ((int)blockIdx.x + k * (int)gridDim.x) * 128 + quarter * 32 + lane;
+        const int v = ((int)blockIdx.x + k * (int)gridDim.x) * P.rows + quarter * 32 + lane;
         // (acc_full implies the stage's loads have landed: the MMA issuer waited for them; this wait is the
         //  epilogue threads' own acquire of the TMA-written logits and returns at once)
         ok = __all_sync(0xffffffffu, mbar_wait(full + stage, ph_full, abort_flag, 9));
         if (!ok) break;
-        const bool live = v < P.vocab;
-        const float *sl = reinterpret_cast<const float *>(sW + stage * stage_bytes + tile_bytes) + quarter * 32 + lane;
+        const bool live = quarter * 32 + lane < P.rows && v < P.vocab;
+        const float *sl = reinterpret_cast<const float *>(sW + stage * stage_bytes + tile_bytes) + min(quarter * 32 + lane, P.rows - 1);
 #pragma unroll
         for (int j = 0; j < kMaxBatch / 2; ++j) {
           const int n = 2 * j + nh;
           if (n < P.b) {
-            const float z = __uint_as_float(nh ? acc[2 * j + 1] : acc[2 * j]) + sl[n * 128];
+            const float z = __uint_as_float(nh ? acc[2 * j + 1] : acc[2 * j]) + sl[n * P.rows];
             if (kSample) {
               if (live) P.z_out[(size_t)n * P.vocab + v] = z;       // a warp writes 32 consecutive entries of one row
             } else if (live && (z > bz[j] || (bv[j] < 0 && z == z))) {
@@ -239,7 +251,8 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         if (lane == 0) mbar_arrive(empty + stage);
         if (++stage == P.stages) { stage = 0; ph_full ^= 1u; }
       }
-      if (!ok || kSample) break;
+      if (kSample) break;
+      // (a warp whose wait ran out takes the others along at the next barrier)
       // step maximum: warp reduction, CTA reduction through shared memory, then ONE atomic per request and CTA,
       // each request on its own 128-byte line (atomics on one line are serialised by a single L2 unit)
 #pragma unroll
@@ -255,28 +268,31 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
           if (lane == 0) s_red[quarter * kMaxBatch + n] = x;
         }
       }
-      ok = epi_sync();
+      ok = epi_sync(ok);
       if (!ok) break;
-      if ((int)threadIdx.x < P.b) {
-        unsigned long long x = s_red[threadIdx.x];
+      // ---- grid barrier: every CTA's maxima of this step are in before anyone reads them.  Warp 0 leaves the CTA's and counts the CTA in,
+      // one lane polls; the others sleep on the named barrier.
+      if (warp == 0) {
+        if (lane < P.b) {
+          unsigned long long x = s_red[lane];
 #pragma unroll
-        for (int w = 1; w < 4; ++w) x = s_red[w * kMaxBatch + threadIdx.x] > x ? s_red[w * kMaxBatch + threadIdx.x] : x;
-        atomicMax(P.best + ((size_t)step * kMaxBatch + threadIdx.x) * kBestStride, x);
-      }
-      // ---- grid barrier: every CTA's maxima of this step are in before anyone reads them
-      __threadfence();
-      ok = epi_sync();
-      if (!ok) break;
-      if (threadIdx.x == 0) {
-        atomicAdd(P.barrier, 1u);
-        const unsigned int target = (unsigned int)(step + 1) * gridDim.x;
-        const uint64_t t0 = global_timer_ns();
-        while (*reinterpret_cast<volatile unsigned int *>(P.barrier) < target) {
-          if (*abort_flag || global_timer_ns() - t0 > kWaitLimitNs) { *abort_flag = 7; break; }
+          for (int w = 1; w < 4; ++w) x = s_red[w * kMaxBatch + lane] > x ? s_red[w * kMaxBatch + lane] : x;
+          atomicMax(P.best + ((size_t)step * kMaxBatch + lane) * kBestStride, x);
+          __threadfence();
         }
-        __threadfence();
+        __syncwarp();
+        if (lane == 0) {
+          atomicAdd(P.barrier, 1u);
+          const unsigned int target = (unsigned int)(step + 1) * gridDim.x;
+          const uint64_t t0 = global_timer_ns();
+          for (unsigned int tries = 1; *reinterpret_cast<volatile unsigned int *>(P.barrier) < target; ++tries) {
+            if (tries % 64 == 0 && (*abort_flag || global_timer_ns() - t0 > kWaitLimitNs)) { *abort_flag = 7; break; }
+          }
+          __threadfence();
+        }
+        __syncwarp();
       }
-      ok = epi_sync() && !*abort_flag;
+      ok = epi_sync(!*abort_flag);
     }
     // the last step's winners
     if (!kSample && ok && blockIdx.x == 0 && (int)threadIdx.x < P.b) {
@@ -514,21 +530,28 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
 
   ArParams P;
   memset(&P, 0, sizeof(P));
-  if (!make_tmap_bf16_2d(&P.map_w, h.ar_w, h.rank, h.vocab, (uint64_t)h.rank * 2, 64, 128)) return DPARA_ERR_CUDA;
-  if (!make_tmap_f32_2d(&P.map_l, logits, h.vocab, (uint64_t)h.block * h.b, (uint64_t)h.vocab * 4, 128, h.b <= 16 ? 16 : 32)) return DPARA_ERR_CUDA;
+  // Tile height: as many rounds of the SMs as 128-row tiles take, evenly filled (vocabulary 151936: 1187 tiles of 128 are eight rounds of
+  // the 148 SMs and three tiles; 1310 of 116 are nine rounds of 0.9 the length), but not under 32 rows.
+  int dev = 0, sms = kNumSM;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int rounds = ((h.vocab + 127) / 128 + sms - 1) / sms;
+  P.rows = ((h.vocab + sms * rounds - 1) / (sms * rounds) + 3) / 4 * 4;
+  if (P.rows < 32) P.rows = 32;
+  if (!make_tmap_bf16_2d(&P.map_w, h.ar_w, h.rank, h.vocab, (uint64_t)h.rank * 2, 64, P.rows)) return DPARA_ERR_CUDA;
+  if (!make_tmap_f32_2d(&P.map_l, logits, h.vocab, (uint64_t)h.block * h.b, (uint64_t)h.vocab * 4, P.rows, h.b <= 16 ? 16 : 32)) return DPARA_ERR_CUDA;
   P.logits = logits; P.ar_e = static_cast<const uint16_t *>(h.ar_e); P.bonus = h.bonus; P.next_tokens = h.next_tokens;
   P.best = best; P.barrier = barrier; P.status = status;
   P.b = h.b; P.block = h.block; P.vocab = h.vocab; P.rank = h.rank;
-  P.n_tiles = (h.vocab + 127) / 128;
+  P.n_tiles = (h.vocab + P.rows - 1) / P.rows;
   P.nb = h.b <= 16 ? 16 : 32;
   const int stage_bytes = 128 * h.rank * 2 + P.nb * 128 * 4;
   const int fixed = (h.rank / 64) * P.nb * 128 + 1024 + 2048;   // Ey, alignment slack, barriers and reduction scratch
   P.stages = (227 * 1024 - fixed) / stage_bytes > 4 ? 4 : (227 * 1024 - fixed) / stage_bytes;
   const int smem = P.stages * stage_bytes + fixed;
-  if (cudaFuncSetAttribute(ar_head_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(ar_head_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return DPARA_ERR_CUDA;
-  int dev = 0, sms = kNumSM;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  void (*const kernels[2][4])(ArParams) = {{ar_head_kernel<false, 1>, ar_head_kernel<false, 2>, ar_head_kernel<false, 3>, ar_head_kernel<false, 4>},
+                                           {ar_head_kernel<true, 1>, ar_head_kernel<true, 2>, ar_head_kernel<true, 3>, ar_head_kernel<true, 4>}};
+  void (*const kernel)(ArParams) = kernels[h.uniforms ? 1 : 0][h.rank / 64 - 1];
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return DPARA_ERR_CUDA;
   const int grid = P.n_tiles < sms ? P.n_tiles : sms;
   if (h.uniforms) {
     // ---- sampling: per step the logits z (one-step head kernel), then the draw.  The tickets live in the zeroed 256 bytes
@@ -539,7 +562,7 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
     P.z_out = zstep;
     for (int i = 0; i < h.block; ++i) {
       P.step0 = i;
-      launch_pdl(ar_head_kernel<true>, dim3(grid), dim3(kThreads), (size_t)smem, st, P);
+      launch_pdl(kernel, dim3(grid), dim3(kThreads), (size_t)smem, st, P);
       DPARA_CHECK_LAUNCH();
       launch_pdl(head_sample_kernel, dim3(n_chunks, h.b), dim3(kPickThreads), 0, st, static_cast<const float *>(zstep), h.uniforms, h.next_tokens, part, tick, h.vocab, h.block, i, chunk);
       DPARA_CHECK_LAUNCH();
@@ -549,7 +572,7 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   }
   // cooperative launch: the grid barrier needs every CTA resident (one CTA per SM fits by construction)
   void *args[] = {&P};
-  if (cudaLaunchCooperativeKernel(reinterpret_cast<void *>(ar_head_kernel<false>), dim3(grid), dim3(kThreads), args, smem, st) != cudaSuccess) {
+  if (cudaLaunchCooperativeKernel(reinterpret_cast<void *>(kernel), dim3(grid), dim3(kThreads), args, smem, st) != cudaSuccess) {
     cudaGetLastError();
     return DPARA_ERR_CUDA;
   }
