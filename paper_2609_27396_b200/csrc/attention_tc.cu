@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *merge_flag = reinterpret_cast<volatile int *>(tmem_slot + 2);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // this CTA's items: its slice of the host-built schedule, else items blockIdx.x, blockIdx.x + gridDim.x, ...
   const int team = P.use_seg ? (int)blockIdx.x / P.seg_X : 0;  // (CTAs behind the last whole team have no work)
   const int q_begin = P.use_seg ? (team < P.seg_teams ? (int)P.team_first[team] : 0) : (P.use_sched ? (int)P.cta_first[blockIdx.x] : (int)blockIdx.x);
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       // the Q buffer is free once the previous item's last QK has completed
       ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (k & 1) ^ 1u, abort_flag));
       if (!ok) break;
-      if (lane == 0) {
+      if (elect_one()) {
         const int qrow0 = I.n * A.q_req_rows + A.lo * A.Bq;
         mbar_arrive_expect_tx(q_full, (uint32_t)(I.ntq * Cfg::kTileBytes));
         for (int t = 0; t < I.ntq; ++t) {
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         if (!ok) break;
         uint8_t *dst = sKV + sl * Cfg::kTileBytes;
         if (it < I.n_ctx_it) {
-          if (lane == 0) {
+          if (elect_one()) {
             const int row = (int)(I.c0 + (long long)(I.t0 + it) * 128);
             mbar_arrive_expect_tx(kv_full + sl, Cfg::kTileBytes);
             for (int sb = 0; sb < Cfg::kSlabs; ++sb)
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             fence_proxy_async();
             __syncwarp();
           }
-          if (lane == 0) {
+          if (elect_one()) {
             const int tk = it - I.n_ctx_it;  // tail tile 0: spine rows, then cap0 blocks; tail tile k >= 1: cap blocks
             if (tk == 0) {
               uint32_t bytes = 0;
@@ -445,7 +445,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     // and the issuing thread spends the block's whole execution time issuing it (the queue is shallow); with
     // one thread per tile, one tile's waits and commits overlap the other tile's products and the tensor pipe
     // stays fed.  The two threads meet only through barriers (the S hand-off below, the K/V ring).
-    if (lane == 0) {
+    // The whole warp walks the loop and waits, one lane issues: a wait inside a one-lane branch costs 190..310 clocks when its barrier is
+    // already there, ~95 by a converged warp, and three of them sit on every iteration's chain from scores
+    // to weighted sums (16 requests, 14B-shaped: step 217 -> 211 us; one request 25.8 -> 24.5; four of 32 K context: block 757 -> 746).
+    {
       const int ti = warp - 9;
       constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, false, false);
       constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
@@ -460,43 +463,49 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       bool ok = true, first_qk = (ti == 0);
       auto next_load = [&](int &slot_out) {  // wait for the next tile of the K/V ring (both issuers take every tile, in order)
         slot_out = ring_slot;
-        const bool r = mbar_wait(kv_full + ring_slot, ring_phase, abort_flag, 2);
+        const bool r = __all_sync(0xffffffffu, mbar_wait(kv_full + ring_slot, ring_phase, abort_flag, 2));
         if (++ring_slot == kSlots) { ring_slot = 0; ring_phase ^= 1u; }
         return r;
       };
       // The S buffer comes back from whichever tile's softmax warps loaded it last (also across items).
       auto wait_s_free = [&]() {
         if (first_qk) { first_qk = false; return true; }
-        const bool r = mbar_wait(sf, ph_sf, abort_flag, 3);
+        const bool r = __all_sync(0xffffffffu, mbar_wait(sf, ph_sf, abort_flag, 3));
         ph_sf ^= 1u;
         return r;
       };
       auto issue_qk = [&](int kslot, bool last_it) {
         const uint64_t ka = kdesc0 + (uint64_t)(kslot * kTile16);
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t off = ((kk >> 2) * Cfg::kSlabBytes + (kk & 3) * 32) >> 4;
-          if (kk == 0) mma_ss_c<false>(s_t, qdesc + off, ka + off, idesc_qk);
-          else mma_ss_c<true>(s_t, qdesc + off, ka + off, idesc_qk);
+          for (int kk = 0; kk < D / 16; ++kk) {
+            const uint32_t off = ((kk >> 2) * Cfg::kSlabBytes + (kk & 3) * 32) >> 4;
+            if (kk == 0) mma_ss_c<false>(s_t, qdesc + off, ka + off, idesc_qk);
+            else mma_ss_c<true>(s_t, qdesc + off, ka + off, idesc_qk);
+          }
+          mma_commit(s_full + ti);
+          mma_commit(kv_empty + kslot);        // this tile is done with the K tile
+          if (last_it) mma_commit(q_empty);    // ... and with its Q tile
         }
-        mma_commit(s_full + ti);
-        mma_commit(kv_empty + kslot);        // this tile is done with the K tile
-        if (last_it) mma_commit(q_empty);    // ... and with its Q tile
+        __syncwarp();
       };
       auto issue_pv = [&](int vslot, bool acc) {
         const uint64_t va = vdesc0 + (uint64_t)(vslot * kTile16);
-        mma_ts(o_t, p_t, va, idesc_pv, acc);
+        if (elect_one()) {
+          mma_ts(o_t, p_t, va, idesc_pv, acc);
 #pragma unroll
-        for (int kk = 1; kk < 8; ++kk) mma_ts_c<true>(o_t, p_t + kk * 8, va + (uint64_t)(kk * (2048 >> 4)), idesc_pv);
-        mma_commit(pv_done + ti);
-        mma_commit(kv_empty + vslot);
+          for (int kk = 1; kk < 8; ++kk) mma_ts_c<true>(o_t, p_t + kk * 8, va + (uint64_t)(kk * (2048 >> 4)), idesc_pv);
+          mma_commit(pv_done + ti);
+          mma_commit(kv_empty + vslot);
+        }
+        __syncwarp();
       };
       for (int qi = q_begin; qi < q_end && ok; qi += q_step) {
       const Item I = fetch_item(P, qi);
         if (I.n_iter == 0) continue;
         const int n_iter = I.n_iter;
         int kslot = 0, vslot = 0;
-        ok = mbar_wait(q_full, k & 1, abort_flag, 4);
+        ok = __all_sync(0xffffffffu, mbar_wait(q_full, k & 1, abort_flag, 4));
         ++k;
         if (!ok) break;
         if (ti >= I.ntq) {
@@ -504,9 +513,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           // after its load has landed, so this thread cannot run ahead of the other issuer by a ring cycle)
           for (int q = 0; q < 2 * n_iter && ok; ++q) {
             ok = next_load(kslot);
-            if (ok) mbar_arrive(kv_empty + kslot);
+            if (ok && elect_one()) mbar_arrive(kv_empty + kslot);
+            __syncwarp();
           }
-          if (ok) mbar_arrive(q_empty);
+          if (ok && elect_one()) mbar_arrive(q_empty);
+          __syncwarp();
           continue;
         }
         // per iteration: QK(it + 1), then PV(it) -- the scores of the next iteration are issued as soon as
@@ -522,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             tc_fence_after();
             issue_qk(kslot, it + 2 == n_iter);
           }
-          ok = next_load(vslot) && mbar_wait(p_full + ti, ph_p, abort_flag, 5);
+          ok = next_load(vslot) && __all_sync(0xffffffffu, mbar_wait(p_full + ti, ph_p, abort_flag, 5));
           ph_p ^= 1u;
           if (!ok) break;
           tc_fence_after();
