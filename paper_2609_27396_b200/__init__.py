@@ -106,6 +106,22 @@ def gemm_bf16(a, w, *, epilogue: int = 0, resid=None, want_bf16_copy: bool = Fal
     return (out, out16, st) if out16 is not None else (out, st)
 
 
+lib.dpara_gemm_route.restype = C.c_int
+lib.dpara_gemm_route.argtypes = [C.c_int32] * 8 + [C.POINTER(C.c_int32)]
+EXPORTED.append("dpara_gemm_route")
+
+GEMM_ROUTE = ("few_rows", "tile_rows", "operands", "weight_rows", "ctas", "rounds", "chunk", "slabs")
+
+
+def gemm_route(M: int, N: int, K: int, *, epilogue: int = 0, n_groups: int = 1, split_k: int = 1, row_order: bool = False, one_chain: bool = False):
+    """dpara_gemm_route: the kernel and tiles that a product of these sizes takes, by name (no launch)."""
+    route = (C.c_int32 * 8)()
+    rc = lib.dpara_gemm_route(M, N, K, epilogue, n_groups, split_k, int(row_order), int(one_chain), route)
+    if rc != OK:
+        raise DparaError(rc)
+    return dict(zip(GEMM_ROUTE, route))
+
+
 lib.dpara_selftest_bounded_wait.restype = C.c_int
 lib.dpara_selftest_bounded_wait.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p]
 EXPORTED.append("dpara_selftest_bounded_wait")

@@ -138,7 +138,24 @@ extern "C" int32_t dpara_version(void) { return 1000; }
 
 extern "C" int64_t dpara_kernel_launches(void) { return g_launches.load(std::memory_order_relaxed); }
 
-#include "gemm.cuh"
+#include "gemm_skinny.cuh"
+
+extern "C" dpara_status dpara_gemm_route(int32_t M, int32_t N, int32_t K, int32_t epilogue, int32_t n_groups, int32_t split_k, int32_t row_order,
+                                         int32_t one_chain, int32_t route[8]) {
+  if (!route || n_groups < 1 || split_k < 1) return DPARA_ERR_INVALID_ARG;
+  GemmArgs g{};
+  g.M = M; g.N = N; g.K = K; g.epi = epilogue; g.n_groups = n_groups; g.split_k = split_k; g.one_chain = one_chain;
+  g.perm_block = row_order ? 1 : 0; g.perm_b = g.M;
+  GemmRoute r;
+  const dpara_status s = gemm_route(g, r);
+  if (s != DPARA_OK) return s;
+  const SkinnyShape &k = r.skinny;
+  const long units = r.few ? (long)k.tiles * n_groups : (long)r.n_all * r.pair.t_tiles, at_once = r.few ? k.clusters : r.most;
+  const int rounds = (int)((units + at_once - 1) / at_once);
+  const int few[8] = {1, k.T, k.halves, k.rows, k.split, rounds, k.chunk, k.slabs}, pairs[8] = {0, r.pair.nt, 1, 256, 2, rounds, r.pair.nt, 1};
+  for (int i = 0; i < 8; ++i) route[i] = r.few ? few[i] : pairs[i];
+  return DPARA_OK;
+}
 
 extern "C" dpara_status dpara_gemm_bf16(const dpara_gemm_io *io, int32_t *status_word, void *stream) {
   if (!io) return DPARA_ERR_INVALID_ARG;

@@ -12,6 +12,20 @@ struct SkinnyShape {
   int chunk, stages, slabs, ring_bytes, bar_offset, smem, tmem_cols;
 };
 SkinnyShape skinny_shape(const GemmArgs &g);
+
+struct PairPlan {
+  int t_tiles, nt;   // tiles of activation rows of one product, rows of each
+  double us;         // model
+};
+
+// The kernel and the tiles of a launch, from its sizes (no pointer is looked at).
+struct GemmRoute {
+  int few;               // the kernel for few rows, with `skinny`; else CTA pairs, with `pair`
+  SkinnyShape skinny;
+  PairPlan pair;
+  int n_tiles, n_all, most;   // CTA pairs: weight tiles of one product, of all products and parts of K; pairs of the device
+};
+dpara_status gemm_route(const GemmArgs &g, GemmRoute &r);
 dpara_status launch_gemm_skinny(const GemmArgs &g, const SkinnyShape &sh, int32_t *status, cudaStream_t st);
 
 }  // namespace dpara

@@ -344,11 +344,6 @@ int sm_count() {
   return sms > 1 ? sms : kNumSM;
 }
 
-struct PairPlan {
-  int t_tiles, nt;
-  double us;   // model
-};
-
 // Activation tiles for n_all weight tiles on `most` pairs.  A slab of a tile takes 0.12 + 0.21 nt / 256 us (fill and products; 0.33 at 256
 // rows), or what its weights take from HBM where no other pair reads them in the same round (0.385 when all pairs run), and a launch 6 us
 // beside them; narrower tiles are taken where they even out the rounds or use more pairs (200 x 6144 x 4096: 24 tiles of 208 rows 21.9 us,
@@ -373,29 +368,42 @@ PairPlan pair_plan(int M, int n_all, int nkb, int most) {
 }
 }  // namespace
 
-dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st) {
-  if (g.M <= 0 || g.N <= 0 || g.K <= 0) return DPARA_ERR_INVALID_ARG;
-  if (g.K % kBK != 0 || g.N % 8 != 0) return DPARA_ERR_UNSUPPORTED;
-  if (g.epi < 0 || g.epi > 3 || !g.a || !g.w || !g.out || (g.epi == 1 && !g.resid)) return DPARA_ERR_INVALID_ARG;
-  if (!aligned16(g.a) || !aligned16(g.w) || !aligned16(g.out) || !aligned16(g.resid) || !aligned16(g.out_bf16)) return DPARA_ERR_INVALID_ARG;
-  if (g.n_groups > kGemmMaxGroups) return DPARA_ERR_UNSUPPORTED;
-  GemmKernelParams P;
-  const int w_rows = g.epi == 2 ? 2 * g.N : g.N;
+// Everything about a launch that its sizes decide: refusals, then the kernel and its tiles.
+dpara_status gemm_route(const GemmArgs &g, GemmRoute &r) {
+  if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.epi < 0 || g.epi > 3) return DPARA_ERR_INVALID_ARG;
+  if (g.K % kBK != 0 || g.N % 8 != 0 || g.n_groups > kGemmMaxGroups) return DPARA_ERR_UNSUPPORTED;
+  // (one residual, one bf16 copy and one row order for all products of a launch)
+  if (g.n_groups > 1 && ((g.epi != 0 && g.epi != 3) || g.perm_block)) return DPARA_ERR_UNSUPPORTED;
+  const int nkb = g.K / kBK;
+  if (g.split_k > 1 && (g.epi != 3 || g.M <= kManyRows || g.split_k > nkb || g.perm_block)) return DPARA_ERR_UNSUPPORTED;
   const int cols = g.epi == 2 ? 128 : 256;   // output columns per tile
-  P.n_groups = g.n_groups > 1 ? g.n_groups : 1;
-  P.n_tiles = (g.N + cols - 1) / cols;
-  P.split_k = g.split_k > 1 ? g.split_k : 1;
-  const int nkb = g.K / kBK, n_all = P.n_tiles * P.n_groups * P.split_k;
-  if (P.split_k > 1 && (g.epi != 3 || P.split_k > nkb || g.perm_block)) return DPARA_ERR_UNSUPPORTED;
-  const int most = sm_count() / 2 < kNumSM / 2 ? sm_count() / 2 : kNumSM / 2;
-  const PairPlan plan = pair_plan(g.M, n_all, nkb / P.split_k, most);
+  r.n_tiles = (g.N + cols - 1) / cols;
+  r.n_all = r.n_tiles * (g.n_groups > 1 ? g.n_groups : 1) * (g.split_k > 1 ? g.split_k : 1);
+  r.most = sm_count() / 2 < kNumSM / 2 ? sm_count() / 2 : kNumSM / 2;
+  r.pair = pair_plan(g.M, r.n_all, nkb / (g.split_k > 1 ? g.split_k : 1), r.most);
   // Few rows: single CTAs that share a tile's K range inside clusters.  Above 128 activation rows by the two models (us, pairs / that:
   // 200 rows, 4096 x 12288 44.8 / 30.8, 4096 x 4096 19.8 / 16.1, 6144 x 4096 18.5 / 23.3; 400 rows, 4096 x 4096 21.1 / 22.8).
+  r.few = 0;
   if (g.M <= 512) {
-    const SkinnyShape sh = skinny_shape(g);
-    if (sh.cost >= 0 && (g.M <= kManyRows || 1e-3 * sh.cost + 3.5 < plan.us)) return launch_gemm_skinny(g, sh, status, st);
+    r.skinny = skinny_shape(g);
+    r.few = r.skinny.cost >= 0 && (g.M <= kManyRows || 1e-3 * r.skinny.cost + 3.5 < r.pair.us);
   }
-  P.t_tiles = plan.t_tiles; P.nt = plan.nt;
+  return DPARA_OK;
+}
+
+dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st) {
+  GemmRoute route;
+  const dpara_status checked = gemm_route(g, route);
+  if (checked != DPARA_OK) return checked;
+  if (!g.a || !g.w || !g.out || (g.epi == 1 && !g.resid)) return DPARA_ERR_INVALID_ARG;
+  if (!aligned16(g.a) || !aligned16(g.w) || !aligned16(g.out) || !aligned16(g.resid) || !aligned16(g.out_bf16)) return DPARA_ERR_INVALID_ARG;
+  if (route.few) return launch_gemm_skinny(g, route.skinny, status, st);
+  GemmKernelParams P;
+  const int w_rows = g.epi == 2 ? 2 * g.N : g.N;
+  P.n_groups = g.n_groups > 1 ? g.n_groups : 1;
+  P.split_k = g.split_k > 1 ? g.split_k : 1;
+  P.n_tiles = route.n_tiles;
+  P.t_tiles = route.pair.t_tiles; P.nt = route.pair.nt;
   for (int gi = 0; gi < P.n_groups; ++gi) {
     const void *a = gi ? g.a_g[gi] : g.a, *w = gi ? g.w_g[gi] : g.w;
     void *o = gi ? g.out_g[gi] : g.out;
@@ -411,10 +419,10 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
   P.stages = (kSmemMax - 1024 - kBarBytes - kEpiBytes) / stage_bytes;
   if (P.stages > kMaxStages) P.stages = kMaxStages;
 
-  const long units = (long)P.t_tiles * n_all;
+  const long units = (long)P.t_tiles * route.n_all;
   const int smem = P.stages * stage_bytes + 1024 + kBarBytes + kEpiBytes;
   if (cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return DPARA_ERR_CUDA;
-  launch_pdl(gemm_pair_kernel, dim3(2 * (unsigned)(units < most ? units : most)), dim3(kThreads), smem, st, P);
+  launch_pdl(gemm_pair_kernel, dim3(2 * (unsigned)(units < route.most ? units : route.most)), dim3(kThreads), smem, st, P);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   return DPARA_OK;

@@ -4,6 +4,8 @@ import ctypes as C
 import os
 import re
 
+import pytest
+
 import paper_2609_27396_b200 as dp
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -69,3 +71,24 @@ def test_verify_argument_validation():
     assert dp.lib.dpara_verify_select(C.byref(io4), None, 0, None, None) == dp.ERR_INVALID_ARG      # sampling needs uniforms
     io5 = dp.VerifyIO(2, 4, 100, 2, 8, 7)
     assert dp.lib.dpara_verify_workspace_bytes(C.byref(io5)) == 0                                   # bad mode
+
+
+@pytest.mark.parametrize("kw", [
+    dict(M=256, epilogue=1, n_groups=2),                      # one residual for all products
+    dict(M=256, epilogue=2, n_groups=2),
+    dict(M=256, epilogue=3, n_groups=2, row_order=True),
+    dict(M=128, epilogue=3, split_k=2),                       # the kernel for few rows takes no planes
+    dict(M=256, epilogue=0, split_k=2),
+    dict(M=256, epilogue=3, split_k=2, row_order=True),
+    dict(M=256, epilogue=3, split_k=9),                       # more parts than 64-column slabs of K
+    dict(M=256, epilogue=0, n_groups=9),
+])
+def test_gemm_launches_that_are_refused(kw):
+    with pytest.raises(dp.DparaError) as e:
+        dp.gemm_route(N=512, K=512, **kw)
+    assert e.value.code == dp.ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("kw", [dict(M=256, epilogue=3, n_groups=8, split_k=4), dict(M=8, epilogue=0, n_groups=8, one_chain=True), dict(M=256, epilogue=3, row_order=True)])
+def test_gemm_launches_that_are_taken(kw):
+    assert dp.gemm_route(N=512, K=512, **kw)["rounds"] >= 1
