@@ -8,8 +8,10 @@
 // above the weights' 7.7 / 5.1 / 31 / 15 us at the copy rate: ~1.4 us from the wait to the first products, ~3 us behind the last.  Here
 //   * a tile is one or two operands of R <= 128 weight rows (any multiple of 8: the 128-row operand behind R only makes
 //     accumulator lanes that nobody reads), so that the tiles come out at a whole number of rounds over the SMs;
-//   * a CLUSTER of S CTAs shares a tile, each over its part of K; the parts meet through distributed shared memory, in the order
-//     of the ranks (the same sum every time), and every CTA stores its share of the activation rows;
+//   * where all tiles run at once, a CLUSTER of S CTAs shares a tile, each over its part of K; the parts meet through distributed shared
+//     memory, in the order of the ranks (the same sum every time), and every CTA stores its share of the activation rows.  Not
+//     with several rounds of tiles: the parts' meeting is not hidden behind the next tile (100 rows, 10240 x 5120: 46.0 us in three rounds of
+//     four CTAs a tile, 25.2 in one of single CTAs; 128 rows, 20480 x 8192: 93 and 70), and over 31 shapes it gained 4 % at most;
 //   * a stage of the ring holds the tile's weight rows and T activation rows (M rounded up to 16) of one or two 64-column slabs of K,
 //     one TMA copy per operand.  The stage's barrier and loop cost ~250 clocks of the issuing warp beside 40..60 per product: with one
 //     slab (four products) of a small tile that is more than the products themselves (16 rows, 4096 x 4096: 13.0 -> 11.2 us with two);
@@ -47,7 +49,7 @@ struct SkinnyParams {
   // operands per tile: rows [0, rows) and [rows, 2 rows) of the tile; SwiGLU (always 2): gate rows and up rows
   int out_cols;     // output columns per tile
   int tiles;        // tiles of one product
-  int split;        // cluster size
+  int split;        // cluster size; above 1 only with one round
   int stages, chunk;
   int ring_bytes, bar_offset;
   int w_ready;
@@ -231,9 +233,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + P.bar_offset);
   uint64_t *empty = full + 16;
   uint64_t *acc_full = empty + 16, *acc_empty = acc_full + 2;
-  uint64_t *ready = acc_empty + 2;   // every CTA of the cluster has left its part of this chunk in its buffer
-  uint64_t *freed = ready + 1;       // ... and has read this CTA's
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(freed + 1);
+  uint64_t *ready = acc_empty + 2;   // every CTA of the cluster has left its part in its buffer
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ready + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
   // (through a shuffle: the compiler then knows that these are the same in the whole warp, and works out descriptors and addresses of
@@ -260,7 +261,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
       mbar_init(acc_empty + b, kEpiWarps);
     }
     mbar_init(ready, S);
-    mbar_init(freed, S);
     *abort_flag = 0;
     fence_barrier_init();
   }
@@ -375,7 +375,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
     const uint32_t part_addr = smem_u32(part);
     const int ew = warp < 4 ? warp : warp - 2, quarter = warp & 3;   // epilogue warp 0..7; the TMEM lanes it may read
     int k = 0;
-    uint32_t chunk_no = 0;
     bool live = true;
     for (int unit = cluster; unit < total && live; unit += n_clusters, ++k) {
       const int grp = unit / P.tiles, tile = unit - grp * P.tiles;
@@ -386,10 +385,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
       tc_fence_after();
       const uint32_t taddr = tmem + buf * buf_cols + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-      for (int c0 = 0; c0 < P.T; c0 += P.chunk, ++chunk_no) {
+      for (int c0 = 0; c0 < P.T; c0 += P.chunk) {
         // ---- this CTA's part of activation rows [c0, c0 + chunk) into its buffer, once the last one has been read
-        if (S > 1 && !P.one_round) live = epilogue_bar(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(freed, (chunk_no & 1) ^ 1u, abort_flag, 5))));
-        else if (!P.one_round) named_bar_sync(1, kEpiThreads);
+        if (!P.one_round) named_bar_sync(1, kEpiThreads);
         const int n_here = min(P.chunk, P.T - c0);
         int piece = 0;   // 32 columns each, handed out to the two warps of a TMEM quarter in turn
 #pragma unroll 1
@@ -413,7 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
         live = epilogue_bar(live);
         if (S > 1) {
           if (threadIdx.x < S) mbar_arrive_rank(ready, threadIdx.x);
-          live = epilogue_bar(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(ready, chunk_no & 1, abort_flag, 6))));
+          live = epilogue_bar(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(ready, 0, abort_flag, 6))));
         }
         const int rows_here = min(P.M - c0, n_here);
         if (live) {
@@ -421,10 +419,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
                             P.epi == 2 ? 1 : kHalves, P.epi, P.resid_bf16, P.perm_block, P.perm_b};
           if (S == 1) sk_finish<4, false>(f);
           else sk_finish<2, true>(f);
-        }
-        if (S > 1 && !P.one_round) {
-          live = epilogue_bar(live);   // this CTA has read everybody's part
-          if (threadIdx.x < S) mbar_arrive_rank(freed, threadIdx.x);
         }
       }
     }
@@ -533,7 +527,7 @@ SkinnyShape skinny_shape(const GemmArgs &g) {
         sh.clusters = units < cap[s] ? (int)units : cap[s];
         const long rounds = (units + sh.clusters - 1) / sh.clusters;
         sh.one_round = rounds == 1;
-        if (!sh.one_round && g.M > kManyRows) break;   // (the caller takes such shapes to the CTA pairs)
+        if (!sh.one_round && (s > 1 || g.M > kManyRows)) break;   // (more rows: the caller takes such shapes to the CTA pairs)
         if (!skinny_layout(sh, nkb)) continue;
         const double w_bytes = rows * halves * 128.0, active = (double)sh.clusters * s;
         const double bytes = w_bytes + T * 128.0;
@@ -542,7 +536,7 @@ SkinnyShape skinny_shape(const GemmArgs &g) {
           if (other > slab) slab = other;
         const double tail = 1000 + 15.0 * T * halves, more = rounds - 1;
         const int stages_k = (nkb + sh.slabs - 1) / sh.slabs;
-        sh.cost = rounds * ((stages_k + s - 1) / s * sh.slabs) * slab + tail * (1.0 + 0.2 * more) + (s > 1 ? 800.0 + 150.0 * s + 300.0 * more : 0.0) + (s > 1 && s % 2 ? 1500.0 : 0.0);
+        sh.cost = rounds * ((stages_k + s - 1) / s * sh.slabs) * slab + tail * (1.0 + 0.2 * more) + (s > 1 ? 800.0 + 150.0 * s : 0.0) + (s > 1 && s % 2 ? 1500.0 : 0.0);
         if (best.cost < 0 || sh.cost < best.cost) best = sh;
       }
     }
@@ -565,7 +559,7 @@ dpara_status launch_gemm_skinny(const GemmArgs &g, const SkinnyShape &sh, int32_
   }
   P.M = g.M; P.N = g.N; P.K = g.K; P.epi = g.epi; P.up_row_offset = g.N;
   P.T = sh.T; P.rows = sh.rows; P.out_cols = g.epi == 2 ? sh.rows : sh.rows * sh.halves;
-  P.tiles = sh.tiles; P.split = sh.split; P.stages = sh.stages; P.chunk = sh.chunk; 
+  P.tiles = sh.tiles; P.split = sh.split; P.stages = sh.stages; P.chunk = sh.chunk;
   P.ring_bytes = sh.ring_bytes; P.bar_offset = sh.bar_offset; P.one_round = sh.one_round; P.tmem_cols = sh.tmem_cols;
   P.w_ready = g.w_ready;
   P.resid = g.resid; P.resid_bf16 = g.resid_bf16; P.out_bf16 = g.out_bf16;

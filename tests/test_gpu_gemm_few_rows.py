@@ -68,3 +68,19 @@ def test_same_sum_every_time():
     first, _ = dp.gemm_bf16(a, w, epilogue=3)
     for _ in range(5):
         assert torch.equal(first, dp.gemm_bf16(a, w, epilogue=3)[0])
+
+
+def test_parts_of_k_only_in_one_round():
+    """A host query over the range: where the tiles take several rounds no CTAs share one (the parts' meeting would not be hidden)."""
+    import paper_2609_27396_b200 as dp
+    shared = 0
+    for M in (1, 8, 24, 40, 72, 100, 112, 128, 160, 288, 400):
+        for N in (256, 1024, 4096, 5120, 6144, 10240, 11776, 20480, 50000):
+            for K in (512, 4096, 5120, 8192, 17408):
+                for epilogue in (0, 2):
+                    r = dp.gemm_route(M, N, K, epilogue=epilogue)
+                    if r["few_rows"]:
+                        assert r["ctas"] == 1 or r["rounds"] == 1, (M, N, K, epilogue, r)
+                        assert M <= 128 or r["rounds"] == 1, (M, N, K, epilogue, r)
+                        shared += r["ctas"] > 1
+    assert shared > 100
