@@ -345,8 +345,9 @@ int sm_count() {
 }
 
 // Activation tiles for n_all weight tiles on `most` pairs.  A slab of a tile takes 0.12 + 0.21 nt / 256 us (fill and products; 0.33 at 256
-// rows), or what its weights take from HBM where no other pair reads them in the same round (0.385 when all pairs run), and a launch 6 us
-// beside them; narrower tiles are taken where they even out the rounds or use more pairs (200 x 6144 x 4096: 24 tiles of 208 rows 21.9 us,
+// rows), or what its weights take from HBM (all pairs running: 0.385; 0.27 where two pairs read the same weights and 0.21 where more do, which
+// does not fetch them only once: with 0.385 / t a product of 129 rows, 151936 x 2048, took 17 rounds of 80 rows, 158 us, for 9 of 144, 118; 200 rows,
+// 20480 x 8192, 92 for 86), and a launch 6 us beside them; narrower tiles are taken where they even out the rounds or use more pairs (200 x 6144 x 4096: 24 tiles of 208 rows 21.9 us,
 // 72 of 80 rows 18.5; 1152 x 5120 x 5120: 100 tiles of 240 rows are two rounds of the 74 pairs, the second a third full, 61 us; 140 of 176 rows two
 // rounds of 0.8 the length, 53 us).  Also tried: the tiles of the last rounds shared out by K, their pieces added through L2 by whoever finished
 // last: never faster than this (1152 x 5120 x 17408 165 us against 163, 256 x 151936 x 5120 360 against 355: what the chip saves in
@@ -359,7 +360,7 @@ PairPlan pair_plan(int M, int n_all, int nkb, int most) {
     const int nt = ((M + t - 1) / t + 15) / 16 * 16;
     const long tiles = (long)n_all * t, rounds = (tiles + most - 1) / most;
     double slab = 0.12 + 0.21 * nt / 256.0;
-    const double hbm = 0.385 * (tiles < most ? (double)tiles / most : 1.0) / t;
+    const double hbm = (tiles < most ? (double)tiles / most : 1.0) * (t == 1 ? 0.385 : t == 2 ? 0.27 : 0.21);
     if (hbm > slab) slab = hbm;
     const double us = 6.0 + rounds * nkb * slab;
     if (best.us < 0 || us < 0.97 * best.us) { best.t_tiles = t; best.nt = nt; best.us = us; }

@@ -92,3 +92,11 @@ def test_gemm_launches_that_are_refused(kw):
 @pytest.mark.parametrize("kw", [dict(M=256, epilogue=3, n_groups=8, split_k=4), dict(M=8, epilogue=0, n_groups=8, one_chain=True), dict(M=256, epilogue=3, row_order=True)])
 def test_gemm_launches_that_are_taken(kw):
     assert dp.gemm_route(N=512, K=512, **kw)["rounds"] >= 1
+
+
+@pytest.mark.parametrize("M,rows", [(129, 144), (160, 160), (200, 208)])
+def test_streamed_weights_are_read_by_one_pair(M, rows):
+    """Many rounds of weights: tiles of all activation rows, since pairs that read the same weights do not fetch them once."""
+    for N, K in ((151936, 2048), (151936, 5120), (75968, 4096)):
+        r = dp.gemm_route(M, N, K, epilogue=3)
+        assert r["few_rows"] == 0 and r["tile_rows"] == rows, r
