@@ -100,3 +100,10 @@ def test_streamed_weights_are_read_by_one_pair(M, rows):
     for N, K in ((151936, 2048), (151936, 5120), (75968, 4096)):
         r = dp.gemm_route(M, N, K, epilogue=3)
         assert r["few_rows"] == 0 and r["tile_rows"] == rows, r
+
+
+@pytest.mark.parametrize("M", [200, 256, 512, 1024])
+def test_short_products_take_narrower_tiles(M):
+    """K of one slab: the last tile's epilogue is most of the launch, so the activation rows are cut further than into tiles of 256."""
+    r = dp.gemm_route(M, 264, 64)
+    assert r["few_rows"] == 0 and r["tile_rows"] <= 176 and r["rounds"] == 1, r
