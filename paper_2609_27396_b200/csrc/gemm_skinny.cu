@@ -474,9 +474,11 @@ bool skinny_layout(SkinnyShape &sh, int nkb) {
   sh.chunk = sh.one_round || sh.T * part_row <= 48 * 1024 ? sh.T : 32;
   int behind = sh.one_round ? 0 : sh.chunk * part_row;
   if (behind < kWBytes) behind = kWBytes;
-  // two slabs per stage where that leaves a ring of three, and each CTA of a tile at least one stage
+  // Two slabs per stage where that leaves a ring of three, or of four above 64 activation rows, whose products are long enough to cover a stage's
+  // loop (three stages of two slabs / six of one, us: 88 rows, 5120 x 17408 39.8 / 36.3; 100 rows, 151936 x 5120 284 / 273; but 13 rows,
+  // 151936 x 1664 79.1 / 83.3), and each CTA of a tile at least one stage.
   const int room = kSmemMax - 1024 - kBarBytes - behind;
-  sh.slabs = room / (2 * slab) >= 3 && (nkb + 1) / 2 >= sh.split ? 2 : 1;
+  sh.slabs = room / (2 * slab) >= (sh.T > 64 ? 4 : 3) && (nkb + 1) / 2 >= sh.split ? 2 : 1;
   const int stage = slab * sh.slabs;
   sh.stages = room / stage;
   if (sh.stages > 16) sh.stages = 16;

@@ -107,3 +107,16 @@ def test_short_products_take_narrower_tiles(M):
     """K of one slab: the last tile's epilogue is most of the launch, so the activation rows are cut further than into tiles of 256."""
     r = dp.gemm_route(M, 264, 64)
     assert r["few_rows"] == 0 and r["tile_rows"] <= 176 and r["rounds"] == 1, r
+
+
+def test_rings_of_the_kernel_for_few_rows():
+    """Two slabs per stage leave a ring of three stages, of four above 64 activation rows, beside what lies behind the ring (at least 16 KB)."""
+    two = 0
+    for M in (1, 16, 17, 40, 64, 72, 100, 128):
+        for N, K in ((264, 512), (6144, 4096), (5120, 17408), (20480, 8192), (151936, 5120), (151936, 64)):
+            r = dp.gemm_route(M, N, K, epilogue=3)
+            assert r["few_rows"] == 1 and r["slabs"] in (1, 2)
+            two += r["slabs"] == 2
+            stage = 2 * 128 * (r["operands"] * r["weight_rows"] + r["tile_rows"])
+            assert r["slabs"] == 1 or (3 if M <= 64 else 4) * stage <= (227 - 16) * 1024, (M, N, K, r)
+    assert two > 10
