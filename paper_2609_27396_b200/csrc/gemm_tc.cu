@@ -345,15 +345,18 @@ int sm_count() {
 }
 
 // Activation tiles for n_all weight tiles on `most` pairs.  A slab of a tile takes 0.12 + 0.21 nt / 256 us (fill and products; 0.33 at 256
-// rows), or what its weights take from HBM (all pairs running: 0.385; 0.27 where two pairs read the same weights and 0.21 where more do, which
-// does not fetch them only once: with 0.385 / t a product of 129 rows, 151936 x 2048, took 17 rounds of 80 rows, 158 us, for 9 of 144, 118; 200 rows,
-// 20480 x 8192, 92 for 86), and a launch 6 us beside them.  Up to four slabs the
-// last tile's epilogue decides, 0.013 us a row (K = 64, 264 columns: 256 rows 7.2 us in one tile, 5.1 in three; 1024 rows 7.2 in four, 6.4 in seven;
-// counted at K = 1024 too it took 288 x 1536 SwiGLU outputs from 10.9 to 12.4).  Narrower tiles are taken where they even out the rounds or use more pairs (200 x 6144 x 4096: 24 tiles of 208 rows 21.9 us,
-// 72 of 80 rows 18.5; 1152 x 5120 x 5120: 100 tiles of 240 rows are two rounds of the 74 pairs, the second a third full, 61 us; 140 of 176 rows two
-// rounds of 0.8 the length, 53 us).  Also tried: the tiles of the last rounds shared out by K, their pieces added through L2 by whoever finished
-// last: never faster than this (1152 x 5120 x 17408 165 us against 163, 256 x 151936 x 5120 360 against 355: what the chip saves in
-// idle time it gives back in clocks and in the pieces' traffic).
+// rows), or what its weights take from HBM (all pairs running: 0.385, 0.405 above 208 rows; 0.255 where two pairs read the same weights and
+// 0.21 where more do, which does not fetch them only once), and a launch 6 us beside them.  Up to four slabs the last tile's epilogue
+// decides, 0.013 us a row.  Narrower tiles are taken where that evens out the rounds or uses more pairs.  Measured (us):
+//   200 x 6144 x 4096               24 tiles of 208 rows 21.9, 72 of 80 rows 18.5
+//   1152 x 5120 x 5120              100 tiles of 240 rows (two rounds of 74, the second a third full) 61, 140 of 176 rows (two of 0.8 the length) 53
+//   129 x 151936 x 2048             9 rounds of 144 rows 114, 17 of 80 rows 143
+//   200 x 20480 x 8192              2 rounds of 208 rows 85, 3 of 112 rows 91
+//   256 x 12288 x 4096, SwiGLU      2 rounds of 256 rows 57.8, 3 of 128 rows 55.3;  200 rows: 2 rounds of 208 rows 52.4, 3 of 112 rows 54.3
+//   256 x 264 x 64                  one tile of 256 rows 7.2, three of 96 rows 5.1;  288 x 1536 x 1024 SwiGLU: three of 96 rows 10.9, four of 80 12.4
+// Also tried: the tiles of the last rounds shared out by K, their pieces added through L2 by whoever finished last: never faster
+// than this (1152 x 5120 x 17408 165 us against 163, 256 x 151936 x 5120 360 against 355: what the chip saves in idle time it gives back in
+// clocks and in the pieces' traffic).
 PairPlan pair_plan(int M, int n_all, int nkb, int most) {
   PairPlan best{};
   best.us = -1;
@@ -363,7 +366,7 @@ PairPlan pair_plan(int M, int n_all, int nkb, int most) {
     const int nt = ((M + t - 1) / t + 15) / 16 * 16;
     const long tiles = (long)n_all * t, rounds = (tiles + most - 1) / most;
     double slab = 0.12 + 0.21 * nt / 256.0;
-    const double hbm = (tiles < most ? (double)tiles / most : 1.0) * (t == 1 ? 0.385 : t == 2 ? 0.27 : 0.21);
+    const double hbm = (tiles < most ? (double)tiles / most : 1.0) * (t == 1 ? (nt > 208 ? 0.405 : 0.385) : t == 2 ? 0.255 : 0.21);
     if (hbm > slab) slab = hbm;
     const double us = 6.0 + rounds * nkb * slab, whole = nkb <= 4 ? us + 0.013 * nt : us;
     if (best.us < 0 || whole < 0.97 * best_whole) { best.t_tiles = t; best.nt = nt; best.us = us; best_whole = whole; }

@@ -102,6 +102,12 @@ def test_streamed_weights_are_read_by_one_pair(M, rows):
         assert r["few_rows"] == 0 and r["tile_rows"] == rows, r
 
 
+def test_few_rounds_of_streamed_weights():
+    """Two rounds of all 256 rows or three of half of them: the latter, as long as three rounds are enough."""
+    assert dp.gemm_route(256, 12288, 4096, epilogue=2)["tile_rows"] == 128
+    assert dp.gemm_route(256, 17408, 5120, epilogue=2)["tile_rows"] == 256
+
+
 @pytest.mark.parametrize("M", [200, 256, 512, 1024])
 def test_short_products_take_narrower_tiles(M):
     """K of one slab: the last tile's epilogue is most of the launch, so the activation rows are cut further than into tiles of 256."""
