@@ -35,9 +35,10 @@ def _run(ci, use_rope=True, knorm=True):
     nl = len(ci.w_kv)
     kc, vc = [_dev(x) for x in ci.k_cache], [_dev(x) for x in ci.v_cache]
     lens = torch.from_numpy(ci.ctx_len.copy()).cuda()
+    gains = {id(g): _dev(g) for g in ci.norm_w}      # (layers given one array share one device gain, and with it the normalised rows)
     plan = dp.CachePlan(batch=ci.features.shape[0], n_rows=ci.features.shape[1], w_kv=[_dev(w) for w in ci.w_kv], k_ctx=kc, v_ctx=vc,
                         row_start=torch.from_numpy(ci.row_start).cuda(), capacity=torch.from_numpy(ci.capacity).cuda(), ctx_len=lens,
-                        norm_w=[_dev(g) for g in ci.norm_w], knorm_w=[_dev(g) for g in ci.knorm_w] if knorm else None, use_rope=use_rope)
+                        norm_w=[gains[id(g)] for g in ci.norm_w], knorm_w=[_dev(g) for g in ci.knorm_w] if knorm else None, use_rope=use_rope)
     plan.run(_dev(ci.features), torch.from_numpy(ci.accept_len).cuda())
     torch.cuda.synchronize()
     return [_host(k) for k in kc], [_host(v) for v in vc], lens.cpu().numpy(), int(plan.status.item())
@@ -75,6 +76,22 @@ def _check(ci, use_rope=True, knorm=True, capacity=None):
 ])
 def test_append_parity(lens, J, F, Hkv, D, layers):
     ci = W.make_cache_inputs(lens, J, F, Hkv, D, layers, 21)
+    ci.accept_len[0] = J - 1
+    ci.accept_len[1] = 0
+    _check(ci)
+
+
+@pytest.mark.parametrize("lens,J,layers,gain_of", [
+    ((50, 9, 31), 9, 10, [0] * 10),                                # one gain: nothing but the row-wise kernel between the two launches
+    ((50, 9, 31), 9, 10, [0, 0, 1, 1, 2, 2, 2, 3, 3, 4]),          # gains that change inside the first launch, over its end and inside the second
+    ((40,) * 8, 16, 9, [0, 1, 2, 3, 4, 5, 6, 7, 8]),               # 128 rows, a gain for every layer, one layer left over
+])
+def test_append_few_rows_of_more_layers_than_a_launch_takes(lens, J, layers, gain_of):
+    """At most 128 candidate rows: layers go in launches of eight that leave bf16 rows in one buffer."""
+    import paper_2609_27396_b200 as dp
+    assert dp.gemm_route(len(lens) * J, 2 * 4 * 128, 512, epilogue=0, n_groups=8, one_chain=True)["few_rows"] == 1
+    ci = W.make_cache_inputs(lens, J, 512, 4, 128, layers, 33)
+    ci.norm_w = [ci.norm_w[g] for g in gain_of]
     ci.accept_len[0] = J - 1
     ci.accept_len[1] = 0
     _check(ci)
