@@ -31,13 +31,19 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
     if (e_ != cudaSuccess) return DPARA_ERR_CUDA;              \
   } while (0)
 
-// Programmatic dependent launch.  Every kernel of this library runs pdl_wait() (blocks until the kernels before it have
-// completed and their writes are visible) BEFORE it reads or writes any global memory, then pdl_launch_dependents() (the
-// next kernel on the stream may be set up and its CTAs made resident as SMs free up); launched through launch_pdl the
-// kernel's launch latency and set-up then overlap its predecessor.  Wait first, trigger second: a dependent is only ever
-// released by a kernel whose own predecessors are complete, so a dependent that reads some of its inputs before its own
-// wait (the early-start form of verify/select) can race with nothing older than its immediate predecessor.  Without the
-// launch attribute both instructions do nothing.
+// Programmatic dependent launch.  THE RULE for every kernel of this library: a CTA runs pdl_launch_dependents() only after a pdl_wait() of
+// its own (which blocks until the kernels before it have completed and their writes are visible), or never.  A kernel launched through launch_pdl behind
+// it is then released, and its launch latency and set-up overlap this one's tail, only when everything older than the kernel
+// in FRONT of it is complete: ahead of its own pdl_wait() it can race with that one kernel and with nothing else.  Most kernels touch global memory
+// only behind their wait.  These read ahead of it, and what they read may not be written by the kernel directly in front:
+//   kernel                                  reads ahead of its wait                in front of it, by the order its call launches them
+//   gemm_skinny_kernel with w_ready         weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
+//   qk_norm_rope_kernel                     context offsets or lengths             the QKV product
+//   append_rows_kernel                      accept_len, ctx_len, capacity          the projection
+//   ar_head_kernel, sampling, steps > 0     W, base logits (its producer warp)     head_sample_kernel of the step before
+//   verify kernels, early-start form        all but the representations; they also use their workspace   what the caller queued: the flag is its promise
+// Moving a trigger ahead of a wait, or a kernel that writes one of these directly in front of its reader, makes a race.
+// Without the launch attribute both instructions do nothing.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
