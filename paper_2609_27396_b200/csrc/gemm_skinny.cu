@@ -85,17 +85,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity
 __device__ __forceinline__ void mbar_arrive_rank(uint64_t *bar, uint32_t rank) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(map_to_cta(smem_u32(bar), rank)) : "memory");
 }
-// Barrier among the 256 epilogue threads that also makes `live` the same in all of them.
-__device__ __forceinline__ bool epilogue_bar(bool live) {
-  uint32_t all;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-      "barrier.red.and.pred q, 1, 256, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(all) : "r"((uint32_t)live) : "memory");
-  return all != 0;
-}
-__device__ __forceinline__ float sk_silu(float g) { return g / (1.0f + __expf(-g)); }
 
 // Sum over the cluster's parts of four outputs of kU activation rows each, rank 0 first: the loads of four parts in flight, then their
 // additions.  `addr`: shared-memory addresses in this CTA.
@@ -176,7 +165,7 @@ __device__ __forceinline__ void sk_finish(const Finish P) {
         if (in && j < rows_here) {
           const float4 g = x[2 * u], up = x[2 * u + 1];
           *reinterpret_cast<uint2 *>(static_cast<uint16_t *>(P.out) + (size_t)(c0 + j) * P.N + col) =
-              make_uint2(pack_bf16(sk_silu(g.x) * up.x, sk_silu(g.y) * up.y), pack_bf16(sk_silu(g.z) * up.z, sk_silu(g.w) * up.w));
+              make_uint2(pack_bf16(silu(g.x) * up.x, silu(g.y) * up.y), pack_bf16(silu(g.z) * up.z, silu(g.w) * up.w));
         }
       }
     }
@@ -381,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
       const int buf = n_buf == 2 ? k & 1 : 0;
       const uint32_t use = n_buf == 2 ? k >> 1 : k;
       // one warp asks for the accumulator, the others sleep on the named barrier: eight polling warps slow down the two that issue
-      live = epilogue_bar(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, use & 1, abort_flag, 4)));
+      live = named_bar_all_256(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, use & 1, abort_flag, 4)));
       tc_fence_after();
       const uint32_t taddr = tmem + buf * buf_cols + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
@@ -408,10 +397,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_skinny_kernel(const __grid_c
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty + buf);
         }
-        live = epilogue_bar(live);
+        live = named_bar_all_256(live);
         if (S > 1) {
           if (threadIdx.x < S) mbar_arrive_rank(ready, threadIdx.x);
-          live = epilogue_bar(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(ready, 0, abort_flag, 6))));
+          live = named_bar_all_256(live && (warp != 0 || __all_sync(0xffffffffu, mbar_wait_cluster(ready, 0, abort_flag, 6))));
         }
         const int rows_here = min(P.M - c0, n_here);
         if (live) {
@@ -567,9 +556,10 @@ dpara_status launch_gemm_skinny(const GemmArgs &g, const SkinnyShape &sh, int32_
   P.resid = g.resid; P.resid_bf16 = g.resid_bf16; P.out_bf16 = g.out_bf16;
   P.perm_block = g.epi == 3 ? g.perm_block : 0; P.perm_b = g.perm_b;
   P.status = status;
-  void (*const kernels[2][3])(SkinnyParams) = {{gemm_skinny_kernel<1, 1, 1>, gemm_skinny_kernel<2, 1, 1>, gemm_skinny_kernel<1, 2, 1>},
-                                               {gemm_skinny_kernel<1, 1, 2>, gemm_skinny_kernel<2, 1, 2>, gemm_skinny_kernel<1, 2, 2>}};
-  void (*const kernel)(SkinnyParams) = kernels[sh.slabs - 1][sh.halves == 2 ? 1 : sh.T > 256 ? 2 : 0];
+  // (above 256 rows a ring of four stages of two slabs never fits)
+  void (*const kernel)(SkinnyParams) = sh.T > 256       ? gemm_skinny_kernel<1, 2, 1>
+                                       : sh.halves == 2 ? (sh.slabs == 2 ? gemm_skinny_kernel<2, 1, 2> : gemm_skinny_kernel<2, 1, 1>)
+                                                        : (sh.slabs == 2 ? gemm_skinny_kernel<1, 1, 2> : gemm_skinny_kernel<1, 1, 1>);
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return DPARA_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];

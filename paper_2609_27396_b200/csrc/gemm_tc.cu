@@ -54,18 +54,7 @@ struct GemmKernelParams {
   int perm_block, perm_b;
 };
 
-__device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
 
-// Barrier among the 256 epilogue threads that also makes `live` the same in all of them.
-__device__ __forceinline__ bool epi_bar(bool live) {
-  uint32_t all;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-      "barrier.red.and.pred q, 1, 256, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(all) : "r"((uint32_t)live) : "memory");
-  return all != 0;
-}
 
 // A unit of work: a tile of one of the products, or one part of its K range (the parts of a tile are neighbours).
 struct Unit {
@@ -112,7 +101,7 @@ __device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const float own = __uint_as_float(up_side ? r[16 + j] : r[j]), other = theirs[j * 32];
-        const float v = silu_f(up_side ? other : own) * (up_side ? own : other);
+        const float v = silu(up_side ? other : own) * (up_side ? own : other);
         if (j0 + j < rows_all && col < P.N) out[(size_t)(j0 + j) * P.N] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
       }
       named_bar_sync(bar, 64);
@@ -318,7 +307,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
     for (int unit = pair; unit < units && live; unit += pairs, ++k) {
       const int buf = k & 1;
       // one warp asks for the accumulator, the others sleep on the named barrier
-      live = epi_bar(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (k >> 1) & 1, abort_flag, 5)));
+      live = named_bar_all_256(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (k >> 1) & 1, abort_flag, 5)));
       tc_fence_after();
       const uint32_t taddr = tmem + buf * 256 + ((uint32_t)(quarter * 32) << 16);
       if (live) gemm_epilogue(P, taddr, Unit(P, unit, nkb), rank, exchange, quarter, turn, lane);

@@ -45,8 +45,7 @@ __device__ __forceinline__ uint32_t head_key(float f) {
 
 struct ArParams {
   CUtensorMap map_w;
-  CUtensorMap map_l;          // base logits [block * b][vocab] fp32, box = one tile's columns x nb rows
-  const float *logits;        // [block][b][vocab]: the rows one step reads are contiguous
+  CUtensorMap map_l;          // base logits [block * b][vocab] fp32 (the rows one step reads are contiguous), box = one tile's columns x nb rows
   const uint16_t *ar_e;       // [vocab][rank]
   const int32_t *bonus;       // [b]
   int32_t *next_tokens;       // [b][block]
@@ -164,16 +163,6 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
     int kt = 0, stage = 0;
     bool ok = true;
     uint32_t ph_full = 0;
-    // barrier of the epilogue warps (orders their shared-memory writes); all of them pass it with the same answer, so that they leave together
-    auto epi_sync = [&](bool good) {
-      uint32_t all;
-      asm volatile(
-          "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-          "barrier.red.and.pred q, 1, 256, p;\n\t"
-          "selp.u32 %0, 1, 0, q;\n\t}"
-          : "=r"(all) : "r"((uint32_t)good) : "memory");
-      return all != 0;
-    };
     for (int step = step_begin; step < step_end && ok; ++step) {
       // previous tokens: the bonus for the first step, else the winners of the previous step
       if (threadIdx.x < kMaxBatch) {
@@ -197,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         }
         s_tok[threadIdx.x] = tok;
       }
-      epi_sync(true);
+      named_bar_all_256(true);   // (orders the epilogue warps' shared-memory writes; below it also makes them leave together)
       // Ey[n][k] = E[tok_n][k] in the K-major 128-byte-swizzle layout the MMA reads: slab = k / 64, row n at
       // 128 B pitch, 16-byte chunk c of the row stored at chunk position c ^ (n & 7); rows n >= b are zero
       const int chunks_per_row = P.rank / 8;
@@ -268,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
           if (lane == 0) s_red[quarter * kMaxBatch + n] = x;
         }
       }
-      ok = epi_sync(ok);
+      ok = named_bar_all_256(ok);
       if (!ok) break;
       // ---- grid barrier: every CTA's maxima of this step are in before anyone reads them.  Warp 0 leaves the CTA's and counts the CTA in,
       // one lane polls; the others sleep on the named barrier.
@@ -292,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         }
         __syncwarp();
       }
-      ok = epi_sync(!*abort_flag);
+      ok = named_bar_all_256(!*abort_flag);
     }
     // the last step's winners
     if (!kSample && ok && blockIdx.x == 0 && (int)threadIdx.x < P.b) {
@@ -539,7 +528,7 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   if (P.rows < 32) P.rows = 32;
   if (!make_tmap_bf16_2d(&P.map_w, h.ar_w, h.rank, h.vocab, (uint64_t)h.rank * 2, 64, P.rows)) return DPARA_ERR_CUDA;
   if (!make_tmap_f32_2d(&P.map_l, logits, h.vocab, (uint64_t)h.block * h.b, (uint64_t)h.vocab * 4, P.rows, h.b <= 16 ? 16 : 32)) return DPARA_ERR_CUDA;
-  P.logits = logits; P.ar_e = static_cast<const uint16_t *>(h.ar_e); P.bonus = h.bonus; P.next_tokens = h.next_tokens;
+  P.ar_e = static_cast<const uint16_t *>(h.ar_e); P.bonus = h.bonus; P.next_tokens = h.next_tokens;
   P.best = best; P.barrier = barrier; P.status = status;
   P.b = h.b; P.block = h.block; P.vocab = h.vocab; P.rank = h.rank;
   P.n_tiles = (h.vocab + P.rows - 1) / P.rows;
