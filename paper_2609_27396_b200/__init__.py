@@ -17,7 +17,7 @@ LIB_PATH = os.path.join(_HERE, "libdpara.so")
 
 if not os.path.exists(LIB_PATH):
     raise ImportError(
-        f"{LIB_PATH} is missing: build it with `python -m paper_2609_27396_b200.build` "
+        f"{LIB_PATH} is missing: build it with `python paper_2609_27396_b200/build.py` "
         "(nvcc, sm_100a). This package has no CPU fallback.")
 
 lib = C.CDLL(LIB_PATH)

@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     // stays fed.  The two threads meet only through barriers (the S hand-off below, the K/V ring).
     // The whole warp walks the loop and waits, one lane issues: a wait inside a one-lane branch costs 190..310 clocks when its barrier is
     // already there, ~95 by a converged warp, and three of them sit on every iteration's chain from scores
-    // to weighted sums (16 requests, 14B-shaped: step 217 -> 211 us; one request 25.8 -> 24.5; four of 32 K context: block 757 -> 746).
+    // to weighted sums (step with verify/select, both sides in turn: 16 requests, 14B-shaped, 255.8 -> 249.2 us; one request 25.3 -> 23.8).
     {
       const int ti = warp - 9;
       constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, false, false);

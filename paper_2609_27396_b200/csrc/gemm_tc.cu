@@ -2,8 +2,9 @@
 // (fewer: gemm_skinny.cu).
 //
 // A pair of CTAs (a cluster of two, tcgen05 cta_group::2) computes a tile of 256 weight rows x nt activation rows (nt <= 256).  The
-// WEIGHTS are the rows of the product, so that nt can be any multiple of 16: a batch of 1152 rows is five tiles of 240, 288 rows are
-// two of 144 (256-row tiles of activations computed 1280 and 512 rows there).  Per 64-wide slab of K each CTA holds 128 of the weight
+// WEIGHTS are the rows of the product, so that nt can be any multiple of 16 (256-row tiles of activations computed 1280 rows for 1152
+// and 512 for 288); pair_plan chooses it by the weights' shape too: 1152 rows are five tiles of 240 against 17408 x 5120 (SwiGLU) and seven of 176
+// against 5120 x 5120, 288 rows two of 144 against 12288 x 4096 (SwiGLU) and three of 96 against 6144 x 4096.  Per 64-wide slab of K each CTA holds 128 of the weight
 // rows and HALF of the activation rows (128-byte swizzle) and the accumulator of its own 128 weight rows; the even CTA's thread
 // issues M = 256 products that read both halves.  These shapes are bound by the L2 -> shared-memory fill and by power: a pair pulls
 // 64 KB per slab for 256 x 256 outputs.  Each CTA's producer fetches its own halves with ordinary tiled copies and counts the bytes
