@@ -40,7 +40,8 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 //   gemm_skinny_kernel with w_ready         weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
 //   qk_norm_rope_kernel                     context offsets or lengths             the QKV product
 //   append_rows_kernel                      accept_len, ctx_len, capacity          the projection
-//   ar_head_kernel, sampling, steps > 0     W, base logits (its producer warp)     head_sample_kernel of the step before
+//   gemm_skinny_kernel, the LM head         weights                                head_clear_kernel
+//   ar_head_kernel                          W of the head loop                     the LM head's product
 //   verify kernels, early-start form        all but the representations; they also use their workspace   what the caller queued: the flag is its promise
 // Moving a trigger ahead of a wait, or a kernel that writes one of these directly in front of its reader, makes a race.
 // Without the launch attribute both instructions do nothing.

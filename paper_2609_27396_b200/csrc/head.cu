@@ -1,39 +1,63 @@
 // The critical-path remainder T_Head (Alg. 1 after the barrier; Sec. 3.2 "Loss" for the head's form):
 //   base logits  l = h W_lm^T  of the SELECTED branch (b * d rows), one tensor-core GEMM with an fp32 store;
-//   head loop    z_i = l_i + W E(y_{i-1}),  y_i = argmax z_i,  y_0 = bonus,  i = 1..d  (greedy).
+//   head loop    z_i = l_i + W E(y_{i-1}),  y_0 = bonus,  i = 1..d;  y_i = argmax z_i (greedy) or y_i ~ softmax(z_i) (App. C:
+//                temperature 1, top-p 1) by inverse CDF from a supplied uniform.
 //
-// The loop is d dependent steps, each a skinny product: all vocab rows of W (vocab x rank, bf16) against the b
-// embedding rows E(y_{i-1}) -- 0.6 GFLOP and one pass over W (78 MB at vocab 151 936, rank 256, which stays in
-// L2) per step.  ONE persistent cooperative kernel runs all d steps:
-//   warp 8      TMA producer: streams this CTA's tiles of W (at most 128 rows) through a ring of shared-memory stages (the
-//               tiles do not depend on the tokens, so the ring runs ahead across steps), and with each tile the
-//               b x 128 block of base logits it will be added to (plain loads of those from the epilogue queued
-//               behind the deep W stream and cost 1.6 us each; as part of the stage they cost nothing);
-//   warp 9      one thread issues tcgen05.mma: D[128 vocab rows][nb] = W_tile[128][rank] * Ey[nb][rank]^T
-//               (M = 128, N = nb = 16 or 32, both operands K-major in shared memory, 128-byte swizzle);
-//   warps 0-7   build Ey in shared memory at the start of a step (gather of E rows, swizzled by hand), then for
-//               every tile: tcgen05.ld the accumulator (thread = vocab row; warps w and w + 4 share the 32 rows
-//               of a TMEM lane quarter and take the even / odd requests), add the base logit of each request
-//               (from the stage), keep the running (value, index) maximum per request -- a thread meets its
-//               rows in increasing order, so a strict compare keeps the lowest index; at the end of the step a
-//               warp reduction, a CTA reduction and one 64-bit atomicMax per request and CTA.
-// Between steps the CTAs meet at a grid barrier (a counter in global memory; the launch is cooperative, so all
-// CTAs are resident; the wait is bounded by wall time and gives up with DPARA_STATUS_TIMEOUT).
-// A maximum is carried as (order-preserving key of z) << 32 | ~index: the largest packed value is the largest
-// logit, lowest index on ties; NaN ranks below every number.
+// The loop is d dependent steps, each a skinny product: all vocab rows of W (vocab x rank, bf16: 78 MB at vocab 151 936, rank 256) against
+// the b embedding rows E(y_{i-1}).  ONE persistent cooperative kernel runs all d steps; CTA c owns the vocabulary entries
+// [c T R, (c + 1) T R) as T tiles of R <= 128.  What bounds a step is shared memory (a tile of W written by its copy and read by its product takes
+// ~1050 clocks, where its products alone would be done in 640) and the chain last product -> maxima of all CTAs -> token -> row of
+// E -> first product (~5000 clocks, 850 of them one round trip to L2, 900 the row, and the slowest CTA sets the pace).  So
+//   * as many of a CTA's tiles as tensor memory holds (three of nine at rank 256) are put there once and stay: the products read
+//     their A operand from it (10 clocks per product of N = 16 against 40 from shared memory), and a step streams the others only.  The
+//     ring that streams them is filled while the chain runs;
+//   * the CTAs meet through DATA: each publishes its maximum per request as one 64-bit word with the step's tag, and the warp
+//     that needs a request's winner polls that request's words of all CTAs.  No atomic, no fence, no counter, no second
+//     round trip for the value; the same warp then fetches the row of E, so that no barrier of the CTA lies in between;
+//   * sampling takes the same launch: z stays on the SM, and what a step exchanges is a sum per CTA and request and the token drawn (before: z
+//     through memory and a second launch for the draw).
+// Measured (16 steps, vocabulary 151 936, rank 256, this kernel before -> now): 16 requests greedy 233 -> 178 us, 8 requests sampling
+// 330 -> 226 us; one request, 8 steps 85 -> 73 us.  Tried: a pause between the copies of the next step's tiles (the polls are not slowed down by
+// them: 13.1 -> 13.5 thousand clocks a step); maxima of 16 requests per warp in place of 8 (the exchange is bound by its instructions: +1000).
+// Warps:
+//   8           streams the tiles of W that do not stay (they do not depend on the tokens: it runs ahead across steps);
+//   10          streams the base logits, [b][R] per tile, on a ring of its own (plain loads of those from the epilogue queued behind the
+//               deep W stream and cost 1.6 us each);
+//   9           issues tcgen05.mma: D[128 vocab rows][kNb] = W_tile[128][rank] * Ey[kNb][rank]^T (M = 128, N = kNb = 16 or 32);
+//   0-7         epilogue: thread = vocab row; warps w and w + 4 share the 32 rows of a TMEM lane quarter and take the even / odd
+//               requests.  Warp w also does what is per request for requests w, w + 8, ...: publishes, polls, draws, builds Ey.
+// Order of a CTA's tiles in a step: first as many streamed ones as the ring holds (their slots are refilled from then on), then the ones in
+// tensor memory, then the rest; the vocabulary follows that order, so that a thread meets its rows in increasing order and a strict
+// compare keeps the lowest index.
+// Greedy: a maximum travels as (order-preserving key of z) << 32 | ~index: the largest word is the largest logit, lowest index on ties; NaN
+// ranks below every number.
+// Sampling: z replaces the base logit where that lies (shared memory; the call's workspace where a step's logits do not fit), each
+// CTA publishes its weight sum per request and the exponent it is relative to; every CTA finds the CTA the threshold u * (sum of all) falls into by the
+// same arithmetic, and that one finds the crossing entry and publishes the token.  Weights are fp32 (relative error ~1e-7, far below the fp32
+// logits' own), their sums carry 44 bits and more behind the point.
+// All waits are bounded by wall time and give up with DPARA_STATUS_TIMEOUT; the launch is cooperative, so all CTAs are resident.
 #include "gemm.cuh"
 #include "head.cuh"
 #include "sm100_ptx.cuh"
+
+#include <math.h>
 
 namespace dpara {
 using namespace ptx;
 
 namespace {
-constexpr int kThreads = 320;  // warps 0-7 epilogue, 8 TMA producer, 9 MMA issuer
-constexpr int kEpiWarps = 8, kProducerWarp = 8, kMmaWarp = 9;
+constexpr int kThreads = 352;  // warps 0-7 epilogue, 8 W, 9 MMA issuer, 10 base logits
+constexpr int kEpiWarps = 8, kWeightWarp = 8, kMmaWarp = 9, kLogitWarp = 10;
 constexpr int kMaxBatch = 32;
-constexpr int kAccCols = 32;  // TMEM columns per accumulator buffer (nb <= 32)
-constexpr int kBestStride = 16;  // 64-bit words between two requests' maxima: one 128-byte line (one L2 atomic unit) each
+constexpr int kResidentCol = 128;                  // accumulators in TMEM columns [0, 128); behind them the tiles of W that stay
+constexpr int kMaxAccBufs = kResidentCol / 16;
+constexpr int kMaxStages = 4, kMaxLogitSlots = 16;
+constexpr int kCtasPerLane = (kNumSM + 31) / 32;
+constexpr int kCtaStride = 32 * kCtasPerLane;      // words of one request: a slot per CTA, whole 128-byte lines
+constexpr int kReplicas = 8;
+constexpr unsigned long long kTagMask = 63;
+constexpr int kTagBits = 6;                        // step / 2 + 1 (two buffers in turn, at most 64 steps)
+constexpr int kBarBytes = 3072;                    // barriers and the reduction scratch
 
 __device__ __forceinline__ uint32_t head_key(float f) {
   if (f != f) return 0u;                    // NaN below everything
@@ -41,252 +65,596 @@ __device__ __forceinline__ uint32_t head_key(float f) {
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
+
+__device__ __forceinline__ unsigned long long load_word(const unsigned long long *p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void publish(unsigned long long *p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// Polls until each of the lane's words (at(i) null: none) carries the step's tag; the whole warp calls it.
+template <int kN, typename At>
+__device__ __forceinline__ bool poll_words(At at, uint32_t tag, unsigned long long (&v)[kN], volatile int *abort_flag) {
+  constexpr uint32_t kMask = (uint32_t)kTagMask;
+#pragma unroll
+  for (int i = 0; i < kN; ++i) v[i] = 0ull;
+  uint64_t t0 = 0;
+#pragma unroll 1
+  for (unsigned int tries = 0;; ++tries) {
+    bool all = true;
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+      const unsigned long long *p = at(i);
+      if (p && ((uint32_t)v[i] & kMask) != tag) v[i] = load_word(p);
+    }
+#pragma unroll
+    for (int i = 0; i < kN; ++i) all = all && (!at(i) || ((uint32_t)v[i] & kMask) == tag);
+    if (__all_sync(0xffffffffu, all)) return true;
+    if (tries == 0) t0 = global_timer_ns();
+    if (tries % 64 == 63 && __any_sync(0xffffffffu, *abort_flag || global_timer_ns() - t0 > kWaitLimitNs)) {
+      *abort_flag = 7;
+      return false;
+    }
+  }
+}
+
+// ---- sampling.  The weight of a logit z is 2^(z log2(e) - E) with a whole exponent E of the CTA's own (the largest weight is in (1/2, 1]), so that
+// weights of different CTAs differ by a power of two; sums are whole numbers of 2^-F, F = 62 - log2(vocabulary) bits (44 at 151 936), and are
+// brought to the largest E by shifts.  The fp64 pipe has no part in it: with fp64 sums of exp(z - max) and their
+// fp64 exponentials a draw took 4 us more.
+constexpr long long kNoWeight = -(1ll << 50), kInfinite = 1ll << 50;   // E of a CTA without a number above -inf; with an infinite one
+struct Scale {
+  float m = 0.f, e = 0.f;
+  long long exponent = kNoWeight;
+  __device__ __forceinline__ Scale() {}
+  __device__ __forceinline__ explicit Scale(float top) : m(top), exponent(top > 0.f ? kInfinite : kNoWeight) {
+    if (!finite()) return;
+    if (far()) {
+      // (codes that keep the order and are more than 62 apart from one another and from every other exponent)
+      const long long code = (1ll << 40) + ((long long)__float_as_uint(fabsf(m)) << 8);
+      exponent = m > 0.f ? code : -code;
+    } else {
+      e = ceilf(m * 1.4426950408889634f);
+      exponent = (long long)e;
+    }
+  }
+  __device__ __forceinline__ bool finite() const { return m > -INFINITY && m < INFINITY; }
+  // from here on neighbouring floats are 256 apart: only the largest has weight
+  __device__ __forceinline__ bool far() const { return fabsf(m) >= 2147483648.f; }
+  __device__ __forceinline__ float weight(float z) const {
+    if (far()) return z == m ? 1.f : 0.f;
+    z = fmaxf(z, -INFINITY);   // (NaN: no weight)
+    return ex2(fmaf(z, kLog2eLo, fmaf(z, kLog2eHi, -e)));
+  }
+  static constexpr float kLog2eHi = 1.44269502162933349609375f, kLog2eLo = 1.92596299112661746887e-8f;   // log2(e) in two floats
+};
+// Two sums of floats with the rounding errors of their additions kept beside them (Knuth's TwoSum on pairs): 2^-46 and better.
+struct TwoSum {
+  uint64_t s = 0, c = 0;
+  __device__ __forceinline__ void add(uint64_t x) {
+    const uint64_t minus = pack2(-1.f, -1.f), t = add2(s, x), y = fma2(s, minus, t);
+    c = add2(c, add2(fma2(fma2(y, minus, t), minus, s), fma2(y, minus, x)));
+    s = t;
+  }
+  __device__ __forceinline__ unsigned long long fixed(float unit) const {
+    float a, b, x, y;
+    unpack2(s, a, b);
+    unpack2(c, x, y);
+    const long long v = (__float2ll_rn(a * unit) + __float2ll_rn(b * unit)) + (__float2ll_rn(x * unit) + __float2ll_rn(y * unit));
+    return v > 0 ? (unsigned long long)v : 0ull;
+  }
+};
+// v brought from its exponent to one that is `up` larger
+__device__ __forceinline__ unsigned long long lowered(unsigned long long v, long long up) { return up > 63 ? 0ull : v >> up; }
+__device__ __forceinline__ unsigned long long warp_scan(unsigned long long v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+// floor(u * total), total < 2^62; anything that is not in [0, 1): total (which makes the last entry with weight the one drawn)
+__device__ __forceinline__ unsigned long long threshold(float u, unsigned long long total) {
+  if (!(u >= 0.f && u < 1.f)) return total;
+  const uint32_t bits = __float_as_uint(u) & 0x7fffffffu, field = bits >> 23;
+  const unsigned long long mant = field ? (bits & 0x7fffffu) | 0x800000u : bits;
+  const int down = 150 - (int)(field ? field : 1u);   // u = mant * 2^-down, down >= 24
+  const unsigned long long lo = mant * total, hi = __umul64hi(mant, total);
+  if (down < 64) return (hi << (64 - down)) | (lo >> down);
+  return down < 128 ? hi >> (down - 64) : 0ull;
+}
+
+template <int kCols>
+__device__ __forceinline__ void load_acc(uint32_t taddr, uint32_t (&r)[kCols]) {
+  if constexpr (kCols == 8) tmem_ld8(taddr, r);
+  else tmem_ld16(taddr, r);
+}
 }  // namespace
 
 struct ArParams {
   CUtensorMap map_w;
-  CUtensorMap map_l;          // base logits [block * b][vocab] fp32 (the rows one step reads are contiguous), box = one tile's columns x nb rows
-  const uint16_t *ar_e;       // [vocab][rank]
-  const int32_t *bonus;       // [b]
-  int32_t *next_tokens;       // [b][block]
-  unsigned long long *best;   // [block][kMaxBatch][kBestStride], zeroed before the launch
-  unsigned int *barrier;      // zeroed before the launch
+  CUtensorMap map_l;              // base logits [block * b][vocab] fp32 (the rows one step reads are contiguous), box = R columns x b rows
+  const uint16_t *ar_w, *ar_e;    // [vocab][rank]
+  const int32_t *bonus;           // [b]
+  const float *uniforms;          // [b][block]
+  int32_t *next_tokens;           // [b][block]
+  // What the CTAs exchange, zero before the launch: words [2 (step parity)][replica][b][1, sampling: 2][CTA], drawn [2][replica][kMaxBatch]
+  unsigned long long *words, *drawn;
+  float *z;                       // sampling where z does not fit in shared memory: [b][vocab]
   int32_t *status;
-  int b, block, vocab, rank, n_tiles, nb, stages;
-  int rows;                   // vocabulary rows per tile (<= 128, a multiple of 4)
-  float *z_out;               // sampling: [b][vocab] fp32, the logits z of step `step0`
-  int step0;                  // sampling: the one step this launch computes
+  int b, block, vocab;
+  int rows, tiles;                // R (a multiple of 4), T
+  int resident;                   // tiles that stay in tensor memory
+  int stages, logit_slots, slab_bytes, logit_bytes, logit_off, e_off, bar_off;
+  int z_in_place;                 // sampling: a step's base logits all have slots, z replaces them there
+  float unit;                     // sampling: 2^F
 };
 
-// kSample = false: the whole greedy loop in one cooperative launch.  kSample = true: ONE step (P.step0) of the sampling
-// loop -- the same producer / MMA / epilogue pipeline, but the epilogue writes z = l + W E(y_prev) to P.z_out instead of
-// tracking maxima, the previous tokens come from P.next_tokens (written by the draw of the step before), and there is no
-// grid barrier (the draw is a launch of its own).
-template <bool kSample, int kSlabs>
+template <bool kSample, int kSlabs, int kNb>
 __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_constant__ ArParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int tile_bytes = 128 * P.rank * 2;
-  const int lg_bytes = P.nb * 128 * 4;                   // base logits of one tile: [nb rows][128 vocab entries] fp32
-  const int stage_bytes = tile_bytes + lg_bytes;
-  constexpr int slabs = kSlabs;                          // rank / 64
-  uint8_t *sW = smem;                                    // ring of stages: W tile [slab][128 rows][128 B], then the logits block
-  uint8_t *sE = smem + P.stages * stage_bytes;           // Ey: [slab][nb rows][128 B]
-  uint64_t *bars = reinterpret_cast<uint64_t *>(sE + slabs * P.nb * 128);
-  uint64_t *full = bars, *empty = bars + 4, *acc_full = bars + 8, *acc_empty = bars + 10, *e_ready = bars + 12;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 14);
+  constexpr int kRank = kSlabs * 64, kHalf = kNb / 2, kPer = kNb / kEpiWarps, kTileCols = kRank / 2, kAccBufs = kResidentCol / kNb;
+  uint8_t *sW = smem;                                    // ring of tiles of W, [slab][R rounded up to 8][128 B]
+  uint8_t *sE = smem + P.e_off;                          // Ey: [slab][kNb rows][128 B]
+  uint8_t *sL = smem + P.logit_off;                      // slots of base logits, [b][R] fp32 each
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + P.bar_off);
+  uint64_t *full = bars, *empty = full + kMaxStages, *l_full = empty + kMaxStages, *l_empty = l_full + kMaxLogitSlots,
+           *acc_full = l_empty + kMaxLogitSlots, *acc_empty = acc_full + kMaxAccBufs, *e_ready = acc_empty + kMaxAccBufs;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(e_ready + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  int *s_tok = reinterpret_cast<int *>(tmem_slot + 2);   // [kMaxBatch] previous tokens of this step
-  unsigned long long *s_red = reinterpret_cast<unsigned long long *>(s_tok + kMaxBatch);  // [4 warps][kMaxBatch]
+  unsigned long long *s_red = reinterpret_cast<unsigned long long *>(bars + 64);  // [kEpiWarps][kMaxBatch]
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 4; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1 + kEpiWarps); }  // released by the MMA commit and the epilogue warps
-    for (int a = 0; a < 2; ++a) { mbar_init(acc_full + a, 1); mbar_init(acc_empty + a, kEpiWarps); }
+    for (int s = 0; s < kMaxStages; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
+    for (int s = 0; s < kMaxLogitSlots; ++s) { mbar_init(l_full + s, 1); mbar_init(l_empty + s, kEpiWarps); }
+    for (int a = 0; a < kAccBufs; ++a) { mbar_init(acc_full + a, 1); mbar_init(acc_empty + a, kEpiWarps); }
     mbar_init(e_ready, kEpiWarps);
     *abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == kMmaWarp) { tmem_alloc(tmem_slot, 64); tmem_relinquish(); }
+  if (warp == kMmaWarp) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-  // Nothing above touches global memory.  In the sampling loop's later steps the kernel in front is the draw of the step before, let
-  // go only when everything before it had ended: W and the base logits are there, and the producer fills its ring while the draw runs.  (The
-  // warps that read tokens and write z wait; only they let the next kernel go.)
-  if (!kSample || P.step0 == 0 || warp < kEpiWarps) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
-  // this CTA's tiles: blockIdx.x, blockIdx.x + gridDim.x, ... (the same in every step)
-  const int my_tiles = (P.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int step_begin = kSample ? P.step0 : 0, step_end = kSample ? P.step0 + 1 : P.block;
 
-  if (warp == kProducerWarp) {
-    // ------------------------------------------------------------------ producer
-    // (this warp and the next: the whole warp walks the loop and waits, one lane issues; a wait inside a one-lane branch costs two to
-    // three times as many clocks)
+  const int v0 = (int)blockIdx.x * P.tiles * P.rows;      // this CTA's first vocabulary entry
+  const int count = min(P.vocab - v0, P.tiles * P.rows);  // its entries (>= 1: the grid ends with the vocabulary)
+  const int my_tiles = (count + P.rows - 1) / P.rows;
+  const int n_res = min(P.resident, my_tiles), n_str = my_tiles - n_res;
+  const int lead = min(P.stages, n_str);                  // positions [lead, lead + n_res) of a step are the tiles that stay
+  const int n_ctas = gridDim.x;
+  const int slots = P.z_in_place ? my_tiles : P.logit_slots;   // in place: tile k of a step in slot k
+
+  if (warp == kWeightWarp) {
+    // ------------------------------------------------------------------ W (no kernel of this call writes it: no wait for the one in front)
     prefetch_tensormap(&P.map_w);
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true;
-    const uint32_t tx = (uint32_t)(slabs * P.rows * 128 + P.nb * P.rows * 4);
-    for (int step = step_begin; step < step_end && ok; ++step) {
-      for (int k = 0; k < my_tiles; ++k) {
+    const uint32_t tx = (uint32_t)(kSlabs * P.rows * 128);
+#pragma unroll 1
+    for (int step = 0; step < P.block && ok; ++step)
+#pragma unroll 1
+      for (int k = 0; k < n_str; ++k) {
         ok = __all_sync(0xffffffffu, mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2));
         if (!ok) break;
-        const int row0 = ((int)blockIdx.x + k * (int)gridDim.x) * P.rows;
+        const int row0 = v0 + (k < lead ? k : k + n_res) * P.rows;
         if (elect_one()) {
-          uint8_t *dst = sW + stage * stage_bytes;
+          uint8_t *dst = sW + stage * kSlabs * P.slab_bytes;
           mbar_arrive_expect_tx(full + stage, tx);
 #pragma unroll
-          for (int sb = 0; sb < slabs; ++sb) tma_load_2d(dst + sb * 16384, &P.map_w, full + stage, sb * 64, row0);
-          tma_load_2d(dst + tile_bytes, &P.map_l, full + stage, row0, step * P.b);
+          for (int sb = 0; sb < kSlabs; ++sb) tma_load_2d(dst + sb * P.slab_bytes, &P.map_w, full + stage, sb * 64, row0);
         }
         __syncwarp();
         if (++stage == P.stages) { stage = 0; ph ^= 1u; }
       }
-    }
-  } else if (warp == kMmaWarp) {
-    // ------------------------------------------------------------------ MMA issuer
-    const uint32_t idesc = idesc_bf16_f32(128, P.nb, false, false);
-    const uint64_t desc = smem_desc_sw128(smem_u32(sW), 16, 1024);
-    const uint32_t w_lo0 = (uint32_t)desc, e_lo = w_lo0 + ((uint32_t)(sE - sW) >> 4), hi = (uint32_t)(desc >> 32);
-    const uint32_t e_slab = (uint32_t)(P.nb * 128) >> 4, stage_units = (uint32_t)stage_bytes >> 4;
-    int stage = 0, kt = 0;
+  } else if (warp == kLogitWarp) {
+    // ------------------------------------------------------------------ base logits
+    prefetch_tensormap(&P.map_l);
+    pdl_wait();
+    int slot = 0;
     uint32_t ph = 0;
     bool ok = true;
-    for (int step = step_begin; step < step_end && ok; ++step) {
-      ok = __all_sync(0xffffffffu, mbar_wait(e_ready, (step - step_begin) & 1, abort_flag, 3));   // Ey of this step is in shared memory
-      for (int k = 0; k < my_tiles && ok; ++k, ++kt) {
-        const int buf = kt & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + buf, ((kt >> 1) & 1) ^ 1u, abort_flag, 4) && mbar_wait(full + stage, ph, abort_flag, 5));
+    const uint32_t tx = (uint32_t)(P.b * P.rows * 4);
+#pragma unroll 1
+    for (int step = 0; step < P.block && ok; ++step)
+#pragma unroll 1
+      for (int k = 0; k < my_tiles; ++k) {
+        ok = __all_sync(0xffffffffu, mbar_wait(l_empty + slot, ph ^ 1u, abort_flag, 3));
         if (!ok) break;
-        tc_fence_after();
         if (elect_one()) {
-          const uint32_t w_lo = w_lo0 + stage * stage_units;
-#pragma unroll
-          for (int kk = 0; kk < slabs * 4; ++kk)
-            mma_ss_lo(tmem + buf * kAccCols, w_lo + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4), e_lo + (kk >> 2) * e_slab + (kk & 3) * 2, hi, idesc, kk > 0);
-          mma_commit(empty + stage);
-          mma_commit(acc_full + buf);
+          mbar_arrive_expect_tx(l_full + slot, tx);
+          tma_load_2d(sL + slot * P.logit_bytes, &P.map_l, l_full + slot, v0 + k * P.rows, step * P.b);
         }
         __syncwarp();
-        if (++stage == P.stages) { stage = 0; ph ^= 1u; }
+        if (++slot == slots) { slot = 0; ph ^= 1u; }
+      }
+  } else if (warp == kMmaWarp) {
+    // ------------------------------------------------------------------ MMA issuer (the whole warp walks and waits, one lane issues: a wait
+    // inside a one-lane branch costs two to three times as many clocks)
+    const uint32_t idesc = idesc_bf16_f32(128, kNb, false, false);
+    const uint64_t desc = smem_desc_sw128(smem_u32(sW), 16, 1024);
+    const uint32_t w_lo0 = (uint32_t)desc, e_lo = w_lo0 + ((uint32_t)P.e_off >> 4), hi = (uint32_t)(desc >> 32);
+    constexpr uint32_t e_slab = (uint32_t)(kNb * 128) >> 4;
+    const uint32_t w_slab = (uint32_t)P.slab_bytes >> 4;
+    int stage = 0, buf = 0;
+    uint32_t ph = 0, ph_acc = 0;
+    bool ok = true, there = false;
+#pragma unroll 1
+    for (int step = 0; step < P.block && ok; ++step) {
+      ok = __all_sync(0xffffffffu, mbar_wait(e_ready, step & 1, abort_flag, 4));   // Ey of this step is in shared memory
+#pragma unroll 1
+      for (int k = 0; k < my_tiles && ok; ++k) {
+        const bool stays = k >= lead && k < lead + n_res;
+        // (Ey of a step is there when the accumulators of the step before have all been read)
+        if (k >= kAccBufs) ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + buf, ph_acc ^ 1u, abort_flag, 5));
+        const uint32_t acc = tmem + buf * kNb;
+        if (stays) {
+          tc_fence_after();
+          if (ok && elect_one()) {
+            const uint32_t a = tmem + kResidentCol + (k - lead) * kTileCols;
+#pragma unroll
+            for (int kk = 0; kk < kSlabs * 4; ++kk) mma_ts_lo(acc, a + kk * 8, e_lo + (kk >> 2) * e_slab + (kk & 3) * 2, hi, idesc, kk > 0);
+            mma_commit(acc_full + buf);
+          }
+          __syncwarp();
+        } else {
+          if (!__all_sync(0xffffffffu, there)) ok = __all_sync(0xffffffffu, mbar_wait(full + stage, ph, abort_flag, 6)) && ok;
+          if (!ok) break;
+          const int cur = stage;
+          if (++stage == P.stages) { stage = 0; ph ^= 1u; }
+          there = mbar_test(full + stage, ph);    // (the next one's barrier is asked before this one's products go out)
+          tc_fence_after();
+          if (elect_one()) {
+            const uint32_t w_lo = w_lo0 + cur * kSlabs * w_slab;
+#pragma unroll
+            for (int kk = 0; kk < kSlabs * 4; ++kk)
+              mma_ss_lo(acc, w_lo + (kk >> 2) * w_slab + (kk & 3) * 2, e_lo + (kk >> 2) * e_slab + (kk & 3) * 2, hi, idesc, kk > 0);
+            mma_commit(empty + cur);
+            mma_commit(acc_full + buf);
+          }
+          __syncwarp();
+        }
+        if (++buf == kAccBufs) { buf = 0; ph_acc ^= 1u; }
       }
     }
   } else {
-    // ------------------------------------------------------------------ Ey build + epilogue: thread = vocab row of the tile
-    const int quarter = warp & 3, nh = warp >> 2;  // TMEM lane quarter; this warp takes requests n = 2 j + nh
-    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-    int kt = 0, stage = 0;
-    bool ok = true;
-    uint32_t ph_full = 0;
-    for (int step = step_begin; step < step_end && ok; ++step) {
-      // previous tokens: the bonus for the first step, else the winners of the previous step
-      if (threadIdx.x < kMaxBatch) {
-        int tok = 0;
-        if ((int)threadIdx.x < P.b) {
-          if (step == 0) {
-            tok = P.bonus[threadIdx.x];
-            if (tok < 0 || tok >= P.vocab) {
-              if (P.status) atomicOr(reinterpret_cast<unsigned int *>(P.status), DPARA_STATUS_BAD_TOKEN);
-              tok = 0;
-            }
-          } else if (kSample) {
-            tok = __ldcg(P.next_tokens + (size_t)threadIdx.x * P.block + (step - 1));
-            if (tok < 0 || tok >= P.vocab) tok = 0;
-          } else {
-            const unsigned long long w = __ldcg(P.best + ((size_t)(step - 1) * kMaxBatch + threadIdx.x) * kBestStride);
-            tok = (int)(0xffffffffu - (uint32_t)(w & 0xffffffffull));
-            if (w == 0ull) tok = 0;  // (all-NaN row)
-            if (blockIdx.x == 0) P.next_tokens[(size_t)threadIdx.x * P.block + (step - 1)] = tok;
-          }
-        }
-        s_tok[threadIdx.x] = tok;
-      }
-      named_bar_all_256(true);   // (orders the epilogue warps' shared-memory writes; below it also makes them leave together)
-      // Ey[n][k] = E[tok_n][k] in the K-major 128-byte-swizzle layout the MMA reads: slab = k / 64, row n at
-      // 128 B pitch, 16-byte chunk c of the row stored at chunk position c ^ (n & 7); rows n >= b are zero
-      const int chunks_per_row = P.rank / 8;
-      for (int q = threadIdx.x; q < P.nb * chunks_per_row; q += kEpiWarps * 32) {
-        const int n = q / chunks_per_row, c = q % chunks_per_row;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (n < P.b) v = *reinterpret_cast<const uint4 *>(P.ar_e + (size_t)s_tok[n] * P.rank + c * 8);
-        const int sb = c >> 3, cc = c & 7;
-        *reinterpret_cast<uint4 *>(sE + sb * (P.nb * 128) + n * 128 + ((cc ^ (n & 7)) << 4)) = v;
-      }
-      fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(e_ready);
-
-      float bz[kMaxBatch / 2];
-      int bv[kMaxBatch / 2];
+    // ------------------------------------------------------------------ epilogue, exchange, Ey
+    const int quarter = warp & 3, nh = warp >> 2;  // TMEM lane quarter; column nh * kHalf + j holds request 2 j + nh
+    const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+    // The tiles that stay: thread = row, 32 words (64 of K) at a time, in the layout of a bf16 A operand (lane = row, column = two
+    // neighbouring elements).  Rows behind the tile or the vocabulary only make accumulator lanes that nobody reads.
+#pragma unroll 1
+    for (int i = 0; i < n_res; ++i) {
+      const int row = min(v0 + (lead + i) * P.rows + min(quarter * 32 + lane, P.rows - 1), P.vocab - 1);
+      const uint4 *src = reinterpret_cast<const uint4 *>(P.ar_w + (size_t)row * kRank);
+#pragma unroll 1
+      for (int sb = nh; sb < kSlabs; sb += 2) {
+        uint32_t r[32];
 #pragma unroll
-      for (int j = 0; j < kMaxBatch / 2; ++j) { bz[j] = -INFINITY; bv[j] = -1; }
-      for (int k = 0; k < my_tiles; ++k, ++kt) {
-        const int buf = kt & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (kt >> 1) & 1, abort_flag, 6));
+        for (int q = 0; q < 8; ++q) {
+          const uint4 x = __ldg(src + sb * 8 + q);
+          r[4 * q] = x.x; r[4 * q + 1] = x.y; r[4 * q + 2] = x.z; r[4 * q + 3] = x.w;
+        }
+        tmem_st32(lanes + kResidentCol + i * kTileCols + sb * 32, r);
+      }
+    }
+    tmem_wait_st();
+    tc_fence_before();
+    // Ey[pos][k] = E[tok][k] in the K-major 128-byte-swizzle layout the MMA reads: slab = k / 64, row at 128 B pitch, 16-byte chunk c of the
+    // row stored at chunk position c ^ (row & 7)
+    auto put_row = [&](int n, bool live, int tok) {
+      const int pos = (n & 1) * kHalf + (n >> 1);
+      if (lane < kRank / 8) {
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (live) v = __ldg(reinterpret_cast<const uint4 *>(P.ar_e + (size_t)tok * kRank + lane * 8));
+        *reinterpret_cast<uint4 *>(sE + (lane >> 3) * (kNb * 128) + pos * 128 + (((lane & 7) ^ (pos & 7)) << 4)) = v;
+      }
+    };
+    pdl_wait();
+    pdl_launch_dependents();
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int n = warp + kEpiWarps * q;
+      int tok = 0;
+      if (n < P.b) {
+        tok = P.bonus[n];
+        if (tok < 0 || tok >= P.vocab) {
+          if (P.status && lane == 0) atomicOr(reinterpret_cast<unsigned int *>(P.status), DPARA_STATUS_BAD_TOKEN);
+          tok = 0;
+        }
+      }
+      put_row(n, n < P.b, tok);
+    }
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(e_ready);
+
+    const int z_row = kSample && !P.z_in_place ? P.vocab : P.rows;   // floats between two requests' z of a tile
+    const int z_tile = P.z_in_place ? P.logit_bytes / 4 : P.rows;      // ... and between two tiles'
+    const int mine_n = (P.b - nh + 1) / 2;                           // this warp's requests 2 j + nh
+    int buf = 0, slot = 0;
+    uint32_t ph_acc = 0, ph_l = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int step = 0; step < P.block && ok; ++step) {
+      float bz[kHalf];
+      int bv[kHalf];
+#pragma unroll
+      for (int j = 0; j < kHalf; ++j) { bz[j] = -INFINITY; bv[j] = -1; }
+#pragma unroll 1
+      for (int k = 0; k < my_tiles; ++k) {
+        ok = __all_sync(0xffffffffu, mbar_wait(l_full + slot, ph_l, abort_flag, 9) && mbar_wait(acc_full + buf, ph_acc, abort_flag, 8));
         if (!ok) break;
         tc_fence_after();
-        uint32_t acc[32];
-        tmem_ld32(taddr + buf * kAccCols, acc);
+        uint32_t acc[kHalf];
+        load_acc<kHalf>(lanes + buf * kNb + nh * kHalf, acc);
+        const int r = quarter * 32 + lane, v = v0 + k * P.rows + r;
+        const bool live = r < P.rows && v < P.vocab;
+        float *sl = reinterpret_cast<float *>(sL + slot * P.logit_bytes) + nh * P.rows + min(r, P.rows - 1);
+        float *zt = kSample && !P.z_in_place ? P.z + (size_t)nh * P.vocab + v : sl;
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty + buf);
-        const int v = ((int)blockIdx.x + k * (int)gridDim.x) * P.rows + quarter * 32 + lane;
-        // (acc_full implies the stage's loads have landed: the MMA issuer waited for them; this wait is the
-        //  epilogue threads' own acquire of the TMA-written logits and returns at once)
-        ok = __all_sync(0xffffffffu, mbar_wait(full + stage, ph_full, abort_flag, 9));
-        if (!ok) break;
-        const bool live = quarter * 32 + lane < P.rows && v < P.vocab;
-        const float *sl = reinterpret_cast<const float *>(sW + stage * stage_bytes + tile_bytes) + min(quarter * 32 + lane, P.rows - 1);
+        if (++buf == kAccBufs) { buf = 0; ph_acc ^= 1u; }
+        // four requests at a time: their loads and compares in flight together
 #pragma unroll
-        for (int j = 0; j < kMaxBatch / 2; ++j) {
-          const int n = 2 * j + nh;
-          if (n < P.b) {
-            const float z = __uint_as_float(nh ? acc[2 * j + 1] : acc[2 * j]) + sl[n * P.rows];
+        for (int j4 = 0; j4 < kHalf; j4 += 4) {
+          if (j4 >= mine_n) break;
+          float l[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) l[u] = sl[2 * min(j4 + u, mine_n - 1) * P.rows];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int j = j4 + u;
+            const float z = __uint_as_float(acc[j]) + l[u];
             if (kSample) {
-              if (live) P.z_out[(size_t)n * P.vocab + v] = z;       // a warp writes 32 consecutive entries of one row
+              if (live && j < mine_n) zt[(size_t)(2 * j) * z_row] = z;
+              bz[j] = live ? fmaxf(bz[j], z) : bz[j];   // (fmaxf drops NaN)
             } else if (live && (z > bz[j] || (bv[j] < 0 && z == z))) {
               // larger, or the first number this thread sees (NaN never wins; -inf can, at the lowest index)
               bz[j] = z; bv[j] = v;
             }
           }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty + stage);
-        if (++stage == P.stages) { stage = 0; ph_full ^= 1u; }
+        if (!kSample || !P.z_in_place) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(l_empty + slot);
+        }
+        if (++slot == slots) { slot = 0; ph_l ^= 1u; }
       }
-      if (kSample) break;
-      // (a warp whose wait ran out takes the others along at the next barrier)
-      // step maximum: warp reduction, CTA reduction through shared memory, then ONE atomic per request and CTA,
-      // each request on its own 128-byte line (atomics on one line are serialised by a single L2 unit)
+      // ---- maxima of the CTA: by warp, then over the four quarters
 #pragma unroll
-      for (int j = 0; j < kMaxBatch / 2; ++j) {
-        const int n = 2 * j + nh;
-        if (n < P.b) {
-          unsigned long long x = bv[j] < 0 ? 0ull : (((unsigned long long)head_key(bz[j]) << 32) | (unsigned long long)(0xffffffffu - (uint32_t)bv[j]));
+      for (int j4 = 0; j4 < kHalf; j4 += 4) {
+        if (j4 >= mine_n) break;
+        uint32_t key[4], best[4], low[4];
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
-            x = y > x ? y : x;
-          }
-          if (lane == 0) s_red[quarter * kMaxBatch + n] = x;
+        for (int u = 0; u < 4; ++u) key[u] = !kSample && bv[j4 + u] < 0 ? 0u : head_key(bz[j4 + u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) best[u] = __reduce_max_sync(0xffffffffu, key[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) low[u] = kSample ? 0u : __reduce_max_sync(0xffffffffu, key[u] == best[u] && key[u] ? 0xffffffffu - (uint32_t)bv[j4 + u] : 0u);
+        if (lane < 4) {
+          const unsigned long long x = lane == 0 ? ((unsigned long long)best[0] << 32) | low[0] : lane == 1 ? ((unsigned long long)best[1] << 32) | low[1]
+                                     : lane == 2 ? ((unsigned long long)best[2] << 32) | low[2] : ((unsigned long long)best[3] << 32) | low[3];
+          s_red[quarter * kMaxBatch + min(2 * (j4 + lane) + nh, kMaxBatch - 1)] = x;
         }
       }
+      // (a warp whose wait ran out takes the others along)
       ok = named_bar_all_256(ok);
       if (!ok) break;
-      // ---- grid barrier: every CTA's maxima of this step are in before anyone reads them.  Warp 0 leaves the CTA's and counts the CTA in,
-      // one lane polls; the others sleep on the named barrier.
-      if (warp == 0) {
-        if (lane < P.b) {
-          unsigned long long x = s_red[lane];
+      const bool last = step + 1 == P.block;
+      unsigned long long top[kPer];
 #pragma unroll
-          for (int w = 1; w < 4; ++w) x = s_red[w * kMaxBatch + lane] > x ? s_red[w * kMaxBatch + lane] : x;
-          atomicMax(P.best + ((size_t)step * kMaxBatch + lane) * kBestStride, x);
-          __threadfence();
-        }
-        __syncwarp();
-        if (lane == 0) {
-          atomicAdd(P.barrier, 1u);
-          const unsigned int target = (unsigned int)(step + 1) * gridDim.x;
-          const uint64_t t0 = global_timer_ns();
-          for (unsigned int tries = 1; *reinterpret_cast<volatile unsigned int *>(P.barrier) < target; ++tries) {
-            if (tries % 64 == 0 && (*abort_flag || global_timer_ns() - t0 > kWaitLimitNs)) { *abort_flag = 7; break; }
-          }
-          __threadfence();
-        }
-        __syncwarp();
+      for (int q = 0; q < kPer; ++q) {
+        const int n = warp + kEpiWarps * q;
+        const unsigned long long x = s_red[(lane & 3) * kMaxBatch + n];
+        const uint32_t hi32 = __reduce_max_sync(0xffffffffu, (uint32_t)(x >> 32));
+        top[q] = (unsigned long long)hi32 << 32;
+        if (!kSample) top[q] |= __reduce_max_sync(0xffffffffu, (uint32_t)(x >> 32) == hi32 ? (uint32_t)x : 0u);
       }
-      ok = named_bar_all_256(!*abort_flag);
-    }
-    // the last step's winners
-    if (!kSample && ok && blockIdx.x == 0 && (int)threadIdx.x < P.b) {
-      const unsigned long long w = __ldcg(P.best + ((size_t)(P.block - 1) * kMaxBatch + threadIdx.x) * kBestStride);
-      P.next_tokens[(size_t)threadIdx.x * P.block + (P.block - 1)] = w == 0ull ? 0 : (int)(0xffffffffu - (uint32_t)(w & 0xffffffffull));
+      // this step's words: the two buffers in turn (a CTA writes a step's words when it has seen all of the step before, so those two steps
+      // older have been read), every word in kReplicas copies, of which a CTA polls one
+      const uint32_t tag = (uint32_t)(step >> 1) + 1u;
+      constexpr int kWords = kSample ? 2 : 1;
+      const size_t copy_words = (size_t)P.b * kWords * kCtaStride;
+      unsigned long long *const words = P.words + (size_t)(step & 1) * kReplicas * copy_words;
+      const unsigned long long *const my_words = words + (blockIdx.x % kReplicas) * copy_words;
+      int tok[kPer];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) tok[q] = 0;
+      if (!kSample) {
+        unsigned long long got[kPer * kCtasPerLane];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+          const int n = warp + kEpiWarps * q;
+          // key << 32 | ~(entry of the CTA's range) << 6 | tag
+          const uint32_t entry = 0xffffffffu - (uint32_t)top[q] - (uint32_t)v0;
+          if (n < P.b && lane < kReplicas)
+            publish(words + lane * copy_words + (size_t)n * kCtaStride + blockIdx.x, (top[q] >> 32 << 32) | (uint32_t)(~entry << kTagBits) | tag);
+        }
+        if (last && blockIdx.x != 0) break;     // (CTA 0 writes the last winners)
+        ok = poll_words([&](int i) -> const unsigned long long * {
+          const int n = warp + kEpiWarps * (i / kCtasPerLane), c = lane + 32 * (i % kCtasPerLane);
+          return n < P.b && c < n_ctas ? my_words + (size_t)n * kCtaStride + c : nullptr;
+        }, tag, got, abort_flag);
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+          unsigned long long x = 0ull;
+#pragma unroll
+          for (int i = 0; i < kCtasPerLane; ++i) {
+            const unsigned long long w = got[q * kCtasPerLane + i];
+            const uint32_t v = ((~(uint32_t)w) >> kTagBits) + (uint32_t)((lane + 32 * i) * P.tiles * P.rows);
+            const unsigned long long y = w >> 32 ? (w >> 32 << 32) | (0xffffffffu - v) : 0ull;
+            x = y > x ? y : x;
+          }
+          const uint32_t hi32 = __reduce_max_sync(0xffffffffu, (uint32_t)(x >> 32));
+          const uint32_t lo32 = __reduce_max_sync(0xffffffffu, (uint32_t)(x >> 32) == hi32 ? (uint32_t)x : 0u);
+          const int n = warp + kEpiWarps * q;
+          tok[q] = hi32 ? (int)(0xffffffffu - lo32) : 0;      // (no number in the row: 0)
+          if (blockIdx.x == 0 && n < P.b && lane == 0 && ok) P.next_tokens[(size_t)n * P.block + step] = tok[q];
+        }
+      } else {
+        // weight sums: lane l has the groups of four entries [l per_lane, (l + 1) per_lane) of the CTA's range (an odd number of them: no bank
+        // conflicts), three groups at a time
+        const int groups = count >> 2, tile_groups = P.rows >> 2, per_lane = ((groups + 31) >> 5) | 1, seg = 4 * per_lane;
+        unsigned long long mine[kPer];
+        unsigned long long got[kPer * 2 * kCtasPerLane];   // per request: the lane's CTAs' sums, then their exponents
+        const float *const z0 = P.z_in_place ? reinterpret_cast<const float *>(sL) : P.z + v0;
+        auto z_at = [&](int n, int e) { const int t = e / P.rows; return z0 + (size_t)n * z_row + (size_t)t * z_tile + (e - t * P.rows); };
+        Scale ref[kPer];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+          const int n = warp + kEpiWarps * q;
+          mine[q] = 0ull;
+          if (n < P.b) {
+            const uint32_t key = (uint32_t)(top[q] >> 32);
+            ref[q] = Scale(__uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key));
+            if (ref[q].finite()) {
+              int g = lane * per_lane, t = g / tile_groups, r = g - t * tile_groups;
+              const int g1 = min(groups, g + per_lane);
+              const float *const zn = z0 + (size_t)n * z_row;
+              TwoSum sum[2];
+#pragma unroll 1
+              for (; g < g1; g += 3) {
+                float4 x[3];
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                  x[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                  if (g + u < g1) x[u] = *reinterpret_cast<const float4 *>(zn + (size_t)t * z_tile + 4 * r);
+                  if (++r == tile_groups) { r = 0; ++t; }
+                }
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                  sum[0].add(pack2(ref[q].weight(x[u].x), ref[q].weight(x[u].y)));
+                  sum[1].add(pack2(ref[q].weight(x[u].z), ref[q].weight(x[u].w)));
+                }
+              }
+              mine[q] = sum[0].fixed(P.unit) + sum[1].fixed(P.unit);
+            }
+            unsigned long long s = mine[q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane < kReplicas) {
+              unsigned long long *const to = words + lane * copy_words + (size_t)(2 * n) * kCtaStride + blockIdx.x;
+              // (the sum's lowest bits travel with the exponent)
+              publish(to, (s & ~kTagMask) | tag);
+              publish(to + kCtaStride, (unsigned long long)ref[q].exponent << 2 * kTagBits | (s & kTagMask) << kTagBits | tag);
+            }
+          }
+        }
+        ok = poll_words([&](int i) -> const unsigned long long * {
+          const int q2 = i / kCtasPerLane, n = warp + kEpiWarps * (q2 / 2), c = lane * kCtasPerLane + i % kCtasPerLane;
+          return n < P.b && c < n_ctas ? my_words + (size_t)(2 * n + (q2 & 1)) * kCtaStride + c : nullptr;
+        }, tag, got, abort_flag);
+        if (ok) {
+#pragma unroll
+          for (int q = 0; q < kPer; ++q) {
+            const int n = warp + kEpiWarps * q;
+            if (n >= P.b) break;
+            unsigned long long s_all[kCtasPerLane];
+            long long e_all[kCtasPerLane], top_e = kNoWeight;
+#pragma unroll
+            for (int i = 0; i < kCtasPerLane; ++i) {
+              const bool has = lane * kCtasPerLane + i < n_ctas;
+              const unsigned long long sum = got[(2 * q) * kCtasPerLane + i], exponent = got[(2 * q + 1) * kCtasPerLane + i];
+              s_all[i] = has ? (sum & ~kTagMask) | (exponent >> kTagBits & kTagMask) : 0ull;
+              e_all[i] = has ? (long long)exponent >> 2 * kTagBits : kNoWeight;
+              top_e = e_all[i] > top_e ? e_all[i] : top_e;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              const long long t = __shfl_xor_sync(0xffffffffu, top_e, o);
+              top_e = t > top_e ? t : top_e;
+            }
+            int owner = 0, pick = 0;
+            if (top_e > kNoWeight && top_e < kInfinite) {
+              unsigned long long run = 0ull;
+#pragma unroll
+              for (int i = 0; i < kCtasPerLane; ++i) {
+                s_all[i] = lowered(s_all[i], top_e - e_all[i]);
+                run += s_all[i];
+              }
+              const unsigned long long inc = warp_scan(run, lane), total = __shfl_sync(0xffffffffu, inc, 31);
+              const unsigned long long T = threshold(P.uniforms[(size_t)n * P.block + step], total);
+              // the CTA the threshold falls into; if there is none, the last one with weight
+              unsigned long long before = inc - run, base = 0ull;
+              int found = -1;
+#pragma unroll
+              for (int i = 0; i < kCtasPerLane; ++i) {
+                if (s_all[i] && (T >= total || (before <= T && T - before < s_all[i]))) { found = lane * kCtasPerLane + i; base = before; }
+                before += s_all[i];
+              }
+              const unsigned int who = __ballot_sync(0xffffffffu, found >= 0);   // (not empty: the largest weight of the row is above 1/2)
+              const int src = 31 - __clz(who);
+              owner = __shfl_sync(0xffffffffu, found, src);
+              base = __shfl_sync(0xffffffffu, base, src);
+              if (owner == (int)blockIdx.x) {
+                // the lane whose entries the threshold falls into, then the entry
+                const long long up = top_e - ref[q].exponent;
+                const unsigned long long w = lowered(mine[q], up), from = base + (warp_scan(w, lane) - w);
+                unsigned int hit = __ballot_sync(0xffffffffu, w && from <= T && T - from < w);
+                if (!hit) hit = __ballot_sync(0xffffffffu, w != 0ull);
+                const int hl = 31 - __clz(hit ? hit : 1u);
+                unsigned long long acc = __shfl_sync(0xffffffffu, from, hl);
+                const int e0 = hl * seg, e1 = min(count, e0 + seg);
+                pick = -1;
+                int tail = e0;                                           // the last entry with weight
+#pragma unroll 1
+                for (int c0 = e0; c0 < e1 && pick < 0; c0 += 32) {
+                  unsigned long long x = 0ull;
+                  if (c0 + lane < e1) x = lowered(__float2ull_rn(ref[q].weight(*z_at(n, c0 + lane)) * P.unit), up);
+                  const unsigned long long in = warp_scan(x, lane);
+                  const unsigned int over = __ballot_sync(0xffffffffu, x && acc + in > T), some = __ballot_sync(0xffffffffu, x != 0ull);
+                  if (over) pick = c0 + __ffs(over) - 1;
+                  if (some) tail = c0 + 31 - __clz(some);
+                  acc += __shfl_sync(0xffffffffu, in, 31);
+                }
+                if (pick < 0) pick = tail;
+                pick += v0;
+              }
+            }
+            if (owner == (int)blockIdx.x && lane == 0) {
+              P.next_tokens[(size_t)n * P.block + step] = pick;
+            }
+            if (owner == (int)blockIdx.x && lane < kReplicas)
+              publish(P.drawn + ((step & 1) * kReplicas + lane) * kMaxBatch + n, (unsigned long long)pick << kTagBits | tag);
+          }
+        }
+        if (P.z_in_place) {
+          // z has been read: the slots go back (they were written here, and copies will write them next)
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) for (int k = 0; k < my_tiles; ++k) mbar_arrive(l_empty + k);
+        }
+        if (last) break;
+        unsigned long long token[1] = {0ull};
+        const unsigned long long *const mine_drawn =
+            lane < kPer && warp + kEpiWarps * lane < P.b ? P.drawn + ((step & 1) * kReplicas + blockIdx.x % kReplicas) * kMaxBatch + warp + kEpiWarps * lane : nullptr;
+        ok = ok && poll_words([&](int) { return mine_drawn; }, tag, token, abort_flag);
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) tok[q] = __shfl_sync(0xffffffffu, (int)(token[0] >> kTagBits), q);
+      }
+      if (last) break;
+      if (ok) {
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+          const int n = warp + kEpiWarps * q;
+          if (n < P.b) put_row(n, true, tok[q]);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(e_ready);
+      } else {
+        named_bar_all_256(false);   // (this warp's part of the next step's barrier: the others leave there)
+      }
     }
   }
   // ------------------------------------------------------------------ teardown
@@ -296,203 +664,38 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
   if (*abort_flag) {
     if (threadIdx.x == 0) {
       if (P.status) atomicOr(reinterpret_cast<unsigned int *>(P.status), DPARA_STATUS_TIMEOUT);
+#pragma unroll 1
       for (int k = 0; k < 4096; ++k) __nanosleep(256);  // copies that may still be in flight get a bounded time to land
     }
     __syncthreads();
   }
-  if (warp == kMmaWarp) tmem_dealloc(tmem, 64);
+  if (warp == kMmaWarp) tmem_dealloc(tmem, 512);
 }
 
-// ------------------------------------------------------------------------------------------------ sampling head loop
-// y_i ~ softmax(z_i) with a supplied uniform (App. C: temperature 1, top-p 1).  Two launches per step: the head kernel
-// above in its one-step form writes z = l_i + W E(y_{i-1}) (fp32, [b][vocab]), then the draw, spread over
-// (vocabulary chunk, request) CTAs: each CTA leaves its chunk's maximum m_c and weight sum s_c = sum exp(z - m_c) and
-// takes a ticket; the CTA that takes a request's last ticket (no CTA ever waits) rescales the chunk sums to the row
-// maximum, finds the chunk the threshold u * total falls into, rescans that one chunk in vocabulary order for the
-// crossing element, writes the token and puts the ticket back to zero.
-// Exponentials are fp32 (relative error ~1e-7, far below the fp32 logits' own), every sum is fp64.
 namespace {
-constexpr int kPickThreads = 256;
-constexpr int kPickMaxChunks = 256;          // one chunk per thread in the finishing CTA
-
-struct PickPart { float m; float pad; double s; };
-
-__host__ __device__ inline int pick_chunk_elems(int vocab) {
-  int chunk = 2048;
-  while ((vocab + chunk - 1) / chunk > kPickMaxChunks) chunk *= 2;
-  return chunk;
-}
-
-__device__ __forceinline__ double warp_sum(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-
-// inclusive block scan of one double per thread (kPickThreads threads); returns the inclusive value, total in *total
-__device__ __forceinline__ double block_scan(double x, double *s_warp, double *total) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double inc = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const double t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  __syncthreads();                       // s_warp free again
-  if (lane == 31) s_warp[w] = inc;
-  __syncthreads();
-  double before = 0.0, tot = 0.0;
-#pragma unroll
-  for (int k = 0; k < kPickThreads / 32; ++k) { if (k < w) before += s_warp[k]; tot += s_warp[k]; }
-  *total = tot;
-  return before + inc;
-}
-
-__global__ void __launch_bounds__(kPickThreads) head_sample_kernel(const float *__restrict__ z, const float *__restrict__ uniforms,
-                                                                   int32_t *__restrict__ next_tokens, PickPart *__restrict__ part,
-                                                                   unsigned int *__restrict__ tick, int vocab, int block,
-                                                                   int step, int chunk) {
-  const int n = blockIdx.y, c = blockIdx.x, n_chunks = gridDim.x, tid = threadIdx.x;
-  const float *row = z + (size_t)n * vocab;
+// Clears the words that the loop's CTAs exchange.  A kernel and not a memset: the LM head then starts behind it without a gap, and may read its weights
+// ahead of its wait.
+__global__ void __launch_bounds__(256) head_clear_kernel(uint4 *words, size_t n) {
   pdl_wait();
   pdl_launch_dependents();
-  __shared__ float s_max[kPickThreads / 32];
-  __shared__ double s_warp[kPickThreads / 32];
-  __shared__ int s_flag;
-  __shared__ int s_tok;
-  __shared__ double s_base;
-
-  // ---- phase 1: this chunk's maximum and weight sum (vocab % 8 == 0 and chunk % 1024 == 0: float4 loads never straddle)
-  const int c0 = c * chunk, c1 = min(vocab, c0 + chunk);
-  float mx = -INFINITY;
-  for (int v = c0 + tid * 4; v < c1; v += kPickThreads * 4) {
-    const float4 x = __ldcg(reinterpret_cast<const float4 *>(row + v));
-    mx = fmaxf(mx, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));          // fmaxf drops NaN operands
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((tid & 31) == 0) s_max[tid >> 5] = mx;
-  __syncthreads();
-  mx = s_max[0];
-#pragma unroll
-  for (int w = 1; w < kPickThreads / 32; ++w) mx = fmaxf(mx, s_max[w]);
-  double loc = 0.0;
-  if (mx > -INFINITY && mx < INFINITY) {
-    for (int v = c0 + tid * 4; v < c1; v += kPickThreads * 4) {
-      const float4 x = __ldcg(reinterpret_cast<const float4 *>(row + v));
-      if (x.x == x.x) loc += (double)expf(x.x - mx);
-      if (x.y == x.y) loc += (double)expf(x.y - mx);
-      if (x.z == x.z) loc += (double)expf(x.z - mx);
-      if (x.w == x.w) loc += (double)expf(x.w - mx);
-    }
-  }
-  loc = warp_sum(loc);
-  if ((tid & 31) == 0) s_warp[tid >> 5] = loc;
-  __syncthreads();
-  if (tid == 0) {
-    double s = 0.0;
-    for (int w = 0; w < kPickThreads / 32; ++w) s += s_warp[w];
-    PickPart pp; pp.m = mx; pp.pad = 0.f; pp.s = s;
-    part[(size_t)n * kPickMaxChunks + c] = pp;
-    __threadfence();
-    s_flag = atomicAdd(tick + n, 1u) == (unsigned)(n_chunks - 1);
-  }
-  __syncthreads();
-  if (!s_flag) return;
-  __threadfence();
-
-  // ---- phase 2 (the CTA that took the request's last ticket): thread t holds chunk t
-  float m_c = -INFINITY;
-  double s_c = 0.0;
-  if (tid < n_chunks) {
-    const uint4 raw = __ldcg(reinterpret_cast<const uint4 *>(part + (size_t)n * kPickMaxChunks + tid));
-    m_c = __uint_as_float(raw.x);
-    s_c = __hiloint2double((int)raw.w, (int)raw.z);
-  }
-  float M = m_c;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-  __syncthreads();
-  if ((tid & 31) == 0) s_max[tid >> 5] = M;
-  if (tid == 0) { s_tok = -1; s_flag = -1; }
-  __syncthreads();
-  M = s_max[0];
-#pragma unroll
-  for (int w = 1; w < kPickThreads / 32; ++w) M = fmaxf(M, s_max[w]);
-  int tok = 0;
-  if (M > -INFINITY && M < INFINITY) {
-    const double scale = (m_c > -INFINITY) ? exp((double)m_c - (double)M) : 0.0;
-    const double S = s_c * scale;
-    double total;
-    const double inc = block_scan(S, s_warp, &total);
-    const double T = (double)uniforms[(size_t)n * block + step] * total;
-    // the chunk the threshold falls into; when rounding puts the threshold at or past the total, the last chunk with weight
-    if (S > 0.0 && inc - S <= T && T < inc) { s_flag = tid; s_base = inc - S; }
-    __syncthreads();
-    if (s_flag < 0) {
-      if (S > 0.0) atomicMax(&s_flag, tid);
-      __syncthreads();
-      if (tid == s_flag) s_base = inc - S;
-      __syncthreads();
-    }
-    const int cs = s_flag;                               // >= 0: total > 0 because the row maximum is finite
-    __syncthreads();
-    if (tid == cs) { s_max[0] = m_c; s_warp[0] = scale; }
-    __syncthreads();
-    const float mcs = s_max[0];
-    const double scs = s_warp[0];
-    double running = s_base;
-    const int r0 = cs * chunk, r1 = min(vocab, r0 + chunk);
-    int last_w = -1;                                     // the last element with weight seen by this thread
-    for (int v0 = r0; v0 < r1; v0 += kPickThreads * 4) {
-      const int v = v0 + tid * 4;
-      double w[4] = {0.0, 0.0, 0.0, 0.0};
-      if (v < r1) {
-        const float4 x = __ldcg(reinterpret_cast<const float4 *>(row + v));
-        if (x.x == x.x) w[0] = (double)expf(x.x - mcs) * scs;
-        if (x.y == x.y) w[1] = (double)expf(x.y - mcs) * scs;
-        if (x.z == x.z) w[2] = (double)expf(x.z - mcs) * scs;
-        if (x.w == x.w) w[3] = (double)expf(x.w - mcs) * scs;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) if (w[k] > 0.0) last_w = v + k;
-      }
-      const double l4 = (w[0] + w[1]) + (w[2] + w[3]);
-      double sub_total;
-      const double inc4 = block_scan(l4, s_warp, &sub_total);
-      double acc = running + inc4 - l4;
-      if (l4 > 0.0 && acc <= T && T < acc + l4) {
-        int pick = -1;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (pick < 0 && w[k] > 0.0) { acc += w[k]; if (acc > T) pick = v + k; }
-        }
-        if (pick < 0) pick = last_w;                     // rounding inside the four: their last with weight
-        s_tok = pick;
-      }
-      __syncthreads();
-      if (s_tok >= 0) break;
-      running += sub_total;
-    }
-    if (s_tok < 0) {
-      // summation order put the threshold past this chunk's end: its last element with weight
-      atomicMax(&s_tok, last_w);
-      __syncthreads();
-    }
-    tok = s_tok < 0 ? 0 : s_tok;
-  }
-  if (tid == 0) {
-    next_tokens[(size_t)n * block + step] = tok;
-    tick[n] = 0u;                                        // the next step finds the ticket at zero
-  }
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) words[i] = make_uint4(0, 0, 0, 0);
 }
+
+size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+constexpr size_t kDrawnWords = 2 * kReplicas * kMaxBatch;
+size_t words_bytes(int b) { return ((size_t)2 * kReplicas * b * 2 * kCtaStride + kDrawnWords) * sizeof(unsigned long long); }
 }  // namespace
 
 size_t head_workspace_bytes(int b, int block, int vocab) {
   if (b <= 0 || block <= 0 || vocab <= 0) return 0;
-  const size_t logits = (((size_t)b * block * vocab * sizeof(float)) + 255) & ~size_t(255);
-  const size_t zstep = (((size_t)b * vocab * sizeof(float)) + 255) & ~size_t(255);   // sampling: one step's logits
-  return logits + (size_t)block * kMaxBatch * kBestStride * sizeof(unsigned long long) + 256 + zstep +
-         (size_t)kMaxBatch * kPickMaxChunks * sizeof(PickPart);
+  return align256((size_t)b * block * vocab * sizeof(float)) + words_bytes(b) + align256((size_t)b * vocab * sizeof(float));
+}
+
+template <int kNb>
+static void (*ar_kernel(bool sample, int slabs))(ArParams) {
+  static void (*const k[2][4])(ArParams) = {{ar_head_kernel<false, 1, kNb>, ar_head_kernel<false, 2, kNb>, ar_head_kernel<false, 3, kNb>, ar_head_kernel<false, 4, kNb>},
+                                           {ar_head_kernel<true, 1, kNb>, ar_head_kernel<true, 2, kNb>, ar_head_kernel<true, 3, kNb>, ar_head_kernel<true, 4, kNb>}};
+  return k[sample][slabs - 1];
 }
 
 dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cudaStream_t st) {
@@ -502,11 +705,26 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   if (!aligned16(h.sel_reps) || !aligned16(h.w_lm) || !aligned16(h.ar_w) || !aligned16(h.ar_e) || !aligned16(workspace)) return DPARA_ERR_INVALID_ARG;
   uint8_t *ws = static_cast<uint8_t *>(workspace);
   float *logits = reinterpret_cast<float *>(ws);
-  const size_t logits_bytes = (((size_t)h.b * h.block * h.vocab * sizeof(float)) + 255) & ~size_t(255);
-  unsigned long long *best = reinterpret_cast<unsigned long long *>(ws + logits_bytes);
-  unsigned int *barrier = reinterpret_cast<unsigned int *>(best + (size_t)h.block * kMaxBatch * kBestStride);
-  float *zstep = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(barrier) + 256);
-  if (cudaMemsetAsync(best, 0, (size_t)h.block * kMaxBatch * kBestStride * sizeof(unsigned long long) + 256, st) != cudaSuccess) return DPARA_ERR_CUDA;
+  unsigned long long *words = reinterpret_cast<unsigned long long *>(ws + align256((size_t)h.b * h.block * h.vocab * sizeof(float)));
+
+  ArParams P;
+  memset(&P, 0, sizeof(P));
+  // Tile height: as many rounds of the SMs as 128-row tiles take, evenly filled (vocabulary 151936: 1187 tiles of 128 are eight rounds of
+  // the 148 SMs and three tiles; 1333 of 114, rounded up to 116, are nine rounds of 0.9 the length), but not under 32 rows.
+  int dev = 0, sms = kNumSM;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (sms > kNumSM || sms < 1) sms = kNumSM;
+  P.tiles = ((h.vocab + 127) / 128 + sms - 1) / sms;
+  P.rows = ((h.vocab + sms * P.tiles - 1) / (sms * P.tiles) + 3) / 4 * 4;
+  if (P.rows < 32) P.rows = 32;
+  const int grid = (h.vocab + P.tiles * P.rows - 1) / (P.tiles * P.rows);
+  const int slabs = h.rank / 64, nb = h.b <= 16 ? 16 : 32;
+  const bool sample = h.uniforms != nullptr;
+
+  const size_t vecs = (kDrawnWords + (size_t)2 * kReplicas * h.b * (sample ? 2 : 1) * kCtaStride) / 2;   // 16 bytes each
+  launch_pdl(head_clear_kernel, dim3((unsigned)(vecs < 148 * 256 ? (vecs + 255) / 256 : 148)), dim3(256), 0, st, reinterpret_cast<uint4 *>(words), vecs);
+  DPARA_CHECK_LAUNCH();
+  count_launches(1);
 
   // base logits of the selected branches, fp32, stored step-major [block][b][vocab] (GEMM row n * block + i goes
   // to row i * b + n): the b rows a step reads then lie in one contiguous range instead of b ranges
@@ -514,54 +732,61 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   GemmArgs g;
   g.a = h.sel_reps; g.w = h.w_lm; g.M = h.b * h.block; g.N = h.vocab; g.K = h.hidden; g.epi = 3;
   g.resid = nullptr; g.resid_bf16 = 0; g.out = logits; g.out_bf16 = nullptr; g.perm_block = h.block; g.perm_b = h.b;
+  g.w_ready = 1;   // the kernel in front clears words of the workspace
   dpara_status rc = launch_gemm_tc(g, status, st);
   if (rc != DPARA_OK) return rc;
 
-  ArParams P;
-  memset(&P, 0, sizeof(P));
-  // Tile height: as many rounds of the SMs as 128-row tiles take, evenly filled (vocabulary 151936: 1187 tiles of 128 are eight rounds of
-  // the 148 SMs and three tiles; 1310 of 116 are nine rounds of 0.9 the length), but not under 32 rows.
-  int dev = 0, sms = kNumSM;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int rounds = ((h.vocab + 127) / 128 + sms - 1) / sms;
-  P.rows = ((h.vocab + sms * rounds - 1) / (sms * rounds) + 3) / 4 * 4;
-  if (P.rows < 32) P.rows = 32;
   if (!make_tmap_bf16_2d(&P.map_w, h.ar_w, h.rank, h.vocab, (uint64_t)h.rank * 2, 64, P.rows)) return DPARA_ERR_CUDA;
-  if (!make_tmap_f32_2d(&P.map_l, logits, h.vocab, (uint64_t)h.block * h.b, (uint64_t)h.vocab * 4, P.rows, h.b <= 16 ? 16 : 32)) return DPARA_ERR_CUDA;
-  P.ar_e = static_cast<const uint16_t *>(h.ar_e); P.bonus = h.bonus; P.next_tokens = h.next_tokens;
-  P.best = best; P.barrier = barrier; P.status = status;
-  P.b = h.b; P.block = h.block; P.vocab = h.vocab; P.rank = h.rank;
-  P.n_tiles = (h.vocab + P.rows - 1) / P.rows;
-  P.nb = h.b <= 16 ? 16 : 32;
-  const int stage_bytes = 128 * h.rank * 2 + P.nb * 128 * 4;
-  const int fixed = (h.rank / 64) * P.nb * 128 + 1024 + 2048;   // Ey, alignment slack, barriers and reduction scratch
-  P.stages = (227 * 1024 - fixed) / stage_bytes > 4 ? 4 : (227 * 1024 - fixed) / stage_bytes;
-  const int smem = P.stages * stage_bytes + fixed;
-  void (*const kernels[2][4])(ArParams) = {{ar_head_kernel<false, 1>, ar_head_kernel<false, 2>, ar_head_kernel<false, 3>, ar_head_kernel<false, 4>},
-                                           {ar_head_kernel<true, 1>, ar_head_kernel<true, 2>, ar_head_kernel<true, 3>, ar_head_kernel<true, 4>}};
-  void (*const kernel)(ArParams) = kernels[h.uniforms ? 1 : 0][h.rank / 64 - 1];
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return DPARA_ERR_CUDA;
-  const int grid = P.n_tiles < sms ? P.n_tiles : sms;
-  if (h.uniforms) {
-    // ---- sampling: per step the logits z (one-step head kernel), then the draw.  The tickets live in the zeroed 256 bytes
-    // after the greedy path's barrier word (kMaxBatch words from byte 128).
-    unsigned int *tick = barrier + 32;
-    PickPart *part = reinterpret_cast<PickPart *>(reinterpret_cast<uint8_t *>(zstep) + ((((size_t)h.b * h.vocab * sizeof(float)) + 255) & ~size_t(255)));
-    const int chunk = pick_chunk_elems(h.vocab), n_chunks = (h.vocab + chunk - 1) / chunk;
-    P.z_out = zstep;
-    for (int i = 0; i < h.block; ++i) {
-      P.step0 = i;
-      launch_pdl(kernel, dim3(grid), dim3(kThreads), (size_t)smem, st, P);
-      DPARA_CHECK_LAUNCH();
-      launch_pdl(head_sample_kernel, dim3(n_chunks, h.b), dim3(kPickThreads), 0, st, static_cast<const float *>(zstep), h.uniforms, h.next_tokens, part, tick, h.vocab, h.block, i, chunk);
-      DPARA_CHECK_LAUNCH();
-      count_launches(2);
-    }
-    return DPARA_OK;
+  if (!make_tmap_f32_2d(&P.map_l, logits, h.vocab, (uint64_t)h.block * h.b, (uint64_t)h.vocab * 4, P.rows, h.b)) return DPARA_ERR_CUDA;
+  P.ar_w = static_cast<const uint16_t *>(h.ar_w); P.ar_e = static_cast<const uint16_t *>(h.ar_e);
+  int bits = 0;
+  while (bits < 31 && ((h.vocab - 1) >> bits) != 0) ++bits;
+  P.unit = ldexpf(1.f, 62 - bits);
+  P.bonus = h.bonus; P.uniforms = h.uniforms; P.next_tokens = h.next_tokens;
+  P.drawn = words; P.words = words + kDrawnWords; P.status = status;
+  P.z = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(words) + words_bytes(h.b));
+  P.b = h.b; P.block = h.block; P.vocab = h.vocab;
+  // Tiles that stay: what fits behind the accumulators; one step alone reads W once either way.
+  P.resident = h.block > 1 ? (512 - kResidentCol) / (32 * slabs) : 0;
+  if (P.resident > P.tiles) P.resident = P.tiles;
+  P.slab_bytes = (P.rows + 7) / 8 * 1024;
+  P.logit_bytes = (h.b * P.rows * 4 + 127) / 128 * 128;
+  const int tile_bytes = slabs * P.slab_bytes, e_bytes = slabs * nb * 128, room = 227 * 1024 - 1024 - e_bytes - kBarBytes;
+  const int streamed = P.tiles - P.resident, most = streamed < 1 ? 1 : (streamed < kMaxStages ? streamed : kMaxStages);
+  auto stages_with = [&](int slots) {
+    const int n = (room - slots * P.logit_bytes) / tile_bytes;
+    return n < 0 ? 0 : (n < most ? n : most);
+  };
+  if (sample && P.tiles <= kMaxLogitSlots && stages_with(P.tiles) >= (most < 2 ? most : 2)) {
+    P.z_in_place = 1;
+    P.logit_slots = P.tiles;
+  } else {
+    // two to four slots of base logits, as many as cost the ring of W nothing
+    P.logit_slots = 2;
+    while (P.logit_slots < 4 && stages_with(P.logit_slots + 1) == stages_with(2)) ++P.logit_slots;
   }
-  // cooperative launch: the grid barrier needs every CTA resident (one CTA per SM fits by construction)
-  void *args[] = {&P};
-  if (cudaLaunchCooperativeKernel(reinterpret_cast<void *>(kernel), dim3(grid), dim3(kThreads), args, smem, st) != cudaSuccess) {
+  P.stages = stages_with(P.logit_slots);
+  P.e_off = P.stages * tile_bytes;
+  P.logit_off = P.e_off + e_bytes;
+  P.bar_off = P.logit_off + P.logit_slots * P.logit_bytes;
+  int smem = P.bar_off + kBarBytes + 1024;
+  if (smem < P.e_off + 128 * 128 + 1024) smem = P.e_off + 128 * 128 + 1024;   // (a product reads 128 rows of a slab, however many were filled)
+  void (*const kernel)(ArParams) = nb == 16 ? ar_kernel<16>(sample, slabs) : ar_kernel<32>(sample, slabs);
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) return DPARA_ERR_CUDA;
+  // cooperative: the CTAs wait for one another's words, so every one has to be resident (one per SM fits by construction)
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, kernel, P) != cudaSuccess) {
     cudaGetLastError();
     return DPARA_ERR_CUDA;
   }
