@@ -37,7 +37,7 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
   return v;
 }
 
-// Copy of the selected branch: reps[n][r] -> selected[n], `bytes` per request.
+// Copy of the selected branch: reps[n][r] -> selected[n], `bytes` per request; by `nthreads` threads in all.
 __device__ __forceinline__ void gather_branch(const uint8_t *__restrict__ reps, uint8_t *__restrict__ selected, int n,
                                               size_t req_bytes, int r, size_t bytes, int tid, int nthreads) {
   const uint8_t *src = reps + (size_t)n * req_bytes + (size_t)r * bytes;
@@ -317,20 +317,30 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampling_kernel(const Verif
   const int end = min(P.V, base + kSampChunk);
   unsigned long long a0 = 0, a1 = 0;
   if (P.vec_ok) {
+    constexpr int kPieces = kSampChunk / (kVsThreads * 4);
+    float4 pv[kPieces], qv[kPieces];
 #pragma unroll
-    for (int it = 0; it < kSampChunk / (kVsThreads * 4); ++it) {
-      int idx = base + (it * kVsThreads + tid) * 4;
+    for (int it = 0; it < kPieces; ++it) {
+      const int idx = base + (it * kVsThreads + tid) * 4;
+      pv[it] = qv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (idx < end) {
-        float4 pv = __ldg(reinterpret_cast<const float4 *>(prow + idx));
-        float4 qv = residual ? __ldg(reinterpret_cast<const float4 *>(qrow + idx)) : pv;
-        unsigned long long w0, w1;
-        weights_of(pv.x, qv.x, residual, w0, w1); a0 += w0; a1 += w1;
-        weights_of(pv.y, qv.y, residual, w0, w1); a0 += w0; a1 += w1;
-        weights_of(pv.z, qv.z, residual, w0, w1); a0 += w0; a1 += w1;
-        weights_of(pv.w, qv.w, residual, w0, w1); a0 += w0; a1 += w1;
+        pv[it] = __ldg(reinterpret_cast<const float4 *>(prow + idx));
+        if (residual) qv[it] = __ldg(reinterpret_cast<const float4 *>(qrow + idx));
       }
     }
+    // The accepted length is known: every CTA copies its share of the selected branch while its rows are on their way (one CTA copied all of
+    // it behind the draw, 128 KB a request at b = 8: with the wide loads of the crossing chunk below the call 23.9 -> 9.3 us).  An early start may not read it yet.
+    if (P.reps && !P.early) gather_branch(P.reps, P.selected, n, P.req_bytes, r, P.rep_bytes, c * kVsThreads + tid, P.nchunks * kVsThreads);
+#pragma unroll
+    for (int it = 0; it < kPieces; ++it) {
+      unsigned long long w0, w1;
+      weights_of(pv[it].x, qv[it].x, residual, w0, w1); a0 += w0; a1 += w1;
+      weights_of(pv[it].y, qv[it].y, residual, w0, w1); a0 += w0; a1 += w1;
+      weights_of(pv[it].z, qv[it].z, residual, w0, w1); a0 += w0; a1 += w1;
+      weights_of(pv[it].w, qv[it].w, residual, w0, w1); a0 += w0; a1 += w1;
+    }
   } else {
+    if (P.reps && !P.early) gather_branch(P.reps, P.selected, n, P.req_bytes, r, P.rep_bytes, c * kVsThreads + tid, P.nchunks * kVsThreads);
     for (int idx = base + tid; idx < end; idx += kVsThreads) {
       unsigned long long w0, w1;
       weights_of(prow[idx], qrow[idx], residual, w0, w1);
@@ -357,6 +367,7 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampling_kernel(const Verif
 
   // ---- last CTA of request n: total weight, threshold, locate the crossing
   if (P.early) pdl_wait();     // before the branch is read and before the request's part of the call completes
+  const float u_draw = P.uniforms[(size_t)n * P.J + g];   // (on its way while the sums are read)
   __threadfence();
   __shared__ unsigned long long s_T, s_basepref;
   __shared__ int s_chunk, s_which, s_tok;
@@ -382,7 +393,7 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampling_kernel(const Verif
       const unsigned long long Wt = which ? W1 : W0;
       // a uniform is m * 2^-24 with m < 2^24; anything at or above 1 is taken as the largest uniform, so the
       // threshold stays below the total weight and the draw inside the vocabulary
-      unsigned int m = __float2uint_rn(fminf(P.uniforms[(size_t)n * P.J + g], 1.0f) * 16777216.0f);
+      unsigned int m = __float2uint_rn(fminf(u_draw, 1.0f) * 16777216.0f);
       m = m > 16777215u ? 16777215u : m;
       const unsigned long long lo = (unsigned long long)m * Wt;  // low 64 bits
       const unsigned long long hi = __umul64hi((unsigned long long)m, Wt);
@@ -416,7 +427,7 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampling_kernel(const Verif
       unsigned long long Wt = which ? W1 : W0;
       // a uniform is m * 2^-24 with m < 2^24; anything at or above 1 is taken as the largest uniform, so the
       // threshold stays below the total weight and the draw inside the vocabulary
-      unsigned int m = __float2uint_rn(fminf(P.uniforms[(size_t)n * P.J + g], 1.0f) * 16777216.0f);
+      unsigned int m = __float2uint_rn(fminf(u_draw, 1.0f) * 16777216.0f);
       m = m > 16777215u ? 16777215u : m;
       unsigned long long lo = (unsigned long long)m * Wt;  // low 64 bits
       unsigned long long hi = __umul64hi((unsigned long long)m, Wt);
@@ -441,11 +452,32 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampling_kernel(const Verif
     const int per = kSampChunk / kVsThreads;
     unsigned long long w[kSampChunk / kVsThreads];
     unsigned long long loc = 0;
+    // (16-byte loads where the rows allow it: element by element a warp's lanes, 64 bytes apart, took sixteen times as many sectors)
+    float pe[kSampChunk / kVsThreads], qe[kSampChunk / kVsThreads];
+    if (P.vec_ok) {
+#pragma unroll
+      for (int e = 0; e < per; e += 4) {
+        const int idx = cb + tid * per + e;
+        float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), qv = pv;
+        if (idx < P.V) {
+          pv = __ldg(reinterpret_cast<const float4 *>(prow + idx));
+          if (residual) qv = __ldg(reinterpret_cast<const float4 *>(qrow + idx));
+        }
+        pe[e] = pv.x; pe[e + 1] = pv.y; pe[e + 2] = pv.z; pe[e + 3] = pv.w;
+        qe[e] = qv.x; qe[e + 1] = qv.y; qe[e + 2] = qv.z; qe[e + 3] = qv.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < per; ++e) {
+        const int idx = cb + tid * per + e;
+        pe[e] = idx < P.V ? prow[idx] : 0.f;
+        qe[e] = idx < P.V && residual ? qrow[idx] : 0.f;
+      }
+    }
 #pragma unroll
     for (int e = 0; e < per; ++e) {
-      int idx = cb + tid * per + e;
-      unsigned long long w0 = 0, w1 = 0;
-      if (idx < P.V) weights_of(prow[idx], qrow[idx], residual, w0, w1);
+      unsigned long long w0, w1;
+      weights_of(pe[e], qe[e], residual, w0, w1);
       w[e] = which ? w1 : w0;
       loc += w[e];
     }
@@ -495,7 +527,7 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampling_kernel(const Verif
   __syncthreads();
   for (int i = tid; i < 2 * P.nchunks; i += kVsThreads) P.ws64[(size_t)n * P.nchunks * 2 + i] = 0ull;
   if (tid == 0) P.counters[n] = 0u;
-  if (P.reps) gather_branch(P.reps, P.selected, n, P.req_bytes, r, P.rep_bytes, tid, kVsThreads);
+  if (P.reps && P.early) gather_branch(P.reps, P.selected, n, P.req_bytes, r, P.rep_bytes, tid, kVsThreads);
 }
 
 // Greedy: 16-byte loads in flight per thread.  As many as possible (fewer, larger CTAs amortise the reduction
