@@ -4,14 +4,16 @@
 // Per drafter layer: rmsnorm of the candidate feature rows -> one tensor-core GEMM against the layer's [keys | values]
 // projection -> a row-wise kernel that applies the per-head key norm and the rotary embedding at the row's position
 // and writes the r + 1 accepted rows of every request behind the filled part of that layer's cache.  One layer's product
-// is skinny (a few hundred rows against a 2 Hkv D x F weight: 8 output tiles at the benchmark shape), so with more than
-// 128 rows up to eight layers go into ONE grouped launch, their K ranges cut in parts where that evens out the rounds;
-// the parts leave fp32 partial sums and ONE row-wise launch for the same layers adds them (rounding the sum to bf16, as
-// a single product's bf16 store would).  The accepted
+// is skinny (a few hundred rows against a 2 Hkv D x F weight: 8 output tiles at the benchmark shape), so up to eight
+// layers go into ONE grouped launch, with more than 128 rows and few layers their K ranges cut in parts; the parts leave
+// fp32 partial sums and ONE row-wise launch for the same layers adds them (rounding the sum to bf16, as a single
+// product's bf16 store does).  The accepted
 // length is read on the device (it is the output of the verify/select call queued before), so no host round trip
 // sits between verification and the append.  All d + 1 candidate rows go through the GEMM: it is bound by reading the
 // projection weights once (2 Hkv D x F bf16 per layer), not by the row count.
 #include <math.h>
+
+#include <algorithm>
 
 #include "gemm.cuh"
 #include "layer.cuh"
@@ -19,9 +21,8 @@
 namespace dpara {
 
 struct AppendParams {
-  const uint16_t *kv;       // n_parts == 0: layer g of the launch: [b * J][2 * Hkv * D] bf16, [keys | values] of every candidate row, from kv + g * part_stride
-  const float *kv_parts;    // layer g of the launch: [n_parts][b * J][2 * Hkv * D] fp32 partial sums from kv_parts + g * n_parts * part_stride
-  int n_parts;
+  const uint16_t *kv;       // no parts: layer g of the launch: [b * J][2 * Hkv * D] bf16, [keys | values] of every candidate row, from kv + g * part_stride
+  const float *kv_parts;    // layer g of the launch: [parts][b * J][2 * Hkv * D] fp32 partial sums from kv_parts + g * parts * part_stride
   size_t part_stride;       // elements between two parts (two layers' rows)
   // per layer of the launch (blockIdx.y)
   const uint16_t *knorm_w[kGemmMaxGroups];  // [D] or null
@@ -34,15 +35,17 @@ struct AppendParams {
   double inv_freq[64];      // theta^(-2 d / D), d < D / 2, worked out on the host in double precision
 };
 
-// One CTA per (candidate row (request n, draft position i), layer of the launch); rows above the accepted length leave at once.
+// One CTA per (candidate row (request n, draft position i), layer of the launch); rows above the accepted length leave at once.  What a row takes is
+// round trips to memory, so a thread has all it needs of a head (or of its piece of v) in flight before the first addition: kParts is a template
+// argument (0: bf16 rows), a lane owns four neighbouring elements of either half of a key head and D / 8 lanes share the head.
+// With 4-byte loads in a loop over a run-time number of parts the launch took 18 us of the 256-row call of five layers; that call 54.7 -> 44.7 with the plan below.
+template <int kParts>
 __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) {
   extern __shared__ float s_cs[];  // cos[D/2], sin[D/2]
   const int n = blockIdx.x / P.J, i = blockIdx.x % P.J, tid = threadIdx.x, g = blockIdx.y;
   // Outcome, length and angles before the wait: the kernel in front is the projection, which writes none of them, and it lets this one
   // go only when everything before it has ended (256 rows, five layers: 57.0 -> 54.5 us).
   const uint16_t *knorm_w = P.knorm_w[g];
-  const uint16_t *kv = P.kv + (size_t)g * P.part_stride;
-  const float *kv_parts = P.kv_parts + (size_t)g * P.n_parts * P.part_stride;
   const int r = P.accept_len[n];
   const long long L = P.ctx_len[n];
   const bool fits = r >= 0 && r < P.J && L + r + 1 <= P.capacity[n];
@@ -56,6 +59,7 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
       s_cs[half + d] = (float)sn;
     }
   }
+  const size_t row = (size_t)((fits ? P.row_start[n] : 0) + L + i);
   pdl_wait();
   pdl_launch_dependents();
   if (!fits) {  // does not fit (or no valid outcome): the request is left alone
@@ -63,63 +67,91 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
     return;
   }
   if (i > r) return;  // rejected suffix: dropped
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31;
-  const size_t row = (size_t)(P.row_start[n] + L + i);
-  const size_t src_off = (size_t)blockIdx.x * 2 * P.Hkv * P.D;
-  // element `e` of this candidate row as the bf16 value the projection stores (split K: the rounded sum of the parts)
-  auto kv_at = [&](size_t e) -> float {
-    if (P.n_parts == 0) return bf16_bits_to_float(kv[src_off + e]);
-    float acc = 0.f;
-    for (int s = 0; s < P.n_parts; ++s) acc += __ldg(kv_parts + (size_t)s * P.part_stride + src_off + e);
-    return __bfloat162float(__float2bfloat16_rn(acc));
-  };
-  const int E = P.D / 64;  // pairs (d, d + D/2) per lane
-  for (int h = warp; h < P.Hkv; h += 4) {
-    const size_t ks = (size_t)h * P.D;
-    uint16_t *kd = P.k_cache[g] + (row * P.Hkv + h) * P.D;
-    float x1[2], x2[2], ss = 0.f;
-    for (int e = 0; e < E; ++e) {
-      const int d = lane + 32 * e;
-      x1[e] = kv_at(ks + d);
-      x2[e] = kv_at(ks + d + half);
-      ss += x1[e] * x1[e] + x2[e] * x2[e];
-    }
-    if (knorm_w) {
+  const size_t src = (size_t)blockIdx.x * 2 * P.Hkv * P.D;
+  const uint16_t *kv = P.kv + (size_t)g * P.part_stride + src;
+  const float *kv_parts = P.kv_parts + (size_t)g * kParts * P.part_stride + src;
+  constexpr int kLoads = kParts ? kParts : 1;
+  struct Raw { float4 v[kLoads]; };
+  // four neighbouring elements: their loads ...
+  auto fetch = [&](int e, Raw &raw) {
+    if (kParts == 0) {
+      const uint2 w = *reinterpret_cast<const uint2 *>(kv + e);
+      raw.v[0] = make_float4(bf16lo(w.x), bf16hi(w.x), bf16lo(w.y), bf16hi(w.y));
+    } else {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      for (int s = 0; s < kLoads; ++s) raw.v[s] = __ldg(reinterpret_cast<const float4 *>(kv_parts + (size_t)s * P.part_stride + e));
+    }
+  };
+  // ... and their values as the bf16 the projection stores (split K: the rounded sum of the parts)
+  auto value = [&](const Raw &raw, float (&x)[4]) {
+    float4 a = raw.v[0];
+#pragma unroll
+    for (int s = 1; s < kLoads; ++s) { a.x += raw.v[s].x; a.y += raw.v[s].y; a.z += raw.v[s].z; a.w += raw.v[s].w; }
+    const float y[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) x[e] = __bfloat162float(__float2bfloat16_rn(y[e]));
+  };
+  const int per_head = P.D / 8, sub = tid % per_head, step = 128 / per_head;   // lanes of a head; heads of the CTA at a time
+  const int vs = P.Hkv * P.D, d = 4 * sub;
+  // the first pieces of v are on their way while the keys are worked on
+  Raw va, vb;
+  const int c0 = tid * 4;
+  if (kParts && c0 < vs) fetch(vs + c0, va);
+  if (kParts && c0 + 512 < vs) fetch(vs + c0 + 512, vb);
+  for (int h0 = 0; h0 < P.Hkv; h0 += step) {
+    const int h = h0 + tid / per_head;
+    const bool has = h < P.Hkv;      // (all lanes of a warp take part in the sums, also those behind the last head)
+    Raw lo, hi;
+    float x1[4] = {}, x2[4] = {};
+    if (has) { fetch(h * P.D + d, lo); fetch(h * P.D + half + d, hi); }
+    uint2 g1 = make_uint2(0x3f803f80u, 0x3f803f80u), g2 = g1;
+    if (knorm_w) { g1 = *reinterpret_cast<const uint2 *>(knorm_w + d); g2 = *reinterpret_cast<const uint2 *>(knorm_w + half + d); }
+    if (h0 == 0) __syncthreads();   // (the angles)
+    if (has) { value(lo, x1); value(hi, x2); }
+    if (knorm_w) {
+      float ss = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) ss += x1[e] * x1[e] + x2[e] * x2[e];
+      for (int o = per_head / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
       const float rs = rsqrtf(ss / (float)P.D + P.eps);
-      for (int e = 0; e < E; ++e) {
-        const int d = lane + 32 * e;
-        x1[e] = __bfloat162float(__float2bfloat16_rn(x1[e] * rs * bf16_bits_to_float(knorm_w[d])));
-        x2[e] = __bfloat162float(__float2bfloat16_rn(x2[e] * rs * bf16_bits_to_float(knorm_w[d + half])));
+      const float f1[4] = {bf16lo(g1.x), bf16hi(g1.x), bf16lo(g1.y), bf16hi(g1.y)}, f2[4] = {bf16lo(g2.x), bf16hi(g2.x), bf16lo(g2.y), bf16hi(g2.y)};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        x1[e] = __bfloat162float(__float2bfloat16_rn(x1[e] * rs * f1[e]));
+        x2[e] = __bfloat162float(__float2bfloat16_rn(x2[e] * rs * f2[e]));
       }
     }
-    for (int e = 0; e < E; ++e) {
-      const int d = lane + 32 * e;
-      float y1 = x1[e], y2 = x2[e];
+    float y1[4], y2[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      y1[e] = x1[e]; y2[e] = x2[e];
       if (P.use_rope) {
-        const float cs = s_cs[d], sn = s_cs[half + d];
-        y1 = x1[e] * cs - x2[e] * sn;
-        y2 = x2[e] * cs + x1[e] * sn;
+        const float cs = s_cs[d + e], sn = s_cs[half + d + e];
+        y1[e] = x1[e] * cs - x2[e] * sn;
+        y2[e] = x2[e] * cs + x1[e] * sn;
       }
-      kd[d] = __bfloat16_as_ushort(__float2bfloat16_rn(y1));
-      kd[d + half] = __bfloat16_as_ushort(__float2bfloat16_rn(y2));
+    }
+    if (has) {
+      uint16_t *kd = P.k_cache[g] + (row * P.Hkv + h) * P.D;
+      *reinterpret_cast<uint2 *>(kd + d) = make_uint2(pack_bf16(y1[0], y1[1]), pack_bf16(y1[2], y1[3]));
+      *reinterpret_cast<uint2 *>(kd + half + d) = make_uint2(pack_bf16(y2[0], y2[1]), pack_bf16(y2[2], y2[3]));
     }
   }
-  const size_t vs = (size_t)P.Hkv * P.D;
   uint16_t *vd = P.v_cache[g] + row * P.Hkv * P.D;
-  if (P.n_parts == 0) {
-    for (int c = tid * 8; c < P.Hkv * P.D; c += 128 * 8) *reinterpret_cast<uint4 *>(vd + c) = *reinterpret_cast<const uint4 *>(kv + src_off + vs + c);
-  } else {
-    for (int c = tid * 4; c < P.Hkv * P.D; c += 128 * 4) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int s = 0; s < P.n_parts; ++s) {
-        const float4 x = __ldg(reinterpret_cast<const float4 *>(kv_parts + (size_t)s * P.part_stride + src_off + vs + c));
-        acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-      }
-      *reinterpret_cast<uint2 *>(vd + c) = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
-    }
+  if (kParts == 0) {
+    for (int c = tid * 8; c < vs; c += 128 * 8) *reinterpret_cast<uint4 *>(vd + c) = *reinterpret_cast<const uint4 *>(kv + vs + c);
+    return;
+  }
+  auto put = [&](int c, const Raw &raw) {
+    float x[4];
+    value(raw, x);
+    *reinterpret_cast<uint2 *>(vd + c) = make_uint2(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]));
+  };
+  if (c0 < vs) put(c0, va);
+  if (c0 + 512 < vs) put(c0 + 512, vb);
+  for (int c = c0 + 1024; c < vs; c += 512) {
+    fetch(vs + c, va);
+    put(c, va);
   }
 }
 
@@ -134,25 +166,35 @@ __global__ void append_commit_kernel(int64_t *ctx_len, const int64_t *capacity, 
   }
 }
 
-// Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores (at most 128 rows: the
-// kernel for few rows takes all layers at once, one chain of sums over K each; the whole call, 8 rows, five layers of 2048 x 4096: 192 us with a
-// product a layer, 38 now).  The parts are chosen to minimise
-// rounds x (K slabs per part + ~8 slabs' worth of fixed cost per work unit) over the CTA pairs.
+// Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores, one chain of sums over K each (at most
+// 128 rows: the kernel for few rows takes all layers at once; the whole call, 8 rows, five layers of 2048 x 4096: 192 us with a product a layer,
+// 38 now).  More rows: the CTA pairs, K in parts where the layers' tiles alone leave pairs idle.  Model in us: rounds of the pairs x (0.33 a
+// slab + 3 a unit), and 2.3 for every plane of partial sums written and read back.  Measured, whole call in graph replay, 256 rows against
+// 2048 x 5120 (us; no parts / 2 / 3 / 4 / 6 / 8): one layer 26.7 / 20.0 / 18.1 / 18.0 / 19.4 / 19.1, two 29.0 / 22.0 / 23.3 / 21.8 / 27.0 / 25.8, three 31.0 /
+// 29.3 / 25.5 / 32.8 / .., five 41.8 / 44.5 / 41.1 / 45.5 / 49.9 / 55.7, eight 48.9 / 53.2 / 57.8 / 62.7 / ..
+constexpr int kMaxParts = 4;
 static void cache_group_plan(const dpara_cache_io *io, int layers_left, int *group, int *parts) {
   const int M = io->batch * io->n_rows, N = 2 * io->n_kv_heads * io->head_dim;
   *group = layers_left < kGemmMaxGroups ? layers_left : kGemmMaxGroups;
   *parts = 0;
   if (M <= 128) return;
   const int tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = kNumSM / 2, nkb = io->feat_dim / 64;
-  int best = 1;
-  long best_cost = -1;
-  for (int s = 1; s <= 8; s *= 2) {
+  double best = 0;
+  for (int s = 1; s <= kMaxParts; ++s) {
     if (s > 1 && nkb / s < 4) break;
     const long units = (long)*group * tiles * s;
-    const long cost = ((units + pairs - 1) / pairs) * (nkb / s + 8);
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
+    const double us = ((units + pairs - 1) / pairs) * (((nkb + s - 1) / s) * 0.33 + 3.0) + (s > 1 ? 2.3 * s : 0.0);
+    if (s == 1 || us < best) { best = us; *parts = s > 1 ? s : 0; }
   }
-  *parts = best;
+}
+
+static void (*append_rows_of(int parts))(AppendParams) {
+  switch (parts) {
+    case 0: return append_rows_kernel<0>;
+    case 2: return append_rows_kernel<2>;
+    case 3: return append_rows_kernel<3>;
+    default: return append_rows_kernel<kMaxParts>;
+  }
 }
 
 // normalised copies of the feature rows: one per run of layers that share the input norm
@@ -167,17 +209,15 @@ size_t cache_append_workspace_bytes(const dpara_cache_io *io) {
   const size_t M = (size_t)io->batch * io->n_rows, N = (size_t)2 * io->n_kv_heads * io->head_dim;
   int group, parts;
   cache_group_plan(io, io->n_layers, &group, &parts);
-  if (!parts) return (size_t)cache_norm_slots(io) * align_up(M * io->feat_dim * 2, 256) + align_up((size_t)group * M * N * 2, 256);
-  // planes of partial sums: the first launch has the most layers, the last (smaller) one may cut K in more parts --
-  // sized for the larger of the two
-  size_t planes = (size_t)group * parts;
+  auto rows_bytes = [&](int layers, int p) { return align_up((size_t)layers * M * N * (p ? 4 * p : 2), 256); };
+  size_t rows = rows_bytes(group, parts);
+  // (the first launch has the most layers, the last (smaller) one may cut K in more parts: sized for the larger of the two)
   const int rest = io->n_layers % kGemmMaxGroups;
   if (io->n_layers > kGemmMaxGroups && rest) {
-    int g2, p2;
-    cache_group_plan(io, rest, &g2, &p2);
-    planes = planes > (size_t)g2 * p2 ? planes : (size_t)g2 * p2;
+    cache_group_plan(io, rest, &group, &parts);
+    rows = std::max(rows, rows_bytes(group, parts));
   }
-  return (size_t)cache_norm_slots(io) * align_up(M * io->feat_dim * 2, 256) + align_up(planes * M * N * 4, 256);
+  return (size_t)cache_norm_slots(io) * align_up(M * io->feat_dim * 2, 256) + rows;
 }
 
 dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int32_t *status_word, cudaStream_t st) {
@@ -222,8 +262,9 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
     dpara_status s = launch_gemm_tc(g, status_word, st);
     if (s != DPARA_OK) return s;
     P.kv = kv;
-    P.kv_parts = reinterpret_cast<const float *>(kv); P.n_parts = parts;
-    launch_pdl(append_rows_kernel, dim3(M, group), dim3(128), io->head_dim * sizeof(float), st, P);
+    P.kv_parts = reinterpret_cast<const float *>(kv); 
+    void (*const rows)(AppendParams) = append_rows_of(parts);
+    launch_pdl(rows, dim3(M, group), dim3(128), io->head_dim * sizeof(float), st, P);
     DPARA_CHECK_LAUNCH();
     count_launches(1);
     l0 += group;
