@@ -198,3 +198,19 @@ def test_early_start_behind_the_attention_kernel(mode):
         for f in ("accept_len", "bonus", "gather_idx", "out_tokens", "selected"):
             assert torch.equal(getattr(plain, f), getattr(early, f)), (rnd, f)
         assert plain.status.item() == early.status.item() == 0
+
+
+@pytest.mark.parametrize("b,J,V", [
+    (1, 1, 16),          # one CTA
+    (4, 37, 10000),      # 148 CTAs; rows 32 .. 36: the second word of the decision
+    (3, 7, 151936),      # 210 CTAs, ten to a row
+    (12, 37, 4096),      # 444 CTAs: as many as run at once
+    (7, 64, 1000),       # 448: more than run at once, the form that decides row by row
+])
+def test_greedy_in_one_wave_and_above(b, J, V):
+    """Calls whose CTAs all run at once leave a slot per CTA and take one ticket per request; deciding rows at both ends, drafts outside the vocabulary."""
+    v = W.make_verify_inputs(W.VerifyShape(b, J, V, 3, 64, "greedy", 0.9, 1.0), 50 + b, force_full=[0], force_zero=[b - 1] if b > 1 else [])
+    if J > 3 and b > 2:
+        v.draft_tokens[1, J - 2] = V
+        v.draft_tokens[2, 0] = -1
+    _check(v, 0)
