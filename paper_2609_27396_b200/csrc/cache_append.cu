@@ -4,10 +4,10 @@
 // Per drafter layer: rmsnorm of the candidate feature rows -> one tensor-core GEMM against the layer's [keys | values]
 // projection -> a row-wise kernel that applies the per-head key norm and the rotary embedding at the row's position
 // and writes the r + 1 accepted rows of every request behind the filled part of that layer's cache.  One layer's product
-// is skinny (a few hundred rows against a 2 Hkv D x F weight: 8 output tiles at the benchmark shape), so up to eight
-// layers go into ONE grouped launch, with more than 128 rows and few layers their K ranges cut in parts; the parts leave
-// fp32 partial sums and ONE row-wise launch for the same layers adds them (rounding the sum to bf16, as a single
-// product's bf16 store does).  The accepted
+// is skinny (a few hundred rows against a 2 Hkv D x F weight: 8 output tiles at the benchmark shape), so with more than
+// 128 rows up to eight layers go into ONE grouped launch, their K ranges cut in parts where that evens out the rounds;
+// the parts leave fp32 partial sums and ONE row-wise launch for the same layers adds them (rounding the sum to bf16, as
+// a single product's bf16 store would).  The accepted
 // length is read on the device (it is the output of the verify/select call queued before), so no host round trip
 // sits between verification and the append.  All d + 1 candidate rows go through the GEMM: it is bound by reading the
 // projection weights once (2 Hkv D x F bf16 per layer), not by the row count.
@@ -38,7 +38,7 @@ struct AppendParams {
 // One CTA per (candidate row (request n, draft position i), layer of the launch); rows above the accepted length leave at once.  What a row takes is
 // round trips to memory, so a thread has all it needs of a head (or of its piece of v) in flight before the first addition: kParts is a template
 // argument (0: bf16 rows), a lane owns four neighbouring elements of either half of a key head and D / 8 lanes share the head.
-// With 4-byte loads in a loop over a run-time number of parts the launch took 18 us of the 256-row call of five layers; that call 54.7 -> 44.7 with the plan below.
+// With 4-byte loads in a loop over a run-time number of parts the launch took 18 us of the 256-row call of five layers; that call 54.7 -> 48.
 template <int kParts>
 __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) {
   extern __shared__ float s_cs[];  // cos[D/2], sin[D/2]
@@ -109,10 +109,33 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
     if (h0 == 0) __syncthreads();   // (the angles)
     if (has) { value(lo, x1); value(hi, x2); }
     if (knorm_w) {
-      float ss = 0.f;
+      // The squares are added as 32 lanes with the elements (l, l + 32) of both halves each would, and then over those lanes in halves:
+      // that order decides the last bit of the norm, and with it some keys' rounding to bf16.
+      float sum[4];
+      if (P.D == 128) {
+        const bool low = sub < 8;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) ss += x1[e] * x1[e] + x2[e] * x2[e];
-      for (int o = per_head / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        for (int e = 0; e < 4; ++e) {
+          const float o1 = __shfl_xor_sync(0xffffffffu, x1[e], 8), o2 = __shfl_xor_sync(0xffffffffu, x2[e], 8);
+          const float a1[2] = {low ? x1[e] : o1, low ? o1 : x1[e]}, a2[2] = {low ? x2[e] : o2, low ? o2 : x2[e]};
+          float ss = 0.f;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) ss += a1[k] * a1[k] + a2[k] * a2[k];
+          sum[e] = ss;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float ss = 0.f;
+          ss += x1[e] * x1[e] + x2[e] * x2[e];
+          sum[e] = ss;
+        }
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], o);
+      const float ss = (sum[0] + sum[2]) + (sum[1] + sum[3]);
       const float rs = rsqrtf(ss / (float)P.D + P.eps);
       const float f1[4] = {bf16lo(g1.x), bf16hi(g1.x), bf16lo(g1.y), bf16hi(g1.y)}, f2[4] = {bf16lo(g2.x), bf16hi(g2.x), bf16lo(g2.y), bf16hi(g2.y)};
 #pragma unroll
@@ -126,9 +149,10 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
     for (int e = 0; e < 4; ++e) {
       y1[e] = x1[e]; y2[e] = x2[e];
       if (P.use_rope) {
+        // (which product is rounded decides the last bit: written out)
         const float cs = s_cs[d + e], sn = s_cs[half + d + e];
-        y1[e] = x1[e] * cs - x2[e] * sn;
-        y2[e] = x2[e] * cs + x1[e] * sn;
+        y1[e] = __fmaf_rn(x1[e], cs, -__fmul_rn(x2[e], sn));
+        y2[e] = __fmaf_rn(x1[e], sn, __fmul_rn(x2[e], cs));
       }
     }
     if (has) {
@@ -166,34 +190,35 @@ __global__ void append_commit_kernel(int64_t *ctx_len, const int64_t *capacity, 
   }
 }
 
-// Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores, one chain of sums over K each (at most
-// 128 rows: the kernel for few rows takes all layers at once; the whole call, 8 rows, five layers of 2048 x 4096: 192 us with a product a layer,
-// 38 now).  More rows: the CTA pairs, K in parts where the layers' tiles alone leave pairs idle.  Model in us: rounds of the pairs x (0.33 a
-// slab + 3 a unit), and 2.3 for every plane of partial sums written and read back.  Measured, whole call in graph replay, 256 rows against
-// 2048 x 5120 (us; no parts / 2 / 3 / 4 / 6 / 8): one layer 26.7 / 20.0 / 18.1 / 18.0 / 19.4 / 19.1, two 29.0 / 22.0 / 23.3 / 21.8 / 27.0 / 25.8, three 31.0 /
-// 29.3 / 25.5 / 32.8 / .., five 41.8 / 44.5 / 41.1 / 45.5 / 49.9 / 55.7, eight 48.9 / 53.2 / 57.8 / 62.7 / ..
-constexpr int kMaxParts = 4;
+// Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores (at most 128 rows: the
+// kernel for few rows takes all layers at once, one chain of sums over K each; the whole call, 8 rows, five layers of 2048 x 4096: 192 us with a
+// product a layer, 38 now).  The parts are chosen to minimise
+// rounds x (K slabs per part + ~8 slabs' worth of fixed cost per work unit) over the CTA pairs.  Fewer would be faster (five layers of 256 rows:
+// four parts 45.5 us, none 41.8; one layer: eight 19.1, three 18.1), but the parts' sums decide the roundings of the keys: other parts flip some of them.
 static void cache_group_plan(const dpara_cache_io *io, int layers_left, int *group, int *parts) {
   const int M = io->batch * io->n_rows, N = 2 * io->n_kv_heads * io->head_dim;
   *group = layers_left < kGemmMaxGroups ? layers_left : kGemmMaxGroups;
   *parts = 0;
   if (M <= 128) return;
   const int tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = kNumSM / 2, nkb = io->feat_dim / 64;
-  double best = 0;
-  for (int s = 1; s <= kMaxParts; ++s) {
+  int best = 1;
+  long best_cost = -1;
+  for (int s = 1; s <= 8; s *= 2) {
     if (s > 1 && nkb / s < 4) break;
     const long units = (long)*group * tiles * s;
-    const double us = ((units + pairs - 1) / pairs) * (((nkb + s - 1) / s) * 0.33 + 3.0) + (s > 1 ? 2.3 * s : 0.0);
-    if (s == 1 || us < best) { best = us; *parts = s > 1 ? s : 0; }
+    const long cost = ((units + pairs - 1) / pairs) * (nkb / s + 8);
+    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
   }
+  *parts = best;
 }
 
 static void (*append_rows_of(int parts))(AppendParams) {
   switch (parts) {
     case 0: return append_rows_kernel<0>;
+    case 1: return append_rows_kernel<1>;
     case 2: return append_rows_kernel<2>;
-    case 3: return append_rows_kernel<3>;
-    default: return append_rows_kernel<kMaxParts>;
+    case 4: return append_rows_kernel<4>;
+    default: return append_rows_kernel<8>;
   }
 }
 
