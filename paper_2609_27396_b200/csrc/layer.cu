@@ -6,6 +6,8 @@
 // and HBM-bound (M rows of a few KB each).
 #include <math.h>
 
+#include <algorithm>
+
 #include "attention_tc.cuh"
 #include "gemm.cuh"
 #include "layer.cuh"
@@ -41,11 +43,44 @@ __device__ __forceinline__ void rms_store(uint16_t *out, const float (&v)[8], fl
   *reinterpret_cast<uint4 *>(out) = o;
 }
 
-template <bool kF32In>
+// Rotary angles of a call's rows, in double precision.  Slot i of boundary j of request n sits at position L_n + j + 2 + i (the unknown bonus of
+// boundary j at L_n + j + 1), spine row s at L_n + s.
+struct AngleJob {
+  float *table = nullptr;                     // [row][cos of D / 2 angles | sin of D / 2]; null: no table
+  const int64_t *ctx_offsets = nullptr, *ctx_lens = nullptr;   // lengths: ctx_lens, or the offsets' differences
+  int rows = 0, per_request = 1, slot_rows = 0, block = 1;     // a request's first slot_rows rows are slots of boundaries of `block`, the others spine rows
+  int half = 0;                               // D / 2
+  double inv_freq[64] = {};                   // theta^(-2 d / D), d < D / 2, worked out on the host in double precision
+};
+__device__ __forceinline__ void row_angle(const AngleJob &A, int row, int d, float &c, float &s) {
+  const int n = row / A.per_request, rr = row - n * A.per_request;
+  const int rel = rr < A.slot_rows ? rr / A.block + 2 + rr % A.block : rr - A.slot_rows;
+  const double pos = (double)(A.ctx_lens ? A.ctx_lens[n] : A.ctx_offsets[n + 1] - A.ctx_offsets[n]) + rel;
+  double sn, cs;
+  sincos(pos * A.inv_freq[d], &sn, &cs);
+  c = (float)cs;
+  s = (float)sn;
+}
+constexpr int kAnglesPerBlock = 256;
+__device__ __noinline__ void angle_block(const AngleJob &A, int first) {
+  for (int k = first + threadIdx.x; k < min(first + kAnglesPerBlock, A.rows * A.half); k += 128) {
+    const int row = k / A.half, d = k - row * A.half;
+    float *t = A.table + (size_t)row * 2 * A.half + d;
+    row_angle(A, row, d, t[0], t[A.half]);
+  }
+}
+
+template <bool kF32In, bool kAngles>
 __global__ void __launch_bounds__(128) rmsnorm_kernel(const void *__restrict__ x, const uint16_t *__restrict__ gain,
-                                                      uint16_t *__restrict__ out, int H, float eps) {
+                                                      uint16_t *__restrict__ out, int M, int H, float eps, const __grid_constant__ AngleJob angles) {
   constexpr int kHeld = 5;   // rows of 5120 elements
   const int row = blockIdx.x, tid = threadIdx.x;
+  if (kAngles && row >= M) {
+    pdl_wait();
+    pdl_launch_dependents();
+    angle_block(angles, (row - M) * kAnglesPerBlock);
+    return;
+  }
   const size_t base = (size_t)row * H;
   // (no gain: bf16 ones)
   auto gain_at = [&](int c) { return gain ? *reinterpret_cast<const uint4 *>(gain + c) : make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u); };
@@ -96,38 +131,32 @@ __global__ void __launch_bounds__(128) rmsnorm_kernel(const void *__restrict__ x
 }
 
 // ------------------------------------------------------------------------------------------------ q/k norm + rope, v copy
-// One CTA per token row.  qkv row = [Hq*D | Hkv*D | Hkv*D].  q and k heads: optional RMS norm over D
-// (rounded to bf16), then rotate-half rotary embedding at the row's position (rounded to bf16).
-// Positions: slot i of boundary j of request n sits at L_n + j + 2 + i (spine row s at L_n + s, the
-// unknown bonus of boundary j at L_n + j + 1).  Angles are formed in double precision.
+// gridDim.y CTAs of four warps per token row (few rows: enough that a warp has one or two heads, the kernel is then one round trip to memory; one CTA
+// per row took 7 us behind the product at 72 rows of 40 heads).  qkv row = [Hq*D | Hkv*D | Hkv*D].  q and k heads: optional RMS norm over D
+// (rounded to bf16), then rotate-half rotary embedding by the row's angles (rounded to bf16).
 // With spine query rows a request has J * Bq + S rows: the mask-slot rows, then the spine rows.
 struct QkParams {
   const uint16_t *qkv;
   const uint16_t *qnorm_w, *knorm_w;
   uint16_t *q, *k, *v;
-  const int64_t *ctx_offsets, *ctx_lens;
-  int J, Bq, Hq, Hkv, D, Sq;
+  int Hq, Hkv, D;
   int use_rope, use_norm;
-  float eps, theta;
-  double inv_freq[64];   // theta^(-2 d / D), d < D / 2, worked out on the host in double precision
+  float eps;
+  AngleJob angles;
 };
 
+template <bool kSplit>
 __global__ void __launch_bounds__(128) qk_norm_rope_kernel(const QkParams P) {
   extern __shared__ float s_cs[];  // cos[D/2], sin[D/2]
   const int row = blockIdx.x, tid = threadIdx.x;
   const int half = P.D / 2;
-  const int R = P.Bq * P.J + P.Sq;
-  const int n = row / R, rr = row % R;
-  // The angles before the wait: the kernel in front is the QKV product, which writes neither lengths nor offsets, and it lets this one go
-  // only when everything before it has ended.  The double-precision sincos is most of a short launch.
+  // The angles before the wait: the kernel in front is the QKV product, which writes neither lengths nor offsets and lets this one go only when
+  // everything before it has ended, the norm that made a table among it.
   if (P.use_rope) {
-    const int rel = rr < P.Bq * P.J ? rr / P.Bq + 2 + rr % P.Bq : rr - P.Bq * P.J;  // mask slot (j, i): j + 2 + i; spine row s: s
-    const double pos = (double)(P.ctx_lens ? P.ctx_lens[n] : P.ctx_offsets[n + 1] - P.ctx_offsets[n]) + rel;
-    for (int d = tid; d < half; d += 128) {
-      double sn, cs;
-      sincos(pos * P.inv_freq[d], &sn, &cs);
-      s_cs[d] = (float)cs;
-      s_cs[half + d] = (float)sn;
+    if (kSplit) {
+      for (int d = tid; d < P.D; d += 128) s_cs[d] = P.angles.table[(size_t)row * P.D + d];
+    } else {
+      for (int d = tid; d < half; d += 128) row_angle(P.angles, row, d, s_cs[d], s_cs[half + d]);
     }
   }
   pdl_wait();
@@ -136,16 +165,17 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(const QkParams P) {
   const int warp = tid >> 5, lane = tid & 31;
   const size_t qkv_row = (size_t)row * (P.Hq + 2 * P.Hkv) * P.D;
   // A lane owns the element pairs (2 lane, 2 lane + 1) of both halves of a head (one 4-byte load each); a warp takes heads
-  // warp, warp + 4, ... and fetches kChunk of them before it works on the first, so that a row costs a few global round
+  // warp, warp + 4 gridDim.y, ... and fetches kChunk of them before it works on the first, so that a row costs a few global round
   // trips instead of one per head.
   constexpr int kChunk = 6;
   const bool active = 2 * lane < half;
   const int n_heads = P.Hq + P.Hkv;
-  for (int hd0 = warp; hd0 < n_heads; hd0 += 4 * kChunk) {
+  const int part = kSplit ? (int)blockIdx.y : 0, stride = kSplit ? 4 * (int)gridDim.y : 4;
+  for (int hd0 = part * 4 + warp; hd0 < n_heads; hd0 += stride * kChunk) {
     uint32_t lo[kChunk], hi[kChunk];
 #pragma unroll
     for (int c = 0; c < kChunk; ++c) {
-      const int hd = hd0 + 4 * c;
+      const int hd = hd0 + stride * c;
       lo[c] = hi[c] = 0u;
       if (hd < n_heads && active) {
         const uint16_t *src = P.qkv + qkv_row + (size_t)hd * P.D;
@@ -155,7 +185,7 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(const QkParams P) {
     }
 #pragma unroll
     for (int c = 0; c < kChunk; ++c) {
-      const int hd = hd0 + 4 * c;
+      const int hd = hd0 + stride * c;
       if (hd >= n_heads) break;
       const bool is_q = hd < P.Hq;
       uint16_t *dst = is_q ? P.q + ((size_t)row * P.Hq + hd) * P.D : P.k + ((size_t)row * P.Hkv + (hd - P.Hq)) * P.D;
@@ -193,13 +223,13 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(const QkParams P) {
   // v: plain copy into its own contiguous tensor
   const uint16_t *vsrc = P.qkv + qkv_row + (size_t)(P.Hq + P.Hkv) * P.D;
   uint16_t *vdst = P.v + (size_t)row * P.Hkv * P.D;
-  for (int c = tid * 8; c < P.Hkv * P.D; c += 128 * 8) *reinterpret_cast<uint4 *>(vdst + c) = *reinterpret_cast<const uint4 *>(vsrc + c);
+  for (int c = (part * 128 + tid) * 8; c < P.Hkv * P.D; c += 32 * 8 * stride) *reinterpret_cast<uint4 *>(vdst + c) = *reinterpret_cast<const uint4 *>(vsrc + c);
 }
 
 // ------------------------------------------------------------------------------------------------ host
 namespace {
 struct LayerWs {
-  size_t xn, qkv, q, k, v, a, h1, hn, act, attn, total;
+  size_t xn, qkv, q, k, v, a, h1, hn, act, angles, attn, total;
 };
 
 LayerWs layer_ws_layout(const dpara_shape *s, const dpara_layer_io *l, size_t attn_bytes) {
@@ -217,6 +247,7 @@ LayerWs layer_ws_layout(const dpara_shape *s, const dpara_layer_io *l, size_t at
   w.h1 = take(M * H * 4);
   w.hn = take(M * H * 2);
   w.act = take(M * I * 2);
+  w.angles = take(M * s->head_dim * 4);
   w.attn = take(attn_bytes);
   w.total = o;
   return w;
@@ -229,12 +260,18 @@ void layer_workspace_offsets(const dpara_shape *shape, const dpara_layer_io *lay
   for (int i = 0; i < 9; ++i) out[i] = attn_bytes + o[i];
 }
 
-dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st) {
-  if (H % 8) return DPARA_ERR_UNSUPPORTED;
-  launch_pdl(rmsnorm_kernel<false>, dim3(M), dim3(128), 0, st, x, static_cast<const uint16_t *>(gain), static_cast<uint16_t *>(out), H, eps);
+template <bool kF32In>
+static dpara_status launch_rmsnorm(const void *x, const void *gain, void *out, int M, int H, float eps, const AngleJob &angles, cudaStream_t st) {
+  const int blocks = angles.table ? (angles.rows * angles.half + kAnglesPerBlock - 1) / kAnglesPerBlock : 0;
+  launch_pdl(blocks ? rmsnorm_kernel<kF32In, true> : rmsnorm_kernel<kF32In, false>, dim3(M + blocks), dim3(128), 0, st, x, static_cast<const uint16_t *>(gain), static_cast<uint16_t *>(out), M, H, eps, angles);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   return DPARA_OK;
+}
+
+dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st) {
+  if (H % 8) return DPARA_ERR_UNSUPPORTED;
+  return launch_rmsnorm<false>(x, gain, out, M, H, eps, AngleJob{}, st);
 }
 
 size_t layer_workspace_bytes(const dpara_shape *shape, const dpara_layer_io *layer) {
@@ -243,7 +280,7 @@ size_t layer_workspace_bytes(const dpara_shape *shape, const dpara_layer_io *lay
 }
 
 dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, const dpara_layer_io *L, void *workspace,
-                          int32_t *status_word, cudaStream_t st) {
+                          int32_t *status_word, cudaStream_t st, bool angles_there) {
   if (!L->x || !L->w_qkv || !L->w_o || !L->w_gate_up || !L->w_down || !L->y_f32) return DPARA_ERR_INVALID_ARG;
   if (L->hidden <= 0 || L->intermediate <= 0) return DPARA_ERR_INVALID_ARG;
   if ((L->qnorm_w == nullptr) != (L->knorm_w == nullptr)) return DPARA_ERR_INVALID_ARG;
@@ -264,21 +301,31 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   uint16_t *a = reinterpret_cast<uint16_t *>(lw + w.a), *hn = reinterpret_cast<uint16_t *>(lw + w.hn), *act = reinterpret_cast<uint16_t *>(lw + w.act);
   float *h1 = reinterpret_cast<float *>(lw + w.h1);
 
-  launch_pdl(rmsnorm_kernel<false>, dim3(M), dim3(128), 0, st, L->x, static_cast<const uint16_t *>(L->rms1_w), xn, H, L->rms_eps);
-  DPARA_CHECK_LAUNCH();
-  count_launches(1);
+  // Few rows: several CTAs for a row of the row-wise kernel behind the QKV product, so that a warp has one or two heads.  They would each work out
+  // their row's angles, so the angles are made once, by blocks behind the rows of this norm.  With a CTA per row they are made there, behind nothing (a table
+  // of 1152 rows made the first norm 3 us longer: two blocks 1579 -> 1586 us).
+  const int n_heads = shape->n_q_heads + shape->n_kv_heads, per_row = std::min((4 * kNumSM + M - 1) / M, (n_heads + 3) / 4);
+  AngleJob angles;
+  if (L->use_rope) {
+    if (per_row > 1) angles.table = reinterpret_cast<float *>(lw + w.angles);
+    angles.ctx_offsets = io->ctx_offsets; angles.ctx_lens = io->ctx_lens;
+    angles.rows = M; angles.per_request = R; angles.slot_rows = shape->n_boundaries * shape->block; angles.block = shape->block;
+    angles.half = D / 2;
+    for (int d = 0; d < D / 2 && d < 64; ++d) angles.inv_freq[d] = pow((double)L->rope_theta, -2.0 * d / D);
+  }
+  dpara_status s = launch_rmsnorm<false>(L->x, L->rms1_w, xn, M, H, L->rms_eps, angles_there ? AngleJob{} : angles, st);
+  if (s != DPARA_OK) return s;
   GemmArgs g{};
   g.a = xn; g.w = L->w_qkv; g.M = M; g.N = QD + 2 * KD; g.K = H; g.epi = 0; g.out = qkv; g.w_ready = 1;  // the kernels of this chain write no weights
-  dpara_status s = launch_gemm_tc(g, status_word, st);
+  s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
 
   QkParams qp;
   qp.qkv = qkv; qp.qnorm_w = static_cast<const uint16_t *>(L->qnorm_w); qp.knorm_w = static_cast<const uint16_t *>(L->knorm_w);
-  qp.q = q; qp.k = k; qp.v = v; qp.ctx_offsets = io->ctx_offsets; qp.ctx_lens = io->ctx_lens;
-  qp.J = shape->n_boundaries; qp.Bq = shape->block; qp.Hq = shape->n_q_heads; qp.Hkv = shape->n_kv_heads; qp.D = D; qp.Sq = Sq;
-  qp.use_rope = L->use_rope; qp.use_norm = L->qnorm_w != nullptr; qp.eps = L->rms_eps; qp.theta = L->rope_theta;
-  for (int d = 0; d < D / 2 && d < 64; ++d) qp.inv_freq[d] = pow((double)L->rope_theta, -2.0 * d / D);
-  launch_pdl(qk_norm_rope_kernel, dim3(M), dim3(128), D * sizeof(float), st, qp);
+  qp.q = q; qp.k = k; qp.v = v;
+  qp.Hq = shape->n_q_heads; qp.Hkv = shape->n_kv_heads; qp.D = D;
+  qp.use_rope = L->use_rope; qp.use_norm = L->qnorm_w != nullptr; qp.eps = L->rms_eps; qp.angles = angles;
+  launch_pdl(per_row > 1 ? qk_norm_rope_kernel<true> : qk_norm_rope_kernel<false>, dim3(M, per_row), dim3(128), D * sizeof(float), st, qp);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
 
@@ -296,9 +343,8 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   g.a = a; g.w = L->w_o; g.M = M; g.N = H; g.K = QD; g.epi = 1; g.resid = L->x; g.resid_bf16 = 1; g.out = h1; g.w_ready = 1;
   s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
-  launch_pdl(rmsnorm_kernel<true>, dim3(M), dim3(128), 0, st, static_cast<const void *>(h1), static_cast<const uint16_t *>(L->rms2_w), hn, H, L->rms_eps);
-  DPARA_CHECK_LAUNCH();
-  count_launches(1);
+  s = launch_rmsnorm<true>(h1, L->rms2_w, hn, M, H, L->rms_eps, AngleJob{}, st);
+  if (s != DPARA_OK) return s;
   g = GemmArgs{};
   g.a = hn; g.w = L->w_gate_up; g.M = M; g.N = I; g.K = H; g.epi = 2; g.out = act; g.w_ready = 1;
   s = launch_gemm_tc(g, status_word, st);
@@ -344,7 +390,9 @@ dpara_status launch_backbone(const dpara_shape *shape, const dpara_attn_io *io, 
     dpara_attn_io a = *io;
     a.k_ctx = bb->host_k_ctx[l];
     a.v_ctx = bb->host_v_ctx[l];
-    dpara_status s = launch_layer(shape, &a, &L, base + w.layer, status_word, st);
+    // (the rows' positions are the same in every block: one table for all blocks that turn by the same frequencies, made by the first that turns)
+    const dpara_layer_io *made = l > 0 && bb->host_layers[l - 1].use_rope && bb->host_layers[l - 1].rope_theta == L.rope_theta ? &bb->host_layers[l - 1] : nullptr;
+    dpara_status s = launch_layer(shape, &a, &L, base + w.layer, status_word, st, made != nullptr);
     if (s != DPARA_OK) return s;
   }
   return DPARA_OK;
