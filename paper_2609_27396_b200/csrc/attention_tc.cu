@@ -339,10 +339,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   const int q_begin = P.use_seg ? (team < P.seg_teams ? (int)P.team_first[team] : 0) : (P.use_sched ? (int)P.cta_first[blockIdx.x] : (int)blockIdx.x);
   const int q_end = P.use_seg ? (team < P.seg_teams ? (int)P.team_first[team + 1] : 0) : (P.use_sched ? (int)P.cta_first[blockIdx.x + 1] : P.n_items);
   const int q_step = (P.use_seg || P.use_sched) ? 1 : (int)gridDim.x;
-  pdl_wait();  // nothing above touches global memory
-  pdl_launch_dependents();
-  // (a CTA of a cluster must not leave early: its peers meet it at the cluster barriers below)
-  if (P.nsplit == 1 && A.status_word && (*reinterpret_cast<volatile int32_t *>(A.status_word) & (int32_t)DPARA_STATUS_TIMEOUT)) return;
+  // A split launch of a small batch is a chain of latencies: its barriers, TMEM and the producer's first item (whose decode reads cold parameters) come
+  // ahead of the wait for the kernel in front.  Only the producer reads what that kernel may have written; the softmax warps
+  // wait before they write.  (A CTA of a cluster does not look at the status: it must not leave early, its peers meet it at the cluster barriers below.)
+  const bool wait_late = P.nsplit > 1 && P.use_ctx_p;
+  if (!wait_late) {
+    pdl_wait();  // nothing above touches global memory
+    pdl_launch_dependents();
+    if (P.nsplit == 1 && A.status_word && (*reinterpret_cast<volatile int32_t *>(A.status_word) & (int32_t)DPARA_STATUS_TIMEOUT)) return;
+  }
 
   if (threadIdx.x == 0) {
     // K/V slots and the Q buffer are released by BOTH MMA issuers
@@ -376,6 +381,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     bool ok = true;
     for (int qi = q_begin; qi < q_end && ok; qi += q_step) {
       const Item I = fetch_item(P, qi);
+      if (wait_late) {   // (one item per CTA)
+        pdl_wait();
+        pdl_launch_dependents();
+      }
       if (I.n_iter == 0) continue;
       // the Q buffer is free once the previous item's last QK has completed
       ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (k & 1) ^ 1u, abort_flag));
@@ -678,6 +687,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
 
       // ---- output of this item (the MMA issuer cannot touch O_t again before this tile's next p_full arrive)
       if (!ok) break;
+      if (wait_late) pdl_wait();
       const Item I = fetch_item(P, qi);
       const uint32_t geo = tile_geo(I, t);
       const int ji = geo_ji0(geo) + (r >> geo_hs(geo));
@@ -762,11 +772,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   // its unnormalised rows and (max, sum) to its scratch slot (which stays in L2); after a cluster barrier CTA
   // `rank` merges 256 / nsplit of the rows from all peers' slots and writes the final output.  No second launch.
   if (P.nsplit > 1) {
+    const Item I = decode_item(P, blockIdx.x);
     __threadfence();
     __syncwarp();
     cluster_sync_all();
     if (warp < 8 && !*abort_flag) {
-      const Item I = decode_item(P, blockIdx.x);
       const uint32_t rank = cluster_ctarank();
       const int rows_per = I.ntq * 128 / P.nsplit;  // the item's rows (one tile or two), shared out over the cluster
       merge_pieces<D>(P, I, P.nsplit, (int)rank * rows_per, rows_per, threadIdx.x);
