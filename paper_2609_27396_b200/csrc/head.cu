@@ -53,8 +53,10 @@ constexpr int kResidentCol = 128;                  // accumulators in TMEM colum
 constexpr int kMaxAccBufs = kResidentCol / 16;
 constexpr int kMaxStages = 4, kMaxLogitSlots = 16;
 constexpr int kCtasPerLane = (kNumSM + 31) / 32;
+constexpr int kCopies = 8;                         // of every word of the greedy loop
 constexpr int kCtaStride = 32 * kCtasPerLane;      // words of one request: a slot per CTA, whole 128-byte lines
-constexpr int kReplicas = 8;
+// Sampling: lane l looks after CTAs 5 l .. 5 l + 4 (the scan goes through them in the vocabulary's order) and reads slots l, 32 + l, ...
+__device__ __forceinline__ int slot_of(int cta) { return cta % kCtasPerLane * 32 + cta / kCtasPerLane; }
 constexpr unsigned long long kTagMask = 63;
 constexpr int kTagBits = 6;                        // step / 2 + 1 (two buffers in turn, at most 64 steps)
 constexpr int kBarBytes = 3072;                    // barriers and the reduction scratch
@@ -181,7 +183,7 @@ struct ArParams {
   const int32_t *bonus;           // [b]
   const float *uniforms;          // [b][block]
   int32_t *next_tokens;           // [b][block]
-  // What the CTAs exchange, zero before the launch: words [2 (step parity)][replica][b][1, sampling: 2][CTA], drawn [2][replica][kMaxBatch]
+  // What the CTAs exchange, zero before the launch: words [2 (step parity)], greedy [kCopies][b][CTA], sampling [b][2][slot of a CTA]; drawn [2][kMaxBatch]
   unsigned long long *words, *drawn;
   float *z;                       // sampling where z does not fit in shared memory: [b][vocab]
   int32_t *status;
@@ -461,12 +463,13 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         if (!kSample) top[q] |= __reduce_max_sync(0xffffffffu, (uint32_t)(x >> 32) == hi32 ? (uint32_t)x : 0u);
       }
       // this step's words: the two buffers in turn (a CTA writes a step's words when it has seen all of the step before, so those two steps
-      // older have been read), every word in kReplicas copies, of which a CTA polls one
+      // older have been read), in kCopies copies of which a CTA polls one.  (Sampling: one copy, read in whole lines; eight, read with a stride of
+      // five words, took 16 us more over 16 steps of 8 requests.)
       const uint32_t tag = (uint32_t)(step >> 1) + 1u;
-      constexpr int kWords = kSample ? 2 : 1;
+      constexpr int kWords = kSample ? 2 : 1, copies = kSample ? 1 : kCopies;
       const size_t copy_words = (size_t)P.b * kWords * kCtaStride;
-      unsigned long long *const words = P.words + (size_t)(step & 1) * kReplicas * copy_words;
-      const unsigned long long *const my_words = words + (blockIdx.x % kReplicas) * copy_words;
+      unsigned long long *const words = P.words + (size_t)(step & 1) * copies * copy_words;
+      const unsigned long long *const my_words = words + blockIdx.x % copies * copy_words;
       int tok[kPer];
 #pragma unroll
       for (int q = 0; q < kPer; ++q) tok[q] = 0;
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
           const int n = warp + kEpiWarps * q;
           // key << 32 | ~(entry of the CTA's range) << 6 | tag
           const uint32_t entry = 0xffffffffu - (uint32_t)top[q] - (uint32_t)v0;
-          if (n < P.b && lane < kReplicas)
+          if (n < P.b && lane < copies)
             publish(words + lane * copy_words + (size_t)n * kCtaStride + blockIdx.x, (top[q] >> 32 << 32) | (uint32_t)(~entry << kTagBits) | tag);
         }
         if (last && blockIdx.x != 0) break;     // (CTA 0 writes the last winners)
@@ -542,8 +545,8 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
             unsigned long long s = mine[q];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane < kReplicas) {
-              unsigned long long *const to = words + lane * copy_words + (size_t)(2 * n) * kCtaStride + blockIdx.x;
+            if (lane < copies) {
+              unsigned long long *const to = words + lane * copy_words + (size_t)(2 * n) * kCtaStride + slot_of(blockIdx.x);
               // (the sum's lowest bits travel with the exponent)
               publish(to, (s & ~kTagMask) | tag);
               publish(to + kCtaStride, (unsigned long long)ref[q].exponent << 2 * kTagBits | (s & kTagMask) << kTagBits | tag);
@@ -552,7 +555,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         }
         ok = poll_words([&](int i) -> const unsigned long long * {
           const int q2 = i / kCtasPerLane, n = warp + kEpiWarps * (q2 / 2), c = lane * kCtasPerLane + i % kCtasPerLane;
-          return n < P.b && c < n_ctas ? my_words + (size_t)(2 * n + (q2 & 1)) * kCtaStride + c : nullptr;
+          return n < P.b && c < n_ctas ? my_words + (size_t)(2 * n + (q2 & 1)) * kCtaStride + i % kCtasPerLane * 32 + lane : nullptr;
         }, tag, got, abort_flag);
         if (ok) {
 #pragma unroll
@@ -622,10 +625,9 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
               }
             }
             if (owner == (int)blockIdx.x && lane == 0) {
+              publish(P.drawn + (step & 1) * kMaxBatch + n, (unsigned long long)pick << kTagBits | tag);
               P.next_tokens[(size_t)n * P.block + step] = pick;
             }
-            if (owner == (int)blockIdx.x && lane < kReplicas)
-              publish(P.drawn + ((step & 1) * kReplicas + lane) * kMaxBatch + n, (unsigned long long)pick << kTagBits | tag);
           }
         }
         if (P.z_in_place) {
@@ -637,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         if (last) break;
         unsigned long long token[1] = {0ull};
         const unsigned long long *const mine_drawn =
-            lane < kPer && warp + kEpiWarps * lane < P.b ? P.drawn + ((step & 1) * kReplicas + blockIdx.x % kReplicas) * kMaxBatch + warp + kEpiWarps * lane : nullptr;
+            lane < kPer && warp + kEpiWarps * lane < P.b ? P.drawn + (step & 1) * kMaxBatch + warp + kEpiWarps * lane : nullptr;
         ok = ok && poll_words([&](int) { return mine_drawn; }, tag, token, abort_flag);
 #pragma unroll
         for (int q = 0; q < kPer; ++q) tok[q] = __shfl_sync(0xffffffffu, (int)(token[0] >> kTagBits), q);
@@ -682,8 +684,8 @@ __global__ void __launch_bounds__(256) head_clear_kernel(uint4 *words, size_t n)
 }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
-constexpr size_t kDrawnWords = 2 * kReplicas * kMaxBatch;
-size_t words_bytes(int b) { return ((size_t)2 * kReplicas * b * 2 * kCtaStride + kDrawnWords) * sizeof(unsigned long long); }
+constexpr size_t kDrawnWords = 2 * kMaxBatch;
+size_t words_bytes(int b) { return ((size_t)2 * kCopies * b * kCtaStride + kDrawnWords) * sizeof(unsigned long long); }
 }  // namespace
 
 size_t head_workspace_bytes(int b, int block, int vocab) {
@@ -721,7 +723,7 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   const int slabs = h.rank / 64, nb = h.b <= 16 ? 16 : 32;
   const bool sample = h.uniforms != nullptr;
 
-  const size_t vecs = (kDrawnWords + (size_t)2 * kReplicas * h.b * (sample ? 2 : 1) * kCtaStride) / 2;   // 16 bytes each
+  const size_t vecs = (kDrawnWords + (size_t)2 * h.b * (sample ? 2 : kCopies) * kCtaStride) / 2;   // 16 bytes each
   launch_pdl(head_clear_kernel, dim3((unsigned)(vecs < 148 * 256 ? (vecs + 255) / 256 : 148)), dim3(256), 0, st, reinterpret_cast<uint4 *>(words), vecs);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
