@@ -40,12 +40,14 @@ constexpr int kEpiBytes = kEpiWarps * 16 * 32 * 4;   // 16 activation rows of 32
 struct GemmKernelParams {
   CUtensorMap map_w[kGemmMaxGroups];   // one entry per product of a grouped launch (a plain launch uses entry 0)
   CUtensorMap map_a[kGemmMaxGroups];
+  CUtensorMap map_tail;                // activations in boxes of a tail unit's rows (one product)
   void *out_g[kGemmMaxGroups];
   int n_groups;
   int M, N, K;
   int epi;
   int up_row_offset;
   int nt, t_tiles, n_tiles;            // activation rows per tile; tiles of one product
+  int main_units, tail_split, nt_tail; // kTail: tiles from main_units on are cut into tail_split units of nt_tail activation rows
   int stages;
   int split_k;                         // > 1 (fp32 store only): the K range in split_k parts, part s writes plane s of [split_k][M][N] partial sums
   const void *resid;
@@ -57,17 +59,38 @@ struct GemmKernelParams {
 
 
 
-// A unit of work: a tile of one of the products, or one part of its K range (the parts of a tile are neighbours).
+// A unit of work: a tile of one of the products, one part of its K range (the parts of a tile are neighbours), or (kTail, one product) some of its
+// activation rows.
+template <bool kTail>
 struct Unit {
-  int grp, tile, ks, kb0, kb1;
+  int grp, tile, ks, kb0, kb1, row0, nt, rows;
+  bool tail;
   __device__ __forceinline__ Unit(const GemmKernelParams &P, int unit, int nkb) {
-    const int per_group = P.t_tiles * P.n_tiles * P.split_k;
-    grp = unit / per_group;
-    unit -= grp * per_group;
-    tile = unit / P.split_k;
-    ks = unit - tile * P.split_k;
-    kb0 = ks * nkb / P.split_k;
-    kb1 = (ks + 1) * nkb / P.split_k;
+    int sub = 0;
+    tail = kTail && unit >= P.main_units;
+    if (tail) {
+      const int k = (unit - P.main_units) / P.tail_split;
+      sub = unit - P.main_units - k * P.tail_split;
+      unit = P.main_units + k;
+    }
+    if (kTail) {
+      grp = ks = kb0 = 0;
+      kb1 = nkb;
+      tile = unit;
+    } else {
+      const int per_group = P.t_tiles * P.n_tiles * P.split_k;
+      grp = unit / per_group;
+      unit -= grp * per_group;
+      tile = unit / P.split_k;
+      ks = unit - tile * P.split_k;
+      kb0 = ks * nkb / P.split_k;
+      kb1 = (ks + 1) * nkb / P.split_k;
+    }
+    const int first = tile % P.t_tiles * P.nt;
+    nt = tail ? P.nt_tail : P.nt;
+    row0 = tail ? first + sub * P.nt_tail : first;
+    // (a tile's last tail unit may reach behind the tile, the last tile behind the last row; nothing left: no rows)
+    rows = min(min(P.M, first + P.nt) - row0, nt);
   }
 };
 
@@ -76,10 +99,10 @@ struct Unit {
 // what these products are short of (per slab the products read 64 bytes and the copies write 64 bytes per clock of the 128 an SM
 // has): a transposing buffer here cost 4 % of the whole product.  The two warps of a TMEM quarter take the blocks in turn, and the
 // residual rows of a block are on their way while the one before is worked on.
-__device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_t taddr, const Unit &w, int rank, float *exchange, int quarter, int turn, int lane) {
+template <bool kTail>
+__device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_t taddr, const Unit<kTail> &w, int rank, float *exchange, int quarter, int turn, int lane) {
   const int grp = w.grp, tile = w.tile;
-  const int t_tile = tile % P.t_tiles, n_tile = tile / P.t_tiles;
-  const int row0 = t_tile * P.nt, rows_all = min(P.M - row0, P.nt);
+  const int n_tile = tile / P.t_tiles, row0 = w.row0, rows_all = w.rows;
   if (P.epi == 2) {
     // quarters 0 and 1 have gate columns, 2 and 3 the matching up columns: each warp of such a pair hands 16 of the 32 activation rows to the
     // other and finishes the other 16
@@ -186,6 +209,7 @@ __device__ __forceinline__ void gemm_epilogue(const GemmKernelParams &P, uint32_
   }
 }
 
+template <bool kTail>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pair_kernel(const __grid_constant__ GemmKernelParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -203,7 +227,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
   const int rank = __shfl_sync(0xffffffffu, (int)cluster_ctarank(), 0);
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   const int nkb = P.K / kBK;
-  const int units = P.t_tiles * P.n_tiles * P.split_k * P.n_groups;
+  const int tiles = P.t_tiles * P.n_tiles * P.split_k * P.n_groups, units = kTail ? P.main_units + (tiles - P.main_units) * P.tail_split : tiles;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < P.stages; ++s) {
@@ -240,15 +264,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true, there = false;
-    const uint32_t tx = 2u * (uint32_t)stage_bytes;
-    const int half_t = P.nt / 2;
     // (tile id = weight tile * t_tiles + activation tile: the pairs running together cover all activation rows of a few weight tiles)
     for (int unit = pair; unit < units && ok; unit += pairs) {
-      const Unit w(P, unit, nkb);
-      const int grp = w.grp, t_tile = w.tile % P.t_tiles, n_tile = w.tile / P.t_tiles;
+      const Unit<kTail> w(P, unit, nkb);
+      const uint32_t tx = 2u * (uint32_t)(kWBytes + w.nt * 64);
+      const int grp = w.grp, n_tile = w.tile / P.t_tiles;
       const int wrow = P.epi == 2 ? n_tile * 128 + rank * 64 : n_tile * 256 + rank * 128;
-      const int arow = t_tile * P.nt + rank * half_t;
-      const CUtensorMap *map_w = &P.map_w[grp], *map_a = &P.map_a[grp];
+      const int arow = w.row0 + rank * (w.nt / 2);
+      const CUtensorMap *map_w = &P.map_w[grp], *map_a = w.tail ? &P.map_tail : &P.map_a[grp];
       const bool swiglu = P.epi == 2;
 #pragma unroll 1
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
@@ -269,14 +292,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
     }
   } else if (warp == 5) {
     if (rank == 0) {
-      const uint32_t idesc = idesc_bf16_f32(2 * kRows, P.nt, false, false);
       const uint64_t desc = smem_desc_sw128(smem_u32(smem), 16, 1024);
       const uint32_t w_lo = (uint32_t)desc, a_lo = w_lo + (kWBytes >> 4), hi = (uint32_t)(desc >> 32), stage_units = (uint32_t)stage_bytes >> 4;
       int stage = 0, k = 0;
       uint32_t ph = 0;
       bool ok = true, there = false;
       for (int unit = pair; unit < units && ok; unit += pairs, ++k) {
-        const Unit w(P, unit, nkb);
+        const Unit<kTail> w(P, unit, nkb);
+        const uint32_t idesc = idesc_bf16_f32(2 * kRows, w.nt, false, false);
         const int buf = k & 1;
         ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + buf, ((k >> 1) & 1) ^ 1u, abort_flag, 3));  // both CTAs' epilogues of tile k - 2 are done
         if (!ok) break;
@@ -311,7 +334,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
       live = named_bar_all_256(warp != 0 || __all_sync(0xffffffffu, mbar_wait(acc_full + buf, (k >> 1) & 1, abort_flag, 5)));
       tc_fence_after();
       const uint32_t taddr = tmem + buf * 256 + ((uint32_t)(quarter * 32) << 16);
-      if (live) gemm_epilogue(P, taddr, Unit(P, unit, nkb), rank, exchange, quarter, turn, lane);
+      if (live) gemm_epilogue<kTail>(P, taddr, Unit<kTail>(P, unit, nkb), rank, exchange, quarter, turn, lane);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(acc_empty + buf);
@@ -388,6 +411,22 @@ dpara_status gemm_route(const GemmArgs &g, GemmRoute &r) {
   return DPARA_OK;
 }
 
+// The tiles of a last round that has few of them (at most a third of the pairs): each in `split` parts of its activation rows, on pairs that would have
+// nothing to do.  Every part reads the tile's weights again (from L2), so only as many as L2 serves beside.  256 x 151936 x 5120: 594 tiles are eight
+// rounds of 74 pairs and two tiles; with the head loop behind it 559.8 -> 552.3 us (about a quarter of what the round took: the pairs drift apart over
+// eight rounds).  1024 x 12288 x 4096 SwiGLU, five rounds and 14 tiles: the block around it 873.6 -> 864.9.
+static bool tail_plan(const GemmArgs &g, const GemmRoute &r, GemmKernelParams &P) {
+  const long units = (long)r.pair.t_tiles * r.n_all;
+  const int left = (int)(units % r.most), at_once = 48;
+  if (g.n_groups > 1 || g.split_k > 1 || units < r.most || left == 0 || 2 * left > at_once) return false;
+  P.nt_tail = (r.pair.nt / (at_once / left) + 15) / 16 * 16;
+  if (P.nt_tail < 32) P.nt_tail = 32;
+  if (P.nt_tail >= r.pair.nt) return false;
+  P.tail_split = (r.pair.nt + P.nt_tail - 1) / P.nt_tail;
+  P.main_units = (int)(units - left);
+  return true;
+}
+
 dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st) {
   GemmRoute route;
   const dpara_status checked = gemm_route(g, route);
@@ -401,6 +440,8 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
   P.split_k = g.split_k > 1 ? g.split_k : 1;
   P.n_tiles = route.n_tiles;
   P.t_tiles = route.pair.t_tiles; P.nt = route.pair.nt;
+  const bool tail = tail_plan(g, route, P);
+  if (tail && !make_tmap_bf16_2d(&P.map_tail, g.a, g.K, g.M, (uint64_t)g.K * 2, kBK, P.nt_tail / 2)) return DPARA_ERR_CUDA;
   for (int gi = 0; gi < P.n_groups; ++gi) {
     const void *a = gi ? g.a_g[gi] : g.a, *w = gi ? g.w_g[gi] : g.w;
     void *o = gi ? g.out_g[gi] : g.out;
@@ -418,8 +459,9 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
 
   const long units = (long)P.t_tiles * route.n_all;
   const int smem = P.stages * stage_bytes + 1024 + kBarBytes + kEpiBytes;
-  if (cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return DPARA_ERR_CUDA;
-  launch_pdl(gemm_pair_kernel, dim3(2 * (unsigned)(units < route.most ? units : route.most)), dim3(kThreads), smem, st, P);
+  void (*const kernel)(GemmKernelParams) = tail ? gemm_pair_kernel<true> : gemm_pair_kernel<false>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return DPARA_ERR_CUDA;
+  launch_pdl(kernel, dim3(2 * (unsigned)(units < route.most ? units : route.most)), dim3(kThreads), smem, st, P);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   return DPARA_OK;

@@ -51,3 +51,29 @@ def test_swiglu(M, I, K):
     got = out.float().cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 2 ** -7 * np.abs(ref) + 1e-3), float(np.abs(got - ref).max())
     assert int(st.item()) == 0
+
+
+# activation rows, columns, K, epilogue, tiles left in the last round, activation rows of the units that each of those is cut into
+@pytest.mark.parametrize("M,N,K,epi,left,rows", [
+    (1152, 15760, 320, 3, 14, 80),      # three units of 80 rows for 240
+    (980, 18952, 320, 0, 4, 32),        # eight of 32 for 256; the last tile has 212 rows, its last unit none
+    (980, 18952, 320, 1, 4, 32),
+    (600, 10440, 320, 2, 24, 112),      # two of 112 for 208
+    (1152, 7856, 320, 2, 14, 80),
+])
+def test_last_round_of_few_tiles(M, N, K, epi, left, rows):
+    """The tiles of a nearly empty last round are cut along their activation rows."""
+    import paper_2609_27396_b200 as dp
+    nt = dp.gemm_route(M, N, K, epilogue=epi)["tile_rows"]
+    units = -(-M // nt) * -(-N // (128 if epi == 2 else 256))
+    assert units > 74 and units % 74 == left and rows == max(32, (nt // (48 // left) + 15) // 16 * 16)
+    rng = np.random.default_rng(M + N + K + epi)
+    a, w = _bits(rng, (M, K), 1.0), _bits(rng, (2 * N if epi == 2 else N, K), 0.08)
+    x, y = OA.bf16_bits_to_f64(a), OA.bf16_bits_to_f64(w)
+    r32 = rng.standard_normal((M, N)).astype(np.float32) if epi == 1 else None
+    got, st = dp.gemm_bf16(_dev(a), _dev(w), epilogue=epi, resid=torch.from_numpy(r32).cuda() if epi == 1 else None)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    got = got.float().cpu().numpy().astype(np.float64)
+    ref = OL.swiglu_linear(x, y) if epi == 2 else OL.linear(x, y) + (r32 if epi == 1 else 0)
+    assert np.all(np.abs(got - ref) <= {0: 2 ** -8, 1: 0, 2: 2 ** -7, 3: 0}[epi] * np.abs(ref) + (1e-3 if epi == 2 else 1e-4))
