@@ -39,7 +39,7 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 //   kernel                                  reads ahead of its wait                in front of it, by the order its call launches them
 //   gemm_skinny_kernel with w_ready         weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
 //   qk_norm_rope_kernel                     context offsets or lengths, angles     the QKV product
-//   append_rows_kernel                      accept_len, ctx_len, capacity          the projection
+//   append_rows_kernel                      accept_len, ctx_len, capacity, row_start   the projection
 //   gemm_skinny_kernel, the LM head         weights                                head_clear_kernel
 //   ar_head_kernel                          W of the head loop                     the LM head's product
 //   verify kernels, early-start form        all but the representations; they also use their workspace   what the caller queued: the flag is its promise

@@ -17,7 +17,7 @@
 //   * sampling takes the same launch: z stays on the SM, and what a step exchanges is a sum per CTA and request and the token drawn (before: z
 //     through memory and a second launch for the draw).
 // Measured (16 steps, vocabulary 151 936, rank 256, this kernel before -> now): 16 requests greedy 233 -> 178 us, 8 requests sampling
-// 330 -> 226 us; one request, 8 steps 85 -> 73 us.  Tried: a pause between the copies of the next step's tiles (the polls are not slowed down by
+// 330 -> 213 us; one request, 8 steps 85 -> 73 us.  Tried: a pause between the copies of the next step's tiles (the polls are not slowed down by
 // them: 13.1 -> 13.5 thousand clocks a step); maxima of 16 requests per warp in place of 8 (the exchange is bound by its instructions: +1000).
 // Warps:
 //   8           streams the tiles of W that do not stay (they do not depend on the tokens: it runs ahead across steps);
