@@ -303,8 +303,9 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
 
   // Few rows: several CTAs for a row of the row-wise kernel behind the QKV product, so that a warp has one or two heads.  They would each work out
   // their row's angles, so the angles are made once, by blocks behind the rows of this norm.  With a CTA per row they are made there, behind nothing (a table
-  // of 1152 rows made the first norm 3 us longer: two blocks 1579 -> 1586 us).
-  const int n_heads = shape->n_q_heads + shape->n_kv_heads, per_row = std::min((4 * kNumSM + M - 1) / M, (n_heads + 3) / 4);
+  // of 1152 rows made the first norm 3 us longer: two blocks 1579 -> 1586 us), and up to 16 heads are few enough for one CTA's warps (144 rows of 6 heads:
+  // 220.0 -> 221.4 us when split).
+  const int n_heads = shape->n_q_heads + shape->n_kv_heads, per_row = n_heads <= 16 ? 1 : std::min((4 * kNumSM + M - 1) / M, (n_heads + 3) / 4);
   AngleJob angles;
   if (L->use_rope) {
     if (per_row > 1) angles.table = reinterpret_cast<float *>(lw + w.angles);

@@ -115,7 +115,7 @@ def test_angles_are_made_once_for_blocks_that_turn_alike():
     import paper_2609_27396_b200 as dp
     g = torch.Generator(device="cuda").manual_seed(3)
     bf = lambda sigma, *shape: (sigma * torch.randn(*shape, device="cuda", generator=g)).to(torch.bfloat16)  # noqa: E731
-    b, J, Bq, Hq, Hkv, D, H, I = 2, 3, 4, 4, 2, 64, 256, 512
+    b, J, Bq, Hq, Hkv, D, H, I = 2, 3, 4, 16, 4, 64, 256, 512     # 20 heads: a table is only made above 16
     off, rows = [0, 70, 75], J * Bq + J
     shape = dict(n_boundaries=J, block=Bq, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D)
     turns = [dict(rope_theta=1e6), dict(rope_theta=1e6), dict(rope_theta=1e4), dict(use_rope=False), dict(rope_theta=1e4), dict(rope_theta=1e4)]
