@@ -269,8 +269,10 @@ dpara_status dpara_verify_select_static(const dpara_verify_io *io, int32_t *stat
  * language-model head on shipped hidden states right before the head loop).  uniforms == NULL: greedy decoding (Table 1),
  * y_i is the lowest index holding the maximum of z_i; NaN ranks below every number.  uniforms != NULL: sampling (App. C:
  * temperature 1, top-p 1), y_i is drawn from softmax(z_i) by the inverse CDF in vocabulary order with the supplied
- * uniform u = uniforms[n][i-1] = m * 2^-24: the lowest v with sum_{v' <= v} w_v' > u * sum w, w_v = exp(z_v - max z)
- * (exponentials and sums in double precision; NaN logits weigh nothing).
+ * uniform u = uniforms[n][i-1] = m * 2^-24: the lowest v with sum_{v' <= v} w_v' > u * sum w, w_v = exp(z_v - max z).
+ * Exponentials have the precision of fp32 and the range of double, sums are double: u = 0 draws the lowest v with any weight in
+ * that range.  NaN logits weigh nothing; a u outside [0, 1) draws the last v with weight; a row without a logit above -inf, or
+ * with one of +inf, gives token 0.
  *   sel_reps     device [b][block][hidden] bf16: the selected branches (the `selected` output of dpara_verify_select)
  *   w_lm         device [vocab][hidden] bf16 (weights stored [out][in])
  *   ar_w, ar_e   device [vocab][rank] bf16: W (one row per vocabulary entry) and E (one row per token)

@@ -17,7 +17,8 @@
 //   * sampling takes the same launch: z stays on the SM, and what a step exchanges is a sum per CTA and request and the token drawn (before: z
 //     through memory and a second launch for the draw).
 // Measured (16 steps, vocabulary 151 936, rank 256, this kernel before -> now): 16 requests greedy 233 -> 178 us, 8 requests sampling
-// 330 -> 213 us; one request, 8 steps 85 -> 73 us.  Tried: a pause between the copies of the next step's tiles (the polls are not slowed down by
+// 330 -> 230 us (213 with weights as powers of two and their sums in fixed point, which lost light entries and failed for logits above 2^23);
+// one request, 8 steps 85 -> 73 us.  Tried: a pause between the copies of the next step's tiles (the polls are not slowed down by
 // them: 13.1 -> 13.5 thousand clocks a step); maxima of 16 requests per warp in place of 8 (the exchange is bound by its instructions: +1000).
 // Warps:
 //   8           streams the tiles of W that do not stay (they do not depend on the tokens: it runs ahead across steps);
@@ -32,9 +33,9 @@
 // Greedy: a maximum travels as (order-preserving key of z) << 32 | ~index: the largest word is the largest logit, lowest index on ties; NaN
 // ranks below every number.
 // Sampling: z replaces the base logit where that lies (shared memory; the call's workspace where a step's logits do not fit), each
-// CTA publishes its weight sum per request and the exponent it is relative to; every CTA finds the CTA the threshold u * (sum of all) falls into by the
-// same arithmetic, and that one finds the crossing entry and publishes the token.  Weights are fp32 (relative error ~1e-7, far below the fp32
-// logits' own), their sums carry 44 bits and more behind the point.
+// CTA publishes its weight sum per request and the maximum it is relative to; every CTA finds the CTA the threshold u * (sum of all) falls into by the
+// same arithmetic, and that one finds the crossing entry and publishes the token.  Weights are fp32 exponentials (their argument is rounded: 6e-8 of
+// its size, beside the logits' own error), sums fp64.
 // All waits are bounded by wall time and give up with DPARA_STATUS_TIMEOUT; the launch is cooperative, so all CTAs are resident.
 #include "gemm.cuh"
 #include "head.cuh"
@@ -102,71 +103,27 @@ __device__ __forceinline__ bool poll_words(At at, uint32_t tag, unsigned long lo
   }
 }
 
-// ---- sampling.  The weight of a logit z is 2^(z log2(e) - E) with a whole exponent E of the CTA's own (the largest weight is in (1/2, 1]), so that
-// weights of different CTAs differ by a power of two; sums are whole numbers of 2^-F, F = 62 - log2(vocabulary) bits (44 at 151 936), and are
-// brought to the largest E by shifts.  The fp64 pipe has no part in it: with fp64 sums of exp(z - max) and their
-// fp64 exponentials a draw took 4 us more.
-constexpr long long kNoWeight = -(1ll << 50), kInfinite = 1ll << 50;   // E of a CTA without a number above -inf; with an infinite one
-struct Scale {
-  float m = 0.f, e = 0.f;
-  long long exponent = kNoWeight;
-  __device__ __forceinline__ Scale() {}
-  __device__ __forceinline__ explicit Scale(float top) : m(top), exponent(top > 0.f ? kInfinite : kNoWeight) {
-    if (!finite()) return;
-    if (far()) {
-      // (codes that keep the order and are more than 62 apart from one another and from every other exponent)
-      const long long code = (1ll << 40) + ((long long)__float_as_uint(fabsf(m)) << 8);
-      exponent = m > 0.f ? code : -code;
-    } else {
-      e = ceilf(m * 1.4426950408889634f);
-      exponent = (long long)e;
-    }
-  }
-  __device__ __forceinline__ bool finite() const { return m > -INFINITY && m < INFINITY; }
-  // from here on neighbouring floats are 256 apart: only the largest has weight
-  __device__ __forceinline__ bool far() const { return fabsf(m) >= 2147483648.f; }
-  __device__ __forceinline__ float weight(float z) const {
-    if (far()) return z == m ? 1.f : 0.f;
-    z = fmaxf(z, -INFINITY);   // (NaN: no weight)
-    return ex2(fmaf(z, kLog2eLo, fmaf(z, kLog2eHi, -e)));
-  }
-  static constexpr float kLog2eHi = 1.44269502162933349609375f, kLog2eLo = 1.92596299112661746887e-8f;   // log2(e) in two floats
-};
-// Two sums of floats with the rounding errors of their additions kept beside them (Knuth's TwoSum on pairs): 2^-46 and better.
-struct TwoSum {
-  uint64_t s = 0, c = 0;
-  __device__ __forceinline__ void add(uint64_t x) {
-    const uint64_t minus = pack2(-1.f, -1.f), t = add2(s, x), y = fma2(s, minus, t);
-    c = add2(c, add2(fma2(fma2(y, minus, t), minus, s), fma2(y, minus, x)));
-    s = t;
-  }
-  __device__ __forceinline__ unsigned long long fixed(float unit) const {
-    float a, b, x, y;
-    unpack2(s, a, b);
-    unpack2(c, x, y);
-    const long long v = (__float2ll_rn(a * unit) + __float2ll_rn(b * unit)) + (__float2ll_rn(x * unit) + __float2ll_rn(y * unit));
-    return v > 0 ? (unsigned long long)v : 0ull;
-  }
-};
-// v brought from its exponent to one that is `up` larger
-__device__ __forceinline__ unsigned long long lowered(unsigned long long v, long long up) { return up > 63 ? 0ull : v >> up; }
-__device__ __forceinline__ unsigned long long warp_scan(unsigned long long v, int lane) {
+// ---- sampling.  A logit's weight is exp(z - m) against the maximum m of its CTA's entries, in fp32 where that is a normal number and in fp64 below;
+// every sum is fp64.  A CTA's sum travels with its m, and exp(m - largest m) in fp64 brings it beside the others'.
+constexpr float kDeep = -87.f;
+__device__ __noinline__ double deep_weight(float z, float m) { return exp((double)z - (double)m); }
+// (NaN: no weight)
+__device__ __forceinline__ double weight(float z, float m) {
+  z = fmaxf(z, -INFINITY);
+  return z - m < kDeep ? deep_weight(z, m) : (double)expf(z - m);
+}
+__device__ __forceinline__ double warp_scan(double v, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long t = __shfl_up_sync(0xffffffffu, v, o);
+    const double t = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += t;
   }
   return v;
 }
-// floor(u * total), total < 2^62; anything that is not in [0, 1): total (which makes the last entry with weight the one drawn)
-__device__ __forceinline__ unsigned long long threshold(float u, unsigned long long total) {
-  if (!(u >= 0.f && u < 1.f)) return total;
-  const uint32_t bits = __float_as_uint(u) & 0x7fffffffu, field = bits >> 23;
-  const unsigned long long mant = field ? (bits & 0x7fffffu) | 0x800000u : bits;
-  const int down = 150 - (int)(field ? field : 1u);   // u = mant * 2^-down, down >= 24
-  const unsigned long long lo = mant * total, hi = __umul64hi(mant, total);
-  if (down < 64) return (hi << (64 - down)) | (lo >> down);
-  return down < 128 ? hi >> (down - 64) : 0ull;
+// The sum of the lanes before this one, from the sums up to each: the next lane starts where this one ends, so that no threshold falls between two.
+__device__ __forceinline__ double before_lane(double inclusive, int lane) {
+  const double t = __shfl_up_sync(0xffffffffu, inclusive, 1);
+  return lane ? t : 0.0;
 }
 
 template <int kCols>
@@ -192,7 +149,6 @@ struct ArParams {
   int resident;                   // tiles that stay in tensor memory
   int stages, logit_slots, slab_bytes, logit_bytes, logit_off, e_off, bar_off;
   int z_in_place;                 // sampling: a step's base logits all have slots, z replaces them there
-  float unit;                     // sampling: 2^F
 };
 
 template <bool kSample, int kSlabs, int kNb>
@@ -508,48 +464,62 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
         // weight sums: lane l has the groups of four entries [l per_lane, (l + 1) per_lane) of the CTA's range (an odd number of them: no bank
         // conflicts), three groups at a time
         const int groups = count >> 2, tile_groups = P.rows >> 2, per_lane = ((groups + 31) >> 5) | 1, seg = 4 * per_lane;
-        unsigned long long mine[kPer];
-        unsigned long long got[kPer * 2 * kCtasPerLane];   // per request: the lane's CTAs' sums, then their exponents
+        double mine[kPer];
+        float own_m[kPer];
+        unsigned long long got[kPer * 2 * kCtasPerLane];   // per request: the lane's CTAs' sums, then their maxima
         const float *const z0 = P.z_in_place ? reinterpret_cast<const float *>(sL) : P.z + v0;
         auto z_at = [&](int n, int e) { const int t = e / P.rows; return z0 + (size_t)n * z_row + (size_t)t * z_tile + (e - t * P.rows); };
-        Scale ref[kPer];
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
           const int n = warp + kEpiWarps * q;
-          mine[q] = 0ull;
+          mine[q] = 0.0;
+          own_m[q] = -INFINITY;
           if (n < P.b) {
             const uint32_t key = (uint32_t)(top[q] >> 32);
-            ref[q] = Scale(__uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key));
-            if (ref[q].finite()) {
+            const float m = __uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key);
+            own_m[q] = m;
+            if (m > -INFINITY && m < INFINITY) {
               int g = lane * per_lane, t = g / tile_groups, r = g - t * tile_groups;
               const int g1 = min(groups, g + per_lane);
               const float *const zn = z0 + (size_t)n * z_row;
-              TwoSum sum[2];
+              double sum[2] = {0.0, 0.0};
 #pragma unroll 1
               for (; g < g1; g += 3) {
                 float4 x[3];
+                float low = m;
 #pragma unroll
                 for (int u = 0; u < 3; ++u) {
-                  x[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                  x[u] = make_float4(m, m, m, m);
                   if (g + u < g1) x[u] = *reinterpret_cast<const float4 *>(zn + (size_t)t * z_tile + 4 * r);
                   if (++r == tile_groups) { r = 0; ++t; }
+                  x[u].x = fmaxf(x[u].x, -INFINITY); x[u].y = fmaxf(x[u].y, -INFINITY); x[u].z = fmaxf(x[u].z, -INFINITY); x[u].w = fmaxf(x[u].w, -INFINITY);
+                  low = fminf(low, fminf(fminf(x[u].x, x[u].y), fminf(x[u].z, x[u].w)));
                 }
+                if (low - m >= kDeep) {
 #pragma unroll
-                for (int u = 0; u < 3; ++u) {
-                  sum[0].add(pack2(ref[q].weight(x[u].x), ref[q].weight(x[u].y)));
-                  sum[1].add(pack2(ref[q].weight(x[u].z), ref[q].weight(x[u].w)));
+                  for (int u = 0; u < 3; ++u) {
+                    const double w0 = expf(x[u].x - m), w1 = expf(x[u].y - m), w2 = expf(x[u].z - m), w3 = expf(x[u].w - m);
+                    if (g + u < g1) { sum[0] += w0; sum[1] += w1; sum[0] += w2; sum[1] += w3; }
+                  }
+                } else {
+#pragma unroll 1
+                  for (int e = 0; e < 12 && g + (e >> 2) < g1; ++e) {
+                    const float4 y = e < 4 ? x[0] : e < 8 ? x[1] : x[2];
+                    sum[0] += weight((e & 3) == 0 ? y.x : (e & 3) == 1 ? y.y : (e & 3) == 2 ? y.z : y.w, m);
+                  }
                 }
               }
-              mine[q] = sum[0].fixed(P.unit) + sum[1].fixed(P.unit);
+              mine[q] = sum[0] + sum[1];
             }
-            unsigned long long s = mine[q];
+            double s = mine[q];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane < copies) {
               unsigned long long *const to = words + lane * copy_words + (size_t)(2 * n) * kCtaStride + slot_of(blockIdx.x);
-              // (the sum's lowest bits travel with the exponent)
-              publish(to, (s & ~kTagMask) | tag);
-              publish(to + kCtaStride, (unsigned long long)ref[q].exponent << 2 * kTagBits | (s & kTagMask) << kTagBits | tag);
+              const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
+              // (the sum's lowest bits travel with the maximum)
+              publish(to, (bits & ~kTagMask) | tag);
+              publish(to + kCtaStride, (unsigned long long)__float_as_uint(m) << 32 | (bits & kTagMask) << kTagBits | tag);
             }
           }
         }
@@ -562,65 +532,72 @@ __global__ void __launch_bounds__(kThreads, 1) ar_head_kernel(const __grid_const
           for (int q = 0; q < kPer; ++q) {
             const int n = warp + kEpiWarps * q;
             if (n >= P.b) break;
-            unsigned long long s_all[kCtasPerLane];
-            long long e_all[kCtasPerLane], top_e = kNoWeight;
+            double s_all[kCtasPerLane];
+            float m_all[kCtasPerLane], top_m = -INFINITY;
 #pragma unroll
             for (int i = 0; i < kCtasPerLane; ++i) {
               const bool has = lane * kCtasPerLane + i < n_ctas;
-              const unsigned long long sum = got[(2 * q) * kCtasPerLane + i], exponent = got[(2 * q + 1) * kCtasPerLane + i];
-              s_all[i] = has ? (sum & ~kTagMask) | (exponent >> kTagBits & kTagMask) : 0ull;
-              e_all[i] = has ? (long long)exponent >> 2 * kTagBits : kNoWeight;
-              top_e = e_all[i] > top_e ? e_all[i] : top_e;
+              const unsigned long long sum = got[(2 * q) * kCtasPerLane + i], max = got[(2 * q + 1) * kCtasPerLane + i];
+              s_all[i] = has ? __longlong_as_double((long long)((sum & ~kTagMask) | (max >> kTagBits & kTagMask))) : 0.0;
+              m_all[i] = has ? __uint_as_float((uint32_t)(max >> 32)) : -INFINITY;
+              top_m = fmaxf(top_m, m_all[i]);
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              const long long t = __shfl_xor_sync(0xffffffffu, top_e, o);
-              top_e = t > top_e ? t : top_e;
-            }
-            int owner = 0, pick = 0;
-            if (top_e > kNoWeight && top_e < kInfinite) {
-              unsigned long long run = 0ull;
+            for (int o = 16; o > 0; o >>= 1) top_m = fmaxf(top_m, __shfl_xor_sync(0xffffffffu, top_m, o));
+            int owner = 0, pick = 0;    // (no number above -inf, or an infinite one: token 0)
+            if (top_m > -INFINITY && top_m < INFINITY) {
+              double run = 0.0;
 #pragma unroll
               for (int i = 0; i < kCtasPerLane; ++i) {
-                s_all[i] = lowered(s_all[i], top_e - e_all[i]);
+                s_all[i] *= exp((double)m_all[i] - (double)top_m);
                 run += s_all[i];
               }
-              const unsigned long long inc = warp_scan(run, lane), total = __shfl_sync(0xffffffffu, inc, 31);
-              const unsigned long long T = threshold(P.uniforms[(size_t)n * P.block + step], total);
-              // the CTA the threshold falls into; if there is none, the last one with weight
-              unsigned long long before = inc - run, base = 0ull;
-              int found = -1;
+              const double inc = warp_scan(run, lane), total = __shfl_sync(0xffffffffu, inc, 31);
+              // (a uniform that is not in [0, 1) makes the last entry with weight the one drawn)
+              const float u = P.uniforms[(size_t)n * P.block + step];
+              const double T = u >= 0.f && u < 1.f ? (double)u * total : (double)INFINITY;
+              // the first CTA whose end lies above the threshold; if rounding left none, the last one with weight.  (There is one: the sum of
+              // the CTA with the largest m is at least 1.)
+              double from = before_lane(inc, lane), base = 0.0, tail_base = 0.0;
+              int found = -1, tail = -1;
 #pragma unroll
               for (int i = 0; i < kCtasPerLane; ++i) {
-                if (s_all[i] && (T >= total || (before <= T && T - before < s_all[i]))) { found = lane * kCtasPerLane + i; base = before; }
-                before += s_all[i];
+                const double to = from + s_all[i];
+                if (s_all[i] > 0.0) {
+                  tail = lane * kCtasPerLane + i; tail_base = from;
+                  if (found < 0 && to > T) { found = tail; base = from; }
+                }
+                from = to;
               }
-              const unsigned int who = __ballot_sync(0xffffffffu, found >= 0);   // (not empty: the largest weight of the row is above 1/2)
-              const int src = 31 - __clz(who);
+              unsigned int who = __ballot_sync(0xffffffffu, found >= 0);
+              int src = __ffs(who) - 1;
+              if (!who) {
+                found = tail; base = tail_base;
+                src = 31 - __clz(__ballot_sync(0xffffffffu, tail >= 0));
+              }
               owner = __shfl_sync(0xffffffffu, found, src);
               base = __shfl_sync(0xffffffffu, base, src);
               if (owner == (int)blockIdx.x) {
-                // the lane whose entries the threshold falls into, then the entry
-                const long long up = top_e - ref[q].exponent;
-                const unsigned long long w = lowered(mine[q], up), from = base + (warp_scan(w, lane) - w);
-                unsigned int hit = __ballot_sync(0xffffffffu, w && from <= T && T - from < w);
-                if (!hit) hit = __ballot_sync(0xffffffffu, w != 0ull);
-                const int hl = 31 - __clz(hit ? hit : 1u);
-                unsigned long long acc = __shfl_sync(0xffffffffu, from, hl);
+                // the lane whose entries the threshold falls into, then the entry, by the same rule
+                const double scale = exp((double)own_m[q] - (double)top_m), w = mine[q] * scale, lane_inc = warp_scan(w, lane), lane_from = before_lane(lane_inc, lane);
+                unsigned int hit = __ballot_sync(0xffffffffu, w > 0.0 && base + lane_inc > T);
+                int hl = __ffs(hit) - 1;
+                if (!hit) hl = 31 - __clz(__ballot_sync(0xffffffffu, w > 0.0));
+                double acc = base + __shfl_sync(0xffffffffu, lane_from, hl);
                 const int e0 = hl * seg, e1 = min(count, e0 + seg);
                 pick = -1;
-                int tail = e0;                                           // the last entry with weight
+                int last_entry = e0;                                     // the last entry with weight
 #pragma unroll 1
                 for (int c0 = e0; c0 < e1 && pick < 0; c0 += 32) {
-                  unsigned long long x = 0ull;
-                  if (c0 + lane < e1) x = lowered(__float2ull_rn(ref[q].weight(*z_at(n, c0 + lane)) * P.unit), up);
-                  const unsigned long long in = warp_scan(x, lane);
-                  const unsigned int over = __ballot_sync(0xffffffffu, x && acc + in > T), some = __ballot_sync(0xffffffffu, x != 0ull);
+                  double x = 0.0;
+                  if (c0 + lane < e1) x = weight(*z_at(n, c0 + lane), own_m[q]);
+                  const double in = warp_scan(x * scale, lane);
+                  const unsigned int some = __ballot_sync(0xffffffffu, x > 0.0), over = __ballot_sync(0xffffffffu, x > 0.0 && acc + in > T);
                   if (over) pick = c0 + __ffs(over) - 1;
-                  if (some) tail = c0 + 31 - __clz(some);
+                  if (some) last_entry = c0 + 31 - __clz(some);
                   acc += __shfl_sync(0xffffffffu, in, 31);
                 }
-                if (pick < 0) pick = tail;
+                if (pick < 0) pick = last_entry;
                 pick += v0;
               }
             }
@@ -741,9 +718,6 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   if (!make_tmap_bf16_2d(&P.map_w, h.ar_w, h.rank, h.vocab, (uint64_t)h.rank * 2, 64, P.rows)) return DPARA_ERR_CUDA;
   if (!make_tmap_f32_2d(&P.map_l, logits, h.vocab, (uint64_t)h.block * h.b, (uint64_t)h.vocab * 4, P.rows, h.b)) return DPARA_ERR_CUDA;
   P.ar_w = static_cast<const uint16_t *>(h.ar_w); P.ar_e = static_cast<const uint16_t *>(h.ar_e);
-  int bits = 0;
-  while (bits < 31 && ((h.vocab - 1) >> bits) != 0) ++bits;
-  P.unit = ldexpf(1.f, 62 - bits);
   P.bonus = h.bonus; P.uniforms = h.uniforms; P.next_tokens = h.next_tokens;
   P.drawn = words; P.words = words + kDrawnWords; P.status = status;
   P.z = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(words) + words_bytes(h.b));

@@ -87,3 +87,50 @@ def test_sampling_of_unusual_logits(fill, special):
                 w = np.where(np.isnan(z), 0.0, np.exp(z - np.nanmax(z)))
                 c = np.cumsum(w) / w.sum()
                 assert w[got] > 0 and c[got] - w[got] / w.sum() - 1e-6 <= u[n, i] <= c[got] + 1e-6, (n, i, got, want)
+
+
+def _sample_row(row, u):
+    """The tokens and the status of a call whose logits are `row` (bf16) in every step of both requests, with the uniforms u [2][block]."""
+    vocab, block = len(row), u.shape[1]
+    w_lm = torch.zeros(vocab, 64, dtype=torch.bfloat16)
+    w_lm[:, 0] = row
+    reps = torch.zeros(2, block, 64, dtype=torch.bfloat16)
+    reps[:, :, 0] = 1.0
+    zero = torch.zeros(vocab, 64, dtype=torch.bfloat16, device="cuda")
+    toks, plan = dp.draft_head(reps.cuda(), w_lm.cuda(), zero, zero, torch.zeros(2, dtype=torch.int32, device="cuda"), uniforms=torch.from_numpy(u).cuda())
+    torch.cuda.synchronize()
+    return toks.cpu().numpy(), plan.status.item()
+
+
+# Neighbouring values of these sizes are 65536 and more apart, 32768 at the smallest: an entry weighs 1 or nothing, and the tokens are the oracle's
+@pytest.mark.parametrize("block", [1, 4])
+@pytest.mark.parametrize("at", ["one", "two", "all"])
+@pytest.mark.parametrize("top", [1e7, -1e7, 1e8, -1e8, 188743680.0, -754974720.0, 1551892480.0, -1585446912.0, 1.5e9, -1.5e9, 2.0 ** 31, -3e38, 3e38])
+def test_sampling_of_large_logits(top, at, block):
+    row = torch.full((8192,), top, dtype=torch.bfloat16)
+    if at != "all":
+        keep = [4099] if at == "one" else [130, 8190]
+        below = row[0].view(torch.int16) + (-1 if top > 0 else 1)          # the next bf16 towards -inf
+        row[[v for v in range(8192) if v not in keep]] = below.view(torch.bfloat16)
+    u = np.array([[0.0, 0.3, 0.75, 1 - 2.0 ** -24], [0.5, 0.11, 0.9, 0.49999]], np.float32)[:, :block]
+    toks, status = _sample_row(row, u)
+    assert status == 0
+    z = row.double().numpy()
+    assert toks.tolist() == [[H.sample_from_logits(z, float(x)) for x in r] for r in u]
+
+
+@pytest.mark.parametrize("row", [
+    {0: -200.0, 8191: 90.0},                       # the lightest entry is e^-290 of the row
+    {0: -600.0, 1: -480.0, 2: -350.0, 3: 0.0},     # ... and its neighbours in the same CTA's range are not much heavier
+    {40: -104.0, 41: 0.0},                         # below the smallest fp32
+    {5000: -87.0, 5001: -86.5, 5002: 0.0},
+])
+def test_sampling_of_light_entries(row):
+    """At u = 0 the lowest entry with any weight in double precision, however light; one step of the uniform further the heavy one."""
+    full = torch.full((8192,), -float("inf"), dtype=torch.bfloat16)
+    for v, z in row.items():
+        full[v] = z
+    toks, status = _sample_row(full, np.array([[0.0, 2.0 ** -24], [2.0 ** -24, 0.0]], np.float32))
+    assert status == 0
+    low, heavy = min(row), max(row, key=row.get)
+    assert toks.tolist() == [[low, heavy], [heavy, low]]
