@@ -316,7 +316,8 @@ dpara_status dpara_draft_head(const dpara_head_io *io, void *workspace, size_t w
  *                 norm_w [feat_dim] and knorm_w [D] bf16 gains (array or entries may be NULL), k_ctx / v_ctx caches
  *   row_start, capacity   device [b] int64;   ctx_len   device [b] int64, in/out
  * Workspace: dpara_cache_append_workspace_bytes(), 16-byte aligned, private to the call while it runs.
- * Errors: INVALID_ARG, UNSUPPORTED (head_dim not 64/128, feat_dim % 64 != 0), WORKSPACE, CUDA. */
+ * Errors: INVALID_ARG (null pointers, a bf16 tensor that is not 16-byte aligned, the gains among them), UNSUPPORTED (head_dim not 64/128,
+ * feat_dim % 64 != 0), WORKSPACE, CUDA. */
 typedef struct {
   int32_t batch, n_rows, feat_dim, n_kv_heads, head_dim, n_layers;
   const void *features;

@@ -325,7 +325,7 @@ extern "C" dpara_status dpara_cache_append(const dpara_cache_io *io, void *works
     return DPARA_ERR_INVALID_ARG;
   for (int l = 0; l < io->n_layers; ++l)
     if (!io->host_w_kv[l] || !io->host_k_ctx[l] || !io->host_v_ctx[l] || !aligned16(io->host_w_kv[l]) || !aligned16(io->host_k_ctx[l]) ||
-        !aligned16(io->host_v_ctx[l]))
+        !aligned16(io->host_v_ctx[l]) || (io->host_norm_w && !aligned16(io->host_norm_w[l])) || (io->host_knorm_w && !aligned16(io->host_knorm_w[l])))
       return DPARA_ERR_INVALID_ARG;
   if (!aligned16(io->features)) return DPARA_ERR_INVALID_ARG;
   if (!workspace || workspace_bytes < cache_append_workspace_bytes(io) || !aligned16(workspace)) return DPARA_ERR_WORKSPACE;

@@ -126,3 +126,22 @@ def test_rings_of_the_kernel_for_few_rows():
             stage = 2 * 128 * (r["operands"] * r["weight_rows"] + r["tile_rows"])
             assert r["slabs"] == 1 or (3 if M <= 64 else 4) * stage <= (227 - 16) * 1024, (M, N, K, r)
     assert two > 10
+
+
+def _append_of_two_layers(**kw):
+    """The host's answer to an append whose pointers are 4096 except for those given; without a workspace, so that nothing is launched."""
+    n = 2
+    d = dict(features=4096, w_kv=[4096] * n, norm=[4096] * n, knorm=[4096] * n, k=[4096] * n, v=[4096] * n)
+    d.update(kw)
+    tabs = [(C.c_void_p * n)(*d[k]) for k in ("w_kv", "norm", "knorm", "k", "v")]
+    io = dp.CacheIO(1, 4, 128, 2, 64, n, d["features"], 4096, *[C.addressof(t) for t in tabs], 4096, 4096, 4096, 1e-6, 1e6, 1)
+    return dp.lib.dpara_cache_append(C.byref(io), None, 0, None, None)
+
+
+def test_append_refuses_misaligned_tensors():
+    assert _append_of_two_layers() == dp.ERR_WORKSPACE                                  # nothing else is wrong
+    assert _append_of_two_layers(norm=[None, 4096], knorm=[4096, None]) == dp.ERR_WORKSPACE
+    for name in ("w_kv", "norm", "knorm", "k", "v"):
+        for off in (2, 8):
+            assert _append_of_two_layers(**{name: [4096, 4096 + off]}) == dp.ERR_INVALID_ARG, (name, off)
+    assert _append_of_two_layers(features=4098) == dp.ERR_INVALID_ARG
