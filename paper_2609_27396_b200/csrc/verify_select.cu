@@ -606,11 +606,14 @@ static int chunks_of(const dpara_verify_io *io) {
 }
 
 // Greedy: do all CTAs run at once?  (Three per SM are resident in the form with the most loads per thread, more in the others.)
-static bool one_wave_of(const dpara_verify_io *io) { return (long long)io->batch * io->n_boundaries * chunks_of(io) <= 3 * kNumSM; }
+constexpr int kOneWave = 3 * kNumSM;
+static bool one_wave_of(const dpara_verify_io *io) { return (long long)io->batch * io->n_boundaries * chunks_of(io) <= kOneWave; }
 
-// workspace: [64-bit area][counters]
+// workspace: [64-bit area][counters].  Greedy: a key per row or a slot per CTA of one wave, and room for the most slots whatever the sizes, so that the
+// workspace of a larger call serves a smaller one.
 static size_t ws64_count(const dpara_verify_io *io) {
-  if (io->mode == 0) return (size_t)io->batch * io->n_boundaries * (one_wave_of(io) ? chunks_of(io) : 1);
+  const size_t rows = (size_t)io->batch * io->n_boundaries;
+  if (io->mode == 0) return rows > kOneWave ? rows : kOneWave;
   return (size_t)io->batch * chunks_of(io) * 2;
 }
 

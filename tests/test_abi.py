@@ -145,3 +145,14 @@ def test_append_refuses_misaligned_tensors():
         for off in (2, 8):
             assert _append_of_two_layers(**{name: [4096, 4096 + off]}) == dp.ERR_INVALID_ARG, (name, off)
     assert _append_of_two_layers(features=4098) == dp.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_workspace_of_a_larger_select_serves_a_smaller_one(mode):
+    """A program that sizes one workspace for its largest batch calls with fewer requests and boundaries too."""
+    need = lambda b, J, V: dp.lib.dpara_verify_workspace_bytes(C.byref(dp.VerifyIO(b, J, V, 2, 64, mode)))
+    for V in (1, 1000, 20000, 60000, 151936):
+        for J in (1, 2, 5, 16, 37, 64):
+            for b in list(range(1, 80)) + [150, 444, 445]:
+                most = need(b, J, V)
+                assert need(b + 1, J, V) >= most and (J == 64 or need(b, J + 1, V) >= most) and need(b, J, V + 5000) >= most, (b, J, V)
