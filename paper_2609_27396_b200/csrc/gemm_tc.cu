@@ -411,13 +411,15 @@ dpara_status gemm_route(const GemmArgs &g, GemmRoute &r) {
   return DPARA_OK;
 }
 
-// The tiles of a last round that has few of them (at most a third of the pairs): each in `split` parts of its activation rows, on pairs that would have
-// nothing to do.  Every part reads the tile's weights again (from L2), so only as many as L2 serves beside.  256 x 151936 x 5120: 594 tiles are eight
-// rounds of 74 pairs and two tiles; with the head loop behind it 559.8 -> 552.3 us (about a quarter of what the round took: the pairs drift apart over
-// eight rounds).  1024 x 12288 x 4096 SwiGLU, five rounds and 14 tiles: the block around it 873.6 -> 864.9.
+// The tiles of a last round that has few of them (at most a third of the pairs): each in up to `at_once` / left parts of its activation rows, on pairs that
+// would have nothing to do.  Every part reads the tile's weights again (from L2), so only about two thirds of the pairs are given one.  Against whole
+// tiles, 109 products of 129 to 1152 rows with 1 to 24 tiles left of 74, stores and SwiGLU, weights from HBM: 1.057x (geometric mean), faster by
+// more than the spread in all but three, slower by more than it in none.  1.13 behind one round of tiles, 1.07 behind two or three, 1.035 behind four to nine (the pairs drift
+// apart, and the whole tiles of a last round start early on some); 1.068 with 1 to 8 tiles left, 1.058 with 9 to 16, 1.044 with 17 to 24.  For
+// instance 207 x 23112 x 1088 22.0 -> 19.7 us, 498 x 9920 x 2752 SwiGLU 54.9 -> 48.6, 1014 x 14784 x 4544 SwiGLU 196 -> 190.
 static bool tail_plan(const GemmArgs &g, const GemmRoute &r, GemmKernelParams &P) {
   const long units = (long)r.pair.t_tiles * r.n_all;
-  const int left = (int)(units % r.most), at_once = 48;
+  const int left = (int)(units % r.most), at_once = r.most * 13 / 20;   // 48 of 74 pairs
   if (g.n_groups > 1 || g.split_k > 1 || units < r.most || left == 0 || 2 * left > at_once) return false;
   P.nt_tail = (r.pair.nt / (at_once / left) + 15) / 16 * 16;
   if (P.nt_tail < 32) P.nt_tail = 32;
