@@ -303,8 +303,9 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
 
   // Few rows: several CTAs for a row of the row-wise kernel behind the QKV product, so that a warp has one or two heads.  They would each work out
   // their row's angles, so the angles are made once, by blocks behind the rows of this norm.  With a CTA per row they are made there, behind nothing (a table
-  // of 1152 rows made the first norm 3 us longer: two blocks 1579 -> 1586 us), and up to 16 heads are few enough for one CTA's warps (144 rows of 6 heads:
-  // 220.0 -> 221.4 us when split).
+  // of 1152 rows made the first norm 3 us longer: two blocks 1579 -> 1586 us), and up to 16 heads are few enough for one CTA's warps.  What several CTAs save a
+  // block of 25, 72, 144, 288 or 429 rows: 2.0 to 5.6 us at 40 heads, 1.5 to 4.0 at 32, 0.1 to 2.4 at 24, 0.3 to 1.6 at 20, -0.3 to 0.7 at 16; at 12, 10 and 8 they
+  // lose 0.6 to 0.7 at 429 rows and mostly do not show at the others (-1.1 to 0.7, runs differ by up to 1).
   const int n_heads = shape->n_q_heads + shape->n_kv_heads, per_row = n_heads <= 16 ? 1 : std::min((4 * kNumSM + M - 1) / M, (n_heads + 3) / 4);
   AngleJob angles;
   if (L->use_rope) {
