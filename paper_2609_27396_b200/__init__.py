@@ -152,12 +152,16 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return t.data_ptr()
 
 
+# The current stream's handle as a number: the Stream object that torch.cuda.current_stream() makes is 3 us of a call's host time, which is what bounds
+# small calls (draft and verify of one tiny request: 21.7 us of host, 12 of GPU).  A private name of torch, so the public way stands behind it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
-    """The stream's handle; without one that of the current stream, asked for as a number: the Stream object that torch.cuda.current_stream()
-    makes is 3 us of a call's host time, which is what bounds small calls (draft and verify of one tiny request: 21.7 us of host, 12 of GPU)."""
+    """The stream's handle; without one that of the current stream of the current device."""
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return _raw_stream(torch.cuda.current_device()) if _raw_stream else torch.cuda.current_stream().cuda_stream
 
 
 def _host_offsets(ctx_offsets: Sequence[int]):

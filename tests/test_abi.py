@@ -156,3 +156,15 @@ def test_workspace_of_a_larger_select_serves_a_smaller_one(mode):
             for b in list(range(1, 80)) + [150, 444, 445]:
                 most = need(b, J, V)
                 assert need(b + 1, J, V) >= most and (J == 64 or need(b, J + 1, V) >= most) and need(b, J, V + 5000) >= most, (b, J, V)
+
+
+@pytest.mark.parametrize("raw", [None, lambda device: 100 + device])
+def test_stream_handle_with_and_without_the_raw_query(monkeypatch, raw):
+    class Stream:
+        cuda_stream = 103
+    monkeypatch.setattr(dp, "_raw_stream", raw)
+    monkeypatch.setattr(dp.torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(dp.torch.cuda, "current_stream", lambda: Stream)
+    assert dp._stream_ptr(None) == 103
+    Stream.cuda_stream = 7
+    assert dp._stream_ptr(Stream) == 7
