@@ -58,6 +58,14 @@ extern "C" dpara_status dpara_layer_workspace_layout(const dpara_shape *shape, c
   return DPARA_OK;
 }
 
+// What a block's kernels read and write with wide accesses; `first`, `last`: in its stack (the tensors between blocks are the workspace's).
+// The head norms' gains are read four bytes at a time.
+static bool layer_aligned(const dpara_layer_io &L, bool first, bool last) {
+  auto aligned4 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; };
+  return aligned16(L.w_qkv) && aligned16(L.w_o) && aligned16(L.w_gate_up) && aligned16(L.w_down) && aligned16(L.rms1_w) && aligned16(L.rms2_w) &&
+         aligned4(L.qnorm_w) && aligned4(L.knorm_w) && (!first || aligned16(L.x)) && (!last || (aligned16(L.y_f32) && aligned16(L.y_bf16)));
+}
+
 extern "C" dpara_status dpara_draft_all_boundaries(const dpara_shape *shape, const dpara_attn_io *io,
                                                    const dpara_layer_io *layer, void *workspace, size_t workspace_bytes,
                                                    int32_t *status_word, void *stream) {
@@ -80,6 +88,7 @@ extern "C" dpara_status dpara_draft_all_boundaries(const dpara_shape *shape, con
   if (!aligned16(io->k_ctx) || !aligned16(io->v_ctx) || !aligned16(io->k_spine) || !aligned16(io->v_spine) ||
       !aligned16(io->q) || !aligned16(io->k_blk) || !aligned16(io->v_blk) || !aligned16(io->out))
     return DPARA_ERR_INVALID_ARG;
+  if (layer && !layer_aligned(*layer, true, true)) return DPARA_ERR_INVALID_ARG;
   const size_t need = dpara_draft_workspace_bytes(shape, io->host_ctx_offsets, layer, layer != nullptr);
   if (need > 0 && (!workspace || workspace_bytes < need || !aligned16(workspace))) return DPARA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -112,6 +121,7 @@ extern "C" dpara_status dpara_draft_backbone(const dpara_shape *shape, const dpa
   for (int l = 0; l < bb->n_layers; ++l) {
     if (bb->host_layers[l].hidden != bb->host_layers[0].hidden || bb->host_layers[l].intermediate != bb->host_layers[0].intermediate)
       return DPARA_ERR_INVALID_ARG;
+    if (!layer_aligned(bb->host_layers[l], l == 0, l + 1 == bb->n_layers)) return DPARA_ERR_INVALID_ARG;
     if (has_ctx && (!bb->host_k_ctx[l] || !bb->host_v_ctx[l] || !aligned16(bb->host_k_ctx[l]) || !aligned16(bb->host_v_ctx[l])))
       return DPARA_ERR_INVALID_ARG;
   }

@@ -168,3 +168,29 @@ def test_stream_handle_with_and_without_the_raw_query(monkeypatch, raw):
     assert dp._stream_ptr(None) == 103
     Stream.cuda_stream = 7
     assert dp._stream_ptr(Stream) == 7
+
+
+LAYER_POINTERS = ("x", "w_qkv", "w_o", "w_gate_up", "w_down", "rms1_w", "rms2_w", "qnorm_w", "knorm_w", "y_f32", "y_bf16")
+
+
+def _blocks(n_layers, **at):
+    """The host's answer to a block or a stack of blocks whose pointers are 4096 except the last block's given ones; without a workspace, so that nothing is launched."""
+    off = (C.c_int64 * 2)(0, 0)
+    io = dp.AttnIO(ctx_offsets=4096, host_ctx_offsets=C.addressof(off), k_spine=4096, v_spine=4096)
+    ios = [dp.LayerIO(rms_eps=1e-6, rope_theta=1e6, use_rope=1, hidden=128, intermediate=128, **{k: 4096 for k in LAYER_POINTERS}) for _ in range(n_layers or 1)]
+    for name, p in at.items():
+        setattr(ios[-1 if name != "x" else 0], name, p)
+    if not n_layers:
+        return dp.lib.dpara_draft_all_boundaries(C.byref(_shape()), C.byref(io), C.byref(ios[0]), None, 0, None, None)
+    layers, caches = (dp.LayerIO * n_layers)(*ios), (C.c_void_p * n_layers)(*[4096] * n_layers)
+    bb = dp.BackboneIO(n_layers, C.addressof(layers), C.addressof(caches), C.addressof(caches))
+    return dp.lib.dpara_draft_backbone(C.byref(_shape()), C.byref(io), C.byref(bb), None, 0, None, None)
+
+
+@pytest.mark.parametrize("n_layers", [0, 1, 3])
+def test_blocks_refuse_misaligned_tensors(n_layers):
+    assert _blocks(n_layers) == dp.ERR_WORKSPACE                                        # nothing else is wrong
+    assert _blocks(n_layers, rms1_w=None, rms2_w=None, qnorm_w=None, knorm_w=None, y_bf16=None) == dp.ERR_WORKSPACE
+    for name in LAYER_POINTERS:
+        assert _blocks(n_layers, **{name: 4098}) == dp.ERR_INVALID_ARG, name
+    assert _blocks(n_layers, qnorm_w=4100, knorm_w=4104) == dp.ERR_WORKSPACE            # the row-wise kernel takes these
