@@ -134,3 +134,53 @@ def test_sampling_of_light_entries(row):
     assert status == 0
     low, heavy = min(row), max(row, key=row.get)
     assert toks.tolist() == [[low, heavy], [heavy, low]]
+
+
+def _inputs_of_a_call(seed, vocab):
+    inp = W.make_head_inputs(W.HeadShape(3, 6, 64, vocab, 256), seed)
+    t = [dev_bf16(x) for x in (inp.sel_reps, inp.w_lm, inp.ar_w, inp.ar_e)] + [torch.from_numpy(inp.bonus).cuda()]
+    return t, torch.from_numpy(_uniforms(inp.shape, seed)).cuda(), dp.HeadPlan(3, 6, 64, vocab, 256)
+
+
+def test_sampling_and_greedy_on_two_streams():
+    """Calls on two streams with no order between them: each loop needs all its CTAs on the chip at once, and both get that."""
+    calls = [_inputs_of_a_call(5, 60000), _inputs_of_a_call(6, 40000)]
+    want = [[plan.run(*t, uniforms=x).clone() for x in (u, None)] for t, u, plan in calls]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in calls]
+    got = [[], []]
+    for _ in range(12):
+        for i, (t, u, plan) in enumerate(calls):
+            with torch.cuda.stream(streams[i]):
+                got[i].append([plan.run(*t, uniforms=x).clone() for x in (u, None)])
+    torch.cuda.synchronize()
+    for i, (_, _, plan) in enumerate(calls):
+        assert plan.status.item() == 0
+        for g in got[i]:
+            assert torch.equal(g[0], want[i][0]) and torch.equal(g[1], want[i][1]), i
+
+
+@pytest.mark.parametrize("sampling", [False, True])
+def test_head_captured_in_a_graph(sampling):
+    t, u, plan = _inputs_of_a_call(9, 30000)
+    u = u if sampling else None
+    first = plan.run(*t, uniforms=u).clone()
+    t[4].bitwise_xor_(1)
+    if sampling:
+        u.mul_(0.5)
+    second = plan.run(*t, uniforms=u).clone()
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s), torch.cuda.graph(g, stream=s):
+        plan.run(*t, uniforms=u, stream=s)
+    for _ in range(3):
+        plan.next_tokens.fill_(-1)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(plan.next_tokens, second)
+    t[4].bitwise_xor_(1)                             # new inputs in the captured buffers
+    if sampling:
+        u.mul_(2.0)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(plan.next_tokens, first) and plan.status.item() == 0
