@@ -282,7 +282,9 @@ dpara_status dpara_verify_select_static(const dpara_verify_io *io, int32_t *stat
  * bf16 products with fp32 accumulation; z_i = (fp32 base logit) + (fp32 correction), compared in fp32.
  * Workspace: dpara_head_workspace_bytes(b, block, vocab) bytes of device memory, 16-byte aligned, owned by the
  * caller and private to the call while it runs (it holds the fp32 base logits [b * block][vocab], the words the loop's CTAs
- * exchange and room for one step's logits z [b][vocab]).  The loop is ONE persistent kernel, greedy or sampling.
+ * exchange and room for one step's logits z [b][vocab]).  The loop is ONE persistent kernel, greedy or sampling, whose CTAs (at most one
+ * per SM) wait for one another: it is launched so that all run at once, and refused with DPARA_ERR_CUDA where the current context's
+ * share of the GPU cannot hold them.
  * All work is queued on `stream`; nothing is allocated.  Errors: INVALID_ARG (null or misaligned pointer,
  * non-positive size), UNSUPPORTED (b > 32, block > 64, rank not a multiple of 64 or > 256, hidden % 64 != 0,
  * vocab % 8 != 0), CUDA.  A device-side wait that runs out sets DPARA_STATUS_TIMEOUT in *status_word. */
