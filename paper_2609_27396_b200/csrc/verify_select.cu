@@ -46,7 +46,8 @@ __device__ __forceinline__ void gather_branch(const uint8_t *__restrict__ reps, 
     const uint4 *s = reinterpret_cast<const uint4 *>(src);
     uint4 *d = reinterpret_cast<uint4 *>(dst);
     const size_t nv = bytes >> 4;
-    // 8 independent 16-byte loads in flight per thread: the copy is one CTA's job, so latency matters
+    // 8 independent 16-byte loads in flight per thread, for the forms in which one CTA copies (greedy, and an early start); where all of a request's
+    // CTAs do, a branch of 1 MB or less is one load a thread
     size_t i = tid;
     for (; i + 7 * (size_t)nthreads < nv; i += 8 * (size_t)nthreads) {
       uint4 v[8];
