@@ -969,7 +969,7 @@ def main():
             out["head"] = {"workload": "T_Head at %s: b=%d, d=%d, hidden=%d, vocab=%d, head rank=%d (greedy)" % (wl.name, sh.batch, sh.block, sh.hidden, sh.vocab, sh.rank),
                            "head_us": th, "lm_head_us": tl, "ar_loop_us": th - tl, "ar_step_us": (th - tl) / sh.block,
                            "sampling": {"head_us": ts, "ar_loop_us": ts - tl, "ar_step_us": (ts - tl) / sh.block,
-                                        "note": "y_i ~ softmax(z_i) from supplied uniforms (temperature 1): per step one GEMM that writes z_i and one inverse-CDF kernel"},
+                                        "note": "y_i ~ softmax(z_i) from supplied uniforms (temperature 1): the same persistent kernel, which draws by inverse CDF"},
                            "lm_head": {"bound": "hbm", "achieved": lmb / (tl * 1e-6) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                                        "frac": lmb / (tl * 1e-6) / 1e9 / peaks["hbm_gbs"], "bytes": lmb,
                                        "tflops": 2.0 * sh.batch * sh.block * sh.hidden * sh.vocab / (tl * 1e-6) / 1e12},
