@@ -61,6 +61,9 @@ __device__ __forceinline__ int slot_of(int cta) { return cta % kCtasPerLane * 32
 constexpr unsigned long long kTagMask = 63;
 constexpr int kTagBits = 6;                        // step / 2 + 1 (two buffers in turn, at most 64 steps)
 constexpr int kBarBytes = 3072;                    // barriers and the reduction scratch
+// Two loops' CTAs never share an SM: each takes all of its tensor memory and waits for its whole grid, so two loops (of calls on two streams) that each
+// hold some SMs' would wait for one another.  The other kernels that take tensor memory need too many registers to come beside one.
+constexpr int kMoreThanHalfAnSM = 116 * 1024;
 
 __device__ __forceinline__ uint32_t head_key(float f) {
   if (f != f) return 0u;                    // NaN below everything
@@ -747,6 +750,7 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   P.bar_off = P.logit_off + P.logit_slots * P.logit_bytes;
   int smem = P.bar_off + kBarBytes + 1024;
   if (smem < P.e_off + 128 * 128 + 1024) smem = P.e_off + 128 * 128 + 1024;   // (a product reads 128 rows of a slab, however many were filled)
+  if (smem < kMoreThanHalfAnSM) smem = kMoreThanHalfAnSM;
   void (*const kernel)(ArParams) = nb == 16 ? ar_kernel<16>(sample, slabs) : ar_kernel<32>(sample, slabs);
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) return DPARA_ERR_CUDA;
   // cooperative: the CTAs wait for one another's words, so every one has to be resident (one per SM fits by construction)

@@ -136,28 +136,30 @@ def test_sampling_of_light_entries(row):
     assert toks.tolist() == [[low, heavy], [heavy, low]]
 
 
-def _inputs_of_a_call(seed, vocab):
-    inp = W.make_head_inputs(W.HeadShape(3, 6, 64, vocab, 256), seed)
+def _inputs_of_a_call(seed, vocab, rank=256):
+    inp = W.make_head_inputs(W.HeadShape(3, 6, 64, vocab, rank), seed)
     t = [dev_bf16(x) for x in (inp.sel_reps, inp.w_lm, inp.ar_w, inp.ar_e)] + [torch.from_numpy(inp.bonus).cuda()]
-    return t, torch.from_numpy(_uniforms(inp.shape, seed)).cuda(), dp.HeadPlan(3, 6, 64, vocab, 256)
+    return t, torch.from_numpy(_uniforms(inp.shape, seed)).cuda(), dp.HeadPlan(3, 6, 64, vocab, rank)
 
 
-def test_sampling_and_greedy_on_two_streams():
-    """Calls on two streams with no order between them: each loop needs all its CTAs on the chip at once, and both get that."""
-    calls = [_inputs_of_a_call(5, 60000), _inputs_of_a_call(6, 40000)]
-    want = [[plan.run(*t, uniforms=x).clone() for x in (u, None)] for t, u, plan in calls]
+@pytest.mark.parametrize("rank,modes", [(256, "sg"), (64, "sg"), (64, "g"), (128, "g")])
+def test_calls_on_two_streams(rank, modes):
+    """Calls on two streams with no order between them: each loop needs all its CTAs and their tensor memory at once, and both get that."""
+    calls = [_inputs_of_a_call(5, 60000, rank), _inputs_of_a_call(6, 40000, rank)]
+    calls = [(t, [u if m == "s" else None for m in modes], plan) for t, u, plan in calls]
+    want = [[plan.run(*t, uniforms=x).clone() for x in us] for t, us, plan in calls]
     torch.cuda.synchronize()
     streams = [torch.cuda.Stream() for _ in calls]
     got = [[], []]
     for _ in range(12):
-        for i, (t, u, plan) in enumerate(calls):
+        for i, (t, us, plan) in enumerate(calls):
             with torch.cuda.stream(streams[i]):
-                got[i].append([plan.run(*t, uniforms=x).clone() for x in (u, None)])
+                got[i].append([plan.run(*t, uniforms=x).clone() for x in us])
     torch.cuda.synchronize()
     for i, (_, _, plan) in enumerate(calls):
         assert plan.status.item() == 0
         for g in got[i]:
-            assert torch.equal(g[0], want[i][0]) and torch.equal(g[1], want[i][1]), i
+            assert all(torch.equal(x, y) for x, y in zip(g, want[i])), i
 
 
 @pytest.mark.parametrize("sampling", [False, True])
