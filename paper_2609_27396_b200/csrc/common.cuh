@@ -38,6 +38,7 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // only behind their wait.  These read ahead of it, and what they read may not be written by the kernel directly in front:
 //   kernel                                  reads ahead of its wait                in front of it, by the order its call launches them
 //   gemm_skinny_kernel with w_ready         weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
+//   chain_kernel                            weights                                RMS norm, attention or the kernel that makes angles
 //   qk_norm_rope_kernel                     context offsets or lengths, angles     the QKV product
 //   append_rows_kernel                      accept_len, ctx_len, capacity, row_start   the projection
 //   gemm_skinny_kernel, the LM head         weights                                head_clear_kernel

@@ -3,12 +3,13 @@
 //   rmsnorm -> QKV GEMM -> per-head RMS norm + rotary embedding -> all-boundary attention ->
 //   O GEMM (+x) -> rmsnorm -> gate/up GEMM with fused SiLU*up -> down GEMM (+h1).
 // The GEMMs and the attention are the tensor-core kernels; the three small kernels here are row-wise
-// and HBM-bound (M rows of a few KB each).
+// and HBM-bound (M rows of a few KB each).  Few rows: everything between two attentions is one launch (chain.cu).
 #include <math.h>
 
 #include <algorithm>
 
 #include "attention_tc.cuh"
+#include "chain.cuh"
 #include "gemm.cuh"
 #include "layer.cuh"
 
@@ -51,6 +52,8 @@ struct AngleJob {
   int rows = 0, per_request = 1, slot_rows = 0, block = 1;     // a request's first slot_rows rows are slots of boundaries of `block`, the others spine rows
   int half = 0;                               // D / 2
   double inv_freq[64] = {};                   // theta^(-2 d / D), d < D / 2, worked out on the host in double precision
+  uint32_t *clear = nullptr;                  // the counters of a call's chains, n_clear of them, to zero
+  int n_clear = 0;
 };
 __device__ __forceinline__ void row_angle(const AngleJob &A, int row, int d, float &c, float &s) {
   const int n = row / A.per_request, rr = row - n * A.per_request;
@@ -78,7 +81,9 @@ __global__ void __launch_bounds__(128) rmsnorm_kernel(const void *__restrict__ x
   if (kAngles && row >= M) {
     pdl_wait();
     pdl_launch_dependents();
-    angle_block(angles, (row - M) * kAnglesPerBlock);
+    if (row == M)
+      for (int k = tid; k < angles.n_clear; k += 128) angles.clear[k] = 0u;
+    if (angles.table) angle_block(angles, (row - M) * kAnglesPerBlock);
     return;
   }
   const size_t base = (size_t)row * H;
@@ -229,8 +234,18 @@ __global__ void __launch_bounds__(128) qk_norm_rope_kernel(const QkParams P) {
 // ------------------------------------------------------------------------------------------------ host
 namespace {
 struct LayerWs {
-  size_t xn, qkv, q, k, v, a, h1, hn, act, angles, attn, total;
+  size_t xn, qkv, q, k, v, a, h1, hn, act, angles, attn, planes, total;
 };
+
+ChainShape block_chain(const dpara_shape *s, const dpara_layer_io *l) {
+  const long M = (long)s->batch * (s->n_boundaries * s->block + (s->spine_queries ? s->n_spine : 0));
+  if (M > kChainRows) return ChainShape{};
+  // A block of which 256 MB of weights and more are read for at most 48 rows is HBM's time either way: chain against kernels of their own 0.97 (40 rows, hidden 4096) to 1.01 there,
+  // 1.03 to 1.18 at all other sizes (rows 16 to 126, hidden 512 to 5120).
+  const double weights = 2.0 * l->hidden * ((double)(2 * s->n_q_heads + 2 * s->n_kv_heads) * s->head_dim + 3.0 * l->intermediate);
+  if (M <= 48 && weights > 256e6) return ChainShape{};
+  return chain_shape((int)M, l->hidden, l->intermediate, s->n_q_heads * s->head_dim, s->n_kv_heads * s->head_dim, s->head_dim);
+}
 
 LayerWs layer_ws_layout(const dpara_shape *s, const dpara_layer_io *l, size_t attn_bytes) {
   const size_t M = (size_t)s->batch * (s->n_boundaries * s->block + (s->spine_queries ? s->n_spine : 0));
@@ -249,9 +264,14 @@ LayerWs layer_ws_layout(const dpara_shape *s, const dpara_layer_io *l, size_t at
   w.act = take(M * I * 2);
   w.angles = take(M * s->head_dim * 4);
   w.attn = take(attn_bytes);
+  const ChainShape chain = block_chain(s, l);
+  w.planes = take(chain.ok ? chain.plane_bytes : 0);
   w.total = o;
   return w;
 }
+
+// A call's counters: of every chain of a stack of n blocks, one in front of each attention and one behind the last.
+size_t counter_bytes(int n_blocks) { return (size_t)(n_blocks + 1) * kChainCounterWords * sizeof(uint32_t); }
 }  // namespace
 
 void layer_workspace_offsets(const dpara_shape *shape, const dpara_layer_io *layer, size_t attn_bytes, size_t out[9]) {
@@ -262,7 +282,7 @@ void layer_workspace_offsets(const dpara_shape *shape, const dpara_layer_io *lay
 
 template <bool kF32In>
 static dpara_status launch_rmsnorm(const void *x, const void *gain, void *out, int M, int H, float eps, const AngleJob &angles, cudaStream_t st) {
-  const int blocks = angles.table ? (angles.rows * angles.half + kAnglesPerBlock - 1) / kAnglesPerBlock : 0;
+  const int angle_blocks = angles.table ? (angles.rows * angles.half + kAnglesPerBlock - 1) / kAnglesPerBlock : 0, blocks = angles.n_clear && !angle_blocks ? 1 : angle_blocks;
   launch_pdl(blocks ? rmsnorm_kernel<kF32In, true> : rmsnorm_kernel<kF32In, false>, dim3(M + blocks), dim3(128), 0, st, x, static_cast<const uint16_t *>(gain), static_cast<uint16_t *>(out), M, H, eps, angles);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
@@ -276,14 +296,118 @@ dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int
 
 size_t layer_workspace_bytes(const dpara_shape *shape, const dpara_layer_io *layer) {
   if (layer->hidden <= 0 || layer->intermediate <= 0) return 0;
-  return layer_ws_layout(shape, layer, 0).total;  // the attention's own scratch is added by the caller
+  return layer_ws_layout(shape, layer, 0).total + align_up(counter_bytes(1), 256);  // the attention's own scratch is added by the caller
 }
 
+// The block's pointers into its workspace
+namespace {
+struct BlockBuffers {
+  uint16_t *xn, *qkv, *q, *k, *v, *a, *hn, *act;
+  float *h1, *angles, *planes;
+  BlockBuffers(uint8_t *lw, const LayerWs &w)
+      : xn(reinterpret_cast<uint16_t *>(lw + w.xn)), qkv(reinterpret_cast<uint16_t *>(lw + w.qkv)), q(reinterpret_cast<uint16_t *>(lw + w.q)),
+        k(reinterpret_cast<uint16_t *>(lw + w.k)), v(reinterpret_cast<uint16_t *>(lw + w.v)), a(reinterpret_cast<uint16_t *>(lw + w.a)),
+        hn(reinterpret_cast<uint16_t *>(lw + w.hn)), act(reinterpret_cast<uint16_t *>(lw + w.act)), h1(reinterpret_cast<float *>(lw + w.h1)),
+        angles(reinterpret_cast<float *>(lw + w.angles)), planes(reinterpret_cast<float *>(lw + w.planes)) {}
+};
+
+bool block_args_ok(const dpara_shape *shape, const dpara_layer_io *L) {
+  return L->x && L->w_qkv && L->w_o && L->w_gate_up && L->w_down && L->y_f32 && L->hidden > 0 && L->intermediate > 0 && (L->qnorm_w == nullptr) == (L->knorm_w == nullptr);
+}
+
+AngleJob angle_job(const dpara_shape *shape, const dpara_attn_io *io, const dpara_layer_io *L, int M, int R, float *table) {
+  AngleJob angles;
+  angles.table = table;
+  angles.ctx_offsets = io->ctx_offsets; angles.ctx_lens = io->ctx_lens;
+  angles.rows = M; angles.per_request = R; angles.slot_rows = shape->n_boundaries * shape->block; angles.block = shape->block;
+  angles.half = shape->head_dim / 2;
+  for (int d = 0; d < shape->head_dim / 2 && d < 64; ++d) angles.inv_freq[d] = pow((double)L->rope_theta, -2.0 * d / shape->head_dim);
+  return angles;
+}
+
+dpara_status block_attention(const dpara_shape *shape, const dpara_attn_io *io, const BlockBuffers &B, void *workspace, int32_t *status_word, cudaStream_t st) {
+  const int Sq = shape->spine_queries ? shape->n_spine : 0, R = shape->n_boundaries * shape->block + Sq;
+  dpara_attn_io aio = *io;
+  aio.q = B.q; aio.k_blk = B.k; aio.v_blk = B.v; aio.out = B.a; aio.out_dtype = DPARA_BF16; aio.out_lse = nullptr;
+  if (Sq) {
+    // the spine's keys/values are the block's own: rows J * Bq .. of each request in the k / v buffers
+    const size_t at = (size_t)shape->n_boundaries * shape->block * shape->n_kv_heads * shape->head_dim;
+    aio.k_spine = B.k + at;
+    aio.v_spine = B.v + at;
+  }
+  return launch_attention(shape, &aio, workspace, status_word, st, Sq ? R : 0, Sq ? R : 0);
+}
+
+// Angles of rows that turn by other frequencies than the blocks before
+__global__ void __launch_bounds__(128) angles_kernel(const __grid_constant__ AngleJob A) {
+  pdl_wait();
+  pdl_launch_dependents();
+  angle_block(A, blockIdx.x * kAnglesPerBlock);
+}
+
+// A stack of n blocks of few rows: the norm of its input, then chains and attentions in turn.  block(l), ctx(l): block l with its input and outputs, and its context.
+// DPARA_ERR_UNSUPPORTED: this device cannot hold a chain's grid at once; the caller's other way gives the same results.
+template <typename Block, typename Ctx>
+dpara_status launch_chained(const dpara_shape *shape, const ChainShape &sh, int n, Block block, Ctx ctx, uint8_t *attn_ws, uint8_t *lw, uint32_t *counters,
+                            int32_t *status_word, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < kNumSM) return DPARA_ERR_UNSUPPORTED;
+  const int Sq = shape->spine_queries ? shape->n_spine : 0, R = shape->n_boundaries * shape->block + Sq, M = shape->batch * R;
+  dpara_layer_io L{}, before = block(0);
+  const BlockBuffers B(lw, layer_ws_layout(shape, &before, 0));
+  const dpara_attn_io first_io = ctx(0);
+  AngleJob start = before.use_rope ? angle_job(shape, &first_io, &before, M, R, B.angles) : AngleJob{};
+  start.clear = counters;
+  start.n_clear = (n + 1) * kChainCounterWords;
+  dpara_status s = launch_rmsnorm<false>(before.x, before.rms1_w, B.xn, M, before.hidden, before.rms_eps, start, st);
+  if (s != DPARA_OK) return s;
+  bool made = before.use_rope;
+  float theta = before.rope_theta;   // what the angles were made for
+  for (int l = 0; l <= n; ++l) {
+    ChainArgs c{};
+    c.M = M; c.hidden = before.hidden; c.intermediate = before.intermediate;
+    c.n_q_heads = shape->n_q_heads; c.n_kv_heads = shape->n_kv_heads; c.head_dim = shape->head_dim;
+    c.xn = B.xn; c.qkv = B.qkv; c.q = B.q; c.k = B.k; c.v = B.v; c.a = B.a; c.h1 = B.h1; c.hn = B.hn; c.act = B.act;
+    c.planes = B.planes; c.counters = counters + (size_t)l * kChainCounterWords;
+    if (l > 0) {
+      c.tail = 1;
+      c.x = before.x; c.w_o = before.w_o; c.rms2_w = before.rms2_w; c.w_gate_up = before.w_gate_up; c.w_down = before.w_down; c.eps2 = before.rms_eps;
+      c.y_f32 = l == n ? before.y_f32 : nullptr;   // (between blocks the bf16 rows are all that is read)
+      c.y_bf16 = before.y_bf16;
+    }
+    if (l < n) {
+      L = block(l);
+      c.head = 1;
+      c.rms1_w = L.rms1_w; c.w_qkv = L.w_qkv; c.qnorm_w = L.qnorm_w; c.knorm_w = L.knorm_w; c.eps1 = L.rms_eps; c.use_norm = L.qnorm_w != nullptr;
+      if (L.use_rope) {
+        c.angles = B.angles;
+        if (!made || theta != L.rope_theta) {
+          const dpara_attn_io io = ctx(l);
+          const AngleJob job = angle_job(shape, &io, &L, M, R, B.angles);
+          launch_pdl(angles_kernel, dim3((M * job.half + kAnglesPerBlock - 1) / kAnglesPerBlock), dim3(128), 0, st, job);
+          DPARA_CHECK_LAUNCH();
+          count_launches(1);
+        }
+        made = true;
+        theta = L.rope_theta;
+      }
+      before = L;
+    }
+    s = launch_chain(sh, c, status_word, st);
+    if (s != DPARA_OK) return s;
+    if (l < n) {
+      const dpara_attn_io io = ctx(l);
+      s = block_attention(shape, &io, B, attn_ws, status_word, st);
+      if (s != DPARA_OK) return s;
+    }
+  }
+  return DPARA_OK;
+}
+}  // namespace
+
 dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, const dpara_layer_io *L, void *workspace,
-                          int32_t *status_word, cudaStream_t st, bool angles_there) {
-  if (!L->x || !L->w_qkv || !L->w_o || !L->w_gate_up || !L->w_down || !L->y_f32) return DPARA_ERR_INVALID_ARG;
-  if (L->hidden <= 0 || L->intermediate <= 0) return DPARA_ERR_INVALID_ARG;
-  if ((L->qnorm_w == nullptr) != (L->knorm_w == nullptr)) return DPARA_ERR_INVALID_ARG;
+                          int32_t *status_word, cudaStream_t st, bool angles_there, bool allow_chain) {
+  if (!block_args_ok(shape, L)) return DPARA_ERR_INVALID_ARG;
   if (shape->boundary_lo != 0 || shape->boundary_hi != shape->n_boundaries) return DPARA_ERR_UNSUPPORTED;
   const int Sq = shape->spine_queries ? shape->n_spine : 0;
   const int R = shape->n_boundaries * shape->block + Sq;  // rows per request: mask slots, then (if they are queries) the spine
@@ -292,14 +416,16 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   const int QD = shape->n_q_heads * D, KD = shape->n_kv_heads * D;
   if (H % 64 || I % 64 || QD % 64 || H % 8) return DPARA_ERR_UNSUPPORTED;
   const size_t attn_ws = attention_workspace_bytes(shape, io->host_ctx_offsets);
-  // layout: [attention scratch (as sized by attention_workspace_bytes)] [layer buffers]
+  // layout: [attention scratch (as sized by attention_workspace_bytes)] [layer buffers] [counters]
   uint8_t *base = static_cast<uint8_t *>(workspace);
   const LayerWs w = layer_ws_layout(shape, L, 0);
   uint8_t *lw = base + attn_ws;
-  uint16_t *xn = reinterpret_cast<uint16_t *>(lw + w.xn), *qkv = reinterpret_cast<uint16_t *>(lw + w.qkv);
-  uint16_t *q = reinterpret_cast<uint16_t *>(lw + w.q), *k = reinterpret_cast<uint16_t *>(lw + w.k), *v = reinterpret_cast<uint16_t *>(lw + w.v);
-  uint16_t *a = reinterpret_cast<uint16_t *>(lw + w.a), *hn = reinterpret_cast<uint16_t *>(lw + w.hn), *act = reinterpret_cast<uint16_t *>(lw + w.act);
-  float *h1 = reinterpret_cast<float *>(lw + w.h1);
+  const ChainShape chain = block_chain(shape, L);
+  if (chain.ok && allow_chain) {
+    const dpara_status cs = launch_chained(shape, chain, 1, [&](int) { return *L; }, [&](int) { return *io; }, base, lw, reinterpret_cast<uint32_t *>(lw + w.total), status_word, st);
+    if (cs != DPARA_ERR_UNSUPPORTED) return cs;
+  }
+  const BlockBuffers B(lw, w);
 
   // Few rows: several CTAs for a row of the row-wise kernel behind the QKV product, so that a warp has one or two heads.  They would each work out
   // their row's angles, so the angles are made once, by blocks behind the rows of this norm.  With a CTA per row they are made there, behind nothing (a table
@@ -308,57 +434,44 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   // lose 0.6 to 0.7 at 429 rows and mostly do not show at the others (-1.1 to 0.7, runs differ by up to 1).
   const int n_heads = shape->n_q_heads + shape->n_kv_heads, per_row = n_heads <= 16 ? 1 : std::min((4 * kNumSM + M - 1) / M, (n_heads + 3) / 4);
   AngleJob angles;
-  if (L->use_rope) {
-    if (per_row > 1) angles.table = reinterpret_cast<float *>(lw + w.angles);
-    angles.ctx_offsets = io->ctx_offsets; angles.ctx_lens = io->ctx_lens;
-    angles.rows = M; angles.per_request = R; angles.slot_rows = shape->n_boundaries * shape->block; angles.block = shape->block;
-    angles.half = D / 2;
-    for (int d = 0; d < D / 2 && d < 64; ++d) angles.inv_freq[d] = pow((double)L->rope_theta, -2.0 * d / D);
-  }
-  dpara_status s = launch_rmsnorm<false>(L->x, L->rms1_w, xn, M, H, L->rms_eps, angles_there ? AngleJob{} : angles, st);
+  if (L->use_rope) angles = angle_job(shape, io, L, M, R, per_row > 1 ? B.angles : nullptr);
+  dpara_status s = launch_rmsnorm<false>(L->x, L->rms1_w, B.xn, M, H, L->rms_eps, angles_there ? AngleJob{} : angles, st);
   if (s != DPARA_OK) return s;
   GemmArgs g{};
-  g.a = xn; g.w = L->w_qkv; g.M = M; g.N = QD + 2 * KD; g.K = H; g.epi = 0; g.out = qkv; g.w_ready = 1;  // the kernels of this chain write no weights
+  g.a = B.xn; g.w = L->w_qkv; g.M = M; g.N = QD + 2 * KD; g.K = H; g.epi = 0; g.out = B.qkv; g.w_ready = 1;  // the kernels of this chain write no weights
   s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
 
   QkParams qp;
-  qp.qkv = qkv; qp.qnorm_w = static_cast<const uint16_t *>(L->qnorm_w); qp.knorm_w = static_cast<const uint16_t *>(L->knorm_w);
-  qp.q = q; qp.k = k; qp.v = v;
+  qp.qkv = B.qkv; qp.qnorm_w = static_cast<const uint16_t *>(L->qnorm_w); qp.knorm_w = static_cast<const uint16_t *>(L->knorm_w);
+  qp.q = B.q; qp.k = B.k; qp.v = B.v;
   qp.Hq = shape->n_q_heads; qp.Hkv = shape->n_kv_heads; qp.D = D;
   qp.use_rope = L->use_rope; qp.use_norm = L->qnorm_w != nullptr; qp.eps = L->rms_eps; qp.angles = angles;
   launch_pdl(per_row > 1 ? qk_norm_rope_kernel<true> : qk_norm_rope_kernel<false>, dim3(M, per_row), dim3(128), D * sizeof(float), st, qp);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
 
-  dpara_attn_io aio = *io;
-  aio.q = q; aio.k_blk = k; aio.v_blk = v; aio.out = a; aio.out_dtype = DPARA_BF16; aio.out_lse = nullptr;
-  if (Sq) {
-    // the spine's keys/values are the block's own: rows J * Bq .. of each request in the k / v buffers
-    aio.k_spine = k + (size_t)shape->n_boundaries * shape->block * KD;
-    aio.v_spine = v + (size_t)shape->n_boundaries * shape->block * KD;
-  }
-  s = launch_attention(shape, &aio, base, status_word, st, Sq ? R : 0, Sq ? R : 0);
+  s = block_attention(shape, io, B, base, status_word, st);
   if (s != DPARA_OK) return s;
 
   g = GemmArgs{};
-  g.a = a; g.w = L->w_o; g.M = M; g.N = H; g.K = QD; g.epi = 1; g.resid = L->x; g.resid_bf16 = 1; g.out = h1; g.w_ready = 1;
+  g.a = B.a; g.w = L->w_o; g.M = M; g.N = H; g.K = QD; g.epi = 1; g.resid = L->x; g.resid_bf16 = 1; g.out = B.h1; g.w_ready = 1;
   s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
-  s = launch_rmsnorm<true>(h1, L->rms2_w, hn, M, H, L->rms_eps, AngleJob{}, st);
+  s = launch_rmsnorm<true>(B.h1, L->rms2_w, B.hn, M, H, L->rms_eps, AngleJob{}, st);
   if (s != DPARA_OK) return s;
   g = GemmArgs{};
-  g.a = hn; g.w = L->w_gate_up; g.M = M; g.N = I; g.K = H; g.epi = 2; g.out = act; g.w_ready = 1;
+  g.a = B.hn; g.w = L->w_gate_up; g.M = M; g.N = I; g.K = H; g.epi = 2; g.out = B.act; g.w_ready = 1;
   s = launch_gemm_tc(g, status_word, st);
   if (s != DPARA_OK) return s;
   g = GemmArgs{};
-  g.a = act; g.w = L->w_down; g.M = M; g.N = H; g.K = I; g.epi = 1; g.resid = h1; g.resid_bf16 = 0; g.out = L->y_f32; g.out_bf16 = L->y_bf16; g.w_ready = 1;
+  g.a = B.act; g.w = L->w_down; g.M = M; g.N = H; g.K = I; g.epi = 1; g.resid = B.h1; g.resid_bf16 = 0; g.out = L->y_f32; g.out_bf16 = L->y_bf16; g.w_ready = 1;
   return launch_gemm_tc(g, status_word, st);
 }
 
 // ------------------------------------------------------------------------------------------------ stack of blocks
 namespace {
-struct BackboneWs { size_t x0, x1, yf, layer, total; };
+struct BackboneWs { size_t x0, x1, yf, layer, counters, total; };
 BackboneWs backbone_ws_layout(const dpara_shape *s, const dpara_backbone_io *bb, size_t attn_bytes) {
   const size_t M = (size_t)s->batch * (s->n_boundaries * s->block + (s->spine_queries ? s->n_spine : 0));
   const size_t H = bb->host_layers[0].hidden;
@@ -369,6 +482,7 @@ BackboneWs backbone_ws_layout(const dpara_shape *s, const dpara_backbone_io *bb,
   w.x0 = take(M * H * 2);
   w.x1 = take(M * H * 2);
   w.yf = take(M * H * 4);
+  w.counters = take(counter_bytes(bb->n_layers));
   w.total = o;
   return w;
 }
@@ -384,17 +498,38 @@ dpara_status launch_backbone(const dpara_shape *shape, const dpara_attn_io *io, 
   uint8_t *base = static_cast<uint8_t *>(workspace);
   void *xbuf[2] = {base + w.x0, base + w.x1};
   const int last = bb->n_layers - 1;
-  for (int l = 0; l <= last; ++l) {
+  // block l, with the tensors between blocks in the workspace, and its context
+  auto block = [&](int l) {
     dpara_layer_io L = bb->host_layers[l];
     L.x = l == 0 ? bb->host_layers[0].x : xbuf[(l - 1) & 1];
     L.y_f32 = l == last ? bb->host_layers[last].y_f32 : reinterpret_cast<float *>(base + w.yf);
     L.y_bf16 = l == last ? bb->host_layers[last].y_bf16 : xbuf[l & 1];
+    return L;
+  };
+  auto context = [&](int l) {
     dpara_attn_io a = *io;
     a.k_ctx = bb->host_k_ctx[l];
     a.v_ctx = bb->host_v_ctx[l];
+    return a;
+  };
+  const ChainShape chain = block_chain(shape, &bb->host_layers[0]);
+  bool chained = chain.ok;
+  for (int l = 0; l <= last && chained; ++l) {
+    const dpara_layer_io L = block(l);
+    chained = block_args_ok(shape, &L);   // (else the block is refused below)
+  }
+  if (chained) {
+    const size_t attn_ws = attention_workspace_bytes(shape, io->host_ctx_offsets);
+    const dpara_status s = launch_chained(shape, chain, last + 1, block, context, base + w.layer, base + w.layer + attn_ws, reinterpret_cast<uint32_t *>(base + w.counters),
+                                          status_word, st);
+    if (s != DPARA_ERR_UNSUPPORTED) return s;
+  }
+  for (int l = 0; l <= last; ++l) {
+    const dpara_layer_io L = block(l);
+    const dpara_attn_io a = context(l);
     // (the rows' positions are the same in every block: one table for all blocks that turn by the same frequencies, made by the first that turns)
     const dpara_layer_io *made = l > 0 && bb->host_layers[l - 1].use_rope && bb->host_layers[l - 1].rope_theta == L.rope_theta ? &bb->host_layers[l - 1] : nullptr;
-    dpara_status s = launch_layer(shape, &a, &L, base + w.layer, status_word, st, made != nullptr);
+    dpara_status s = launch_layer(shape, &a, &L, base + w.layer, status_word, st, made != nullptr, false);
     if (s != DPARA_OK) return s;
   }
   return DPARA_OK;

@@ -23,8 +23,8 @@ dpara_status launch_backbone(const dpara_shape *shape, const dpara_attn_io *io, 
 size_t layer_workspace_bytes(const dpara_shape *shape, const dpara_layer_io *layer);
 // byte offsets of xn, qkv, q, k, v, a, h1, hn, act inside the workspace of a full-layer call
 void layer_workspace_offsets(const dpara_shape *shape, const dpara_layer_io *layer, size_t attn_bytes, size_t out[9]);
-// angles_there: the workspace holds the rotary angles of these rows and this theta
+// angles_there: the workspace holds the rotary angles of these rows and this theta.  allow_chain: few rows may go through chain.cu
 dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, const dpara_layer_io *layer, void *workspace,
-                          int32_t *status_word, cudaStream_t st, bool angles_there = false);
+                          int32_t *status_word, cudaStream_t st, bool angles_there = false, bool allow_chain = true);
 
 }  // namespace dpara
