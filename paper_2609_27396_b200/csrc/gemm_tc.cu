@@ -40,7 +40,7 @@ constexpr int kEpiBytes = kEpiWarps * 16 * 32 * 4;   // 16 activation rows of 32
 struct GemmKernelParams {
   CUtensorMap map_w[kGemmMaxGroups];   // one entry per product of a grouped launch (a plain launch uses entry 0)
   CUtensorMap map_a[kGemmMaxGroups];
-  CUtensorMap map_tail;                // activations in boxes of a tail unit's rows (one product)
+  CUtensorMap map_tail[kGemmMaxGroups];   // activations in boxes of a tail unit's rows
   void *out_g[kGemmMaxGroups];
   int n_groups;
   int M, N, K;
@@ -59,8 +59,8 @@ struct GemmKernelParams {
 
 
 
-// A unit of work: a tile of one of the products, one part of its K range (the parts of a tile are neighbours), or (kTail, one product) some of its
-// activation rows.
+// A unit of work: a tile of one of the products, one part of its K range (the parts of a tile are neighbours), or (kTail) some of the activation rows of
+// such a part.
 template <bool kTail>
 struct Unit {
   int grp, tile, ks, kb0, kb1, row0, nt, rows;
@@ -73,19 +73,13 @@ struct Unit {
       sub = unit - P.main_units - k * P.tail_split;
       unit = P.main_units + k;
     }
-    if (kTail) {
-      grp = ks = kb0 = 0;
-      kb1 = nkb;
-      tile = unit;
-    } else {
-      const int per_group = P.t_tiles * P.n_tiles * P.split_k;
-      grp = unit / per_group;
-      unit -= grp * per_group;
-      tile = unit / P.split_k;
-      ks = unit - tile * P.split_k;
-      kb0 = ks * nkb / P.split_k;
-      kb1 = (ks + 1) * nkb / P.split_k;
-    }
+    const int per_group = P.t_tiles * P.n_tiles * P.split_k;
+    grp = unit / per_group;
+    unit -= grp * per_group;
+    tile = unit / P.split_k;
+    ks = unit - tile * P.split_k;
+    kb0 = ks * nkb / P.split_k;
+    kb1 = (ks + 1) * nkb / P.split_k;
     const int first = tile % P.t_tiles * P.nt;
     nt = tail ? P.nt_tail : P.nt;
     row0 = tail ? first + sub * P.nt_tail : first;
@@ -271,7 +265,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
       const int grp = w.grp, n_tile = w.tile / P.t_tiles;
       const int wrow = P.epi == 2 ? n_tile * 128 + rank * 64 : n_tile * 256 + rank * 128;
       const int arow = w.row0 + rank * (w.nt / 2);
-      const CUtensorMap *map_w = &P.map_w[grp], *map_a = w.tail ? &P.map_tail : &P.map_a[grp];
+      const CUtensorMap *map_w = &P.map_w[grp], *map_a = w.tail ? &P.map_tail[grp] : &P.map_a[grp];
       const bool swiglu = P.epi == 2;
 #pragma unroll 1
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
@@ -416,11 +410,12 @@ dpara_status gemm_route(const GemmArgs &g, GemmRoute &r) {
 // tiles, 109 products of 129 to 1152 rows with 1 to 24 tiles left of 74, stores and SwiGLU, weights from HBM: 1.057x (geometric mean), faster by
 // more than the spread in all but three, slower by more than it in none.  1.13 behind one round of tiles, 1.07 behind two or three, 1.035 behind four to nine (the pairs drift
 // apart, and the whole tiles of a last round start early on some); 1.068 with 1 to 8 tiles left, 1.058 with 9 to 16, 1.044 with 17 to 24.  For
-// instance 207 x 23112 x 1088 22.0 -> 19.7 us, 498 x 9920 x 2752 SwiGLU 54.9 -> 48.6, 1014 x 14784 x 4544 SwiGLU 196 -> 190.
+// instance 207 x 23112 x 1088 22.0 -> 19.7 us, 498 x 9920 x 2752 SwiGLU 54.9 -> 48.6, 1014 x 14784 x 4544 SwiGLU 196 -> 190.  Launches of several products or parts
+// of K too: the append of five layers, 256 rows (40 tiles in four parts, 12 units behind two rounds) 48.1 -> 45.5, the same bits.
 static bool tail_plan(const GemmArgs &g, const GemmRoute &r, GemmKernelParams &P) {
   const long units = (long)r.pair.t_tiles * r.n_all;
   const int left = (int)(units % r.most), at_once = r.most * 13 / 20;   // 48 of 74 pairs
-  if (g.n_groups > 1 || g.split_k > 1 || units < r.most || left == 0 || 2 * left > at_once) return false;
+  if (units < r.most || left == 0 || 2 * left > at_once) return false;
   P.nt_tail = (r.pair.nt / (at_once / left) + 15) / 16 * 16;
   if (P.nt_tail < 32) P.nt_tail = 32;
   if (P.nt_tail >= r.pair.nt) return false;
@@ -443,13 +438,13 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
   P.n_tiles = route.n_tiles;
   P.t_tiles = route.pair.t_tiles; P.nt = route.pair.nt;
   const bool tail = tail_plan(g, route, P);
-  if (tail && !make_tmap_bf16_2d(&P.map_tail, g.a, g.K, g.M, (uint64_t)g.K * 2, kBK, P.nt_tail / 2)) return DPARA_ERR_CUDA;
   for (int gi = 0; gi < P.n_groups; ++gi) {
     const void *a = gi ? g.a_g[gi] : g.a, *w = gi ? g.w_g[gi] : g.w;
     void *o = gi ? g.out_g[gi] : g.out;
     if (!a || !w || !o || !aligned16(a) || !aligned16(w) || !aligned16(o)) return DPARA_ERR_INVALID_ARG;
     if (!make_tmap_bf16_2d(&P.map_w[gi], w, g.K, w_rows, (uint64_t)g.K * 2, kBK, g.epi == 2 ? kRows / 2 : kRows)) return DPARA_ERR_CUDA;
     if (!make_tmap_bf16_2d(&P.map_a[gi], a, g.K, g.M, (uint64_t)g.K * 2, kBK, P.nt / 2)) return DPARA_ERR_CUDA;
+    if (tail && !make_tmap_bf16_2d(&P.map_tail[gi], a, g.K, g.M, (uint64_t)g.K * 2, kBK, P.nt_tail / 2)) return DPARA_ERR_CUDA;
     P.out_g[gi] = o;
   }
   P.M = g.M; P.N = g.N; P.K = g.K; P.epi = g.epi; P.up_row_offset = g.N;
