@@ -37,11 +37,11 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // in FRONT of it is complete: ahead of its own pdl_wait() it can race with that one kernel and with nothing else.  Most kernels touch global memory
 // only behind their wait.  These read ahead of it, and what they read may not be written by the kernel directly in front:
 //   kernel                                  reads ahead of its wait                in front of it, by the order its call launches them
-//   gemm_skinny_kernel with w_ready         weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
+//   gemm_skinny_, gemm_pair_kernel, w_ready  weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
 //   chain_kernel                            weights                                RMS norm, attention or the kernel that makes angles
 //   qk_norm_rope_kernel                     context offsets or lengths, angles     the QKV product
 //   append_rows_kernel                      accept_len, ctx_len, capacity, row_start   the projection
-//   gemm_skinny_kernel, the LM head         weights                                head_clear_kernel
+//   the LM head's product                   weights                                head_clear_kernel
 //   ar_head_kernel                          W of the head loop                     the LM head's product
 //   verify kernels, early-start form        all but the representations; they also use their workspace   what the caller queued: the flag is its promise
 // Moving a trigger ahead of a wait, or a kernel that writes one of these directly in front of its reader, makes a race.

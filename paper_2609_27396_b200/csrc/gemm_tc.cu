@@ -49,6 +49,7 @@ struct GemmKernelParams {
   int nt, t_tiles, n_tiles;            // activation rows per tile; tiles of one product
   int main_units, tail_split, nt_tail; // kTail: tiles from main_units on are cut into tail_split units of nt_tail activation rows
   int stages;
+  int w_ready;                         // the first unit's weights may be read ahead of the wait for the kernel in front
   int split_k;                         // > 1 (fp32 store only): the K range in split_k parts, part s writes plane s of [split_k][M][N] partial sums
   const void *resid;
   int resid_bf16;
@@ -244,8 +245,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
   cluster_sync_all();  // both CTAs' barriers exist before anything signals across the pair
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-  pdl_wait();  // nothing above touches global memory: the set-up overlaps the tail of the kernel before
-  pdl_launch_dependents();
+  // (nothing above touches global memory: the set-up overlaps the tail of the kernel before)
 
   // Warps 4 and 5: the whole warp walks the loop and waits, one lane issues, and the barrier of the next stage is asked before this
   // stage's instructions go out (a wait inside a one-lane branch costs two to three times as many clocks, and the tensor pipe
@@ -255,31 +255,61 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
       prefetch_tensormap(&P.map_w[gi]);
       prefetch_tensormap(&P.map_a[gi]);
     }
-    int stage = 0;
-    uint32_t ph = 0;
+    const bool swiglu = P.epi == 2;
+    // (worked out once per unit: a division per stage is what the loop has no time for)
+    struct Source {
+      const CUtensorMap *map_w, *map_a;
+      int wrow, arow;
+      uint32_t tx;
+    };
+    auto source = [&](const Unit<kTail> &w) {
+      const int n_tile = w.tile / P.t_tiles;
+      return Source{&P.map_w[w.grp], w.tail ? &P.map_tail[w.grp] : &P.map_a[w.grp], swiglu ? n_tile * 128 + rank * 64 : n_tile * 256 + rank * 128,
+                    w.row0 + rank * (w.nt / 2), 2u * (uint32_t)(kWBytes + w.nt * 64)};
+    };
+    auto load_w = [&](const Source &s, int kb, int stage) {
+      uint8_t *sw = smem + stage * stage_bytes;
+      if (rank == 0) mbar_arrive_expect_tx(full + stage, s.tx);
+      tma_load_2d_pair(sw, s.map_w, full + stage, kb * kBK, s.wrow);
+      if (swiglu) tma_load_2d_pair(sw + kWBytes / 2, s.map_w, full + stage, kb * kBK, P.up_row_offset + s.wrow);
+    };
+    auto load_a = [&](const Source &s, int kb, int stage) { tma_load_2d_pair(smem + stage * stage_bytes + kWBytes, s.map_a, full + stage, kb * kBK, s.arow); };
+    // The weights of the first unit's first stages ahead of the wait, where nothing in front of this kernel writes them (us, without -> with: round of four requests
+    // 664.5 -> 660; four blocks of 280 rows of hidden 704 360 -> 353, a block of 378 rows of hidden 1600 76.1 -> 75.4; large products as before).
+    int early = 0;
+    if (P.w_ready) {
+      const Unit<kTail> first(P, pair, nkb);
+      const Source s = source(first);
+      early = min(P.stages, first.kb1 - first.kb0);
+      if (elect_one())
+#pragma unroll 1
+        for (int i = 0; i < early; ++i) load_w(s, first.kb0 + i, i);
+      __syncwarp();
+      pdl_wait();
+      if (elect_one())
+#pragma unroll 1
+        for (int i = 0; i < early; ++i) load_a(s, first.kb0 + i, i);
+      __syncwarp();
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    int stage = early == P.stages ? 0 : early, done = early;
+    uint32_t ph = early == P.stages ? 1u : 0u;
     bool ok = true, there = false;
     // (tile id = weight tile * t_tiles + activation tile: the pairs running together cover all activation rows of a few weight tiles)
-    for (int unit = pair; unit < units && ok; unit += pairs) {
+    for (int unit = pair; unit < units && ok; unit += pairs, done = 0) {
       const Unit<kTail> w(P, unit, nkb);
-      const uint32_t tx = 2u * (uint32_t)(kWBytes + w.nt * 64);
-      const int grp = w.grp, n_tile = w.tile / P.t_tiles;
-      const int wrow = P.epi == 2 ? n_tile * 128 + rank * 64 : n_tile * 256 + rank * 128;
-      const int arow = w.row0 + rank * (w.nt / 2);
-      const CUtensorMap *map_w = &P.map_w[grp], *map_a = w.tail ? &P.map_tail[grp] : &P.map_a[grp];
-      const bool swiglu = P.epi == 2;
+      const Source s = source(w);
 #pragma unroll 1
-      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+      for (int kb = w.kb0 + done; kb < w.kb1; ++kb) {
         if (!__all_sync(0xffffffffu, there)) ok = __all_sync(0xffffffffu, mbar_wait(empty + stage, ph ^ 1u, abort_flag, 2));
         if (!ok) break;
         const int cur = stage;
         if (++stage == P.stages) { stage = 0; ph ^= 1u; }
         there = mbar_test(empty + stage, ph ^ 1u);
         if (elect_one()) {
-          uint8_t *sw = smem + cur * stage_bytes;
-          if (rank == 0) mbar_arrive_expect_tx(full + cur, tx);
-          tma_load_2d_pair(sw, map_w, full + cur, kb * kBK, wrow);
-          if (swiglu) tma_load_2d_pair(sw + kWBytes / 2, map_w, full + cur, kb * kBK, P.up_row_offset + wrow);
-          tma_load_2d_pair(sw + kWBytes, map_a, full + cur, kb * kBK, arow);
+          load_w(s, kb, cur);
+          load_a(s, kb, cur);
         }
         __syncwarp();
       }
@@ -319,6 +349,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
       }
     }
   } else {
+    pdl_wait();
     const int quarter = warp & 3, turn = warp >= 4;   // the TMEM lanes a warp may read; which of the two warps that may
     int k = 0;
     bool live = true;
@@ -447,6 +478,7 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
     if (tail && !make_tmap_bf16_2d(&P.map_tail[gi], a, g.K, g.M, (uint64_t)g.K * 2, kBK, P.nt_tail / 2)) return DPARA_ERR_CUDA;
     P.out_g[gi] = o;
   }
+  P.w_ready = g.w_ready && P.split_k == 1;   // (split: 192 rows, three layers of 2048 x 4096: an append of 24.6 us 25.0, the norm in front reads slower)
   P.M = g.M; P.N = g.N; P.K = g.K; P.epi = g.epi; P.up_row_offset = g.N;
   P.resid = g.resid; P.resid_bf16 = g.resid_bf16; P.out_bf16 = g.out_bf16; P.status = status;
   P.perm_block = g.epi == 3 ? g.perm_block : 0; P.perm_b = g.perm_b;
