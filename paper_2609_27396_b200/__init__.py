@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Optional, Sequence
 
 import torch
@@ -169,6 +170,21 @@ def _host_offsets(ctx_offsets: Sequence[int]):
     return arr
 
 
+# The structs of the small calls, packed in one go: a ctypes structure made field by field is a microsecond of a call that is bound by its host time.
+_pack_attn_io = struct.Struct("@10Pi4x3P").pack
+assert struct.calcsize("@10Pi4x3P") == C.sizeof(AttnIO)
+_draft_packed = C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_char_p, C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)(
+    ("dpara_draft_all_boundaries", lib))
+
+
+def _addr(t: Optional[torch.Tensor]) -> int:
+    if t is None:
+        return 0
+    if not t.is_contiguous():
+        raise ValueError("dpara: tensors must be contiguous")
+    return t.data_ptr()
+
+
 class DraftPlan:
     """Fixed-address buffers for repeated draft calls on one shape (shape struct, host and device copies
     of the context offsets, workspace, status word).  Building the plan allocates; calling it does not."""
@@ -208,14 +224,12 @@ class DraftPlan:
 
     def __call__(self, *, q=None, k_ctx=None, v_ctx=None, k_spine=None, v_spine=None, k_blk=None, v_blk=None,
                  out=None, out_lse=None, stream=None) -> None:
-        io = AttnIO(_ptr(q), _ptr(k_ctx), _ptr(v_ctx), self.dev_off.data_ptr(), C.addressof(self.host_off),
-                    _ptr(k_spine), _ptr(v_spine), _ptr(k_blk), _ptr(v_blk), _ptr(out),
-                    F32 if (out is not None and out.dtype == torch.float32) else BF16, _ptr(out_lse),
-                    _ptr(self.dev_lens), C.addressof(self.host_lens) if self.host_lens is not None else None)
-        rc = lib.dpara_draft_all_boundaries(C.byref(self.shape), C.byref(io),
-                                            C.byref(self.layer) if self.layer is not None else None,
-                                            self.workspace.data_ptr(), self.workspace.numel(), self.status.data_ptr(),
-                                            _stream_ptr(stream))
+        io = _pack_attn_io(_addr(q), _addr(k_ctx), _addr(v_ctx), self.dev_off.data_ptr(), C.addressof(self.host_off),
+                           _addr(k_spine), _addr(v_spine), _addr(k_blk), _addr(v_blk), _addr(out),
+                           F32 if (out is not None and out.dtype == torch.float32) else BF16, _addr(out_lse),
+                           _addr(self.dev_lens), C.addressof(self.host_lens) if self.host_lens is not None else 0)
+        rc = _draft_packed(C.addressof(self.shape), io, C.addressof(self.layer) if self.layer is not None else None,
+                           self.workspace.data_ptr(), self.workspace.numel(), self.status.data_ptr(), _stream_ptr(stream))
         if rc != OK:
             raise DparaError(rc)
 

@@ -1,5 +1,6 @@
 // C-ABI entry points of the draft call: argument validation, workspace sizing, kernel selection by shape.
 #include "attention_params.cuh"
+#include "attention_tc.cuh"
 #include "layer.cuh"
 
 #include <atomic>
@@ -89,14 +90,17 @@ extern "C" dpara_status dpara_draft_all_boundaries(const dpara_shape *shape, con
       !aligned16(io->q) || !aligned16(io->k_blk) || !aligned16(io->v_blk) || !aligned16(io->out))
     return DPARA_ERR_INVALID_ARG;
   if (layer && !layer_aligned(*layer, true, true)) return DPARA_ERR_INVALID_ARG;
-  const size_t need = dpara_draft_workspace_bytes(shape, io->host_ctx_offsets, layer, layer != nullptr);
+  // (one plan for the scratch and the launch: of the ~5 us that a small call spends in here planning twice was one)
+  const TcPlan plan = plan_attention_tc(shape, io->host_ctx_offsets, nullptr);
+  size_t need = attention_workspace_bytes(plan);
+  if (layer) need += layer_workspace_bytes(shape, layer);
   if (need > 0 && (!workspace || workspace_bytes < need || !aligned16(workspace))) return DPARA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
   if (layer) return launch_layer(shape, io, layer, workspace, status_word, st);
 
   if (!io->q || !io->out) return DPARA_ERR_INVALID_ARG;
-  return launch_attention(shape, io, workspace, status_word, st);
+  return launch_attention(shape, io, workspace, status_word, st, 0, 0, io->host_ctx_lens ? nullptr : &plan);
 }
 
 extern "C" size_t dpara_backbone_workspace_bytes(const dpara_shape *shape, const int64_t *host_ctx_offsets, const dpara_backbone_io *bb) {

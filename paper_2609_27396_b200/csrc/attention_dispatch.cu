@@ -30,19 +30,17 @@ void fill_attn_params(AttnParams &P, const dpara_shape *s, const dpara_attn_io *
   P.status_word = status_word;
 }
 
-size_t attention_workspace_bytes(const dpara_shape *shape, const int64_t *host_off) {
-  TcPlan plan = plan_attention_tc(shape, host_off, nullptr);
-  return plan.eligible ? align_up(plan.workspace_max_bytes, 256) : 0;
-}
+size_t attention_workspace_bytes(const TcPlan &plan) { return plan.eligible ? align_up(plan.workspace_max_bytes, 256) : 0; }
+size_t attention_workspace_bytes(const dpara_shape *shape, const int64_t *host_off) { return attention_workspace_bytes(plan_attention_tc(shape, host_off, nullptr)); }
 
 dpara_status launch_attention(const dpara_shape *shape, const dpara_attn_io *io, void *workspace, int32_t *status_word,
-                              cudaStream_t st, int blk_req_rows, int spine_req_rows) {
+                              cudaStream_t st, int blk_req_rows, int spine_req_rows, const TcPlan *ready) {
   AttnParams P;
   fill_attn_params(P, shape, io, status_word);
   if (blk_req_rows) P.blk_req_rows = blk_req_rows;
   if (spine_req_rows) P.spine_req_rows = spine_req_rows;
   if (P.hi <= P.lo) return DPARA_OK;
-  TcPlan plan = plan_attention_tc(shape, io->host_ctx_offsets, io->host_ctx_lens);
+  const TcPlan plan = ready ? *ready : plan_attention_tc(shape, io->host_ctx_offsets, io->host_ctx_lens);
   if (!plan.eligible) return DPARA_ERR_UNSUPPORTED;  // group size > 16, block > 64, spine > 64, or more than 2^31 rows
   return launch_attention_tc(P, plan, io->host_ctx_offsets, io->host_ctx_lens, workspace, st);
 }

@@ -18,6 +18,7 @@ struct TcPlan {
 };
 
 // host_ctx_lens may be null (request n fills rows host_ctx_offsets[n] .. host_ctx_offsets[n + 1])
+size_t attention_workspace_bytes(const TcPlan &plan);   // a call's scratch (of a plan without host_ctx_lens)
 TcPlan plan_attention_tc(const dpara_shape *s, const int64_t *host_ctx_offsets, const int64_t *host_ctx_lens);
 dpara_status launch_attention_tc(const AttnParams &A, const TcPlan &plan, const int64_t *host_ctx_offsets,
                                  const int64_t *host_ctx_lens, void *workspace, cudaStream_t st);

@@ -8,8 +8,10 @@ namespace dpara {
 size_t attention_workspace_bytes(const dpara_shape *shape, const int64_t *host_ctx_offsets);
 // blk_req_rows / spine_req_rows: rows from one request's block (spine) keys to the next request's when they differ from
 // J * Bq (S), e.g. when both live in one buffer of J * Bq + S rows per request; 0 = the default
+// plan: plan_attention_tc of this shape and these offsets and lengths, where the caller has it
+struct TcPlan;
 dpara_status launch_attention(const dpara_shape *shape, const dpara_attn_io *io, void *workspace, int32_t *status_word,
-                              cudaStream_t st, int blk_req_rows = 0, int spine_req_rows = 0);
+                              cudaStream_t st, int blk_req_rows = 0, int spine_req_rows = 0, const TcPlan *plan = nullptr);
 
 // out[row] = bf16(x[row] / sqrt(mean(x^2) + eps) * gain) for M rows of H bf16 elements (gain may be null)
 dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st);
