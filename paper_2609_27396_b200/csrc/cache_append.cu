@@ -27,10 +27,11 @@ struct AppendParams {
   // per layer of the launch (blockIdx.y)
   const uint16_t *knorm_w[kGemmMaxGroups];  // [D] or null
   uint16_t *k_cache[kGemmMaxGroups], *v_cache[kGemmMaxGroups];
-  const int64_t *row_start, *capacity, *ctx_len;
+  const int64_t *row_start, *capacity, *ctx_len;   // (ctx_len: the copy of the old lengths)
   const int32_t *accept_len;
   int32_t *status_word;
-  int J, Hkv, D, use_rope;
+  int64_t *new_len;         // the caller's lengths, to be written by the call's last launch (null: not this one)
+  int b, J, Hkv, D, use_rope;
   float eps, theta;
   double inv_freq[64];      // theta^(-2 d / D), d < D / 2, worked out on the host in double precision
 };
@@ -64,6 +65,14 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
   const size_t row = (size_t)((fits ? P.row_start[n] : 0) + L + i);
   pdl_wait();
   pdl_launch_dependents();
+  // L_n += r_n + 1 for the requests that fitted: the old lengths are read from the copy that the call's first kernel made, so nobody is waited for (a kernel of its own
+  // behind this one took 2 us of an append; a ticket, the last CTA writing, as much).
+  if (P.new_len && blockIdx.x == 0 && g == 0)
+    for (int m = tid; m < P.b; m += 128) {
+      const int rm = P.accept_len[m];
+      const long long Lm = P.ctx_len[m];
+      if (rm >= 0 && rm < P.J && Lm + rm + 1 <= P.capacity[m]) P.new_len[m] = Lm + rm + 1;
+    }
   if (!fits) {  // does not fit (or no valid outcome): the request is left alone
     if (i == 0 && g == 0 && tid == 0 && P.status_word) atomicOr(reinterpret_cast<unsigned int *>(P.status_word), DPARA_STATUS_CACHE_FULL);
     return;
@@ -181,17 +190,6 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
   }
 }
 
-// After every layer has read the old lengths: L_n += r_n + 1 for the requests that fitted.
-__global__ void append_commit_kernel(int64_t *ctx_len, const int64_t *capacity, const int32_t *accept_len, int b, int J) {
-  pdl_wait();
-  pdl_launch_dependents();
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < b; n += gridDim.x * blockDim.x) {
-    const int r = accept_len[n];
-    const long long L = ctx_len[n];
-    if (r >= 0 && r < J && L + r + 1 <= capacity[n]) ctx_len[n] = L + r + 1;
-  }
-}
-
 // Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores (at most 128 rows: the
 // kernel for few rows takes all layers at once, one chain of sums over K each; the whole call, 8 rows, five layers of 2048 x 4096: 192 us with a
 // product a layer, 38 now).  The parts are chosen to minimise
@@ -232,6 +230,8 @@ static int cache_norm_slots(const dpara_cache_io *io) {
   return slots;
 }
 
+static size_t lengths_bytes(const dpara_cache_io *io) { return align_up((size_t)io->batch * sizeof(int64_t), 256); }
+
 size_t cache_append_workspace_bytes(const dpara_cache_io *io) {
   const size_t M = (size_t)io->batch * io->n_rows, N = (size_t)2 * io->n_kv_heads * io->head_dim;
   int group, parts;
@@ -244,7 +244,7 @@ size_t cache_append_workspace_bytes(const dpara_cache_io *io) {
     cache_group_plan(io, rest, &group, &parts);
     rows = std::max(rows, rows_bytes(group, parts));
   }
-  return (size_t)cache_norm_slots(io) * align_up(M * io->feat_dim * 2, 256) + rows;
+  return (size_t)cache_norm_slots(io) * align_up(M * io->feat_dim * 2, 256) + rows + lengths_bytes(io);
 }
 
 dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int32_t *status_word, cudaStream_t st) {
@@ -255,10 +255,12 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
   const int slots = cache_norm_slots(io);
   uint8_t *ws = static_cast<uint8_t *>(workspace);
   uint16_t *kv = reinterpret_cast<uint16_t *>(ws + (size_t)slots * xn_bytes);
+  int64_t *old_len = reinterpret_cast<int64_t *>(ws + cache_append_workspace_bytes(io) - lengths_bytes(io));   // copied by the first norm
   AppendParams P;
   memset(&P, 0, sizeof(P));
-  P.row_start = io->row_start; P.capacity = io->capacity; P.ctx_len = io->ctx_len; P.accept_len = io->accept_len;
+  P.row_start = io->row_start; P.capacity = io->capacity; P.ctx_len = old_len; P.accept_len = io->accept_len;
   P.status_word = status_word;
+  P.b = io->batch;
   P.J = io->n_rows; P.Hkv = io->n_kv_heads; P.D = io->head_dim; P.use_rope = io->use_rope;
   P.eps = io->rms_eps; P.theta = io->rope_theta;
   for (int d = 0; d < io->head_dim / 2 && d < 64; ++d) P.inv_freq[d] = pow((double)io->rope_theta, -2.0 * d / io->head_dim);
@@ -275,7 +277,7 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
       const void *gain = io->host_norm_w ? io->host_norm_w[l] : nullptr;
       if (l == 0 || gain != prev_gain) {  // layers that share the input norm share the normalised rows
         ++slot;
-        dpara_status s = launch_rmsnorm_bf16(io->features, gain, ws + (size_t)slot * xn_bytes, M, F, io->rms_eps, st);
+        dpara_status s = launch_rmsnorm_bf16(io->features, gain, ws + (size_t)slot * xn_bytes, M, F, io->rms_eps, st, l == 0 ? io->ctx_len : nullptr, old_len, io->batch);
         if (s != DPARA_OK) return s;
         prev_gain = gain;
       }
@@ -290,15 +292,13 @@ dpara_status launch_cache_append(const dpara_cache_io *io, void *workspace, int3
     if (s != DPARA_OK) return s;
     P.kv = kv;
     P.kv_parts = reinterpret_cast<const float *>(kv);
+    P.new_len = l0 + group == io->n_layers ? io->ctx_len : nullptr;
     void (*const rows)(AppendParams) = append_rows_of(parts);
     launch_pdl(rows, dim3(M, group), dim3(128), io->head_dim * sizeof(float), st, P);
     DPARA_CHECK_LAUNCH();
     count_launches(1);
     l0 += group;
   }
-  launch_pdl(append_commit_kernel, dim3((io->batch + 127) / 128), dim3(128), 0, st, io->ctx_len, io->capacity, io->accept_len, io->batch, io->n_rows);
-  DPARA_CHECK_LAUNCH();
-  count_launches(1);
   return DPARA_OK;
 }
 

@@ -40,7 +40,7 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 //   gemm_skinny_, gemm_pair_kernel, w_ready  weights                                RMS norm, attention or a product (block); RMS norm or append_rows (append)
 //   chain_kernel                            weights                                RMS norm, attention or the kernel that makes angles
 //   qk_norm_rope_kernel                     context offsets or lengths, angles     the QKV product
-//   append_rows_kernel                      accept_len, ctx_len, capacity, row_start   the projection
+//   append_rows_kernel                      accept_len, old lengths, capacity, row_start   the projection
 //   the LM head's product                   weights                                head_clear_kernel
 //   ar_head_kernel                          W of the head loop                     the LM head's product
 //   verify kernels, early-start form        all but the representations; they also use their workspace   what the caller queued: the flag is its promise

@@ -54,6 +54,9 @@ struct AngleJob {
   double inv_freq[64] = {};                   // theta^(-2 d / D), d < D / 2, worked out on the host in double precision
   uint32_t *clear = nullptr;                  // the counters of a call's chains, n_clear of them, to zero
   int n_clear = 0;
+  const int64_t *copy = nullptr;              // lengths to be kept as they were, n_copy of them
+  int64_t *copy_to = nullptr;
+  int n_copy = 0;
 };
 __device__ __forceinline__ void row_angle(const AngleJob &A, int row, int d, float &c, float &s) {
   const int n = row / A.per_request, rr = row - n * A.per_request;
@@ -81,8 +84,10 @@ __global__ void __launch_bounds__(128) rmsnorm_kernel(const void *__restrict__ x
   if (kAngles && row >= M) {
     pdl_wait();
     pdl_launch_dependents();
-    if (row == M)
+    if (row == M) {
       for (int k = tid; k < angles.n_clear; k += 128) angles.clear[k] = 0u;
+      for (int k = tid; k < angles.n_copy; k += 128) angles.copy_to[k] = angles.copy[k];
+    }
     if (angles.table) angle_block(angles, (row - M) * kAnglesPerBlock);
     return;
   }
@@ -282,16 +287,20 @@ void layer_workspace_offsets(const dpara_shape *shape, const dpara_layer_io *lay
 
 template <bool kF32In>
 static dpara_status launch_rmsnorm(const void *x, const void *gain, void *out, int M, int H, float eps, const AngleJob &angles, cudaStream_t st) {
-  const int angle_blocks = angles.table ? (angles.rows * angles.half + kAnglesPerBlock - 1) / kAnglesPerBlock : 0, blocks = angles.n_clear && !angle_blocks ? 1 : angle_blocks;
+  const int angle_blocks = angles.table ? (angles.rows * angles.half + kAnglesPerBlock - 1) / kAnglesPerBlock : 0, blocks = (angles.n_clear || angles.n_copy) && !angle_blocks ? 1 : angle_blocks;
   launch_pdl(blocks ? rmsnorm_kernel<kF32In, true> : rmsnorm_kernel<kF32In, false>, dim3(M + blocks), dim3(128), 0, st, x, static_cast<const uint16_t *>(gain), static_cast<uint16_t *>(out), M, H, eps, angles);
   DPARA_CHECK_LAUNCH();
   count_launches(1);
   return DPARA_OK;
 }
 
-dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st) {
+dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st, const int64_t *copy, int64_t *to, int n_copy) {
   if (H % 8) return DPARA_ERR_UNSUPPORTED;
-  return launch_rmsnorm<false>(x, gain, out, M, H, eps, AngleJob{}, st);
+  AngleJob job;
+  job.copy = copy;
+  job.copy_to = to;
+  job.n_copy = copy ? n_copy : 0;
+  return launch_rmsnorm<false>(x, gain, out, M, H, eps, job, st);
 }
 
 size_t layer_workspace_bytes(const dpara_shape *shape, const dpara_layer_io *layer) {

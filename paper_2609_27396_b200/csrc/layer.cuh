@@ -14,7 +14,8 @@ dpara_status launch_attention(const dpara_shape *shape, const dpara_attn_io *io,
                               cudaStream_t st, int blk_req_rows = 0, int spine_req_rows = 0, const TcPlan *plan = nullptr);
 
 // out[row] = bf16(x[row] / sqrt(mean(x^2) + eps) * gain) for M rows of H bf16 elements (gain may be null)
-dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st);
+// (and copies n_copy lengths)
+dpara_status launch_rmsnorm_bf16(const void *x, const void *gain, void *out, int M, int H, float eps, cudaStream_t st, const int64_t *copy = nullptr, int64_t *to = nullptr, int n_copy = 0);
 
 // a stack of blocks (each reads the previous one's bf16 output and its own context cache)
 size_t backbone_workspace_bytes(const dpara_shape *shape, const int64_t *host_ctx_offsets, const dpara_backbone_io *bb);
