@@ -14,7 +14,7 @@
 // Warps: 0-15 sums, row steps (short chains of dependent instructions: eight warps took twice as long); 16 weights; 17 activations; 18 and 19 products (weights
 // as the rows, M = 128; activation rows as the columns).  A stage is two operands of weights, gate and up of one slab of K or two slabs in turn, and each of the two warps has one
 // of them and an accumulator of its own (two slabs: the sums are added at the end): a single warp took ~750 clocks per stage, two take 500 to 700.
-// Measured, whole stacks of blocks, kernels of their own -> this (us): five blocks of 72 rows, hidden 4096 (385 MB of weights each) 591 -> 576; three blocks of 64 to 128 rows: hidden 512
+// Measured, whole stacks of blocks, kernels of their own -> this (us): five blocks of 72 rows, hidden 4096 (385 MB of weights each) 592 -> 582; three blocks of 64 to 128 rows: hidden 512
 // 151 -> 130 and 169 -> 144, 1024 184 -> 172 and 193 -> 179, 2048 209 -> 201 and 266 -> 256, 3072 257 -> 245, 5120 407 -> 392 and 507 -> 480.  A block of 72 rows of hidden 4096 is
 // 60 us of HBM; the rest is the attention (16), ~4 around it (a cooperative launch does not start ahead of the end of the kernel in front), and the four times that HBM
 // waits for a step.  Tried: asking for the next product's weights in L2 while the ring is full, at once or one stage each 0.5 us, and for the O product's while the attention runs

@@ -691,17 +691,50 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
 
   ArParams P;
   memset(&P, 0, sizeof(P));
-  // Tile height: as many rounds of the SMs as 128-row tiles take, evenly filled (vocabulary 151936: 1187 tiles of 128 are eight rounds of
-  // the 148 SMs and three tiles; 1333 of 114, rounded up to 116, are nine rounds of 0.9 the length), but not under 32 rows.
   int dev = 0, sms = kNumSM;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms > kNumSM || sms < 1) sms = kNumSM;
-  P.tiles = ((h.vocab + 127) / 128 + sms - 1) / sms;
-  P.rows = ((h.vocab + sms * P.tiles - 1) / (sms * P.tiles) + 3) / 4 * 4;
-  if (P.rows < 32) P.rows = 32;
-  const int grid = (h.vocab + P.tiles * P.rows - 1) / (P.tiles * P.rows);
   const int slabs = h.rank / 64, nb = h.b <= 16 ? 16 : 32;
   const bool sample = h.uniforms != nullptr;
+  // Tiles per CTA, and with them the number of CTAs.  A step takes ~0.5 us for each tile of a CTA and ~0.012 for each CTA that the others have to hear from: T tiles of 128 rows on n
+  // CTAs cost 42 T + n, with as few tiles as the SMs allow and up.  Before, all SMs had as many rows as came out evenly (12 steps, us, that / this): vocabulary 5760 73.2 / 58.5 (45
+  // CTAs of 144), 12000 75.8 / 67.0, 30128 90.7 / 87.7; sampling 127.5 / 109.2, 128.6 / 121.9, 145.4 / 137.4; 60000 191 / 178.
+  // Where that leaves fewer than four slots of base logits beside the ring of W, 120 rows on more CTAs (16 requests, 151936 x 256: 498 us with four slots, 517 with two).
+  auto plan = [&](int full) {
+    const int blocks = (h.vocab + full - 1) / full;
+    auto ctas = [&](int t) { return (blocks + t - 1) / t; };
+    P.tiles = (blocks + sms - 1) / sms;
+    while (42 * (P.tiles + 1) + ctas(P.tiles + 1) < 42 * P.tiles + ctas(P.tiles)) ++P.tiles;
+    const int share = ctas(P.tiles) * P.tiles;   // the tiles, evenly filled
+    P.rows = ((h.vocab + share - 1) / share + 3) / 4 * 4;
+    if (P.rows < 32) P.rows = 32;
+    // Tiles that stay: what fits behind the accumulators; one step alone reads W once either way.
+    P.resident = h.block > 1 ? (512 - kResidentCol) / (32 * slabs) : 0;
+    if (P.resident > P.tiles) P.resident = P.tiles;
+    P.slab_bytes = (P.rows + 7) / 8 * 1024;
+    P.logit_bytes = (h.b * P.rows * 4 + 127) / 128 * 128;
+    const int tile_bytes = slabs * P.slab_bytes, room = 227 * 1024 - 1024 - slabs * nb * 128 - kBarBytes;
+    const int streamed = P.tiles - P.resident, most = streamed < 1 ? 1 : (streamed < kMaxStages ? streamed : kMaxStages);
+    auto stages_with = [&](int slots) {
+      const int n = (room - slots * P.logit_bytes) / tile_bytes;
+      return n < 0 ? 0 : (n < most ? n : most);
+    };
+    P.z_in_place = sample && P.tiles <= kMaxLogitSlots && stages_with(P.tiles) >= (most < 2 ? most : 2);
+    if (P.z_in_place) {
+      P.logit_slots = P.tiles;
+    } else {
+      // two to four slots of base logits, as many as cost the ring of W nothing
+      P.logit_slots = 2;
+      while (P.logit_slots < 4 && stages_with(P.logit_slots + 1) == stages_with(2)) ++P.logit_slots;
+    }
+    P.stages = stages_with(P.logit_slots);
+    return P.z_in_place || P.logit_slots == 4;
+  };
+  if (!plan(128)) {
+    const int tiles = P.tiles;
+    if (!plan(120) || P.tiles != tiles) plan(128);
+  }
+  const int grid = (h.vocab + P.tiles * P.rows - 1) / (P.tiles * P.rows);
 
   const size_t vecs = (kDrawnWords + (size_t)2 * h.b * (sample ? 2 : kCopies) * kCtaStride) / 2;   // 16 bytes each
   launch_pdl(head_clear_kernel, dim3((unsigned)(vecs < 148 * 256 ? (vecs + 255) / 256 : 148)), dim3(256), 0, st, reinterpret_cast<uint4 *>(words), vecs);
@@ -725,26 +758,7 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   P.drawn = words; P.words = words + kDrawnWords; P.status = status;
   P.z = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(words) + words_bytes(h.b));
   P.b = h.b; P.block = h.block; P.vocab = h.vocab;
-  // Tiles that stay: what fits behind the accumulators; one step alone reads W once either way.
-  P.resident = h.block > 1 ? (512 - kResidentCol) / (32 * slabs) : 0;
-  if (P.resident > P.tiles) P.resident = P.tiles;
-  P.slab_bytes = (P.rows + 7) / 8 * 1024;
-  P.logit_bytes = (h.b * P.rows * 4 + 127) / 128 * 128;
-  const int tile_bytes = slabs * P.slab_bytes, e_bytes = slabs * nb * 128, room = 227 * 1024 - 1024 - e_bytes - kBarBytes;
-  const int streamed = P.tiles - P.resident, most = streamed < 1 ? 1 : (streamed < kMaxStages ? streamed : kMaxStages);
-  auto stages_with = [&](int slots) {
-    const int n = (room - slots * P.logit_bytes) / tile_bytes;
-    return n < 0 ? 0 : (n < most ? n : most);
-  };
-  if (sample && P.tiles <= kMaxLogitSlots && stages_with(P.tiles) >= (most < 2 ? most : 2)) {
-    P.z_in_place = 1;
-    P.logit_slots = P.tiles;
-  } else {
-    // two to four slots of base logits, as many as cost the ring of W nothing
-    P.logit_slots = 2;
-    while (P.logit_slots < 4 && stages_with(P.logit_slots + 1) == stages_with(2)) ++P.logit_slots;
-  }
-  P.stages = stages_with(P.logit_slots);
+  const int tile_bytes = slabs * P.slab_bytes, e_bytes = slabs * nb * 128;
   P.e_off = P.stages * tile_bytes;
   P.logit_off = P.e_off + e_bytes;
   P.bar_off = P.logit_off + P.logit_slots * P.logit_bytes;
