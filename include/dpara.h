@@ -155,6 +155,8 @@ dpara_status dpara_draft_all_boundaries(const dpara_shape *shape, const dpara_at
  *                 intermediate sizes); x is taken from entry 0 only, y_f32 (required) and y_bf16 from the last entry only
  *   host_k_ctx, host_v_ctx   HOST arrays [n_layers] of DEVICE pointers: each block's context keys/values, all laid out
  *                 by io->ctx_offsets (and io->ctx_lens); io->k_ctx / io->v_ctx are ignored
+ * Up to 128 rows (and in a block of dpara_draft_all_boundaries) what lies between two attentions is one kernel whose CTAs, one per SM, wait for one another: it is
+ * launched so that all run at once; where the current context's share of the GPU cannot hold them, kernels without that need give the same results.
  * Workspace: dpara_backbone_workspace_bytes().  Errors: as dpara_draft_all_boundaries. */
 typedef struct {
   int32_t n_layers;
