@@ -320,8 +320,13 @@ struct BlockBuffers {
         angles(reinterpret_cast<float *>(lw + w.angles)), planes(reinterpret_cast<float *>(lw + w.planes)) {}
 };
 
-bool block_args_ok(const dpara_shape *shape, const dpara_layer_io *L) {
-  return L->x && L->w_qkv && L->w_o && L->w_gate_up && L->w_down && L->y_f32 && L->hidden > 0 && L->intermediate > 0 && (L->qnorm_w == nullptr) == (L->knorm_w == nullptr);
+// What refuses a block, whichever kernels would run it
+dpara_status check_block(const dpara_shape *shape, const dpara_layer_io *L) {
+  if (!L->x || !L->w_qkv || !L->w_o || !L->w_gate_up || !L->w_down || !L->y_f32 || L->hidden <= 0 || L->intermediate <= 0) return DPARA_ERR_INVALID_ARG;
+  if ((L->qnorm_w == nullptr) != (L->knorm_w == nullptr)) return DPARA_ERR_INVALID_ARG;
+  if (shape->boundary_lo != 0 || shape->boundary_hi != shape->n_boundaries) return DPARA_ERR_UNSUPPORTED;   // (the products behind the attention read every row)
+  if (L->hidden % 64 || L->intermediate % 64 || shape->n_q_heads * shape->head_dim % 64) return DPARA_ERR_UNSUPPORTED;
+  return DPARA_OK;
 }
 
 AngleJob angle_job(const dpara_shape *shape, const dpara_attn_io *io, const dpara_layer_io *L, int M, int R, float *table) {
@@ -416,14 +421,13 @@ dpara_status launch_chained(const dpara_shape *shape, const ChainShape &sh, int 
 
 dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, const dpara_layer_io *L, void *workspace,
                           int32_t *status_word, cudaStream_t st, bool angles_there, bool allow_chain) {
-  if (!block_args_ok(shape, L)) return DPARA_ERR_INVALID_ARG;
-  if (shape->boundary_lo != 0 || shape->boundary_hi != shape->n_boundaries) return DPARA_ERR_UNSUPPORTED;
+  const dpara_status refused = check_block(shape, L);
+  if (refused != DPARA_OK) return refused;
   const int Sq = shape->spine_queries ? shape->n_spine : 0;
   const int R = shape->n_boundaries * shape->block + Sq;  // rows per request: mask slots, then (if they are queries) the spine
   const int M = shape->batch * R;
   const int H = L->hidden, I = L->intermediate, D = shape->head_dim;
   const int QD = shape->n_q_heads * D, KD = shape->n_kv_heads * D;
-  if (H % 64 || I % 64 || QD % 64 || H % 8) return DPARA_ERR_UNSUPPORTED;
   const size_t attn_ws = attention_workspace_bytes(shape, io->host_ctx_offsets);
   // layout: [attention scratch (as sized by attention_workspace_bytes)] [layer buffers] [counters]
   uint8_t *base = static_cast<uint8_t *>(workspace);
@@ -525,7 +529,7 @@ dpara_status launch_backbone(const dpara_shape *shape, const dpara_attn_io *io, 
   bool chained = chain.ok;
   for (int l = 0; l <= last && chained; ++l) {
     const dpara_layer_io L = block(l);
-    chained = block_args_ok(shape, &L);   // (else the block is refused below)
+    chained = check_block(shape, &L) == DPARA_OK;   // (else it is refused below)
   }
   if (chained) {
     const size_t attn_ws = attention_workspace_bytes(shape, io->host_ctx_offsets);
