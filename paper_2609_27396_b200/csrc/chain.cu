@@ -605,12 +605,16 @@ ChainShape chain_shape(int M, int hidden, int intermediate, int q_dim, int kv_di
   const int reach = (sh.w_stages * 2 - 1) * sh.op_bytes + 128 * 128 + kBarBytes + 1024;
   if (sh.smem < reach) sh.smem = reach;
   if (sh.smem < 116 * 1024) sh.smem = 116 * 1024;   // (one per SM: it takes all tensor memory and waits for its whole grid)
-  size_t most = (size_t)sh.o.split * hidden;
-  if ((size_t)sh.down.split * hidden > most) most = (size_t)sh.down.split * hidden;
-  if ((size_t)sh.qkv.split * n_qkv > most) most = (size_t)sh.qkv.split * n_qkv;
-  sh.plane_bytes = most * M * sizeof(float);
   sh.ok = 1;
   return sh;
+}
+
+size_t chain_plane_bytes(long M, int hidden, int q_dim, int kv_dim) {
+  if (hidden > kChainHidden) return 0;
+  // (a product's parts are kMaxSplit at most, and all its tiles in all its parts have an SM each)
+  const long n_qkv = q_dim + 2 * kv_dim, widest = hidden > n_qkv ? hidden : n_qkv, of_all_sms = (long)kNumSM * 128;
+  const long columns = kMaxSplit * widest < of_all_sms ? kMaxSplit * widest : of_all_sms;
+  return (size_t)(M < kChainRows ? M : kChainRows) * columns * sizeof(float);
 }
 
 dpara_status launch_chain(const ChainShape &sh, const ChainArgs &a, int32_t *status, cudaStream_t st) {

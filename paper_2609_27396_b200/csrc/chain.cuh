@@ -19,9 +19,11 @@ struct ChainShape {
   ChainTiles o, gate_up, down, qkv;
   int op_bytes, w_stages, a_slots, smem;
   int on_way;             // stages of weights on their way at most
-  size_t plane_bytes;     // partial sums of the product with most of them
 };
 ChainShape chain_shape(int M, int hidden, int intermediate, int q_dim, int kv_dim, int head_dim);
+// Room for the partial sums of a chain of up to M rows: what any tiles of it can need, and as much above kChainRows as at them, so that the scratch of a larger
+// batch serves a smaller one.
+size_t chain_plane_bytes(long M, int hidden, int q_dim, int kv_dim);
 
 struct ChainArgs {
   int M, hidden, intermediate, n_q_heads, n_kv_heads, head_dim;

@@ -269,8 +269,7 @@ LayerWs layer_ws_layout(const dpara_shape *s, const dpara_layer_io *l, size_t at
   w.act = take(M * I * 2);
   w.angles = take(M * s->head_dim * 4);
   w.attn = take(attn_bytes);
-  const ChainShape chain = block_chain(s, l);
-  w.planes = take(chain.ok ? chain.plane_bytes : 0);
+  w.planes = take(chain_plane_bytes((long)M, l->hidden, s->n_q_heads * s->head_dim, s->n_kv_heads * s->head_dim));
   w.total = o;
   return w;
 }

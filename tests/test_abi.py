@@ -194,3 +194,20 @@ def test_blocks_refuse_misaligned_tensors(n_layers):
     for name in LAYER_POINTERS:
         assert _blocks(n_layers, **{name: 4098}) == dp.ERR_INVALID_ARG, name
     assert _blocks(n_layers, qnorm_w=4100, knorm_w=4104) == dp.ERR_WORKSPACE            # the row-wise kernel takes these
+
+
+@pytest.mark.parametrize("hq,hkv,d,hidden,inter", [(40, 8, 128, 5120, 17408), (32, 8, 128, 4096, 12288), (16, 4, 64, 256, 512), (2, 2, 64, 64, 64), (64, 8, 128, 5184, 8192)])
+def test_workspace_of_a_larger_batch_serves_a_smaller_one(hq, hkv, d, hidden, inter):
+    """A serving loop's batch varies under one workspace.  The blocks' part of it (the attention's scratch is asked for by the same query, and not this test's)."""
+    layers = (dp.LayerIO * 3)(*[dp.LayerIO(rms_eps=1e-6, rope_theta=1e6, use_rope=1, hidden=hidden, intermediate=inter) for _ in range(3)])
+    bb = dp.BackboneIO(3, C.addressof(layers), None, None)
+    for j, bq in ((8, 1), (5, 1), (1, 1), (3, 5), (8, 8)):
+        for spine in (0, 1):
+            most = [0, 0]
+            for b in range(1, 140):
+                shape = _shape(batch=b, n_boundaries=j, boundary_hi=j, n_spine=j, block=bq, n_q_heads=hq, n_kv_heads=hkv, head_dim=d, spine_queries=spine)
+                off = C.cast((C.c_int64 * (b + 1))(*[9 * n for n in range(b + 1)]), C.c_void_p)
+                attn = dp.lib.dpara_draft_workspace_bytes(C.byref(shape), off, None, 0)
+                need = [dp.lib.dpara_draft_workspace_bytes(C.byref(shape), off, C.byref(layers[0]), 1) - attn, dp.lib.dpara_backbone_workspace_bytes(C.byref(shape), off, C.byref(bb)) - attn]
+                assert need[0] >= most[0] and need[1] >= most[1], (j, bq, spine, b, need, most)
+                most = need
