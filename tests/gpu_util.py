@@ -40,3 +40,18 @@ def check_verify(res, ref):
     if ref["selected"] is not None:
         assert np.array_equal(host_bits(res["selected"]), ref["selected"])
     assert int(res["status"].item()) == ref["status"]
+
+
+def compile_native(tmp_path, text, objects=()):
+    """A library of this CUDA source, with the library's own flags and headers, linked with object files; loaded."""
+    import ctypes
+    import os
+    import subprocess
+    from paper_2609_27396_b200 import build
+    src, obj, lib = tmp_path / "native.cu", tmp_path / "native.o", tmp_path / "native.so"
+    src.write_text(text)
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    for cmd in ([nvcc, *build.NVCC_FLAGS, "-I", build.CSRC, "-c", "-o", str(obj), str(src)], [nvcc, "-shared", *build.NVCC_FLAGS[:2], "-o", str(lib), str(obj), *objects]):
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(str(lib))
