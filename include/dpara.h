@@ -369,7 +369,7 @@ dpara_status dpara_gemm_bf16(const dpara_gemm_io *io, int32_t *status_word, void
  * clusters -- as the calls of this library launch them; dpara_gemm_bf16 itself is (1, 1, 0, 0).
  * route[0] 1: few activation rows, single CTAs that share a tile's K range inside clusters; 0: CTA pairs.
  * route[1] activation rows per tile, [2] operands of weight rows per tile, [3] weight rows per operand, [4] CTAs per tile, [5] rounds of tiles,
- * [6] activation rows that pass through shared memory at a time, [7] 64-column slabs of K per stage.
+ * [6] activation rows that pass through shared memory at a time (pairs: of a unit of the last round, whose tiles are cut along their rows where they are few), [7] 64-column slabs of K per stage.
  * Errors (those a launch would return): INVALID_ARG, UNSUPPORTED. */
 dpara_status dpara_gemm_route(int32_t M, int32_t N, int32_t K, int32_t epilogue, int32_t n_groups, int32_t split_k, int32_t row_order, int32_t one_chain,
                               int32_t route[8]);

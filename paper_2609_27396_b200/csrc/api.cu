@@ -166,7 +166,7 @@ extern "C" dpara_status dpara_gemm_route(int32_t M, int32_t N, int32_t K, int32_
   const SkinnyShape &k = r.skinny;
   const long units = r.few ? (long)k.tiles * n_groups : (long)r.n_all * r.pair.t_tiles, at_once = r.few ? k.clusters : r.most;
   const int rounds = (int)((units + at_once - 1) / at_once);
-  const int few[8] = {1, k.T, k.halves, k.rows, k.split, rounds, k.chunk, k.slabs}, pairs[8] = {0, r.pair.nt, 1, 256, 2, rounds, r.pair.nt, 1};
+  const int few[8] = {1, k.T, k.halves, k.rows, k.split, rounds, k.chunk, k.slabs}, pairs[8] = {0, r.pair.nt, 1, 256, 2, rounds, r.nt_tail ? r.nt_tail : r.pair.nt, 1};
   for (int i = 0; i < 8; ++i) route[i] = r.few ? few[i] : pairs[i];
   return DPARA_OK;
 }

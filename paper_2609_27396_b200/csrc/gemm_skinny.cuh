@@ -24,6 +24,7 @@ struct GemmRoute {
   SkinnyShape skinny;
   PairPlan pair;
   int n_tiles, n_all, most;   // CTA pairs: weight tiles of one product, of all products and parts of K; pairs of the device
+  int nt_tail, main_units;    // activation rows of the units that the tiles of a nearly empty last round are cut into, whole tiles ahead of them; 0: none are cut
 };
 dpara_status gemm_route(const GemmArgs &g, GemmRoute &r);
 dpara_status launch_gemm_skinny(const GemmArgs &g, const SkinnyShape &sh, int32_t *status, cudaStream_t st);

@@ -411,6 +411,25 @@ PairPlan pair_plan(int M, int n_all, int nkb, int most) {
   }
   return best;
 }
+
+// The tiles of a last round that has few of them (at most a third of the pairs): each in up to `at_once` / left parts of its activation rows, on pairs that
+// would have nothing to do.  Every part reads the tile's weights again (from L2), so only about two thirds of the pairs are given one.  Against whole
+// tiles, 109 products of 129 to 1152 rows with 1 to 24 tiles left of 74, stores and SwiGLU, weights from HBM: 1.057x (geometric mean), faster by
+// more than the spread in all but three, slower by more than it in none.  1.13 behind one round of tiles, 1.07 behind two or three, 1.035 behind four to nine (the pairs drift
+// apart, and the whole tiles of a last round start early on some); 1.068 with 1 to 8 tiles left, 1.058 with 9 to 16, 1.044 with 17 to 24.  For
+// instance 207 x 23112 x 1088 22.0 -> 19.7 us, 498 x 9920 x 2752 SwiGLU 54.9 -> 48.6, 1014 x 14784 x 4544 SwiGLU 196 -> 190.  Launches of several products or parts
+// of K too: the append of five layers, 256 rows (40 tiles in four parts, 12 units behind two rounds) 48.1 -> 45.5, the same bits.
+void tail_plan(GemmRoute &r) {
+  const long units = (long)r.pair.t_tiles * r.n_all;
+  const int left = (int)(units % r.most), at_once = r.most * 13 / 20;   // 48 of 74 pairs
+  r.nt_tail = r.main_units = 0;
+  if (units < r.most || left == 0 || 2 * left > at_once) return;
+  int nt = (r.pair.nt / (at_once / left) + 15) / 16 * 16;
+  if (nt < 32) nt = 32;
+  if (nt >= r.pair.nt) return;
+  r.nt_tail = nt;
+  r.main_units = (int)(units - left);
+}
 }  // namespace
 
 // Everything about a launch that its sizes decide: refusals, then the kernel and its tiles.
@@ -426,6 +445,7 @@ dpara_status gemm_route(const GemmArgs &g, GemmRoute &r) {
   r.n_all = r.n_tiles * (g.n_groups > 1 ? g.n_groups : 1) * (g.split_k > 1 ? g.split_k : 1);
   r.most = sm_count() / 2 < kNumSM / 2 ? sm_count() / 2 : kNumSM / 2;
   r.pair = pair_plan(g.M, r.n_all, nkb / (g.split_k > 1 ? g.split_k : 1), r.most);
+  tail_plan(r);
   // Few rows: single CTAs that share a tile's K range inside clusters.  Above 128 activation rows by the two models (us, pairs / that:
   // 200 rows, 4096 x 12288 44.8 / 30.8, 4096 x 4096 19.8 / 16.1, 6144 x 4096 18.5 / 23.3; 400 rows, 4096 x 4096 21.1 / 22.8).
   r.few = 0;
@@ -434,25 +454,6 @@ dpara_status gemm_route(const GemmArgs &g, GemmRoute &r) {
     r.few = r.skinny.cost >= 0 && (g.M <= kManyRows || 1e-3 * r.skinny.cost + 3.5 < r.pair.us);
   }
   return DPARA_OK;
-}
-
-// The tiles of a last round that has few of them (at most a third of the pairs): each in up to `at_once` / left parts of its activation rows, on pairs that
-// would have nothing to do.  Every part reads the tile's weights again (from L2), so only about two thirds of the pairs are given one.  Against whole
-// tiles, 109 products of 129 to 1152 rows with 1 to 24 tiles left of 74, stores and SwiGLU, weights from HBM: 1.057x (geometric mean), faster by
-// more than the spread in all but three, slower by more than it in none.  1.13 behind one round of tiles, 1.07 behind two or three, 1.035 behind four to nine (the pairs drift
-// apart, and the whole tiles of a last round start early on some); 1.068 with 1 to 8 tiles left, 1.058 with 9 to 16, 1.044 with 17 to 24.  For
-// instance 207 x 23112 x 1088 22.0 -> 19.7 us, 498 x 9920 x 2752 SwiGLU 54.9 -> 48.6, 1014 x 14784 x 4544 SwiGLU 196 -> 190.  Launches of several products or parts
-// of K too: the append of five layers, 256 rows (40 tiles in four parts, 12 units behind two rounds) 48.1 -> 45.5, the same bits.
-static bool tail_plan(const GemmArgs &g, const GemmRoute &r, GemmKernelParams &P) {
-  const long units = (long)r.pair.t_tiles * r.n_all;
-  const int left = (int)(units % r.most), at_once = r.most * 13 / 20;   // 48 of 74 pairs
-  if (units < r.most || left == 0 || 2 * left > at_once) return false;
-  P.nt_tail = (r.pair.nt / (at_once / left) + 15) / 16 * 16;
-  if (P.nt_tail < 32) P.nt_tail = 32;
-  if (P.nt_tail >= r.pair.nt) return false;
-  P.tail_split = (r.pair.nt + P.nt_tail - 1) / P.nt_tail;
-  P.main_units = (int)(units - left);
-  return true;
 }
 
 dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st) {
@@ -468,7 +469,9 @@ dpara_status launch_gemm_tc(const GemmArgs &g, int32_t *status, cudaStream_t st)
   P.split_k = g.split_k > 1 ? g.split_k : 1;
   P.n_tiles = route.n_tiles;
   P.t_tiles = route.pair.t_tiles; P.nt = route.pair.nt;
-  const bool tail = tail_plan(g, route, P);
+  const bool tail = route.nt_tail > 0;
+  P.nt_tail = route.nt_tail; P.main_units = route.main_units;
+  P.tail_split = tail ? (P.nt + P.nt_tail - 1) / P.nt_tail : 1;
   for (int gi = 0; gi < P.n_groups; ++gi) {
     const void *a = gi ? g.a_g[gi] : g.a, *w = gi ? g.w_g[gi] : g.w;
     void *o = gi ? g.out_g[gi] : g.out;
