@@ -42,16 +42,32 @@ def check_verify(res, ref):
     assert int(res["status"].item()) == ref["status"]
 
 
-def compile_native(tmp_path, text, objects=()):
-    """A library of this CUDA source, with the library's own flags and headers, linked with object files; loaded."""
+def compile_native(tmp_path, text, without=None):
+    """A library of this CUDA source, with the library's own flags and headers, loaded.  without: linked with the library's other objects but this one."""
     import ctypes
     import os
     import subprocess
     from paper_2609_27396_b200 import build
-    src, obj, lib = tmp_path / "native.cu", tmp_path / "native.o", tmp_path / "native.so"
-    src.write_text(text)
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    for cmd in ([nvcc, *build.NVCC_FLAGS, "-I", build.CSRC, "-c", "-o", str(obj), str(src)], [nvcc, "-shared", *build.NVCC_FLAGS[:2], "-o", str(lib), str(obj), *objects]):
-        r = subprocess.run(cmd, capture_output=True, text=True)
+
+    def run(*cmd):
+        r = subprocess.run([nvcc, *cmd], capture_output=True, text=True)
         assert r.returncode == 0, r.stderr
+
+    def compile_one(src, obj):
+        run(*build.NVCC_FLAGS, "-I", build.CSRC, "-c", "-o", str(obj), str(src))
+
+    src, lib = tmp_path / "native.cu", tmp_path / "native.so"
+    src.write_text(text)
+    objects = [tmp_path / "native.o"]
+    compile_one(src, objects[0])
+    for s in build.sources() if without else []:
+        name = os.path.basename(s)[:-3]
+        if name != without:
+            obj = os.path.join(build.OBJ, name + ".o")
+            if not os.path.exists(obj):
+                obj = tmp_path / (name + ".o")
+                compile_one(s, obj)
+            objects.append(obj)
+    run("-shared", *build.NVCC_FLAGS[:2], "-o", str(lib), *map(str, objects))
     return ctypes.CDLL(str(lib))

@@ -109,14 +109,15 @@ def test_select_gathers_from_rows_with_a_request_stride():
     assert np.array_equal(plan.selected.cpu().view(torch.int16).numpy().view(np.uint16), ref["selected"])
 
 
-def test_angles_are_made_once_for_blocks_that_turn_alike():
+@pytest.mark.parametrize("b", [2, 10])     # 30 rows: the chain; 150: kernels of their own, several CTAs a row behind the QKV product
+def test_angles_are_made_once_for_blocks_that_turn_alike(b):
     """Blocks with the same theta share the table of angles, another theta or a block without rotation in between makes a new one: a stack gives what its
     blocks give one by one, bit for bit."""
     import paper_2609_27396_b200 as dp
     g = torch.Generator(device="cuda").manual_seed(3)
     bf = lambda sigma, *shape: (sigma * torch.randn(*shape, device="cuda", generator=g)).to(torch.bfloat16)  # noqa: E731
-    b, J, Bq, Hq, Hkv, D, H, I = 2, 3, 4, 16, 4, 64, 256, 512     # 20 heads: a table is only made above 16
-    off, rows = [0, 70, 75], J * Bq + J
+    J, Bq, Hq, Hkv, D, H, I = 3, 4, 16, 4, 64, 256, 512     # 20 heads: a table is only made above 16
+    off, rows = [0] + [70 + 5 * n for n in range(b)], J * Bq + J
     shape = dict(n_boundaries=J, block=Bq, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D)
     turns = [dict(rope_theta=1e6), dict(rope_theta=1e6), dict(rope_theta=1e4), dict(use_rope=False), dict(rope_theta=1e4), dict(rope_theta=1e4)]
     kc, vc = [[bf(1.0, off[-1], Hkv, D) for _ in turns] for _ in range(2)]
@@ -124,7 +125,9 @@ def test_angles_are_made_once_for_blocks_that_turn_alike():
     x = bf(1.0, b, rows, H)
     y, y16 = torch.zeros(b, rows, H, device="cuda"), torch.zeros(b, rows, H, device="cuda", dtype=torch.bfloat16)
     stack = dp.BackbonePlan(ctx_offsets=off, **shape, layers=[dp.make_layer_io(x=x, **k, y_f32=y, y_bf16=y16) for k in w], k_ctx=kc, v_ctx=vc)
+    before = dp.lib.dpara_kernel_launches()
     stack()
+    assert dp.lib.dpara_kernel_launches() - before == (1 + 6 + 7 + 1 if b * rows <= 128 else 8 * 6)   # (the chain: one more launch, for 1e4's angles)
     one, one16, into = torch.zeros_like(y), torch.zeros_like(y16), x.clone()
     for k, a, c in zip(w, kc, vc):
         plan = dp.BackbonePlan(ctx_offsets=off, **shape, layers=[dp.make_layer_io(x=into, **k, y_f32=one, y_bf16=one16)], k_ctx=[a], v_ctx=[c])

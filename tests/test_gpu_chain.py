@@ -100,6 +100,69 @@ def test_chain_takes_one_launch_between_attentions():
     assert alone == 1 + 3 + 4 and dp.lib.dpara_kernel_launches() - before - alone == 8 * 3
 
 
+REFUSED = """
+#define launch_chain launch_chain_as_it_is
+#include "chain.cu"
+#undef launch_chain
+namespace dpara {
+dpara_status launch_chain(const ChainShape &, const ChainArgs &, int32_t *, cudaStream_t) { return DPARA_ERR_UNSUPPORTED; }
+}
+"""
+
+
+@pytest.mark.parametrize("spine_rows,layers", [(True, 3), (False, 1)])
+def test_refused_cooperative_launch(tmp_path, monkeypatch, spine_rows, layers):
+    """Where the grid of the chain cannot be held at once (here: the library with a launch that says so), the same call goes through kernels of their own."""
+    import paper_2609_27396_b200 as dp
+    from gpu_util import compile_native
+    few, many = _case(5, 1, 4, 4, 8, (16, 4, 64), 256, 512, layers, spine_rows=spine_rows)
+    many()
+    lib = compile_native(tmp_path, REFUSED, without="chain")
+    for name in dp.EXPORTED:
+        getattr(lib, name).restype, getattr(lib, name).argtypes = getattr(dp.lib, name).restype, getattr(dp.lib, name).argtypes
+    monkeypatch.setattr(dp, "_draft_packed", type(dp._draft_packed)(("dpara_draft_all_boundaries", lib)))
+    monkeypatch.setattr(dp, "lib", lib)
+    few()
+    torch.cuda.synchronize()
+    assert lib.dpara_kernel_launches() == 1 + 8 * layers      # (the norm ahead of the refused launch)
+    assert int(few.plan.status.item()) == 0 and int(many.plan.status.item()) == 0
+    _agree(few, many)
+
+
+def test_chain_beside_other_streams():
+    """The chain, whose CTAs wait for one another, beside streams that keep the SMs busy: the head loop (a cooperative launch too) behind its LM head, and grids of kernels that hold
+    all SMs, a few of them, or come and go.  What the calls give alone, bit for bit."""
+    import paper_2609_27396_b200 as dp
+    few, _many = _case(21, 1, 2, 8, 7, (16, 4, 128), 1024, 3072, 3)
+    g = torch.Generator(device=DEV).manual_seed(4)
+    bf = lambda sigma, *shape: (sigma * torch.randn(*shape, device=DEV, generator=g)).to(torch.bfloat16)  # noqa: E731
+    b, block, hidden, vocab, rank = 2, 6, 512, 30008, 256
+    head, head_in = dp.HeadPlan(b, block, hidden, vocab, rank), (bf(1.0, b, block, hidden), bf(0.05, vocab, hidden), bf(0.3, vocab, rank), bf(0.3, vocab, rank),
+                                                                 torch.zeros(b, dtype=torch.int32, device=DEV))
+    wide, narrow, x = bf(0.02, 4096, 4096), bf(0.02, 256, 4096), bf(1.0, 512, 4096)
+    few()
+    head.run(*head_in)
+    torch.cuda.synchronize()
+    alone = [t.clone() for t in (few.y, few.y16, head.next_tokens)]
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        with torch.cuda.stream(streams[0]):
+            few()
+        with torch.cuda.stream(streams[1]):
+            head.run(*head_in)
+        with torch.cuda.stream(streams[2]):
+            for _ in range(4):
+                x @ wide.T
+        with torch.cuda.stream(streams[3]):
+            for _ in range(10):
+                x[:64] @ narrow.T
+    torch.cuda.synchronize()
+    assert int(few.plan.status.item()) == 0 and int(head.status.item()) == 0
+    for got, want in zip((few.y, few.y16, head.next_tokens), alone):
+        assert torch.equal(got, want)
+
+
 def test_chains_on_two_streams_and_in_a_graph():
     """Two stacks of the chain in streams without order, then captured in a graph and replayed on other inputs."""
     pairs = [_case(s, 1, 2, 8, 7, (16, 4, 64), 640, 1984, 3) for s in (11, 12)]
