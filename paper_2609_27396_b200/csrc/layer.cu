@@ -242,13 +242,20 @@ struct LayerWs {
   size_t xn, qkv, q, k, v, a, h1, hn, act, angles, attn, planes, total;
 };
 
-ChainShape block_chain(const dpara_shape *s, const dpara_layer_io *l) {
+// The chain of a stack of n_blocks; not ok: kernels of their own.  Times of those / with the chain, called one by one, rows 4 to 128:
+//   blocks     weights of a block, MB:  2..8         13..21       29..58       76..96       144..233     312..386 (to 48 rows, to 64, more)  477..661
+//   five                                1.11..1.21   1.10..1.16   1.06..1.13   1.00..1.06   0.99..1.09   0.95..1.00, 1.00..1.01, 1.00..1.03  1.00..1.09
+//   two, three                          1.05..1.18   1.05..1.13   1.01..1.12   0.99..1.04   0.98..1.08   0.96..1.00, -, 0.99..1.03           0.97..1.06
+//   one                                 0.97..1.11   0.98..1.10   0.95..1.05   0.91..1.01   0.97..1.06   0.94..0.97, 0.96..1.00, 0.96..1.02  0.94..1.14
+// A stack's first and last chain have one and three of the four products, so one block is two launches that do not start ahead of the end of the kernel in front, and the
+// meetings of all CTAs, against seven that do: worth it where launches are what a block is, or beyond the sizes that the kernels of their own fill the SMs with.  At most 32 rows of
+// 21 to 58 MB are 0.95 to 1.01.  In a graph the smallest are 1.03..1.14, the others as they are here.
+ChainShape block_chain(const dpara_shape *s, const dpara_layer_io *l, int n_blocks) {
   const long M = (long)s->batch * (s->n_boundaries * s->block + (s->spine_queries ? s->n_spine : 0));
   if (M > kChainRows) return ChainShape{};
-  // A block of which 256 MB of weights and more are read for at most 48 rows is HBM's time either way: chain against kernels of their own 0.97 (40 rows, hidden 4096) to 1.01 there,
-  // 1.03 to 1.18 at all other sizes (rows 16 to 126, hidden 512 to 5120).
   const double weights = 2.0 * l->hidden * ((double)(2 * s->n_q_heads + 2 * s->n_kv_heads) * s->head_dim + 3.0 * l->intermediate);
-  if (M <= 48 && weights > 256e6) return ChainShape{};
+  if (weights > 256e6 && M <= (n_blocks == 1 ? 64 : 48)) return ChainShape{};
+  if (n_blocks == 1 && weights > (M <= 32 ? 16e6 : 64e6) && weights < 128e6) return ChainShape{};
   return chain_shape((int)M, l->hidden, l->intermediate, s->n_q_heads * s->head_dim, s->n_kv_heads * s->head_dim, s->head_dim);
 }
 
@@ -432,8 +439,8 @@ dpara_status launch_layer(const dpara_shape *shape, const dpara_attn_io *io, con
   uint8_t *base = static_cast<uint8_t *>(workspace);
   const LayerWs w = layer_ws_layout(shape, L, 0);
   uint8_t *lw = base + attn_ws;
-  const ChainShape chain = block_chain(shape, L);
-  if (chain.ok && allow_chain) {
+  const ChainShape chain = allow_chain ? block_chain(shape, L, 1) : ChainShape{};
+  if (chain.ok) {
     const dpara_status cs = launch_chained(shape, chain, 1, [&](int) { return *L; }, [&](int) { return *io; }, base, lw, reinterpret_cast<uint32_t *>(lw + w.total), status_word, st);
     if (cs != DPARA_ERR_UNSUPPORTED) return cs;
   }
@@ -524,7 +531,7 @@ dpara_status launch_backbone(const dpara_shape *shape, const dpara_attn_io *io, 
     a.v_ctx = bb->host_v_ctx[l];
     return a;
   };
-  const ChainShape chain = block_chain(shape, &bb->host_layers[0]);
+  const ChainShape chain = block_chain(shape, &bb->host_layers[0], bb->n_layers);
   bool chained = chain.ok;
   for (int l = 0; l <= last && chained; ++l) {
     const dpara_layer_io L = block(l);

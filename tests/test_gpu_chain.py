@@ -72,13 +72,16 @@ def _agree(few, many):
     (1, 8, 1, 16, (10, 2, 64), 320, 448, 2, False, True, False),       # 17 rows; odd numbers of slabs; no gains, no rotation
     (2, 1, 8, 7, (20, 4, 64), 896, 2432, 2, True, True, True),         # 128 rows: the most
     (1, 1, 8, 15, (8, 8, 128), 1088, 3136, 1, True, True, True),
-    (1, 1, 10, 8, (16, 4, 128), 2048, 6144, 1, True, False, True),     # 80 rows (four stages of activations), block without spine rows
+    (1, 1, 10, 8, (16, 4, 128), 1024, 3072, 1, True, False, True),     # 80 rows (four stages of activations), block without spine rows
     (1, 1, 9, 9, (16, 2, 128), 1536, 4096, 1, True, False, True),      # 81 (three)
     (1, 1, 9, 8, (40, 8, 128), 5120, 17408, 1, True, True, True),      # the widest rows
 ])
 def test_chain_against_kernels_of_their_own(b, more, j, bq, heads, hidden, inter, layers, norm, spine_rows, rope):
+    import paper_2609_27396_b200 as dp
     few, many = _case(7, b, more, j, bq, heads, hidden, inter, layers, norm, spine_rows, rope)
+    before = dp.lib.dpara_kernel_launches()
     few()
+    assert dp.lib.dpara_kernel_launches() - before == 1 + layers + (layers + 1)      # a norm, attentions, chains
     many()
     torch.cuda.synchronize()
     assert int(few.plan.status.item()) == 0 and int(many.plan.status.item()) == 0
@@ -98,6 +101,27 @@ def test_chain_takes_one_launch_between_attentions():
     many()
     torch.cuda.synchronize()
     assert alone == 1 + 3 + 4 and dp.lib.dpara_kernel_launches() - before - alone == 8 * 3
+
+
+@pytest.mark.parametrize("j,bq,heads,hidden,inter,one", [
+    (8, 8, (16, 4, 128), 1536, 4608, True),      # 72 rows, 58 MB of weights
+    (8, 8, (16, 4, 128), 1600, 5120, False),     # 66
+    (8, 3, (8, 2, 64), 768, 2304, True),         # 32 rows, 13 MB
+    (8, 3, (8, 2, 64), 1024, 3072, False),       # 21
+    (11, 2, (8, 2, 64), 1024, 3072, True),       # 33 rows
+])
+def test_one_block_goes_where_it_is_faster(j, bq, heads, hidden, inter, one):
+    """One block of few rows takes the chain by its rows and weights; a stack of two such blocks takes it at all of these sizes."""
+    import paper_2609_27396_b200 as dp
+    for layers in (1, 2):
+        few, many = _case(9, 1, 4, j, bq, heads, hidden, inter, layers)
+        before = dp.lib.dpara_kernel_launches()
+        few()
+        assert dp.lib.dpara_kernel_launches() - before == (2 * layers + 2 if one or layers == 2 else 8)
+        many()
+        torch.cuda.synchronize()
+        assert int(few.plan.status.item()) == 0
+        _agree(few, many)
 
 
 REFUSED = """
