@@ -155,8 +155,11 @@ dpara_status dpara_draft_all_boundaries(const dpara_shape *shape, const dpara_at
  *                 intermediate sizes); x is taken from entry 0 only, y_f32 (required) and y_bf16 from the last entry only
  *   host_k_ctx, host_v_ctx   HOST arrays [n_layers] of DEVICE pointers: each block's context keys/values, all laid out
  *                 by io->ctx_offsets (and io->ctx_lens); io->k_ctx / io->v_ctx are ignored
- * Up to 128 rows (and in a block of dpara_draft_all_boundaries) what lies between two attentions is one kernel whose CTAs, one per SM, wait for one another: it is
- * launched so that all run at once; where the current context's share of the GPU cannot hold them, kernels without that need give the same results.
+ * Up to 128 rows of hidden <= 5120, in a stack and in most sizes of one block (dpara_draft_all_boundaries with a layer too), what lies between two attentions is one kernel
+ * whose CTAs, one per SM, wait for one another.  It is launched so that all run at once, which in a busy GPU means once every SM is free, and other streams' kernels wait until it ends.
+ * At most 48 rows (one block: 64) of more than 256 MB of weights a block, one block of 64 to 128 MB, and of 16 to 64 MB with at most 32 rows go through kernels without that need, as does
+ * a call whose context's share of the GPU cannot hold the CTAs.  The two ways add a product's sums in different orders: results agree up to the roundings to bf16 that
+ * this flips (y of five blocks 0.7 % in the 2-norm, either as near to 64-bit results), not bit for bit.  The choice follows from the sizes and the device: a call repeats itself bit for bit.
  * Workspace: dpara_backbone_workspace_bytes().  Errors: as dpara_draft_all_boundaries. */
 typedef struct {
   int32_t n_layers;

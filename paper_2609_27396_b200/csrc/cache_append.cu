@@ -193,8 +193,8 @@ __global__ void __launch_bounds__(128) append_rows_kernel(const AppendParams P) 
 // Layers per grouped launch and K parts per layer for `layers_left` remaining layers; parts = 0: bf16 stores (at most 128 rows: the
 // kernel for few rows takes all layers at once, one chain of sums over K each; the whole call, 8 rows, five layers of 2048 x 4096: 192 us with a
 // product a layer, 38 now).  The parts are chosen to minimise
-// rounds x (K slabs per part + ~8 slabs' worth of fixed cost per work unit) over the CTA pairs.  Fewer would be faster (five layers of 256 rows:
-// four parts 45.5 us, none 41.8; one layer: eight 19.1, three 18.1), but the parts' sums decide the roundings of the keys: other parts flip some of them.
+// rounds x (K slabs per part + ~8 slabs' worth of fixed cost per work unit) over the CTA pairs.  Fewer are not slower (256 rows, back to back:
+// five layers four parts 43.9 us, none 43.8; one layer eight 29.2, none 21.9), but the parts' sums decide the roundings of the keys: other parts flip some of them.
 static void cache_group_plan(const dpara_cache_io *io, int layers_left, int *group, int *parts) {
   const int M = io->batch * io->n_rows, N = 2 * io->n_kv_heads * io->head_dim;
   *group = layers_left < kGemmMaxGroups ? layers_left : kGemmMaxGroups;

@@ -14,12 +14,16 @@
 // Warps: 0-15 sums, row steps (short chains of dependent instructions: eight warps took twice as long); 16 weights; 17 activations; 18 and 19 products (weights
 // as the rows, M = 128; activation rows as the columns).  A stage is two operands of weights, gate and up of one slab of K or two slabs in turn, and each of the two warps has one
 // of them and an accumulator of its own (two slabs: the sums are added at the end): a single warp took ~750 clocks per stage, two take 500 to 700.
-// Measured, whole stacks of blocks, kernels of their own -> this (us): five blocks of 72 rows, hidden 4096 (385 MB of weights each) 592 -> 582; three blocks of 64 to 128 rows: hidden 512
+// Measured, whole stacks of blocks, kernels of their own -> this (us): five blocks of 72 rows, hidden 4096 (386 MB of weights each) 592 -> 584; three blocks of 64 to 128 rows: hidden 512
 // 151 -> 130 and 169 -> 144, 1024 184 -> 172 and 193 -> 179, 2048 209 -> 201 and 266 -> 256, 3072 257 -> 245, 5120 407 -> 392 and 507 -> 480.  A block of 72 rows of hidden 4096 is
 // 60 us of HBM; the rest is the attention (16), ~4 around it (a cooperative launch does not start ahead of the end of the kernel in front), and the four times that HBM
 // waits for a step.  Tried: asking for the next product's weights in L2 while the ring is full, at once or one stage each 0.5 us, and for the O product's while the attention runs
 // (the row steps, or the attention, get longer by what the product wins); parts of K that start at different slabs in different tiles (no change: the activations are not what a stage waits
 // for); weights of the next product while others still work on this one (the slowest CTA sets the pace).
+// Beside another stream the wait for all SMs shows: six stacks of five blocks of 72 rows beside six passes of library products that read 1 GB of weights (us alone, the other's alone,
+// both together): hidden 4096 3479, 1247, 4806 (kernels of their own 3638, 1242, 4661), 2048 2100, 1256, 3431 (2296, 1248, 3245), 512 1358, 1248, 2526 (1611, 1242, 2518); beside small
+// products (64 x 1024 x 4096) 5602, 4244 and 3436 (5365, 4121, 3551).  Short kernels of another stream wait for a chain's end: twelve runs of six scans of one CTA done after 2890, 1728 and 1182
+// (1121, 708, 705).  Which call takes the chain: layer.cu.
 // All waits are bounded by wall time and give up with DPARA_STATUS_TIMEOUT; the launch is cooperative, so all CTAs are resident.
 #include "chain.cuh"
 #include "gemm.cuh"

@@ -274,8 +274,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_pa
       if (swiglu) tma_load_2d_pair(sw + kWBytes / 2, s.map_w, full + stage, kb * kBK, P.up_row_offset + s.wrow);
     };
     auto load_a = [&](const Source &s, int kb, int stage) { tma_load_2d_pair(smem + stage * stage_bytes + kWBytes, s.map_a, full + stage, kb * kBK, s.arow); };
-    // The weights of the first unit's first stages ahead of the wait, where nothing in front of this kernel writes them (us, without -> with: round of four requests
-    // 664.5 -> 660; four blocks of 280 rows of hidden 704 360 -> 353, a block of 378 rows of hidden 1600 76.1 -> 75.4; large products as before).
+    // The weights of the first unit's first stages ahead of the wait, where nothing in front of this kernel writes them (us, without -> with: four blocks of
+    // 280 rows of hidden 704 250 -> 242, five of 576 of 1024 375 -> 369, a block of 378 of 1600 82.0 -> 80.9, round of four requests 662.6 -> 659.7; larger products and the LM heads: the same).
     int early = 0;
     if (P.w_ready) {
       const Unit<kTail> first(P, pair, nkb);
@@ -418,7 +418,8 @@ PairPlan pair_plan(int M, int n_all, int nkb, int most) {
 // more than the spread in all but three, slower by more than it in none.  1.13 behind one round of tiles, 1.07 behind two or three, 1.035 behind four to nine (the pairs drift
 // apart, and the whole tiles of a last round start early on some); 1.068 with 1 to 8 tiles left, 1.058 with 9 to 16, 1.044 with 17 to 24.  For
 // instance 207 x 23112 x 1088 22.0 -> 19.7 us, 498 x 9920 x 2752 SwiGLU 54.9 -> 48.6, 1014 x 14784 x 4544 SwiGLU 196 -> 190.  Launches of several products or parts
-// of K too: the append of five layers, 256 rows (40 tiles in four parts, 12 units behind two rounds) 48.1 -> 45.5, the same bits.
+// of K too: the append of five layers, 256 rows (40 tiles in four parts, 12 units behind two rounds) 47.3 -> 43.9, 200 rows 43.3 -> 41.4, 407 rows of half the heads 41.1 -> 39.2,
+// 325 rows of 1280 features the same; the same bits.
 void tail_plan(GemmRoute &r) {
   const long units = (long)r.pair.t_tiles * r.n_all;
   const int left = (int)(units % r.most), at_once = r.most * 13 / 20;   // 48 of 74 pairs

@@ -699,7 +699,10 @@ dpara_status launch_head(const HeadArgs &h, void *workspace, int32_t *status, cu
   // Tiles per CTA, and with them the number of CTAs.  A step takes ~0.5 us for each tile of a CTA and ~0.012 for each CTA that the others have to hear from: T tiles of 128 rows on n
   // CTAs cost 42 T + n, with as few tiles as the SMs allow and up.  Before, all SMs had as many rows as came out evenly (12 steps, us, that / this): vocabulary 5760 73.2 / 58.5 (45
   // CTAs of 144), 12000 75.8 / 67.0, 30128 90.7 / 87.7; sampling 127.5 / 109.2, 128.6 / 121.9, 145.4 / 137.4; 60000 191 / 178.
-  // Where that leaves fewer than four slots of base logits beside the ring of W, 120 rows on more CTAs (16 requests, 151936 x 256: 498 us with four slots, 517 with two).
+  // Where that leaves fewer than four slots of base logits beside the ring of W, tiles of 120 rows are taken if they leave four with as many tiles a CTA.  16 steps of hidden 512, us,
+  // 128 rows / 120.  Rank 256: 151936 entries 16 requests 273 / 250, 12 to 15 237..249 / 235..247; 100000 entries 16 requests 220 / 201, 14 199 / 197, 12 189 / 188.  Rank 192: 151936
+  // entries, 13 to 16 requests 236..246 / 233..242.  Where they don't leave four they mostly lose (17 to 32 requests, rank 256: 285..358 / 291..362; ranks 64 to 192 of other vocabularies
+  // up to 8 %), but not always: 16 requests of 128256 entries 242 / 226, rank 192 of 151936 with 17 to 19 306..317 / 284..300.
   auto plan = [&](int full) {
     const int blocks = (h.vocab + full - 1) / full;
     auto ctas = [&](int t) { return (blocks + t - 1) / t; };

@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(128) angles_kernel(const __grid_constant__ Ang
 }
 
 // A stack of n blocks of few rows: the norm of its input, then chains and attentions in turn.  block(l), ctx(l): block l with its input and outputs, and its context.
-// DPARA_ERR_UNSUPPORTED: this device cannot hold a chain's grid at once; the caller's other way gives the same results.
+// DPARA_ERR_UNSUPPORTED: this device cannot hold a chain's grid at once; the caller's other way adds each product's sums in another order and gives the same up to its roundings.
 template <typename Block, typename Ctx>
 dpara_status launch_chained(const dpara_shape *shape, const ChainShape &sh, int n, Block block, Ctx ctx, uint8_t *attn_ws, uint8_t *lw, uint32_t *counters,
                             int32_t *status_word, cudaStream_t st) {
