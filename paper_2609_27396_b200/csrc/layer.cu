@@ -243,13 +243,13 @@ struct LayerWs {
 };
 
 // The chain of a stack of n_blocks; not ok: kernels of their own.  Times of those / with the chain, called one by one, rows 4 to 128:
-//   blocks     weights of a block, MB:  2..8         13..21       29..58       76..96       144..233     312..386 (to 48 rows, to 64, more)  477..661
+//   blocks     weights of a block, MB:  2..8         13..21       29..58       74..96       144..233     312..386 (to 48 rows, to 64, more)  477..661
 //   five                                1.11..1.21   1.10..1.16   1.06..1.13   1.00..1.06   0.99..1.09   0.95..1.00, 1.00..1.01, 1.00..1.03  1.00..1.09
 //   two, three                          1.05..1.18   1.05..1.13   1.01..1.12   0.99..1.04   0.98..1.08   0.96..1.00, -, 0.99..1.03           0.97..1.06
-//   one                                 0.97..1.11   0.98..1.10   0.95..1.05   0.91..1.01   0.97..1.06   0.94..0.97, 0.96..1.00, 0.96..1.02  0.94..1.14
+//   one                                 0.97..1.11   0.97..1.10   0.94..1.05   0.91..1.04   0.97..1.06   0.94..0.98, 0.96..1.00, 0.96..1.02  0.94..1.14
 // A stack's first and last chain have one and three of the four products, so one block is two launches that do not start ahead of the end of the kernel in front, and the
-// meetings of all CTAs, against seven that do: worth it where launches are what a block is, or beyond the sizes that the kernels of their own fill the SMs with.  At most 32 rows of
-// 21 to 58 MB are 0.95 to 1.01.  In a graph the smallest are 1.03..1.14, the others as they are here.
+// meetings of all CTAs, against seven that do: worth it where launches are what a block is, or beyond the sizes that the kernels of their own fill the SMs with.  (One block of at
+// most 32 rows: 0.97 to 1.06 to 13 MB, 0.94 to 1.03 from 21 to 58.)  In a graph the smallest are 1.03..1.14, the others as they are here.
 ChainShape block_chain(const dpara_shape *s, const dpara_layer_io *l, int n_blocks) {
   const long M = (long)s->batch * (s->n_boundaries * s->block + (s->spine_queries ? s->n_spine : 0));
   if (M > kChainRows) return ChainShape{};
